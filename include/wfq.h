@@ -110,7 +110,9 @@ typedef struct {
 
 /* Arithmetic of an apply / of the inner Krylov iterations. */
 enum {
-    WFQ_PREC_FP64 = 0,     /* FP64 operator, complex128 vectors */
+    WFQ_PREC_FP64 = 0,     /* FP64 operator, complex128 vectors (more than 4 columns on a stored
+                              FP64 D: 8 exact digits per operand on the tensor cores, at least
+                              as accurate as FP64 sums) */
     WFQ_PREC_MIXED = 1,    /* D.x from 3 bf16 products (hi.hi + hi.lo + lo.hi) with FP32
                               accumulation on the tensor cores, D from the stored bf16 planes
                               or generated from the coordinates -- or, without stored planes
@@ -120,12 +122,14 @@ enum {
                               residuals use the WFQ_PREC_DF product (on a geometry with no
                               stored D, D regenerated in FP64 once that product's rounding
                               holds a residual at a floor) */
-    WFQ_PREC_DF = 2,       /* wfq_apply and the refinement residuals: complex128 vectors, D.x
-                              with float-pair operands and double-float accumulation (~2^-48
-                              relative per product) on the FP32 pipes: D split from the stored
-                              FP64 D (up to 4 columns: the FP64 GEMV), or read from the stored
-                              FP32 pair planes or symmetric tiles, or regenerated from the
-                              coordinates in double-float (near pairs in FP64) */
+    WFQ_PREC_DF = 2,       /* wfq_apply and the refinement residuals: complex128 vectors, D.x to
+                              double-float accuracy (~2^-48 relative per product) or better:
+                              more than 4 columns on the stored FP64 D or FP32 pair planes by
+                              exact digit slices on the tensor cores (7 signed 8-bit digits of
+                              D and x, integer sums); up to 4 columns the FP64 GEMV of the
+                              stored FP64 D, else float pairs with double-float accumulation on
+                              the FP32 pipes (stored pairs or symmetric tiles, or regenerated
+                              from the coordinates in double-float, near pairs in FP64) */
     WFQ_PREC_FMM = 3       /* wfq_apply only: complex64 vectors, D.x by the fast multipole
                               method built with wfq_fmm_build (near field by Eq. 3, far field
                               1/r by Chebyshev interpolation), FP32 arithmetic */

@@ -172,7 +172,7 @@ static int galloc(wfq_geom *g, T **p, size_t count) {
 }
 
 static void free_geom(wfq_geom *g) {
-    void *ptrs[] = {g->xyz, g->atom64, g->atom32, g->atom32p, g->atomdf, g->eta, g->rowptr, g->col,
+    void *ptrs[] = {g->xyz, g->atom64, g->atom32, g->atom32p, g->atomdf, g->eta, g->dexp, g->rowptr, g->col,
                     g->val64, g->val32, g->D64, g->Dhi, g->Dlo, g->Dfh, g->Dfl,
                     g->Dsym, g->sym_items, g->sym_item_start, g->elem};
     for (void *p : ptrs)
@@ -402,6 +402,17 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
         adf[2 * i + 1] = make_float4(zh, zl, (float)(wfac / eta_h[i]), 0.0f);
     }
     std::vector<float> val32(val.begin(), val.end());
+    // Row exponents of the digit-slice products: D_ij = erf(r / s_ij) / r <= 2 / (sqrt(pi) s_ij)
+    // <= sqrt(2) eta_i, since s_ij >= w_i = sqrt(2 / pi) / eta_i (Eq. 3, Eq. 4).
+    std::vector<int> dexp;
+    if (store & (WFQ_STORE_FP64 | WFQ_STORE_F32X2)) {
+        dexp.resize(n);
+        g->digits_ok = true;
+        for (int64_t i = 0; i < n; ++i) {
+            dexp[i] = std::ilogb(1.4142135623730951 * eta_h[i]) + 1;
+            if (dexp[i] < -kDigitExpMax || dexp[i] > kDigitExpMax) g->digits_ok = false;
+        }
+    }
 
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);
     if ((rc = galloc(g, &g->atom64, n))) return bail(rc);
@@ -409,6 +420,7 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
     if ((rc = galloc(g, &g->atom32p, g->npad))) return bail(rc);
     if ((rc = galloc(g, &g->atomdf, 2 * n))) return bail(rc);
     if ((rc = galloc(g, &g->eta, n))) return bail(rc);
+    if (!dexp.empty() && (rc = galloc(g, &g->dexp, n))) return bail(rc);
     if ((rc = galloc(g, &g->rowptr, n + 1))) return bail(rc);
     if ((rc = galloc(g, &g->col, g->nnz))) return bail(rc);
     if ((rc = galloc(g, &g->val64, g->nnz))) return bail(rc);
@@ -462,6 +474,7 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
     }
     if ((rc = up(g->atomdf, adf.data(), sizeof(float4) * 2 * n))) return bail(rc);
     if ((rc = up(g->eta, eta_h.data(), sizeof(double) * n))) return bail(rc);
+    if ((rc = up(g->dexp, dexp.data(), sizeof(int) * dexp.size()))) return bail(rc);
     if ((rc = up(g->rowptr, rowptr.data(), sizeof(int64_t) * (n + 1)))) return bail(rc);
     if ((rc = up(g->col, col.data(), sizeof(int32_t) * g->nnz))) return bail(rc);
     if ((rc = up(g->val64, val.data(), sizeof(double) * g->nnz))) return bail(rc);
@@ -525,6 +538,7 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     };
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);
     if ((rc = galloc(g, &g->elem, n))) return bail(rc);
+    if ((rc = galloc(g, &g->dexp, n))) return bail(rc);
     if ((rc = galloc(g, &g->rowptr, n + 1))) return bail(rc);   // empty sparse term
     if ((rc = galloc(g, &g->D64, (size_t)n * n))) return bail(rc);
     if (store & WFQ_STORE_BF16X2) {
@@ -551,12 +565,23 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     if (e == cudaSuccess) e = cudaMemcpy(g->elem, el.data(), sizeof(elem64_t) * n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(g->rowptr, 0, sizeof(int64_t) * (n + 1));
     if (e == cudaSuccess) e = cudaMemset(close, 0, sizeof(int));
+    std::vector<int> dexp(n, kDexpNone);
+    if (e == cudaSuccess) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
     if ((rc = launch_build_bem(g, close, nullptr))) return done(rc);
     int close_h = 0;
     e = cudaMemcpy(&close_h, close, sizeof(int), cudaMemcpyDeviceToHost);   // synchronises the build
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM build: ") + cudaGetErrorString(e)));
     if (close_h) return done(fail(WFQ_EINVAL, "two surface elements closer than 1e-8 bohr"));
+    // row exponents: a row of zeros (possible on a flat surface) takes any scale
+    e = cudaMemcpy(dexp.data(), g->dexp, sizeof(int) * n, cudaMemcpyDeviceToHost);
+    g->digits_ok = true;
+    for (int64_t i = 0; i < n; ++i) {
+        if (dexp[i] == kDexpNone) dexp[i] = 0;
+        if (dexp[i] < -kDigitExpMax || dexp[i] > kDigitExpMax) g->digits_ok = false;
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM row exponents: ") + cudaGetErrorString(e)));
     done(WFQ_OK);
     *out = g;
     return WFQ_OK;

@@ -74,9 +74,14 @@ __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restri
 
 // ------------------------------------------------------------------ FP64 stored D: many columns
 
-// U[n x C] = D[n x n] X[n x C], row-major, 64 x 64 tiles, 4 x 4 outputs per thread.
+// U[n x C] = D[n x n] X[n x C], row-major, 64 x 64 tiles, 4 x 4 outputs per thread.  Runs only
+// when only_if is null or *only_if is set: it is what the digit-slice product (gemm_digits.cu)
+// leaves to plain FP64 -- columns with an Inf or NaN, whose signs and NaNs it reproduces, and
+// geometries whose entries lie outside the digits' exponent range.
 __global__ void __launch_bounds__(256) k_dgemm(int64_t n, int64_t C, const double *__restrict__ D,
-                                               const double *__restrict__ X, double *__restrict__ U) {
+                                               const double *__restrict__ X, double *__restrict__ U,
+                                               const int *__restrict__ only_if) {
+    if (only_if && *only_if == 0) return;
     __shared__ double As[16][65];
     __shared__ double Bs[16][64];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -186,68 +191,6 @@ __global__ void __launch_bounds__(256) k_dotf(int64_t n, int64_t C, const atom64
         for (int c = 0; c < 4; ++c) {
             int64_t gc = n0 + tx * 4 + c;
             if (gc < C) U[gi * C + gc] = acc[r][c];
-        }
-    }
-}
-
-// ------------------------------------------------------------------ double-float stored D
-
-// U[n x C] = D[n x n] X[n x C] with double-float products (df_mac): every FP64 operand
-// split into a float pair (hi = fp32(v), lo = fp32(v - hi): 48 significant bits).  This
-// runs on the FP32 pipes, which GB300 has far more of than FP64.  PL: D comes from the
-// stored FP32 pair planes (no FP64 arithmetic at all); else it is split from the FP64 D.
-
-template <bool PL>
-__global__ void __launch_bounds__(256) k_dgemm_df(int64_t n, int64_t C, const double *__restrict__ D,
-                                                  const float *__restrict__ Fh, const float *__restrict__ Fl,
-                                                  int64_t ldf, const double *__restrict__ X, double *__restrict__ U) {
-    __shared__ float Ah[16][64], Al[16][64], Bh[16][64], Bl[16][64];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
-    float sh[4][4] = {}, sl[4][4] = {};
-    for (int64_t k0 = 0; k0 < n; k0 += 16) {
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            const int e = tid + l * 256;
-            const int r = e >> 4, kk = e & 15;
-            const int64_t gi = m0 + r, gk = k0 + kk;
-            if (PL) {
-                const bool in = gi < n && gk < n;
-                Ah[kk][r] = in ? Fh[gi * ldf + gk] : 0.f;
-                Al[kk][r] = in ? Fl[gi * ldf + gk] : 0.f;
-            } else {
-                df_split((gi < n && gk < n) ? D[gi * n + gk] : 0.0, Ah[kk][r], Al[kk][r]);
-            }
-            const int kb = e >> 6, cb = e & 63;
-            const int64_t bk = k0 + kb, bc = n0 + cb;
-            df_split((bk < n && bc < C) ? X[bk * C + bc] : 0.0, Bh[kb][cb], Bl[kb][cb]);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < 16; ++kk) {
-            float ah[4], al[4], bh[4], bl[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                ah[t] = Ah[kk][ty * 4 + t];
-                al[t] = Al[kk][ty * 4 + t];
-                bh[t] = Bh[kk][tx * 4 + t];
-                bl[t] = Bl[kk][tx * 4 + t];
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) df_mac(ah[r], al[r], bh[c], bl[c], sh[r][c], sl[r][c]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int64_t gi = m0 + ty * 4 + r;
-        if (gi >= n) continue;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int64_t gc = n0 + tx * 4 + c;
-            if (gc < C) U[gi * C + gc] = (double)sh[r][c] + (double)sl[r][c];
         }
     }
 }
@@ -401,7 +344,8 @@ int d_gemv_df_mf(const wfq_geom *g, int C, const float *xh, const float *xl, dou
     return WFQ_OK;
 }
 
-// As k_dgemm_df with the D tile generated per use (matrix-free); TN columns per thread.
+// U[n x C] = D[n x n] X[n x C] with double-float products (df_mac) on the FP32 pipes, the D
+// tile generated per use (matrix-free); TN columns per thread.
 template <int TN>
 __global__ void __launch_bounds__(256) k_dotf_df(int64_t n, int64_t C, const float4 *__restrict__ adf,
                                                  const atom64_t *__restrict__ a64, const double *__restrict__ eta,
@@ -489,18 +433,13 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     }
     const int64_t n = g->n, C = 2 * cc;
     if (C <= 8 && g->D64) return d_apply_fp64(g, cc, X, U, s);   // few columns: memory bound, FP64 GEMV
+    if (!g->digits_ok) return g->Dfh ? d_apply_pairs_df(g, cc, X, U, s) : d_apply_fp64(g, cc, X, U, s);
+    // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
+    // pair planes: 8.4 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-    dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
-    if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
-    const double *x = reinterpret_cast<const double *>(X);
-    double *u = reinterpret_cast<double *>(U);
-    if (g->Dfh)
-        k_dgemm_df<true><<<grid, 256, 0, s>>>(n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u);
-    else
-        k_dgemm_df<false><<<grid, 256, 0, s>>>(n, C, g->D64, nullptr, nullptr, 0, x, u);
-    note_launch();
-    WFQ_CUDA(cudaGetLastError());
-    return WFQ_OK;
+    DevBuf<int> bad;
+    WFQ_TRY(bad.alloc(g->ctx, 1, s));
+    return digits_product(g, 7, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), bad.ptr, s);
 }
 
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s) {
@@ -523,8 +462,15 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     } else {
         dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
         if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "FP64 apply: too many rows");
-        if (g->D64) {
-            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u);
+        if (g->D64 && g->digits_ok) {
+            // eight exact digits on the tensor cores; columns that are not finite in FP64.
+            // 10k-atom sphere, 32 real columns: 0.41 ms against 20.5 ms for the FP64 kernel.
+            DevBuf<int> bad;
+            WFQ_TRY(bad.alloc(g->ctx, 1, s));
+            WFQ_TRY(digits_product(g, 8, C, x, u, bad.ptr, s));
+            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, bad.ptr);
+        } else if (g->D64) {
+            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, nullptr);
         } else {
             WFQ_TRY(require_wfq(g));
             k_dotf<<<grid, 256, 0, s>>>(n, C, g->atom64, g->eta, x, u);

@@ -64,6 +64,8 @@ constexpr int64_t kSymTile = 64;
 struct SymItem {
     int I, J0, J1, pad;
 };
+// Row exponents the digit-slice products take: their power-of-two scales stay normal floats.
+constexpr int kDigitExpMax = 60;
 // index of tile (I, J), I <= J, in the row-ordered upper triangle of T x T tiles
 __host__ __device__ inline int64_t sym_tile(int64_t I, int64_t J, int64_t T) { return I * T - I * (I - 1) / 2 + (J - I); }
 
@@ -167,6 +169,8 @@ struct wfq_geom {
                                 // generator reads them as packed FP32x2 operands
     float4 *atomdf = nullptr;   // 2 per atom: (xh, xl, yh, yl), (zh, zl, width, 0) float pairs
     double *eta = nullptr;      // n
+    int *dexp = nullptr;        // n, stored FP64 D or FP32 planes only: |D_ij| < 2^dexp[i]
+    bool digits_ok = false;     // every dexp within +-kDigitExpMax (the digit-slice products)
     wfq::elem64_t *elem = nullptr;   // BEM geometries: n element records
 
     // Kbar CSR (device)
@@ -244,7 +248,9 @@ int build_kbar_csr(int64_t n, const double *xyz, const wfq_params &p, std::vecto
 
 int launch_build_d(const wfq_geom *g, cudaStream_t s);
 // BEM geometries: the operator's entries into the requested storages; *close is set
-// non-zero (device int) when two elements lie closer than 1e-8 bohr.
+// non-zero (device int) when two elements lie closer than 1e-8 bohr.  Also g->dexp, each
+// row's largest exponent (kDexpNone for a row of zeros).
+constexpr int kDexpNone = -2000;
 int launch_build_bem(const wfq_geom *g, int *close, cudaStream_t s);
 int launch_rhs(const wfq_geom *g, int ndir, const double *dirs_dev, double E0, double *R,
                cudaStream_t s);
@@ -262,10 +268,16 @@ int launch_polarizability(const wfq_geom *g, int64_t ncols, const double2 *q, do
 // U = D X in FP64 (stored FP64 D if present, else recomputed from the coordinates).
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
 
-// U = D X with double-float products (FP64 operands split into float pairs, about 48
-// significant bits) when the FP64 D is stored and there are more than 4 columns; else
-// the FP64 kernels.  Used for the refinement residual of mixed-precision solves.
+// U = D X to double-float accuracy (about 48 significant bits) or better: exact digit slices
+// for more than 4 complex columns on stored planes, else double-float or FP64 kernels.  Used
+// for the refinement residual of mixed-precision solves.
 int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
+
+// U = D X for C real columns (row-major) by S = 7 or 8 exact digit slices on the tensor cores
+// (gemm_digits.cu): S = 8 from the FP64 D, S = 7 from the FP32 pair planes, else the FP64 D.
+// Needs g->digits_ok.  bad: device int, set to 1 when a column of X has an Inf or NaN (its
+// results are NaN), else 0.
+int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s);
 
 // U = D X for at most 4 complex columns with double-float products (~2^-48 per product)
 // from the stored float pairs (full planes or symmetric tiles) -- the FP64-grade product of

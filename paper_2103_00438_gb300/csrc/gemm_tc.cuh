@@ -139,7 +139,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 
 // ------------------------------------------------------------------ kernel
 
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+static __global__ void __launch_bounds__(NUM_THREADS, 1)
     k_gemm3_tc(const __grid_constant__ CUtensorMap tm_dhi, const __grid_constant__ CUtensorMap tm_dlo,
                const __grid_constant__ CUtensorMap tm_xhi, const __grid_constant__ CUtensorMap tm_xlo,
                const Params p) {

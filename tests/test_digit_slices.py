@@ -1,0 +1,71 @@
+"""The digit arithmetic of csrc/gemm_digits.cu on the host: an entry as a fixed-point integer, its
+signed 8-bit digits, and their recombination -- exact, in range and within half a unit."""
+import math
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+
+def fixed_point(v, E, S):
+    """v 2^(8S - 2 - E) as an integer: truncated for S = 8, rounded half up in magnitude for S = 7."""
+    q = abs(Fraction(v)) * Fraction(2) ** (8 * S - 2 - E)
+    f = int(q) if S == 8 else (int(2 * q) + 1) // 2
+    return -f if v < 0 else f
+
+
+def biased_pair(h, l, E):
+    """biased<7> of a float pair in units of 2^(E - 53), in float32 steps."""
+    f = np.float32
+    v = f(h * f(2.0 ** (22 - E)))
+    t = f(v + f(12582912.0))
+    r = f(v - f(t - f(12582912.0)))
+    it = int(np.array(t).view(np.int32)) - (0x4b400000 - 0x01010101)
+    ib = int(np.rint(f(r * f(2147483648.0)))) + int(np.rint(f(l * f(2.0 ** (53 - E))))) + 0x00808080
+    assert -2 ** 31 <= ib < 2 ** 31
+    return (it * 2147483648 + ib) % 2 ** 64
+
+
+def digits(biased, S):
+    return [((biased >> (8 * (S - 1 - a))) & 0xff) - 128 for a in range(S)]
+
+
+BIAS = {8: 0x8080808080808080, 7: 0x0080808080808080}
+
+
+@pytest.mark.parametrize("S", [7, 8])
+def test_fp64_entries_recombine(S):
+    rng = np.random.default_rng(1)
+    vals = [0.0, 1.0, -1.0, np.nextafter(2.0, 0), -np.nextafter(2.0, 0), 2.0 ** -60, 5e-324, 1e-310]
+    vals += list(rng.uniform(-2, 2, 300)) + list(rng.standard_normal(300) * 2.0 ** rng.uniform(-40, 0, 300))
+    for v in vals:
+        if abs(v) >= 2:
+            continue
+        f = fixed_point(v, 1, S)
+        d = digits((f + BIAS[S]) % 2 ** 64, S)
+        assert all(-128 <= x <= 127 for x in d)
+        assert sum(x * 256 ** (S - 1 - a) for a, x in enumerate(d)) == f
+        assert abs(Fraction(f) * Fraction(2) ** (1 - (8 * S - 2)) - Fraction(v)) <= Fraction(2) ** (1 - (8 * S - 2))
+
+
+def test_float_pairs_recombine():
+    rng = np.random.default_rng(2)
+    vals = list(rng.uniform(-1, 1, 2000) * 2.0 ** rng.uniform(-30, 0, 2000))
+    vals += [1.0 - 2.0 ** -53, -(1.0 - 2.0 ** -53), 0.5, 0.25 + 2.0 ** -26, 2.0 ** -23 * 1.5, 0.0]
+    for v in vals:
+        h = np.float32(v)
+        l = np.float32(v - float(h))
+        d = digits(biased_pair(h, l, 1), 7)
+        got = Fraction(sum(x * 256 ** (6 - a) for a, x in enumerate(d))) * Fraction(2) ** (1 - 53)
+        want = Fraction(float(h)) + Fraction(float(l))
+        assert abs(got - want) <= Fraction(2) ** (1 - 53)   # two roundings of half a unit
+
+
+def test_accumulators_stay_exact():
+    # 128 atoms, up to 8 digit products of at most 2^14 per weight, and the 32-bit combinations
+    assert 128 * 8 * 128 * 128 <= 2 ** 24
+    s = [(w + 1) * 128 * 2 ** 14 for w in range(8)]
+    assert s[0] * 256 + s[1] < 2 ** 31 and s[2] * 256 + s[3] < 2 ** 31
+    # S = 7: weights 4 to 6 as one float in units of 2^-7 of weight 4 fits 31 bits
+    assert s[4] * 128 + s[5] // 2 + s[6] // 512 < 2 ** 31
+    assert math.log2(s[0]) + 24 + math.log2(2 ** 21 / 128) < 63   # sums of 2^21 atoms
