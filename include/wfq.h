@@ -127,8 +127,10 @@ enum {
                               more than 4 columns on the stored FP64 D or FP32 pair planes by
                               exact digit slices on the tensor cores (7 signed 8-bit digits of
                               D and x, integer sums); up to 4 columns the FP64 GEMV of the
-                              stored FP64 D, else float pairs with double-float accumulation on
-                              the FP32 pipes (stored pairs or symmetric tiles, or regenerated
+                              stored FP64 D, else float pairs: digit slices of the upper
+                              triangle (symmetric tiles, or 3072 atoms and more on the planes;
+                              row bounds sqrt(2) eta_i within a factor of 8), or double-float
+                              accumulation on the FP32 pipes (smaller planes, or D regenerated
                               from the coordinates in double-float, near pairs in FP64) */
     WFQ_PREC_FMM = 3       /* wfq_apply only: complex64 vectors, D.x by the fast multipole
                               method built with wfq_fmm_build (near field by Eq. 3, far field
@@ -366,8 +368,8 @@ int wfq_solve_gmres(wfq_geom *g, int64_t nfreq, const double *omega, int ndir,
  *   prec: precision of the block GMRES(50) that continues, from their iterate, the
  *         columns whose FP64 true residual is still above rel_tol at the end (basis cap
  *         reached, or rounding of the shared process): WFQ_PREC_MIXED or WFQ_PREC_FP64.
- * D comes from the FP32 pair planes (WFQ_STORE_F32X2, fastest), the symmetric tiles
- * (WFQ_STORE_F32X2_SYM), the FP64 D, or -- with none of them stored -- is regenerated from
+ * D comes from the FP32 pair planes (WFQ_STORE_F32X2) or the symmetric tiles
+ * (WFQ_STORE_F32X2_SYM; the two take the same time from 3072 atoms on), the FP64 D, or -- with none of them stored -- is regenerated from
  * the coordinates in double-float for every product (near pairs in FP64; matrix-free).
  * stats: iters = Arnoldi steps the column used plus any continuation's; restarts = 1 +
  * the continuation's when a column was continued.  Other arguments and results as

@@ -1,5 +1,6 @@
 // C ABI of libwfq (include/wfq.h): argument checking, handle management, host/device
 // staging, dispatch to the kernels.
+#include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -179,6 +180,12 @@ static void free_geom(wfq_geom *g) {
         if (p) cudaFree(p);
     fmm_free(g->fmm);
     delete g;
+}
+
+static void set_exponent_range(wfq_geom *g, const std::vector<int> &dexp) {
+    g->dexp_min = *std::min_element(dexp.begin(), dexp.end());
+    g->dexp_max = *std::max_element(dexp.begin(), dexp.end());
+    g->digits_ok = g->dexp_min >= -kDigitExpMax && g->dexp_max <= kDigitExpMax;
 }
 
 static bool finite_all(const double *a, int64_t n) {
@@ -405,13 +412,10 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
     // Row exponents of the digit-slice products: D_ij = erf(r / s_ij) / r <= 2 / (sqrt(pi) s_ij)
     // <= sqrt(2) eta_i, since s_ij >= w_i = sqrt(2 / pi) / eta_i (Eq. 3, Eq. 4).
     std::vector<int> dexp;
-    if (store & (WFQ_STORE_FP64 | WFQ_STORE_F32X2)) {
+    if (store & (WFQ_STORE_FP64 | WFQ_STORE_F32X2 | WFQ_STORE_F32X2_SYM)) {
         dexp.resize(n);
-        g->digits_ok = true;
-        for (int64_t i = 0; i < n; ++i) {
-            dexp[i] = std::ilogb(1.4142135623730951 * eta_h[i]) + 1;
-            if (dexp[i] < -kDigitExpMax || dexp[i] > kDigitExpMax) g->digits_ok = false;
-        }
+        for (int64_t i = 0; i < n; ++i) dexp[i] = std::ilogb(1.4142135623730951 * eta_h[i]) + 1;
+        set_exponent_range(g, dexp);
     }
 
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);
@@ -575,11 +579,9 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     if (close_h) return done(fail(WFQ_EINVAL, "two surface elements closer than 1e-8 bohr"));
     // row exponents: a row of zeros (possible on a flat surface) takes any scale
     e = cudaMemcpy(dexp.data(), g->dexp, sizeof(int) * n, cudaMemcpyDeviceToHost);
-    g->digits_ok = true;
-    for (int64_t i = 0; i < n; ++i) {
+    for (int64_t i = 0; i < n; ++i)
         if (dexp[i] == kDexpNone) dexp[i] = 0;
-        if (dexp[i] < -kDigitExpMax || dexp[i] > kDigitExpMax) g->digits_ok = false;
-    }
+    set_exponent_range(g, dexp);
     if (e == cudaSuccess) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM row exponents: ") + cudaGetErrorString(e)));
     done(WFQ_OK);

@@ -435,7 +435,7 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     if (C <= 8 && g->D64) return d_apply_fp64(g, cc, X, U, s);   // few columns: memory bound, FP64 GEMV
     if (!g->digits_ok) return g->Dfh ? d_apply_pairs_df(g, cc, X, U, s) : d_apply_fp64(g, cc, X, U, s);
     // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
-    // pair planes: 8.4 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.
+    // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     DevBuf<int> bad;
     WFQ_TRY(bad.alloc(g->ctx, 1, s));
@@ -464,7 +464,7 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
         if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "FP64 apply: too many rows");
         if (g->D64 && g->digits_ok) {
             // eight exact digits on the tensor cores; columns that are not finite in FP64.
-            // 10k-atom sphere, 32 real columns: 0.41 ms against 20.5 ms for the FP64 kernel.
+            // 10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
             DevBuf<int> bad;
             WFQ_TRY(bad.alloc(g->ctx, 1, s));
             WFQ_TRY(digits_product(g, 8, C, x, u, bad.ptr, s));

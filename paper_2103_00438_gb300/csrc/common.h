@@ -169,7 +169,8 @@ struct wfq_geom {
                                 // generator reads them as packed FP32x2 operands
     float4 *atomdf = nullptr;   // 2 per atom: (xh, xl, yh, yl), (zh, zl, width, 0) float pairs
     double *eta = nullptr;      // n
-    int *dexp = nullptr;        // n, stored FP64 D or FP32 planes only: |D_ij| < 2^dexp[i]
+    int *dexp = nullptr;        // n, stored FP64 D, FP32 planes or tiles: |D_ij| < 2^dexp[i]
+    int dexp_min = 0, dexp_max = 0;
     bool digits_ok = false;     // every dexp within +-kDigitExpMax (the digit-slice products)
     wfq::elem64_t *elem = nullptr;   // BEM geometries: n element records
 
@@ -278,6 +279,22 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
 // Needs g->digits_ok.  bad: device int, set to 1 when a column of X has an Inf or NaN (its
 // results are NaN), else 0.
 int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s);
+
+// U = D V for C <= 4 real vectors by exact digit slices from the stored float pairs (symmetric
+// tiles or full planes; gemv_digits.cu).  Buffers of one stream's products: digit planes of the
+// vectors (gemv_digits_plane_elems, zeroed once), exponents and largest magnitudes (C each) and
+// the integer sums (2 n C, zeroed once; each product leaves them zeroed).
+struct GemvDigits {
+    uint16_t *planes;
+    int *xexp;
+    unsigned long long *vmax, *acc;
+};
+bool gemv_digits_usable(const wfq_geom *g);
+size_t gemv_digits_plane_elems(const wfq_geom *g);
+// digits of the vectors X (element i of vector c at i si + c sc)
+int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s);
+// U (same indexing) = D times the vectors whose digits are in w
+int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s);
 
 // U = D X for at most 4 complex columns with double-float products (~2^-48 per product)
 // from the stored float pairs (full planes or symmetric tiles) -- the FP64-grade product of

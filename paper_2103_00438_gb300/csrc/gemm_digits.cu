@@ -17,8 +17,8 @@
 //
 // Why: GB300 has about 2 FP64 FMAs per clock per SM (0.5e12/s) and the double-float product
 // costs 12 FP32 operations; the tensor cores do 36 (S = 8) or 28 (S = 7) fp16 digit products
-// in less time than either: 20000 atoms x 384 real columns from the pair planes 8.4 ms (69.9 ms
-// for double-float FMAs), a 10k-atom sphere x 32 real columns in FP64 0.41 ms (20.5 ms).
+// in less time than either: 20000 atoms x 384 real columns from the pair planes 7.3 ms (69.9 ms
+// for double-float FMAs), a 10k-atom sphere x 32 real columns in FP64 0.38 ms (20.5 ms).
 //
 // Structure (one CTA per SM, 28 warps, stream-K over (column group, row tile, 128-atom chunk)):
 //   warps 0-15  epilogue: 8 warps for each of two TMEM slots (S accumulators of 128 x 32), read
@@ -37,9 +37,9 @@
 // back while the other's products run.  A group of one half alternates the slots by chunk.
 // Every barrier wait is bounded, as in gemm_tc.cuh.
 //
-// Bound: the conversion and read-back arithmetic about as much as the MMAs (cnt20k, S = 7: 8.1 ms
-// in this kernel; without the conversions' loads 7.7, with one MMA in seven 6.9, with one
-// read-back column in 16 7.2; the MMAs alone 5.8 = 0.8 of the measured bf16 rate).  Measured
+// Bound: the conversion and read-back arithmetic about as much as the MMAs (cnt20k, S = 7: 7.0 ms
+// in this kernel, 8.1 before the MMAs were issued from a warp-uniform loop; then 7.7 without the
+// conversions' loads, 6.9 with one MMA in seven, 7.2 with one read-back column in 16).  Measured
 // slower: a third D stage, L2 prefetch of the next chunk (0.5 ms), 16-atom D stages (more
 // fences), two converter groups on alternate stages with three register sets (instruction-cache
 // misses), skipping the leading digit plane where it is all zeros.
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int64_t u_begin = dp.units * (int64_t)blockIdx.x / gridDim.x;
     const int64_t u_end = dp.units * ((int64_t)blockIdx.x + 1) / gridDim.x;
 
@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
                 for (uint32_t j = it > DG_STAGES ? it - DG_STAGES : 0; j < it; ++j)
                     tc::mbar_wait(tc::smem_u32(b_full + (j & 1u)), (j >> 1) & 1u, p, 1, &no_abort);
             }
-        } else if (warp == DG_TMA_WARP + 1 && lane == 0) {
+        } else if (warp == DG_TMA_WARP + 1) {
+            const bool el = tc::elect_one();
             // ---------------------------------------------------------- MMA issuer
             uint32_t it = 0, uses = 0, abuf = 0, apar = 0;   // uses: phase of each slot's barriers, a bit each
             bool aborted = false;
@@ -465,26 +466,26 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
                                 // fp16 operands, FP32 accumulator, N = 32 (S - a)
                                 const uint32_t idesc =
                                     (1u << 4) | ((uint32_t)((S - a) * DG_HALF >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-                                tc::umma_bf16(d + (uint32_t)(a * DG_HALF),
+                                if (el) tc::umma_bf16(d + (uint32_t)(a * DG_HALF),
                                               da + (uint64_t)(uint32_t)(a * (DG_A_BYTES >> 4) + ks * 2), db + (uint64_t)(ks * 2),
                                               idesc, (a == 0 && st == 0 && ks == 0) ? 0u : 1u);
                             }
                         }
                         if (st == DG_CHUNK / BK - 1) {
-                            tc::umma_commit(tc::smem_u32(acc_full + slot));
+                            if (el) tc::umma_commit(tc::smem_u32(acc_full + slot));
                             uses ^= 1u << slot;
                         }
                     }
                     if (aborted) break;
-                    tc::umma_commit(tc::smem_u32(a_empty + abuf));
-                    tc::umma_commit(tc::smem_u32(b_empty + s));
+                    if (el) tc::umma_commit(tc::smem_u32(a_empty + abuf));
+                    if (el) tc::umma_commit(tc::smem_u32(b_empty + s));
                     if (++abuf == NA) {
                         abuf = 0;
                         apar ^= 1u;
                     }
                 }
             }
-            tc::umma_commit(tc::smem_u32(drain));
+            if (el) tc::umma_commit(tc::smem_u32(drain));
             volatile int no_abort = 0;
             tc::mbar_wait(tc::smem_u32(drain), 0u, p, 5, &no_abort);
         }

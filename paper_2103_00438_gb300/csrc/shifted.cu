@@ -12,7 +12,8 @@
 // column solves by its own complex Givens QR of the shared real Hbar_j.  One D product of
 // the ndir real Arnoldi vectors per iteration therefore serves all nfreq x ndir columns.
 //
-// Precision: the Arnoldi vectors, Hbar and the rotations are FP64; D is applied with
+// Precision: the Arnoldi vectors, Hbar and the rotations are FP64; D is applied by exact digit
+// slices on the tensor cores (gemv_digits.cu, large structures with stored float pairs) or with
 // double-float products (~2^-48 relative) on the FP32 pipes, from the stored FP32 pair
 // planes (or split from the FP64 D).  Every column's true residual R - (A - zI) q is
 // measured at the end in FP64 from q = sum_k v_k y_k and D q = sum_k (D v_k) y_k, the D
@@ -26,6 +27,7 @@
 
 #include "common.h"
 #include "dfloat.cuh"
+#include "vec_digits.cuh"
 
 namespace wfq {
 namespace {
@@ -198,7 +200,8 @@ __global__ void __launch_bounds__(GV_WARPS * 32, MINB) k_dgemv_df(int64_t n, int
     }
 }
 
-// ---- the same product from the symmetric tiled storage (upper-triangle 64 x 64 tiles):
+// ---- the same product from the symmetric tiled storage (upper-triangle 64 x 64 tiles), for
+// hardnesses too far apart for the digit slices (gemv_digits_usable):
 // every stored tile (I, J), I < J, serves both U_I += D_IJ x_J and U_J += D_IJ^T x_I, so D is
 // read once for the triangle instead of the full matrix -- half the memory; the time is
 // that of the full-plane product (both are bound by issue of the double-float arithmetic:
@@ -471,15 +474,17 @@ constexpr int RU_ELEMS = 32 * RU_EPL;
 // sums are added in a fixed order.  Fused with the next step's reductions of the updated w:
 // NEXT_DOTS -- the partial dots of w with V_0 .. V_{nv-1} for the second Gram-Schmidt pass,
 // partial[(block * nv + k) * C + d]; NEXT_NORM -- the partial squared norm,
-// partial[block * C + d].  Fixed orders throughout.
-enum { NEXT_DOTS = 1, NEXT_NORM = 2 };
+// partial[block * C + d]; NEXT_NORM_MAX -- also the largest |w| of the block, pmax[block * C + d].
+// Fixed orders throughout.
+enum { NEXT_DOTS = 1, NEXT_NORM = 2, NEXT_NORM_MAX = 3 };
 template <int NEXT>
 __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int C, int nv, const double *__restrict__ V,
                                                                  int64_t vstride, const double *__restrict__ coef,
-                                                                 double *__restrict__ w, double *__restrict__ partial) {
+                                                                 double *__restrict__ w, double *__restrict__ partial,
+                                                                 double *__restrict__ pmax) {
     __shared__ double part[RU_SLICES][RU_ELEMS];
     __shared__ double wv[RU_ELEMS];
-    __shared__ double sqw[RU_ELEMS / 32];
+    __shared__ double sqw[RU_ELEMS / 32], mxw[RU_ELEMS / 32];
     const int el = threadIdx.x & 31, sl = threadIdx.x >> 5;
     const int d = blockIdx.y;
     const int64_t i0 = (int64_t)blockIdx.x * RU_ELEMS;
@@ -521,20 +526,38 @@ __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int 
             *we = wn;
         }
         wv[e] = wn;
-        if (NEXT == NEXT_NORM) {
+        if constexpr (NEXT == NEXT_NORM || NEXT == NEXT_NORM_MAX) {
             double sq = wn * wn;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
             if (el == 0) sqw[sl] = sq;
+            if constexpr (NEXT == NEXT_NORM_MAX) {   // magnitudes as integers: order of the bits, NaN and Inf largest
+                unsigned long long mx = (unsigned long long)__double_as_longlong(wn) & 0x7fffffffffffffffull;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+                    mx = o > mx ? o : mx;
+                }
+                if (el == 0) mxw[sl] = __longlong_as_double((long long)mx);
+            }
         }
     }
     __syncthreads();
-    if constexpr (NEXT == NEXT_NORM) {
+    if constexpr (NEXT == NEXT_NORM || NEXT == NEXT_NORM_MAX) {
         if (threadIdx.x == 0) {
             double sq = 0.0;
 #pragma unroll
             for (int q = 0; q < RU_ELEMS / 32; ++q) sq += sqw[q];
             partial[(int64_t)blockIdx.x * C + d] = sq;
+            if constexpr (NEXT == NEXT_NORM_MAX) {
+                unsigned long long mx = 0;
+#pragma unroll
+                for (int q = 0; q < RU_ELEMS / 32; ++q) {
+                    const unsigned long long o = (unsigned long long)__double_as_longlong(mxw[q]);
+                    mx = o > mx ? o : mx;
+                }
+                pmax[(int64_t)blockIdx.x * C + d] = __longlong_as_double((long long)mx);
+            }
         }
         return;
     }
@@ -564,23 +587,53 @@ __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int 
     }
 }
 
+// Where the next D product finds v: float-pair splits (xh, xl), or the digit planes of the
+// digit-slice GEMV (groups of up to 4 directions, gs elements apart) with the exponents xexp.
+struct NextVec {
+    float *xh, *xl;
+    __half *planes;
+    int *xexp;
+    int64_t gs, npad;
+    const double *pmax;   // largest |w| per block of k_rupdate_next
+};
+
 // The norms of the C directions from their nrb partial squares (every block reduces them
 // in the same fixed order: lane-strided sums, a butterfly), H(j + 1, j) = hn[d] = norm
-// (block 0), then v = w / norm with v's float-pair split, as k_rscale.  Four elements
-// per thread.
+// (block 0), then v = w / norm with v's float-pair split, as k_rscale, or its digits (division
+// is monotonic: max |v| is max |w| / norm as computed).  Four elements per thread.
+template <bool DIG>
 __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restrict__ partial, int m, int j,
                               double *__restrict__ H, double *__restrict__ hn, const double *__restrict__ w,
-                              double *__restrict__ v, float *__restrict__ xh, float *__restrict__ xl) {
-    extern __shared__ double nrm[];   // [C]
+                              double *__restrict__ v, NextVec nx) {
+    extern __shared__ double nrm[];   // [C], then C exponents
+    int *vex = reinterpret_cast<int *>(nrm + C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int d = warp; d < C; d += blockDim.x / 32) {
         double sv = 0.0;
-        for (int rb = lane; rb < nrb; rb += 32) sv += partial[(int64_t)rb * C + d];
+        unsigned long long mx = 0;
+        for (int rb = lane; rb < nrb; rb += 32) {
+            sv += partial[(int64_t)rb * C + d];
+            if constexpr (DIG) {
+                const unsigned long long o = (unsigned long long)__double_as_longlong(nx.pmax[(int64_t)rb * C + d]);
+                mx = o > mx ? o : mx;
+            }
+        }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) sv += __shfl_xor_sync(0xffffffffu, sv, off);
+        for (int off = 16; off > 0; off >>= 1) {
+            sv += __shfl_xor_sync(0xffffffffu, sv, off);
+            if constexpr (DIG) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
+                mx = o > mx ? o : mx;
+            }
+        }
         if (lane == 0) {
             const double nr = sqrt(sv);
             nrm[d] = nr;
+            if constexpr (DIG) {
+                const double vm = nr > 0.0 ? __longlong_as_double((long long)mx) / nr : 0.0;
+                vex[d] = vec_exp((unsigned long long)__double_as_longlong(vm) & 0x7fffffffffffffffull);
+                if (blockIdx.x == 0) nx.xexp[d] = vex[d];
+            }
             if (blockIdx.x == 0) {
                 H[((int64_t)d * m + j) * (m + 1) + j + 1] = nr;
                 hn[d] = nr;
@@ -591,15 +644,21 @@ __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restric
     for (int q = 0; q < 4; ++q) {
         const int64_t e = ((int64_t)blockIdx.x * 4 + q) * blockDim.x + threadIdx.x;
         if (e >= n * C) break;
-        const double h = nrm[e / n];
+        const int d = (int)(e / n);
+        const double h = nrm[d];
         const double t = h > 0.0 ? w[e] / h : 0.0;
         v[e] = t;
-        df_split(t, xh[e], xl[e]);
+        if constexpr (DIG) {
+            const int cg = min(4, C - (d & ~3));
+            put_vec_digits(t, vex[d], nx.planes + (d >> 2) * nx.gs + (d & 3) * nx.npad + (e - d * n), cg * nx.npad);
+        } else {
+            df_split(t, nx.xh[e], nx.xl[e]);
+        }
     }
 }
 
 // v[d][i] = w[d][i] / hn[d] (0 when hn = 0: the direction's Krylov space is exhausted),
-// and v's float-pair split (xh, xl) for the next D product
+// and, unless xh is null, v's float-pair split (xh, xl) for the next D product
 __global__ void k_rscale(int64_t n, int C, const double *__restrict__ hn, const double *__restrict__ w,
                          double *__restrict__ v, float *__restrict__ xh, float *__restrict__ xl) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -607,7 +666,7 @@ __global__ void k_rscale(int64_t n, int C, const double *__restrict__ hn, const 
     const double h = hn[e / n];
     const double t = h > 0.0 ? w[e] / h : 0.0;
     v[e] = t;
-    df_split(t, xh[e], xl[e]);
+    if (xh) df_split(t, xh[e], xl[e]);
 }
 
 // ------------------------------------------------------------------ per-shift least squares
@@ -783,6 +842,15 @@ __global__ void k_shift_z(int64_t nc, const double *__restrict__ col_omega, Shif
 
 // ------------------------------------------------------------------ host
 
+// Digit slices (gemv_digits.cu) or double-float multiply-adds for the D products from float
+// pairs.  us per product of 3 vectors, digits with their finish against double-float:
+//   full planes (the upper triangle read)   n = 1985: 21 / 16   3043: 27.5 / 26.7   5017: 45 / 62
+//                                           8007: 80 / 134      20000: 390 / 675
+//   symmetric tiles                         n = 321: 15 / 26    1985: 21 / 58       8007: 84 / 168
+bool use_gemv_digits(const wfq_geom *g) {
+    return gemv_digits_usable(g) && (!g->Dfh || g->n >= 3072);
+}
+
 struct Arnoldi {
     wfq_geom *g;
     cudaStream_t s;
@@ -795,6 +863,11 @@ struct Arnoldi {
     DevBuf<double> partial_f;   // partial reductions of the fused kernels (update + dots / norm)
     int nbru = 0;
     DevBuf<float2> rowpart, colpart;   // symmetric product partial sums
+    bool digits = false;               // D products by digit slices (gemv_digits.cu)
+    DevBuf<uint16_t> planes;           // vector digits, a set for every 4 directions
+    DevBuf<int> xexp;
+    DevBuf<unsigned long long> vmax, acc;
+    DevBuf<double> pmax;
 
     int init(wfq_geom *geom, int ndir, int m, cudaStream_t stream) {
         g = geom;
@@ -803,14 +876,26 @@ struct Arnoldi {
         C = ndir;
         rpb = std::max<int64_t>(1024, round_up((n + 2 * g->ctx->num_sms - 1) / (2 * g->ctx->num_sms), 256));
         nrb = (int)((n + rpb - 1) / rpb);
-        WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
-        WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
+        digits = use_gemv_digits(g);
+        if (digits) {
+            const size_t np = gemv_digits_plane_elems(g) * ((C + 3) / 4);
+            WFQ_TRY(planes.alloc(g->ctx, np, s));
+            WFQ_TRY(xexp.alloc(g->ctx, C, s));
+            WFQ_TRY(vmax.alloc(g->ctx, C, s));
+            WFQ_TRY(acc.alloc(g->ctx, (size_t)8 * n, s));
+            WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
+            WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 8 * n, s));
+        } else {
+            WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
+            WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
+        }
         WFQ_TRY(U.alloc(g->ctx, (size_t)n * C, s));
         WFQ_TRY(partial.alloc(g->ctx, (size_t)nrb * (m + 1) * C, s));
         nbru = (int)((n + RU_ELEMS - 1) / RU_ELEMS);
         WFQ_TRY(partial_f.alloc(g->ctx, (size_t)nbru * (m + 1) * C, s));
         WFQ_TRY(coef.alloc(g->ctx, (size_t)(m + 1) * C, s));
-        if (g->Dsym && !g->Dfh) {
+        if (digits) WFQ_TRY(pmax.alloc(g->ctx, (size_t)nbru * C, s));
+        if (g->Dsym && !g->Dfh && !digits) {
             const int64_t T = g->sym_nt, cg = std::min<int64_t>(C, 4);
             WFQ_TRY(rowpart.alloc(g->ctx, (size_t)g->sym_nitems * kSymTile * cg, s));
             WFQ_TRY(colpart.alloc(g->ctx, (size_t)(T * (T + 1) / 2) * kSymTile * cg, s));
@@ -861,8 +946,29 @@ struct Arnoldi {
         return best;
     }
 
-    // u = D v; xh / xl already hold v's float-pair split (written when v was normalised)
+    GemvDigits work(int d0) const {
+        return GemvDigits{planes.ptr + (size_t)(d0 / 4) * gemv_digits_plane_elems(g), xexp.ptr + d0, vmax.ptr + d0, acc.ptr};
+    }
+    NextVec next() const {
+        return NextVec{xh.ptr, xl.ptr, reinterpret_cast<__half *>(planes.ptr), xexp.ptr, (int64_t)gemv_digits_plane_elems(g),
+                       g->npad, pmax.ptr};
+    }
+    // digits of v [C][n] (the start vectors; later ones get theirs in k_rscale_norm)
+    int split(const double *v) {
+        for (int d0 = 0; digits && d0 < C; d0 += 4)
+            WFQ_TRY(gemv_digits_split(g, std::min(4, C - d0), v + (int64_t)d0 * n, 1, n, work(d0), s));
+        return WFQ_OK;
+    }
+
+    // u = D v; xh / xl (or the digit planes) already hold v (written when v was normalised)
     int dmul(double *u) {
+        if (digits) {
+            for (int d0 = 0; d0 < C; d0 += 4) {
+                KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, 8.0 * (double)n * (double)n);
+                WFQ_TRY(gemv_digits_product(g, std::min(4, C - d0), work(d0), u + (int64_t)d0 * n, 1, n, s));
+            }
+            return WFQ_OK;
+        }
         if (!g->Dsym && !g->Dfh && !g->D64) {   // matrix-free: D regenerated per product
             KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, 0.0);
             for (int d0 = 0; d0 < C; d0 += 4)
@@ -975,6 +1081,27 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
     const int64_t n = g->n;
     const int C = (int)(2 * cc);
     if (!(g->Dfh || g->Dsym)) return fail(WFQ_EUNSUPPORTED, "float-pair product: needs stored pairs");
+    if (use_gemv_digits(g)) {
+        DevBuf<uint16_t> planes;
+        DevBuf<int> xexp;
+        DevBuf<unsigned long long> vmax, acc;
+        const size_t np = gemv_digits_plane_elems(g);
+        WFQ_TRY(planes.alloc(g->ctx, np, s));
+        WFQ_TRY(xexp.alloc(g->ctx, 4, s));
+        WFQ_TRY(vmax.alloc(g->ctx, 4, s));
+        WFQ_TRY(acc.alloc(g->ctx, (size_t)8 * n, s));
+        WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 8 * n, s));
+        const GemvDigits w{planes.ptr, xexp.ptr, vmax.ptr, acc.ptr};
+        KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
+        for (int d0 = 0; d0 < C; d0 += 4) {
+            const int cg = std::min(4, C - d0);
+            // rows past 8 cg and atoms past n stay zero
+            WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
+            WFQ_TRY(gemv_digits_split(g, cg, reinterpret_cast<const double *>(X) + d0, C, 1, w, s));
+            WFQ_TRY(gemv_digits_product(g, cg, w, reinterpret_cast<double *>(U) + d0, C, 1, s));
+        }
+        return WFQ_OK;
+    }
     DevBuf<float> xh, xl;
     DevBuf<double> ud, rowpart, colpart;
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
@@ -1095,6 +1222,7 @@ int solve_gmres_shifted(wfq_geom *g, const SolveArgs &a, cudaStream_t s) {
     k_take_rhs<<<nblk(n * C), 256, 0, s>>>(n, (int)C, R.ptr, ar.U.ptr); note_launch();
     WFQ_TRY(ar.dots(ar.U.ptr, 0, 1, ar.U.ptr, RF_NORM, m, -1, H.ptr, hn.ptr));
     k_rscale<<<nblk(n * C), 256, 0, s>>>(n, (int)C, hn.ptr, ar.U.ptr, V.ptr, ar.xh.ptr, ar.xl.ptr); note_launch();
+    WFQ_TRY(ar.split(V.ptr));
     std::vector<double> rn_h(C), tg(C);
     WFQ_CUDA(cudaMemcpyAsync(rn_h.data(), hn.ptr, sizeof(double) * C, cudaMemcpyDeviceToHost, s));
     WFQ_CUDA(cudaStreamSynchronize(s));   // also completes the cdir_h / om_h uploads
@@ -1145,17 +1273,25 @@ int solve_gmres_shifted(wfq_geom *g, const SolveArgs &a, cudaStream_t s) {
             const int nv = j + 1;
             WFQ_TRY(ar.dots(V.ptr, vstride, nv, w, RF_SET, m, j, H.ptr, hn.ptr));
             k_rupdate_next<NEXT_DOTS><<<dim3((unsigned)ar.nbru, (unsigned)C), 32 * RU_SLICES, 0, s>>>(
-                n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w, ar.partial_f.ptr);
+                n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w, ar.partial_f.ptr, nullptr);
             note_launch();
             k_rdot_fin<<<nblk((int64_t)nv * C * 32), 256, 0, s>>>(ar.nbru, nv, (int)C, RF_ADD, ar.partial_f.ptr, m, j,
                                                                   H.ptr, ar.coef.ptr, hn.ptr);
             note_launch();
-            k_rupdate_next<NEXT_NORM><<<dim3((unsigned)ar.nbru, (unsigned)C), 32 * RU_SLICES, 0, s>>>(
-                n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w, ar.partial_f.ptr);
+            const dim3 gu((unsigned)ar.nbru, (unsigned)C);
+            const size_t sm = (sizeof(double) + sizeof(int)) * C;
+            if (ar.digits) {
+                k_rupdate_next<NEXT_NORM_MAX><<<gu, 32 * RU_SLICES, 0, s>>>(n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w,
+                                                                            ar.partial_f.ptr, ar.pmax.ptr);
+                k_rscale_norm<true><<<nblk(n * C, 1024), 256, sm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
+                                                                       hn.ptr, w, w, ar.next());
+            } else {
+                k_rupdate_next<NEXT_NORM><<<gu, 32 * RU_SLICES, 0, s>>>(n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w,
+                                                                        ar.partial_f.ptr, nullptr);
+                k_rscale_norm<false><<<nblk(n * C, 1024), 256, sm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
+                                                                        hn.ptr, w, w, ar.next());
+            }
             note_launch();
-            k_rscale_norm<<<nblk(n * C, 1024), 256, sizeof(double) * C, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m,
-                                                                             j, H.ptr, hn.ptr, w, w, ar.xh.ptr,
-                                                                             ar.xl.ptr);
             note_launch();
             WFQ_CUDA(cudaEventRecord(side.fork, s));
             WFQ_CUDA(cudaStreamWaitEvent(side.st, side.fork, 0));
