@@ -154,7 +154,7 @@ static __global__ void __launch_bounds__(NUM_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int64_t G = gridDim.x;
     const int64_t u_begin = p.units * (int64_t)blockIdx.x / G;
     const int64_t u_end = p.units * ((int64_t)blockIdx.x + 1) / G;
@@ -216,8 +216,9 @@ static __global__ void __launch_bounds__(NUM_THREADS, 1)
                     mbar_wait(smem_u32(full + s), (uint32_t)((last_it[s] / p.stages) & 1), p, 1, &no_abort);
                 }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
+        const bool el = elect_one();
         const uint32_t idesc = idesc_bf16(BM, p.nchunk);
         int64_t it = 0, seg = 0;
         int64_t u = u_begin;
@@ -247,20 +248,20 @@ static __global__ void __launch_bounds__(NUM_THREADS, 1)
                         const uint64_t b_hi = desc_k_sw64(base + 2 * A_BYTES + boff);
                         const uint64_t b_lo = desc_k_sw64(base + 2 * A_BYTES + p.b_bytes + boff);
                         const uint32_t d = tmem + (uint32_t)(j * p.nchunk);
-                        umma_bf16(d, a_hi, b_hi, idesc, first ? 0u : 1u);
-                        umma_bf16(d, a_hi, b_lo, idesc, 1u);
-                        umma_bf16(d, a_lo, b_hi, idesc, 1u);
+                        if (el) umma_bf16(d, a_hi, b_hi, idesc, first ? 0u : 1u);
+                        if (el) umma_bf16(d, a_hi, b_lo, idesc, 1u);
+                        if (el) umma_bf16(d, a_lo, b_hi, idesc, 1u);
                     }
                     first = false;
                 }
-                umma_commit(smem_u32(empty + s));
+                if (el) umma_commit(smem_u32(empty + s));
             }
             if (aborted) break;
-            umma_commit(smem_u32(acc_full));
+            if (el) umma_commit(smem_u32(acc_full));
             ++seg;
         }
         // every MMA this thread issued has completed once `drain` flips
-        umma_commit(smem_u32(drain));
+        if (el) umma_commit(smem_u32(drain));
         volatile int no_abort = 0;
         mbar_wait(smem_u32(drain), 0u, p, 5, &no_abort);
     } else if (warp >= 2) {
