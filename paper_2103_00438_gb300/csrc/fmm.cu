@@ -52,13 +52,20 @@ struct Fmm {
     int32_t *child_lo = nullptr;     // nbox: children's global index range [lo, hi)
     int32_t *child_hi = nullptr;
     int8_t *octant = nullptr;        // nbox: which child of its parent (bit d: upper half in d)
-    int32_t *il_start = nullptr;     // nbox + 1: interaction list of each box (CSR)
-    int32_t *il_src = nullptr;       // nil: source box (global index)
-    int16_t *il_off = nullptr;       // nil: offset code, sum_d (src_d - tgt_d + 3) 7^d
+    // M2L: the boxes of levels >= 2 by octant (boxes of one octant have the same offsets in the
+    // same order, the slots) and each slot's source box
+    int nslots = 0;                  // 27 (quadtree) or 189 (octree)
+    int64_t nm2l = 0;
+    int32_t oct_first[9] = {};       // first list position of each octant
+    int32_t *m2l_box = nullptr;      // nm2l: global box index
+    int8_t *m2l_level = nullptr;     // nm2l
+    int32_t *m2l_src = nullptr;      // nslots x nm2l: source box, -1: none
+    int16_t *slot_off = nullptr;     // 2^dim x nslots: offset code, sum_d (src_d - tgt_d + 3) 7^d
     int32_t *near_start = nullptr;   // nleaf + 1: near leaves of each leaf (CSR)
     int32_t *near_leaf = nullptr;    // nnear: leaf index
     int8_t *near_delta = nullptr;    // nnear: offset code, sum_d (src_d - tgt_d + 1) 3^d
-    float *T = nullptr;              // 2^dim x P x P: M2M weights [octant][parent node][child node]
+    float *Tm = nullptr;             // 2^dim x P x Pp: M2M weights [octant][child node][parent node]
+    float *Tl = nullptr;             // 2^dim x P x Pp: the same [octant][parent node][child node], for L2L
     float *K = nullptr;              // 7^dim x P x P: M2L kernel for boxes of half-width 1
     float *cheb = nullptr;           // p x p: T_k(x_m)
     size_t bytes = 0;
@@ -120,12 +127,13 @@ int upload(wfq_ctx *ctx, Fmm *f, T **dst, const std::vector<T> &src) {
 struct FmmDev {
     int dim, p, P, L;
     float h;                          // leaf side
-    const int32_t *perm, *leaf_start, *parent, *child_lo, *child_hi, *il_start, *il_src;
+    int nslots;
+    const int32_t *perm, *leaf_start, *parent, *child_lo, *child_hi, *m2l_box, *m2l_src;
     const int32_t *near_start, *near_leaf;
-    const int16_t *il_off;
-    const int8_t *octant, *near_delta;
+    const int16_t *slot_off;
+    const int8_t *octant, *near_delta, *m2l_level;
     const float4 *atl;
-    const float *eta, *T, *K, *cheb;
+    const float *eta, *Tm, *Tl, *K, *cheb;
     int64_t leaf0;                    // global index of the first leaf
 };
 
@@ -152,7 +160,17 @@ __device__ __forceinline__ float node_product(const FmmDev &f, int m, const floa
     return W0[m / (f.p * f.p)] * W1[(m / f.p) % f.p] * W2[m % f.p];
 }
 
-// P2M: one block per leaf; multipole coefficients M[leaf][m][r] = sum_i S(m, y_i) x_i[r].
+// Rows of X in sorted order, padded with zeros to Cp columns (a multiple of 4).
+__global__ void k_fmm_sort_x(int64_t n, int64_t C, int64_t Cp, const int32_t *__restrict__ perm, const float *__restrict__ X,
+                             float *__restrict__ Xs) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * Cp) return;
+    const int64_t k = e / Cp, r = e - k * Cp;
+    Xs[e] = r < C ? X[(int64_t)perm[k] * C + r] : 0.f;
+}
+
+// P2M: one block per leaf; multipole coefficients M[leaf][m][r] = sum_i S(m, y_i) x_i[r]
+// (X in sorted order).
 __global__ void k_fmm_p2m(FmmDev f, int64_t C, const float *__restrict__ X, float *__restrict__ M) {
     extern __shared__ float sm[];
     const int64_t b = blockIdx.x;
@@ -176,7 +194,7 @@ __global__ void k_fmm_p2m(FmmDev f, int64_t C, const float *__restrict__ X, floa
         for (int64_t t = threadIdx.x; t < (int64_t)nk * C; t += blockDim.x) {
             const int k = (int)(t / C);
             const int64_t r = t % C;
-            xs[t] = X[(int64_t)f.perm[c0 + k] * C + r];
+            xs[t] = X[(int64_t)(c0 + k) * C + r];
         }
         __syncthreads();
         for (int64_t o = threadIdx.x; o < PC; o += blockDim.x) {
@@ -192,199 +210,253 @@ __global__ void k_fmm_p2m(FmmDev f, int64_t C, const float *__restrict__ X, floa
     }
 }
 
-// M2M at one level: one block per parent box (global index box0 + blockIdx.x).
-__global__ void k_fmm_m2m(FmmDev f, int64_t C, int64_t box0, float *__restrict__ M) {
+// acc[0..7] += the rows r0 .. r0 + 7 of Tt^T In for one column: Tt is P x Pp (rows past P zero),
+// In this column of a P x Cp array.  Eight rows share each load of In; Tt is uniform in a warp.
+__device__ __forceinline__ void node_rows(int P, int Pp, int64_t Cp, const float *__restrict__ Tt, int r0,
+                                          const float *__restrict__ In, float (&acc)[8]) {
+#pragma unroll 6
+    for (int k = 0; k < P; ++k) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(Tt + (int64_t)k * Pp + r0));
+        const float4 b = __ldg(reinterpret_cast<const float4 *>(Tt + (int64_t)k * Pp + r0 + 4));
+        const float v = In[(int64_t)k * Cp];
+        acc[0] = fmaf(a.x, v, acc[0]);
+        acc[1] = fmaf(a.y, v, acc[1]);
+        acc[2] = fmaf(a.z, v, acc[2]);
+        acc[3] = fmaf(a.w, v, acc[3]);
+        acc[4] = fmaf(b.x, v, acc[4]);
+        acc[5] = fmaf(b.y, v, acc[5]);
+        acc[6] = fmaf(b.z, v, acc[6]);
+        acc[7] = fmaf(b.w, v, acc[7]);
+    }
+}
+
+// M2M at one level: a block per (parent box, 32 columns), its warps over groups of 8 nodes.
+// (One output per thread with two loads per multiply-add took 418 us over the levels of the
+// 250k-atom disk, order 6, 32 columns, against 255; L2L 358 against 219.)
+__global__ void __launch_bounds__(256) k_fmm_m2m(FmmDev f, int Pp, int64_t C, int64_t box0, float *__restrict__ M) {
     const int64_t g = box0 + blockIdx.x;
+    const int64_t r = (int64_t)blockIdx.y * 32 + (threadIdx.x & 31);
+    if (r >= C) return;
     const int64_t PC = (int64_t)f.P * C;
     const int c0 = f.child_lo[g], c1 = f.child_hi[g];
-    for (int64_t o = threadIdx.x; o < PC; o += blockDim.x) {
-        const int m = (int)(o / C);
-        const int64_t r = o % C;
-        float acc = 0.f;
-        for (int ch = c0; ch < c1; ++ch) {
-            const float *Tm = f.T + ((int64_t)f.octant[ch] * f.P + m) * f.P;
-            const float *Mc = M + (int64_t)ch * PC + r;
-            for (int mp = 0; mp < f.P; ++mp) acc = fmaf(Tm[mp], Mc[(int64_t)mp * C], acc);
-        }
-        M[g * PC + o] = acc;
+    for (int r0 = (threadIdx.x >> 5) * 8; r0 < f.P; r0 += blockDim.x / 4) {
+        float acc[8] = {};
+        for (int ch = c0; ch < c1; ++ch)
+            node_rows(f.P, Pp, C, f.Tm + (int64_t)f.octant[ch] * f.P * Pp, r0, M + (int64_t)ch * PC + r, acc);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (r0 + i < f.P) M[g * PC + (int64_t)(r0 + i) * C + r] = acc[i];
     }
 }
 
-// M2L for every box of levels 2..L: one block per (target box, group of 64 columns);
-// thread (tm, tr) owns a 4 x 4 tile of (node, column) outputs.  lvl: first global box of
-// each level, levels 0..L+1 (device copy in constant-size argument).
-struct LevelTable {
-    int64_t first[24];
+// L2L at one level (l >= 3): a block per (box, 32 columns); L[child] += T[oct]^T L[parent].
+__global__ void __launch_bounds__(256) k_fmm_l2l(FmmDev f, int Pp, int64_t C, int64_t box0, float *__restrict__ Lc) {
+    const int64_t g = box0 + blockIdx.x;
+    const int64_t r = (int64_t)blockIdx.y * 32 + (threadIdx.x & 31);
+    if (r >= C) return;
+    const int64_t PC = (int64_t)f.P * C;
+    for (int r0 = (threadIdx.x >> 5) * 8; r0 < f.P; r0 += blockDim.x / 4) {
+        float acc[8] = {};
+        node_rows(f.P, Pp, C, f.Tl + (int64_t)f.octant[g] * f.P * Pp, r0, Lc + (int64_t)f.parent[g] * PC + r, acc);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (r0 + i < f.P) Lc[g * PC + (int64_t)(r0 + i) * C + r] += acc[i];
+    }
+}
+
+// M2L for every box of levels 2..L.  A block takes boxes of one octant, which meet the same
+// offsets slot by slot, so one kernel tile K[offset] in shared memory serves all of them; a lane
+// owns one column of M2L_NB boxes and 2 RP nodes (packed FP32x2 pairs of nodes), reading its
+// column of the sources' multipoles straight from L2 and K as a broadcast.  K[-offset] is the
+// transpose of K[offset] (1 / |x_m - x_s - 2 d| with m and s exchanged), so its rows hold the
+// target nodes of one source node consecutively.  lpb lanes per box (a power of two >= the
+// columns of a block, at most 32).  blockIdx.z: group of 2 RP target nodes.
+//
+// Bound: FP32 FMAs (455544 tiles of 36 x 36 x 32 for the 250k-atom disk, order 6: 0.53 ms) and
+// the K broadcasts (one 16-byte shared load per 8 FMAs of a lane): 1.00 ms.  A block per box with
+// 4 x 4 register tiles, both operands staged, took 4.66 ms.  Unrolling the source nodes by 6
+// keeps enough loads in flight (4: 1.67 ms, 12: 1.02); one box per lane 1.3 to 1.7 ms; prefetching
+// the next nodes into registers 1.5 to 2.1 ms.
+struct M2lGrid {
+    int32_t first[9];   // octant's first list position, then the end
+    int32_t tile[9];    // octant's first block
     float inv_a[24];    // 1 / half-width of the boxes of each level
 };
-constexpr int M2L_KC = 32;    // source nodes per shared-memory stage
-constexpr int M2L_CB = 64;    // columns per block
+constexpr int M2L_WARPS = 8, M2L_NB = 2;
 
-__global__ void k_fmm_m2l(FmmDev f, int64_t C, LevelTable lv, const float *__restrict__ M, float *__restrict__ Lc) {
-    extern __shared__ float sm[];
-    const int64_t t = lv.first[2] + blockIdx.x;
-    int l = 2;
-    while (t >= lv.first[l + 1]) ++l;
-    const float scale = lv.inv_a[l];
-    const int64_t cb = (int64_t)blockIdx.y * M2L_CB;
-    const int ncol = (int)min((int64_t)M2L_CB, C - cb);
-    const int tm = threadIdx.x / (M2L_CB / 4), tr = threadIdx.x % (M2L_CB / 4);
-    const int P = f.P;
-    float *sK = sm;                         // [P][M2L_KC]
-    float *sM = sm + P * M2L_KC;            // [M2L_KC][M2L_CB]
-    float acc[4][4] = {};
+template <int RP>
+__global__ void __launch_bounds__(32 * M2L_WARPS, 2)
+    k_fmm_m2l(FmmDev f, int64_t C, int64_t nm2l, int noct, M2lGrid gr, int lpb, const float *__restrict__ M,
+              float *__restrict__ Lc) {
+    extern __shared__ __align__(16) float sK[];   // [P][2 RP]
+    constexpr int RW = 2 * RP;
+    const int P = f.P, r0 = blockIdx.z * RW;
+    int oc = 0;
+    while (oc + 1 < noct && (int)blockIdx.x >= gr.tile[oc + 1]) ++oc;
+    const int bpw = 32 / lpb;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t col = (int64_t)blockIdx.y * 32 + (lane & (lpb - 1));
     const int64_t PC = (int64_t)P * C;
-    for (int e = f.il_start[t]; e < f.il_start[t + 1]; ++e) {
-        const int64_t s = f.il_src[e];
-        const float *Ko = f.K + (int64_t)f.il_off[e] * P * P;
-        const float *Ms = M + s * PC + cb;
-        for (int k0 = 0; k0 < P; k0 += M2L_KC) {
-            const int nk = min(M2L_KC, P - k0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < P * M2L_KC; q += blockDim.x) {
-                const int m = q / M2L_KC, kk = q % M2L_KC;
-                sK[q] = kk < nk ? Ko[(int64_t)m * P + k0 + kk] : 0.f;
+    int64_t pos[M2L_NB];
+    bool ok[M2L_NB];
+#pragma unroll
+    for (int b = 0; b < M2L_NB; ++b) {
+        pos[b] = gr.first[oc] + (((int64_t)blockIdx.x - gr.tile[oc]) * M2L_WARPS + warp) * (M2L_NB * bpw) + b * bpw + lane / lpb;
+        ok[b] = pos[b] < gr.first[oc + 1] && col < C;
+    }
+    float2 acc[M2L_NB][RP];
+#pragma unroll
+    for (int b = 0; b < M2L_NB; ++b)
+#pragma unroll
+        for (int q = 0; q < RP; ++q) acc[b][q] = make_float2(0.f, 0.f);
+    const int total = f.dim == 2 ? 6 * 8 : 6 * 57;   // offset code of -d: total - code
+    for (int sl = 0; sl < f.nslots; ++sl) {
+        const float *Ko = f.K + (int64_t)(total - f.slot_off[oc * f.nslots + sl]) * P * P;
+        __syncthreads();
+        for (int q = threadIdx.x; q < P * RW; q += blockDim.x) {
+            const int k = q / RW, m = q - k * RW;
+            sK[q] = r0 + m < P ? __ldg(Ko + (int64_t)k * P + r0 + m) : 0.f;
+        }
+        int32_t src[M2L_NB];
+        bool any = false;
+#pragma unroll
+        for (int b = 0; b < M2L_NB; ++b) {
+            src[b] = ok[b] ? __ldg(f.m2l_src + (int64_t)sl * nm2l + pos[b]) : -1;
+            any = any || src[b] >= 0;
+        }
+        __syncthreads();
+        if (!__any_sync(0xffffffffu, any)) continue;
+        const float *Ms[M2L_NB];
+#pragma unroll
+        for (int b = 0; b < M2L_NB; ++b) Ms[b] = M + (int64_t)(src[b] < 0 ? 0 : src[b]) * PC + col;
+#pragma unroll 6
+        for (int k = 0; k < P; ++k) {
+            float2 mv[M2L_NB];
+#pragma unroll
+            for (int b = 0; b < M2L_NB; ++b) {
+                const float v = src[b] >= 0 ? __ldg(Ms[b] + (int64_t)k * C) : 0.f;
+                mv[b] = make_float2(v, v);
             }
-            for (int q = threadIdx.x; q < M2L_KC * M2L_CB; q += blockDim.x) {
-                const int kk = q / M2L_CB, r = q % M2L_CB;
-                sM[q] = (kk < nk && r < ncol) ? Ms[(int64_t)(k0 + kk) * C + r] : 0.f;
-            }
-            __syncthreads();
-            if (tm * 4 < P) {
-                for (int kk = 0; kk < nk; ++kk) {
-                    float kv[4], mv[4];
+            const float2 *kr = reinterpret_cast<const float2 *>(sK + k * RW);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) kv[i] = (tm * 4 + i < P) ? sK[(tm * 4 + i) * M2L_KC + kk] : 0.f;
+            for (int q = 0; q < RP; ++q) {
+                const float2 kv = kr[q];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) mv[j] = sM[kk * M2L_CB + tr * 4 + j];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(kv[i], mv[j], acc[i][j]);
-                }
+                for (int b = 0; b < M2L_NB; ++b) acc[b][q] = __ffma2_rn(kv, mv[b], acc[b][q]);
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int m = tm * 4 + i;
-        if (m >= P) continue;
+    for (int b = 0; b < M2L_NB; ++b) {
+        if (!ok[b]) continue;
+        const float scale = gr.inv_a[f.m2l_level[pos[b]]];
+        float *o = Lc + (int64_t)f.m2l_box[pos[b]] * PC + col;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = tr * 4 + j;
-            if (r < ncol) Lc[t * PC + (int64_t)m * C + cb + r] = scale * acc[i][j];
+        for (int q = 0; q < RP; ++q) {
+            const int m = r0 + 2 * q;
+            if (m < P) o[(int64_t)m * C] = scale * acc[b][q].x;
+            if (m + 1 < P) o[(int64_t)(m + 1) * C] = scale * acc[b][q].y;
         }
     }
 }
 
-// L2L at one level (l >= 3): one block per box; L[child] += T[oct]^T L[parent].
-__global__ void k_fmm_l2l(FmmDev f, int64_t C, int64_t box0, float *__restrict__ Lc) {
-    const int64_t g = box0 + blockIdx.x;
-    const int64_t pg = f.parent[g];
-    const int o8 = f.octant[g];
-    const int64_t PC = (int64_t)f.P * C;
-    for (int64_t o = threadIdx.x; o < PC; o += blockDim.x) {
-        const int m = (int)(o / C);
-        const int64_t r = o % C;
-        const float *Tc = f.T + (int64_t)o8 * f.P * f.P + m;
-        const float *Lp = Lc + pg * PC + r;
-        float acc = 0.f;
-        for (int mp = 0; mp < f.P; ++mp) acc = fmaf(Tc[(int64_t)mp * f.P], Lp[(int64_t)mp * C], acc);
-        Lc[g * PC + o] += acc;
-    }
-}
-
-// L2P and the near field: one block per leaf.  Thread (target atom, group of RC columns).
-constexpr int NF_RC = 8;
-constexpr int NF_SCH = 64;   // source atoms per shared-memory stage
-
-__global__ void k_fmm_l2p_near(FmmDev f, int64_t C, int far, const float *__restrict__ X,
-                               const float *__restrict__ Lc, float *__restrict__ U) {
-    extern __shared__ float sm[];
-    const int64_t b = blockIdx.x;
+// L2P and the near field: a warp per leaf, a lane per target atom, 4 CQ columns (blockIdx.y) in
+// registers, so a pair's D_ij is computed once for them (once per 8 columns before: 1431 us for
+// the 250k-atom disk, order 6, 32 columns, against 726).  Sources, their X rows and the leaf's
+// local coefficients are uniform in the warp and come through L1.
+template <int CQ>
+__global__ void __launch_bounds__(128) k_fmm_l2p_near(FmmDev f, int64_t nleaf, int64_t C, int64_t Cp, int far,
+                                                      const float *__restrict__ Xs, const float *__restrict__ Lc,
+                                                      float *__restrict__ U) {
+    __shared__ float sW[4][3][kMaxP][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t b = (int64_t)blockIdx.x * 4 + warp;
+    if (b >= nleaf) return;
+    const int64_t col0 = (int64_t)blockIdx.y * (4 * CQ);
     const int k0 = f.leaf_start[b], k1 = f.leaf_start[b + 1];
-    const int ng = (int)((C + NF_RC - 1) / NF_RC);
-    const int64_t PC = (int64_t)f.P * C;
-    float4 *ssrc = reinterpret_cast<float4 *>(sm);            // [NF_SCH] (x, y, z, width)
-    float *seta = sm + 4 * NF_SCH;                            // [NF_SCH]
-    float *sx = seta + NF_SCH;                                // [NF_SCH][C]
     const float a = 0.5f * f.h;
-    for (int base = k0; base < k1; base += blockDim.x / ng) {
-        const int i = base + threadIdx.x / ng;
-        const int g = threadIdx.x % ng;
-        const bool act = (threadIdx.x / ng) < blockDim.x / ng && i < k1;
-        float acc[NF_RC];
+    for (int base = k0; base < k1; base += 32) {
+        const int i = base + lane;
+        const bool act = i < k1;
+        const float4 qi = act ? f.atl[i] : make_float4(0.f, 0.f, 0.f, 1.f);
+        float2 lo[CQ], hi[CQ];
 #pragma unroll
-        for (int j = 0; j < NF_RC; ++j) acc[j] = 0.f;
-        float4 qi = make_float4(0.f, 0.f, 0.f, 1.f);
-        float etai = 0.f;
-        if (act) {
-            qi = f.atl[i];
-            etai = f.eta[i];
-            if (far && f.L >= 2) {
-                float W[3][kMaxP];
-                node_weights(f, qi.x / a, W[0]);
-                node_weights(f, qi.y / a, W[1]);
-                if (f.dim == 3) node_weights(f, qi.z / a, W[2]);
-                const float *Lb = Lc + (f.leaf0 + b) * PC;
-                for (int m = 0; m < f.P; ++m) {
-                    const float wm = node_product(f, m, W[0], W[1], W[2]);
+        for (int q = 0; q < CQ; ++q) lo[q] = hi[q] = make_float2(0.f, 0.f);
+        auto add = [&](float d, const float4 *x) {
 #pragma unroll
-                    for (int j = 0; j < NF_RC; ++j) {
-                        const int64_t r = (int64_t)g * NF_RC + j;
-                        if (r < C) acc[j] = fmaf(wm, Lb[(int64_t)m * C + r], acc[j]);
-                    }
+            for (int q = 0; q < CQ; ++q) {
+                if (col0 + 4 * q >= Cp) break;
+                const float4 v = __ldg(x + q);
+                lo[q] = __ffma2_rn(make_float2(d, d), make_float2(v.x, v.y), lo[q]);
+                hi[q] = __ffma2_rn(make_float2(d, d), make_float2(v.z, v.w), hi[q]);
+            }
+        };
+        if (far && f.L >= 2) {
+            const float y[3] = {qi.x / a, qi.y / a, qi.z / a};
+            float tk[kMaxP];
+            for (int d = 0; d < f.dim; ++d) {   // node_weights into shared memory
+                tk[0] = 1.f;
+                if (f.p > 1) tk[1] = y[d];
+                for (int k = 2; k < f.p; ++k) tk[k] = 2.f * y[d] * tk[k - 1] - tk[k - 2];
+                const float inv = 1.f / f.p;
+                for (int m = 0; m < f.p; ++m) {
+                    float s = 0.f;
+                    for (int k = 1; k < f.p; ++k) s = fmaf(f.cheb[m * f.p + k], tk[k], s);
+                    sW[warp][d][m][lane] = inv + 2.f * inv * s;
                 }
             }
+            __syncwarp();
+            const float *Lb = Lc + (f.leaf0 + b) * (int64_t)f.P * Cp + col0;
+            if (f.dim == 2) {
+                for (int m0 = 0; m0 < f.p; ++m0) {
+                    const float w0 = sW[warp][0][m0][lane];
+                    for (int m1 = 0; m1 < f.p; ++m1, Lb += Cp)
+                        add(w0 * sW[warp][1][m1][lane], reinterpret_cast<const float4 *>(Lb));
+                }
+            } else {
+                for (int m0 = 0; m0 < f.p; ++m0)
+                    for (int m1 = 0; m1 < f.p; ++m1) {
+                        const float w01 = sW[warp][0][m0][lane] * sW[warp][1][m1][lane];
+                        for (int m2 = 0; m2 < f.p; ++m2, Lb += Cp)
+                            add(w01 * sW[warp][2][m2][lane], reinterpret_cast<const float4 *>(Lb));
+                    }
+            }
+            __syncwarp();
         }
+        const float etai = act ? f.eta[i] : 0.f;
         for (int e = f.near_start[b]; e < f.near_start[b + 1]; ++e) {
             const int nb = f.near_leaf[e];
             const int dc = f.near_delta[e];
             const float ox = ((dc % 3) - 1) * f.h, oy = ((dc / 3) % 3 - 1) * f.h, oz = (dc / 9 - 1) * f.h;
-            const int s0 = f.leaf_start[nb], s1 = f.leaf_start[nb + 1];
-            for (int c0 = s0; c0 < s1; c0 += NF_SCH) {
-                const int ns = min(NF_SCH, s1 - c0);
-                __syncthreads();
-                for (int q = threadIdx.x; q < ns; q += blockDim.x) {
-                    float4 sj = f.atl[c0 + q];
-                    sj.x += ox;   // source position in the target leaf's frame
-                    sj.y += oy;
-                    sj.z += oz;
-                    ssrc[q] = sj;
-                    seta[q] = f.eta[c0 + q];
+            const int s1 = f.leaf_start[nb + 1];
+            for (int j = f.leaf_start[nb]; j < s1; ++j) {
+                float4 sj = __ldg(f.atl + j);
+                sj.x += ox;   // source position in the target leaf's frame
+                sj.y += oy;
+                sj.z += oz;
+                const float dx = qi.x - sj.x, dy = qi.y - sj.y, dz = qi.z - sj.z;
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const float s2 = fmaf(qi.w, qi.w, sj.w * sj.w);
+                const float rinv = rsqrtf(r2);
+                float d = rinv;                   // erf(r / s) rounds to 1 in FP32 from r = 4 s on
+                if (r2 < 16.f * s2) {
+                    const float sinv = rsqrtf(s2);
+                    // r -> 0 limit of erf(r / s) / r: 2 / (sqrt(pi) s)
+                    d = r2 > 1e-24f ? erff(r2 * rinv * sinv) * rinv : 1.1283791670955126f * sinv;
                 }
-                for (int64_t q = threadIdx.x; q < (int64_t)ns * C; q += blockDim.x)
-                    sx[q] = X[(int64_t)f.perm[c0 + q / C] * C + q % C];
-                __syncthreads();
-                if (!act) continue;
-                for (int jj = 0; jj < ns; ++jj) {
-                    const float4 sj = ssrc[jj];
-                    float d;
-                    if (c0 + jj == i) {
-                        d = etai;
-                    } else {
-                        const float dx = qi.x - sj.x, dy = qi.y - sj.y, dz = qi.z - sj.z;
-                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        const float sinv = rsqrtf(fmaf(qi.w, qi.w, sj.w * sj.w));
-                        if (r2 > 1e-24f) {
-                            const float rinv = rsqrtf(r2);
-                            d = erff(r2 * rinv * sinv) * rinv;
-                        } else {
-                            d = 1.1283791670955126f * sinv;   // r -> 0 limit of erf(r / s) / r: 2 / (sqrt(pi) s)
-                        }
-                    }
-                    const float *xj = sx + (int64_t)jj * C + (int64_t)g * NF_RC;
-#pragma unroll
-                    for (int j = 0; j < NF_RC; ++j)
-                        if ((int64_t)g * NF_RC + j < C) acc[j] = fmaf(d, xj[j], acc[j]);
-                }
+                if (j == i) d = etai;
+                add(d, reinterpret_cast<const float4 *>(Xs + (int64_t)j * Cp + col0));
             }
         }
         if (act) {
-            float *Ui = U + (int64_t)f.perm[i] * C + (int64_t)g * NF_RC;
+            float *Ui = U + (int64_t)f.perm[i] * C + col0;
 #pragma unroll
-            for (int j = 0; j < NF_RC; ++j)
-                if ((int64_t)g * NF_RC + j < C) Ui[j] = acc[j];
+            for (int q = 0; q < CQ; ++q) {
+                const float v[4] = {lo[q].x, lo[q].y, hi[q].x, hi[q].y};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (col0 + 4 * q + j < C) Ui[4 * q + j] = v[j];
+            }
         }
     }
 }
@@ -401,16 +473,19 @@ FmmDev dev_view(const Fmm *f) {
     d.parent = f->parent;
     d.child_lo = f->child_lo;
     d.child_hi = f->child_hi;
-    d.il_start = f->il_start;
-    d.il_src = f->il_src;
+    d.nslots = f->nslots;
+    d.m2l_box = f->m2l_box;
+    d.m2l_level = f->m2l_level;
+    d.m2l_src = f->m2l_src;
+    d.slot_off = f->slot_off;
     d.near_start = f->near_start;
     d.near_leaf = f->near_leaf;
-    d.il_off = f->il_off;
     d.octant = f->octant;
     d.near_delta = f->near_delta;
     d.atl = f->atl;
     d.eta = f->eta;
-    d.T = f->T;
+    d.Tm = f->Tm;
+    d.Tl = f->Tl;
     d.K = f->K;
     d.cheb = f->cheb;
     d.leaf0 = f->lvl0[f->L];
@@ -422,8 +497,8 @@ FmmDev dev_view(const Fmm *f) {
 void fmm_free(Fmm *f) {
     if (!f) return;
     void *ptrs[] = {f->perm, f->leaf_start, f->atl, f->eta, f->parent, f->child_lo, f->child_hi, f->octant,
-                    f->il_start, f->il_src, f->il_off, f->near_start, f->near_leaf, f->near_delta,
-                    f->T, f->K, f->cheb};
+                    f->m2l_box, f->m2l_level, f->m2l_src, f->slot_off, f->near_start, f->near_leaf, f->near_delta,
+                    f->Tm, f->Tl, f->K, f->cheb};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete f;
@@ -462,7 +537,7 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
     }
     const int dim = (mx[2] == mn[2]) ? 2 : 3;
     f->dim = dim;
-    // the M2L kernel's thread tile (4 nodes x 4 columns, <= 1024 threads) bounds the nodes per box
+    // nodes per box the tables and kernels are sized for
     if ((dim == 2 && order > 16) || (dim == 3 && order > 6))
         return fail(WFQ_EINVAL, "FMM order must be <= 16 for a flat structure and <= 6 for a 3D one");
     double wmax = 0.0;
@@ -535,43 +610,65 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
             child_hi[pg] = gi + 1;
         }
 
-    // interaction lists (levels >= 2) and near lists (leaves)
-    std::vector<int32_t> il_start(f->nbox + 1, 0), il_src;
-    std::vector<int16_t> il_off;
-    for (int l = 0; l <= L; ++l)
-        for (size_t q = 0; q < keys[l].size(); ++q) {
-            const int64_t gi = f->lvl0[l] + (int64_t)q;
-            if (l >= 2) {
-                int64_t ct[3] = {0, 0, 0};
-                unmorton(dim, keys[l][q], ct);
-                const int64_t lim = (int64_t)1 << (l - 1);
-                const int nd = dim == 2 ? 9 : 27;
-                for (int u = 0; u < nd; ++u) {
-                    int64_t pn[3] = {ct[0] / 2 + (u % 3) - 1, ct[1] / 2 + (u / 3) % 3 - 1,
-                                     dim == 3 ? ct[2] / 2 + u / 9 - 1 : 0};
-                    bool ok = true;
-                    for (int d = 0; d < dim; ++d) ok = ok && pn[d] >= 0 && pn[d] < lim;
-                    if (!ok) continue;
-                    for (int o = 0; o < (1 << dim); ++o) {
-                        int64_t cc[3] = {0, 0, 0};
-                        int64_t far = 0;
-                        for (int d = 0; d < dim; ++d) {
-                            cc[d] = 2 * pn[d] + ((o >> d) & 1);
-                            far = std::max<int64_t>(far, (int64_t)std::llabs(cc[d] - ct[d]));
-                        }
-                        if (far <= 1) continue;
-                        auto it = index[l].find(morton(dim, cc));
-                        if (it == index[l].end()) continue;
-                        int code = 0, mul = 1;
-                        for (int d = 0; d < dim; ++d, mul *= 7) code += (int)(cc[d] - ct[d] + 3) * mul;
-                        il_src.push_back(it->second);
-                        il_off.push_back((int16_t)code);
-                    }
+    // interaction lists (levels >= 2) and near lists (leaves).  A box's candidates are the children
+    // (o) of its parent's neighbours (u); for boxes of one octant the same (u, o) are adjacent, so
+    // the others, in order, are the octant's slots.
+    const int noct = 1 << dim, nu = dim == 2 ? 9 : 27;
+    f->nslots = dim == 2 ? 27 : 189;
+    std::vector<int16_t> slot_off((size_t)noct * f->nslots);
+    std::vector<int> slot_of((size_t)noct * nu * noct, -1);
+    for (int t = 0; t < noct; ++t) {
+        int sl = 0;
+        for (int u = 0; u < nu; ++u)
+            for (int o = 0; o < noct; ++o) {
+                int far = 0, code = 0, mul = 1;
+                for (int d = 0; d < dim; ++d, mul *= 7) {
+                    const int pn = (d == 0 ? u % 3 : d == 1 ? (u / 3) % 3 : u / 9) - 1;
+                    const int off = 2 * pn + ((o >> d) & 1) - ((t >> d) & 1);
+                    far = std::max(far, std::abs(off));
+                    code += (off + 3) * mul;
                 }
+                if (far <= 1) continue;
+                slot_off[(size_t)t * f->nslots + sl] = (int16_t)code;
+                slot_of[((size_t)t * nu + u) * noct + o] = sl++;
             }
-            il_start[gi + 1] = (int32_t)il_src.size();
+    }
+    std::vector<int32_t> m2l_box;
+    std::vector<int8_t> m2l_level;
+    for (int t = 0; t < noct; ++t) {
+        f->oct_first[t] = (int32_t)m2l_box.size();
+        for (int l = 2; l <= L; ++l)
+            for (int64_t gi = f->lvl0[l]; gi < f->lvl0[l + 1]; ++gi)
+                if (octant[gi] == t) {
+                    m2l_box.push_back((int32_t)gi);
+                    m2l_level.push_back((int8_t)l);
+                }
+    }
+    f->oct_first[noct] = (int32_t)m2l_box.size();
+    f->nm2l = (int64_t)m2l_box.size();
+    std::vector<int32_t> m2l_src((size_t)f->nslots * f->nm2l, -1);
+    for (int64_t q = 0; q < f->nm2l; ++q) {
+        const int l = m2l_level[q], t = octant[m2l_box[q]];
+        int64_t ct[3] = {0, 0, 0};
+        unmorton(dim, keys[l][m2l_box[q] - f->lvl0[l]], ct);
+        const int64_t lim = (int64_t)1 << (l - 1);
+        for (int u = 0; u < nu; ++u) {
+            int64_t pn[3] = {ct[0] / 2 + (u % 3) - 1, ct[1] / 2 + (u / 3) % 3 - 1, dim == 3 ? ct[2] / 2 + u / 9 - 1 : 0};
+            bool ok = true;
+            for (int d = 0; d < dim; ++d) ok = ok && pn[d] >= 0 && pn[d] < lim;
+            if (!ok) continue;
+            for (int o = 0; o < noct; ++o) {
+                const int sl = slot_of[((size_t)t * nu + u) * noct + o];
+                if (sl < 0) continue;
+                int64_t cc[3] = {0, 0, 0};
+                for (int d = 0; d < dim; ++d) cc[d] = 2 * pn[d] + ((o >> d) & 1);
+                auto it = index[l].find(morton(dim, cc));
+                if (it == index[l].end()) continue;
+                m2l_src[(size_t)sl * f->nm2l + q] = it->second;
+                ++f->nil;
+            }
         }
-    f->nil = (int64_t)il_src.size();
+    }
     std::vector<int32_t> near_start(f->nleaf + 1, 0), near_leaf;
     std::vector<int8_t> near_delta;
     for (int64_t q = 0; q < f->nleaf; ++q) {
@@ -619,7 +716,8 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
     auto node = [&](int m, int d) {   // per-dimension node index of node m
         return dim == 2 ? (d == 0 ? m / p : m % p) : (d == 0 ? m / (p * p) : d == 1 ? (m / p) % p : m % p);
     };
-    std::vector<float> T((size_t)(1 << dim) * P * P);
+    const int Pp = (P + 7) / 8 * 8;   // rows of the node tables, in groups of 8
+    std::vector<float> Tm((size_t)(1 << dim) * P * Pp, 0.f), Tl((size_t)(1 << dim) * P * Pp, 0.f);
     {
         std::vector<double> S1((size_t)2 * p * p);   // [bit][parent node][child node]
         std::vector<double> w(p);
@@ -633,7 +731,8 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
                 for (int mc = 0; mc < P; ++mc) {
                     double v = 1.0;
                     for (int d = 0; d < dim; ++d) v *= S1[((size_t)((o >> d) & 1) * p + node(m, d)) * p + node(mc, d)];
-                    T[((size_t)o * P + m) * P + mc] = (float)v;
+                    Tm[((size_t)o * P + mc) * Pp + m] = (float)v;
+                    Tl[((size_t)o * P + m) * Pp + mc] = (float)v;
                 }
     }
     const int noff = dim == 2 ? 49 : 343;
@@ -661,13 +760,15 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
     WFQ_TRY(upload(ctx, f, &f->child_lo, child_lo));
     WFQ_TRY(upload(ctx, f, &f->child_hi, child_hi));
     WFQ_TRY(upload(ctx, f, &f->octant, octant));
-    WFQ_TRY(upload(ctx, f, &f->il_start, il_start));
-    WFQ_TRY(upload(ctx, f, &f->il_src, il_src));
-    WFQ_TRY(upload(ctx, f, &f->il_off, il_off));
+    WFQ_TRY(upload(ctx, f, &f->m2l_box, m2l_box));
+    WFQ_TRY(upload(ctx, f, &f->m2l_level, m2l_level));
+    WFQ_TRY(upload(ctx, f, &f->m2l_src, m2l_src));
+    WFQ_TRY(upload(ctx, f, &f->slot_off, slot_off));
     WFQ_TRY(upload(ctx, f, &f->near_start, near_start));
     WFQ_TRY(upload(ctx, f, &f->near_leaf, near_leaf));
     WFQ_TRY(upload(ctx, f, &f->near_delta, near_delta));
-    WFQ_TRY(upload(ctx, f, &f->T, T));
+    WFQ_TRY(upload(ctx, f, &f->Tm, Tm));
+    WFQ_TRY(upload(ctx, f, &f->Tl, Tl));
     WFQ_TRY(upload(ctx, f, &f->K, K));
     WFQ_TRY(upload(ctx, f, &f->cheb, cheb));
     *out = guard.release();
@@ -677,49 +778,77 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
 int d_apply_fmm(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, cudaStream_t s) {
     const Fmm *f = g->fmm;
     if (!f) return fail(WFQ_EUNSUPPORTED, "WFQ_PREC_FMM needs wfq_fmm_build on this geometry first");
-    const int64_t C = 2 * cc;
+    const int64_t C = 2 * cc, Cp = round_up(C, 4), n = g->n;   // internal rows are padded to 16 bytes
     const FmmDev fd = dev_view(f);
-    const float *Xf = reinterpret_cast<const float *>(X);
-    float *Uf = reinterpret_cast<float *>(U);
-    KScope ks(g->ctx, WFQ_KT_FMM, s, (double)g->n * (double)g->n);
-    DevBuf<float> M, Lc;
-    const int L = f->L;
+    KScope ks(g->ctx, WFQ_KT_FMM, s, (double)n * (double)n);
+    DevBuf<float> M, Lc, Xs;
+    const int L = f->L, P = f->P, Pp = (P + 7) / 8 * 8;
+    const unsigned cols32 = (unsigned)((Cp + 31) / 32);
+    const unsigned node_threads = 32u * (unsigned)std::min(8, (P + 7) / 8);   // M2M, L2L: a warp per 8 nodes
+    WFQ_TRY(Xs.alloc(g->ctx, (size_t)n * Cp, s));
+    k_fmm_sort_x<<<(unsigned)((n * Cp + 255) / 256), 256, 0, s>>>(n, C, Cp, fd.perm, reinterpret_cast<const float *>(X), Xs.ptr);
+    note_launch();
+    WFQ_CUDA(cudaGetLastError());
     if (L >= 2) {
-        const size_t per = (size_t)f->nbox * f->P * C;
+        const size_t per = (size_t)f->nbox * P * Cp;
         WFQ_TRY(M.alloc(g->ctx, per, s));
         WFQ_TRY(Lc.alloc(g->ctx, per, s));
-        const size_t p2m_smem = sizeof(float) * (32 * 3 * kMaxP + 32 * C);
+        const size_t p2m_smem = sizeof(float) * (32 * 3 * kMaxP + 32 * Cp);
         if (p2m_smem > 48 * 1024)
             WFQ_CUDA(cudaFuncSetAttribute(k_fmm_p2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2m_smem));
-        k_fmm_p2m<<<(unsigned)f->nleaf, 128, p2m_smem, s>>>(fd, C, Xf, M.ptr);
+        k_fmm_p2m<<<(unsigned)f->nleaf, 128, p2m_smem, s>>>(fd, Cp, Xs.ptr, M.ptr);
         note_launch();
         WFQ_CUDA(cudaGetLastError());
         for (int l = L - 1; l >= 2; --l) {
-            k_fmm_m2m<<<(unsigned)(f->lvl0[l + 1] - f->lvl0[l]), 128, 0, s>>>(fd, C, f->lvl0[l], M.ptr);
+            k_fmm_m2m<<<dim3((unsigned)(f->lvl0[l + 1] - f->lvl0[l]), cols32), node_threads, 0, s>>>(fd, Pp, Cp, f->lvl0[l], M.ptr);
             note_launch();
         }
-        LevelTable lv{};
-        for (int l = 0; l <= L + 1 && l < 24; ++l) lv.first[l] = f->lvl0[l];
-        for (int l = 0; l <= L && l < 24; ++l) lv.inv_a[l] = (float)(2.0 * std::ldexp(1.0, l) / f->side);
-        const size_t m2l_smem = sizeof(float) * ((size_t)f->P * M2L_KC + M2L_KC * M2L_CB);
-        if (m2l_smem > 48 * 1024)
-            WFQ_CUDA(cudaFuncSetAttribute(k_fmm_m2l, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m2l_smem));
-        const int m2l_threads = ((f->P + 3) / 4) * (M2L_CB / 4);
-        dim3 grid((unsigned)(f->nbox - f->lvl0[2]), (unsigned)((C + M2L_CB - 1) / M2L_CB));
-        k_fmm_m2l<<<grid, m2l_threads, m2l_smem, s>>>(fd, C, lv, M.ptr, Lc.ptr);
+        // lanes per box: the columns of a block rounded up to a power of two
+        int lpb = 4;
+        while (lpb < Cp && lpb < 32) lpb *= 2;
+        const int noct = 1 << f->dim, bpb = M2L_WARPS * M2L_NB * (32 / lpb);
+        M2lGrid gr{};
+        int tiles = 0;
+        for (int t = 0; t < noct; ++t) {
+            gr.first[t] = f->oct_first[t];
+            gr.tile[t] = tiles;
+            tiles += (f->oct_first[t + 1] - f->oct_first[t] + bpb - 1) / bpb;
+        }
+        gr.first[noct] = f->oct_first[noct];
+        for (int l = 0; l <= L && l < 24; ++l) gr.inv_a[l] = (float)(2.0 * std::ldexp(1.0, l) / f->side);
+        // target nodes per block: the choice with the fewest padded nodes, wider first
+        int best = 18;
+        for (int rp : {16, 13, 8})
+            if (round_up(P, 2 * rp) < round_up(P, 2 * best)) best = rp;
+        const dim3 grid((unsigned)tiles, cols32, (unsigned)((P + 2 * best - 1) / (2 * best)));
+        const size_t sm = sizeof(float) * (size_t)P * 2 * best;   // at most 256 x 36 floats
+        const unsigned th = 32 * M2L_WARPS;
+        switch (best) {
+            case 18: k_fmm_m2l<18><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
+            case 16: k_fmm_m2l<16><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
+            case 13: k_fmm_m2l<13><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
+            default: k_fmm_m2l<8><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
+        }
         note_launch();
         WFQ_CUDA(cudaGetLastError());
         for (int l = 3; l <= L; ++l) {
-            k_fmm_l2l<<<(unsigned)(f->lvl0[l + 1] - f->lvl0[l]), 128, 0, s>>>(fd, C, f->lvl0[l], Lc.ptr);
+            k_fmm_l2l<<<dim3((unsigned)(f->lvl0[l + 1] - f->lvl0[l]), cols32), node_threads, 0, s>>>(fd, Pp, Cp, f->lvl0[l], Lc.ptr);
             note_launch();
         }
         WFQ_CUDA(cudaGetLastError());
     }
-    const size_t nf_smem = sizeof(float) * (5 * NF_SCH + (size_t)NF_SCH * C);
-    if (nf_smem > 48 * 1024)
-        WFQ_CUDA(cudaFuncSetAttribute(k_fmm_l2p_near, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nf_smem));
-    k_fmm_l2p_near<<<(unsigned)f->nleaf, 256, nf_smem, s>>>(fd, C, L >= 2 ? 1 : 0, Xf, L >= 2 ? Lc.ptr : nullptr,
-                                                            Uf);
+    // columns per thread: 32, or the fewest multiple of 4 that holds them
+    const unsigned nl4 = (unsigned)((f->nleaf + 3) / 4);
+    const int far = L >= 2 ? 1 : 0;
+    float *Uf = reinterpret_cast<float *>(U);
+    if (Cp > 16)
+        k_fmm_l2p_near<8><<<dim3(nl4, cols32), 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
+    else if (Cp > 8)
+        k_fmm_l2p_near<4><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
+    else if (Cp > 4)
+        k_fmm_l2p_near<2><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
+    else
+        k_fmm_l2p_near<1><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

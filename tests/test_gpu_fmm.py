@@ -140,3 +140,30 @@ def test_fmm_disk1m_sampled_rows_against_exact_rows(W, ctx, orc, S):
         print(f"disk1m order 6, column {c}: max |fmm - exact| / bound {ratio.max():.2e}")
         assert ratio.max() <= 1e-6
     g.close()
+
+
+@pytest.mark.parametrize("flat,orders", [(True, (2, 3, 5, 7)), (False, (2, 3, 4, 5))])
+def test_fmm_columns_do_not_depend_on_their_block(flat, orders):
+    """Every pass treats its columns alike: a block of 17 columns (odd groups of lanes, padded
+    rows, two blocks of columns) and its first 1, 3 and 9 columns agree to the last bit, at
+    orders whose nodes per box leave remainders in the node tiles."""
+    import torch  # noqa: F401
+    from paper_2103_00438_gb300 import structures as S, wfq
+    ctx = wfq.Context(0)
+    xyz = S.graphene_disk(9.0, 0.01, seed=3) if flat else S.nanotube(10, 10, 60)
+    g = wfq.Geometry(ctx, xyz, S.carbon_params(1.84), store=0)
+    om = np.linspace(0.01, 0.1, 17)
+    x = S.random_complex((len(xyz), 17), seed=8).astype(np.complex64)
+    for order in orders:
+        g.fmm_build(order)
+        full = np.empty_like(x)
+        g.apply(om, x, full, prec=wfq.PREC_FMM)
+        for c in (1, 3, 9):
+            y = np.empty((len(xyz), c), dtype=np.complex64)
+            g.apply(om[:c], np.ascontiguousarray(x[:, :c]), y, prec=wfq.PREC_FMM)
+            if c > 4:   # 1 to 4 columns sum the neighbour term across lanes, in another order
+                assert np.array_equal(y, full[:, :c]), (order, c)
+            else:
+                assert np.abs(y - full[:, :c]).max() <= 2e-6 * np.abs(full).max(), (order, c)
+    g.close()
+    ctx.close()
