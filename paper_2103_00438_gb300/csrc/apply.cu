@@ -494,37 +494,56 @@ struct CplxT<float2> {
     using R = float;
 };
 
-// Many columns: one warp per atom row, lanes over complex columns.
+// Many columns: lpc lanes (a power of two, at most 32) per atom row over complex columns, so a
+// warp covers 32 / lpc rows; blockIdx.y: chunk of lpc columns.  A block's rows are consecutive
+// and work on the same columns, so that the neighbours they share come from L1, and four
+// neighbours are gathered at a time.  FP32, us: 20000-atom tube x 192 columns 128 (140 with a
+// warp looping over the chunks of a row), 250k-atom disk x 16 135 (271).  FP64 is bound by the FP64
+// pipe (4 operations per neighbour and column): 1365 for the tube.
 // Y_i = sum_p Kbar_ip (U_j - U_i) - z X_i  (the difference form of Kbar U - P U).
 template <class V, class VAL>
-__global__ void __launch_bounds__(128) k_sparse_cols(int64_t n, int64_t cc,
+__global__ void __launch_bounds__(512) k_sparse_cols(int64_t n, int64_t cc, int lpc,
                                                      const int64_t *__restrict__ rowptr,
                                                      const int32_t *__restrict__ col,
                                                      const VAL *__restrict__ val,
                                                      const V *__restrict__ U, const V *__restrict__ X,
                                                      const double2 *__restrict__ z, V *__restrict__ Y) {
     using R = typename CplxT<V>::R;
-    int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (i >= n) return;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lpc;
+    const int64_t c = (int64_t)blockIdx.y * lpc + (threadIdx.x & (lpc - 1));
+    if (i >= n || c >= cc) return;
     const int64_t p0 = rowptr[i], p1 = rowptr[i + 1];
-    for (int64_t c = lane; c < cc; c += 32) {
-        V ui = U[i * cc + c];
-        R ax = 0, ay = 0;
-        for (int64_t p = p0; p < p1; ++p) {
-            R w = (R)val[p];
-            V uj = U[(int64_t)col[p] * cc + c];
-            ax += w * (uj.x - ui.x);
-            ay += w * (uj.y - ui.y);
+    const V *Uc = U + c;
+    const V ui = Uc[i * cc];
+    R ax = 0, ay = 0;
+    int64_t p = p0;
+    for (; p + 4 <= p1; p += 4) {
+        R w[4];
+        V u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            w[q] = (R)val[p + q];
+            u[q] = Uc[(int64_t)col[p + q] * cc];
         }
-        V xv = X[i * cc + c];
-        double2 zc = z[c];
-        R zr = (R)zc.x, zi = (R)zc.y;
-        V out;
-        out.x = ax - (zr * xv.x - zi * xv.y);
-        out.y = ay - (zr * xv.y + zi * xv.x);
-        Y[i * cc + c] = out;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            ax += w[q] * (u[q].x - ui.x);
+            ay += w[q] * (u[q].y - ui.y);
+        }
     }
+    for (; p < p1; ++p) {
+        const R w = (R)val[p];
+        const V uj = Uc[(int64_t)col[p] * cc];
+        ax += w * (uj.x - ui.x);
+        ay += w * (uj.y - ui.y);
+    }
+    const V xv = X[i * cc + c];
+    const double2 zc = z[c];
+    const R zr = (R)zc.x, zi = (R)zc.y;
+    V out;
+    out.x = ax - (zr * xv.x - zi * xv.y);
+    out.y = ay - (zr * xv.y + zi * xv.x);
+    Y[i * cc + c] = out;
 }
 
 // Few columns (cc <= 4): one warp per atom row, lanes over neighbours.
@@ -615,8 +634,12 @@ static int sparse_shift_impl(const wfq_geom *g, int64_t cc, const V *U, const V 
         case 2: k_sparse_nbrs<V, VAL, 2><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
         case 3: k_sparse_nbrs<V, VAL, 3><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
         case 4: k_sparse_nbrs<V, VAL, 4><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
-        default:
-            k_sparse_cols<V, VAL><<<blocks, 128, 0, s>>>(n, cc, g->rowptr, g->col, val, U, X, z, Y); note_launch();
+        default: {
+            int lpc = 8;
+            while (lpc < cc && lpc < 32) lpc *= 2;
+            const dim3 grid((unsigned)((n * lpc + 511) / 512), (unsigned)((cc + lpc - 1) / lpc));
+            k_sparse_cols<V, VAL><<<grid, 512, 0, s>>>(n, cc, lpc, g->rowptr, g->col, val, U, X, z, Y); note_launch();
+        }
     }
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

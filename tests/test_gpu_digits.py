@@ -158,3 +158,18 @@ def test_hardnesses_far_apart_keep_the_double_float_product(W, ctx, orc, S):
         z = np.array([orc.z_of_omega(w, p) for w in om])
         assert np.all(np.abs(y[i] - ref[i]) <= tau * ((k * (s[q] + s[i])).sum(axis=0) + np.abs(z) * np.abs(x[i])))
 
+
+@pytest.mark.parametrize("ncplx", [5, 8, 9, 16, 17, 32])
+def test_sparse_term_columns_do_not_depend_on_their_block(W, ctx, S, ncplx):
+    """The digit products are exact per column, so an FP64 block of 33 columns and its first
+    ncplx agree to the last bit if the neighbour term's lane layouts (8, 16, 32 columns per row,
+    chunks) do."""
+    n = 341
+    xyz = S.random_cluster(n, seed=21)
+    g = W.Geometry(ctx, xyz, S.sodium_params(), store=W.STORE_FP64)
+    om = np.linspace(0.01, 0.1, 33)
+    x = S.random_complex((n, 33), seed=2)
+    full, part = np.empty_like(x), np.empty((n, ncplx), dtype=complex)
+    g.apply(om, x, full, prec=W.PREC_FP64)
+    g.apply(om[:ncplx], np.ascontiguousarray(x[:, :ncplx]), part, prec=W.PREC_FP64)
+    assert np.array_equal(part, full[:, :ncplx])
