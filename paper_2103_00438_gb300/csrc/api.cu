@@ -173,7 +173,7 @@ static int galloc(wfq_geom *g, T **p, size_t count) {
 }
 
 static void free_geom(wfq_geom *g) {
-    void *ptrs[] = {g->xyz, g->atom64, g->atom32, g->atom32p, g->atomdf, g->eta, g->dexp, g->rowptr, g->col,
+    void *ptrs[] = {g->xyz, g->atom64, g->atom32, g->atom32p, g->atomdf, g->eta, g->rowptr, g->col,
                     g->val64, g->val32, g->D64, g->Dhi, g->Dlo, g->Dfh, g->Dfl,
                     g->Dsym, g->sym_items, g->sym_item_start, g->elem};
     for (void *p : ptrs)
@@ -423,8 +423,12 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
     if ((rc = galloc(g, &g->atom32, g->npad))) return bail(rc);
     if ((rc = galloc(g, &g->atom32p, g->npad))) return bail(rc);
     if ((rc = galloc(g, &g->atomdf, 2 * n))) return bail(rc);
-    if ((rc = galloc(g, &g->eta, n))) return bail(rc);
-    if (!dexp.empty() && (rc = galloc(g, &g->dexp, n))) return bail(rc);
+    // eta, then the row exponents, in one allocation and one upload
+    std::vector<double> eta_up((size_t)n + (dexp.size() + 1) / 2, 0.0);
+    std::copy(eta_h.begin(), eta_h.end(), eta_up.begin());
+    if (!dexp.empty()) std::memcpy(eta_up.data() + n, dexp.data(), sizeof(int) * n);
+    if ((rc = galloc(g, &g->eta, eta_up.size()))) return bail(rc);
+    if (!dexp.empty()) g->dexp = reinterpret_cast<int *>(g->eta + n);
     if ((rc = galloc(g, &g->rowptr, n + 1))) return bail(rc);
     if ((rc = galloc(g, &g->col, g->nnz))) return bail(rc);
     if ((rc = galloc(g, &g->val64, g->nnz))) return bail(rc);
@@ -477,8 +481,7 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
         if ((rc = up(g->atom32p, a32p.data(), sizeof(float4) * g->npad))) return bail(rc);
     }
     if ((rc = up(g->atomdf, adf.data(), sizeof(float4) * 2 * n))) return bail(rc);
-    if ((rc = up(g->eta, eta_h.data(), sizeof(double) * n))) return bail(rc);
-    if ((rc = up(g->dexp, dexp.data(), sizeof(int) * dexp.size()))) return bail(rc);
+    if ((rc = up(g->eta, eta_up.data(), sizeof(double) * eta_up.size()))) return bail(rc);
     if ((rc = up(g->rowptr, rowptr.data(), sizeof(int64_t) * (n + 1)))) return bail(rc);
     if ((rc = up(g->col, col.data(), sizeof(int32_t) * g->nnz))) return bail(rc);
     if ((rc = up(g->val64, val.data(), sizeof(double) * g->nnz))) return bail(rc);
@@ -542,8 +545,8 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     };
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);
     if ((rc = galloc(g, &g->elem, n))) return bail(rc);
-    if ((rc = galloc(g, &g->dexp, n))) return bail(rc);
-    if ((rc = galloc(g, &g->rowptr, n + 1))) return bail(rc);   // empty sparse term
+    if ((rc = galloc(g, &g->rowptr, (n + 1) + (n + 1) / 2))) return bail(rc);   // empty sparse term, row exponents
+    g->dexp = reinterpret_cast<int *>(g->rowptr + n + 1);
     if ((rc = galloc(g, &g->D64, (size_t)n * n))) return bail(rc);
     if (store & WFQ_STORE_BF16X2) {
         if ((rc = galloc(g, &g->Dhi, (size_t)g->npad * g->npad))) return bail(rc);
@@ -569,8 +572,7 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     if (e == cudaSuccess) e = cudaMemcpy(g->elem, el.data(), sizeof(elem64_t) * n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(g->rowptr, 0, sizeof(int64_t) * (n + 1));
     if (e == cudaSuccess) e = cudaMemset(close, 0, sizeof(int));
-    std::vector<int> dexp(n, kDexpNone);
-    if (e == cudaSuccess) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(g->dexp, 0x80, sizeof(int) * n);   // kDexpNone
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
     if ((rc = launch_build_bem(g, close, nullptr))) return done(rc);
     int close_h = 0;
@@ -578,11 +580,16 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM build: ") + cudaGetErrorString(e)));
     if (close_h) return done(fail(WFQ_EINVAL, "two surface elements closer than 1e-8 bohr"));
     // row exponents: a row of zeros (possible on a flat surface) takes any scale
+    std::vector<int> dexp(n);
     e = cudaMemcpy(dexp.data(), g->dexp, sizeof(int) * n, cudaMemcpyDeviceToHost);
+    bool none = false;
     for (int64_t i = 0; i < n; ++i)
-        if (dexp[i] == kDexpNone) dexp[i] = 0;
+        if (dexp[i] == kDexpNone) {
+            dexp[i] = 0;
+            none = true;
+        }
     set_exponent_range(g, dexp);
-    if (e == cudaSuccess) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && none) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM row exponents: ") + cudaGetErrorString(e)));
     done(WFQ_OK);
     *out = g;

@@ -170,6 +170,7 @@ struct wfq_geom {
     float4 *atomdf = nullptr;   // 2 per atom: (xh, xl, yh, yl), (zh, zl, width, 0) float pairs
     double *eta = nullptr;      // n
     int *dexp = nullptr;        // n, stored FP64 D, FP32 planes or tiles: |D_ij| < 2^dexp[i]
+                                // (in the allocation of eta, of rowptr for BEM geometries)
     int dexp_min = 0, dexp_max = 0;
     bool digits_ok = false;     // every dexp within +-kDigitExpMax (the digit-slice products)
     wfq::elem64_t *elem = nullptr;   // BEM geometries: n element records
@@ -251,7 +252,7 @@ int launch_build_d(const wfq_geom *g, cudaStream_t s);
 // BEM geometries: the operator's entries into the requested storages; *close is set
 // non-zero (device int) when two elements lie closer than 1e-8 bohr.  Also g->dexp, each
 // row's largest exponent (kDexpNone for a row of zeros).
-constexpr int kDexpNone = -2000;
+constexpr int kDexpNone = -0x7f7f7f80;   // bytes of 0x80
 int launch_build_bem(const wfq_geom *g, int *close, cudaStream_t s);
 int launch_rhs(const wfq_geom *g, int ndir, const double *dirs_dev, double E0, double *R,
                cudaStream_t s);
