@@ -9,12 +9,14 @@ namespace wfq {
 
 // ------------------------------------------------------------------ FP64 stored D: few columns
 
-// U[i][:] = sum_k D[i][k] X[k][:] for C real columns (C <= 8): each warp owns 4 rows so
-// that every X element read from L2 serves 4 D rows; D rows are read coalesced.
-template <int C>
+// U[i][:] = sum_k D[i][k] X[k][:] for C real columns (C <= 8): each warp owns RW rows so
+// that every X element read from L2 serves RW D rows; D rows are read coalesced.  Bound by the
+// FP64 pipe (1.7 operations per clock per SM), so below 9728 atoms, where 4 rows a warp would
+// leave SMs idle, a warp takes 1 or 2: 1014 atoms, C = 2: 9.5 us, 26.2 with 4 rows.  The order of
+// a row's sum does not depend on RW.
+template <int C, int RW>
 __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restrict__ D,
                                                const double *__restrict__ X, double *__restrict__ U) {
-    constexpr int RW = 4;
     int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     int64_t i0 = warp * RW;
@@ -442,23 +444,37 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     return digits_product(g, 7, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), bad.ptr, s);
 }
 
+template <int C>
+static void launch_dgemv64(int64_t n, const double *D, const double *x, double *u, cudaStream_t s) {
+    auto blocks = [&](int rw) { return (unsigned)(((n + rw - 1) / rw + 7) / 8); };
+    if (n >= 9728)   // 16 warps an SM on 152 SMs
+        k_dgemv<C, 4><<<blocks(4), 256, 0, s>>>(n, D, x, u);
+    else if (n >= 4864)
+        k_dgemv<C, 2><<<blocks(2), 256, 0, s>>>(n, D, x, u);
+    else
+        k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u);
+}
+
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s) {
     const int64_t n = g->n, C = 2 * cc;
+    // The FP64 GEMV takes about 2e-6 n^2 C us (FP64 pipe), the digit slices 45 + 4e-6 n^2 whatever
+    // C is up to 32: from 2 columns and 4096 atoms on the latter (6000 atoms, 2 columns: 188 against
+    // 435 us per apply; 10000 atoms, 4 columns: 463 against 2017).
+    const bool few_by_digits = g->digits_ok && C >= 4 && n >= 4096;
     // no FP64 D but stored float pairs: their double-float product (2^-48 per product, on
     // the FP32 pipes and at 8 or 4 bytes per entry) instead of regenerating D in FP64
     if (!g->D64 && (g->Dfh || g->Dsym) && C <= 8) return d_apply_pairs_df(g, cc, X, U, s);
     const double *x = reinterpret_cast<const double *>(X);
     double *u = reinterpret_cast<double *>(U);
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-    if (g->D64 && C <= 8) {
-        int64_t warps = (n + 3) / 4;
-        unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
+    if (g->D64 && C <= 8 && !few_by_digits) {
         switch (C) {
-            case 2: k_dgemv<2><<<blocks, 256, 0, s>>>(n, g->D64, x, u); note_launch(); break;
-            case 4: k_dgemv<4><<<blocks, 256, 0, s>>>(n, g->D64, x, u); note_launch(); break;
-            case 6: k_dgemv<6><<<blocks, 256, 0, s>>>(n, g->D64, x, u); note_launch(); break;
-            default: k_dgemv<8><<<blocks, 256, 0, s>>>(n, g->D64, x, u); note_launch(); break;
+            case 2: launch_dgemv64<2>(n, g->D64, x, u, s); break;
+            case 4: launch_dgemv64<4>(n, g->D64, x, u, s); break;
+            case 6: launch_dgemv64<6>(n, g->D64, x, u, s); break;
+            default: launch_dgemv64<8>(n, g->D64, x, u, s); break;
         }
+        note_launch();
     } else {
         dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
         if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "FP64 apply: too many rows");

@@ -274,14 +274,32 @@ __device__ void givens_step(const GmresDev &st, int64_t c, int j) {
     const int m = st.m;
     const int64_t na = st.na;
     auto Hp = [&](int i, int jj) { return st.H + ((int64_t)i * m + jj) * na + c; };
-    for (int i = 0; i < j; ++i) {
+    // The rotations' loads do not depend on the chain, so they are issued eight at a time ahead
+    // of it (one at a time each step of the chain waited for three loads).
+    double2 a = *Hp(0, j);
+    int i = 0;
+    for (; i + 8 <= j; i += 8) {
+        double csr[8];
+        double2 snr[8], hr[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            csr[u] = st.cs[(int64_t)(i + u) * na + c];
+            snr[u] = st.sn[(int64_t)(i + u) * na + c];
+            hr[u] = *Hp(i + u + 1, j);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            *Hp(i + u, j) = cadd(cscale(csr[u], a), cmul(snr[u], hr[u]));
+            a = csub(cscale(csr[u], hr[u]), cjmul(snr[u], a));
+        }
+    }
+    for (; i < j; ++i) {
         const double cs = st.cs[(int64_t)i * na + c];
         const double2 sn = st.sn[(int64_t)i * na + c];
-        const double2 a = *Hp(i, j), b = *Hp(i + 1, j);
+        const double2 b = *Hp(i + 1, j);
         *Hp(i, j) = cadd(cscale(cs, a), cmul(sn, b));
-        *Hp(i + 1, j) = csub(cscale(cs, b), cjmul(sn, a));
+        a = csub(cscale(cs, b), cjmul(sn, a));
     }
-    const double2 a = *Hp(j, j);
     const double hb = Hp(j + 1, j)->x;  // a norm: real, >= 0
     const double na_ = sqrt(cabs2(a));
     const double nu = sqrt(na_ * na_ + hb * hb);
@@ -481,18 +499,30 @@ __global__ void k_cycle_cols(int64_t na, const double2 *__restrict__ rnorm, doub
     st.target[c] = fmax(0.5 * tol * bnorm_a[c], inner_red * rn);
 }
 
-// y = R^{-1} g on the first jd rows (R = rotated H); one thread per column
-__global__ void k_backsolve(int64_t na, int jlast, GmresDev st, double2 *__restrict__ y) {
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= na) return;
+// y = R^{-1} g on the first jd rows (R = rotated H), a warp per column, column by column from the
+// last: y_k = y_k / R_kk, then y_l -= R_lk y_k for l < k, lane l mod 32 owning y_l.  (A thread per
+// column waited for two loads per entry: 357 us for 49 steps of one column, 74 now.)
+__global__ void __launch_bounds__(128) k_backsolve(int64_t na, int jlast, GmresDev st, double2 *__restrict__ y) {
+    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (c >= na) return;   // whole warp
     const int m = st.m;
     const int jd = st.done[c] ? st.jdone[c] : (jlast + 1);
-    st.jdone[c] = jd;
-    for (int l = jd - 1; l >= 0; --l) {
-        double2 s = st.g[(int64_t)l * na + c];
-        for (int k = l + 1; k < jd; ++k) s = csub(s, cmul(st.H[((int64_t)l * m + k) * na + c], y[(int64_t)k * na + c]));
-        y[(int64_t)l * na + c] = cdiv(s, st.H[((int64_t)l * m + l) * na + c]);
+    for (int l = lane; l < jd; l += 32) y[(int64_t)l * na + c] = st.g[(int64_t)l * na + c];
+    for (int k = jd - 1; k >= 0; --k) {
+        const int owner = k & 31;
+        double2 yk = czero();
+        if (lane == owner) {
+            yk = cdiv(y[(int64_t)k * na + c], st.H[((int64_t)k * m + k) * na + c]);
+            y[(int64_t)k * na + c] = yk;
+        }
+        yk.x = __shfl_sync(0xffffffffu, yk.x, owner);
+        yk.y = __shfl_sync(0xffffffffu, yk.y, owner);
+        for (int l = lane; l < k; l += 32)
+            y[(int64_t)l * na + c] = csub(y[(int64_t)l * na + c], cmul(st.H[((int64_t)l * m + k) * na + c], yk));
     }
+    __syncwarp();
+    if (lane == 0) st.jdone[c] = jd;
 }
 
 __global__ void k_set_z(int64_t cc, const double *__restrict__ col_omega, ShiftModel zm,
@@ -880,6 +910,9 @@ static int gmres_impl(wfq_geom *g, const SolveArgs &a, cudaStream_t s, GmresOut 
         k_start_basis<VT><<<nblocks(tot), 256, 0, s>>>(tot, (uint32_t)na, cm.ra.ptr, cm.rnorm.ptr, done.ptr, V.ptr); note_launch();
         WFQ_CUDA(cudaGetLastError());
         const RowSplit rs = row_split(n, na, cm.num_sms);
+        // small blocks where larger ones would leave SMs idle: a complex128 projection is bound
+        // by the FP64 pipe (1014 atoms x 1 column: 9.3 us with 32, 13.9 with 256 threads)
+        const int pb = tot < 256u * 2u * (uint32_t)cm.num_sms ? 32 : 256;
         int jlast = -1;
         done_h.assign(na, 0);
         for (int j = 0; j < m && total < a.max_iter; ++j) {
@@ -908,7 +941,7 @@ static int gmres_impl(wfq_geom *g, const SolveArgs &a, cudaStream_t s, GmresOut 
                                                                            cm.tmp.ptr, st, j); note_launch();
                     const double2 *coef = pass == 0 ? hcol : cm.tmp.ptr;
                     const int64_t cstride = pass == 0 ? (int64_t)m * na : na;
-                    k_project<VT><<<nblocks(tot), 256, 0, s>>>(tot, (uint32_t)na, nv, V.ptr + (int64_t)i0 * vstride,
+                    k_project<VT><<<nblocks(tot, pb), pb, 0, s>>>(tot, (uint32_t)na, nv, V.ptr + (int64_t)i0 * vstride,
                                                                vstride, coef, cstride, w); note_launch();
                 }
             }
@@ -925,9 +958,7 @@ static int gmres_impl(wfq_geom *g, const SolveArgs &a, cudaStream_t s, GmresOut 
             if (std::all_of(done_h.begin(), done_h.end(), [](int v) { return v != 0; })) break;
         }
         if (jlast >= 0) {
-            // one thread per column, a serial FP64 chain each: spread over many SMs (few FP64
-            // units per SM on GB300)
-            k_backsolve<<<nblocks(na, 4), 4, 0, s>>>(na, jlast, st, y.ptr); note_launch();
+            k_backsolve<<<nblocks(na * 32, 128), 128, 0, s>>>(na, jlast, st, y.ptr); note_launch();
             k_combine<VT><<<nblocks(tot), 256, 0, s>>>(tot, (uint32_t)na, jlast + 1, V.ptr, vstride, y.ptr, jdone.ptr,
                                                        cm.Ya.ptr); note_launch();
             k_scatter_add<<<nblocks(tot), 256, 0, s>>>(tot, (uint32_t)na, cc, cm.idx.ptr, cm.Ya.ptr, a.q); note_launch();
