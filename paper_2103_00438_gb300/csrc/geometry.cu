@@ -339,30 +339,26 @@ __global__ void k_alpha_partial(int64_t n, int64_t ncols, const double2 *__restr
     for (int k = 0; k < 3; ++k) part[((int64_t)blockIdx.x * ncols + c) * 3 + k] = a[k];
 }
 
+// Pass 2: a warp per output, its lanes over the partials, then a butterfly (fixed order).  An FP64
+// instruction occupies its scheduler's pipe for about 75 clocks whatever its lanes do: a thread per
+// output with a chain of nblk additions took 35 us for 192 columns.
 __global__ void k_alpha_final(int nblk, int64_t ncols, const double2 *__restrict__ part, double E0,
                               double2 *__restrict__ alpha) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (t >= ncols * 3) return;
-    // eight running sums, added in order: one chain of nblk FP64 additions took 36 us
-    double2 p[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) p[k] = make_double2(0.0, 0.0);
-    for (int b = 0; b < nblk; b += 8) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (b + k >= nblk) break;
-            const double2 v = part[(int64_t)(b + k) * ncols * 3 + t];
-            p[k].x += v.x;
-            p[k].y += v.y;
-        }
+    double2 s = {0, 0};
+    for (int b = lane; b < nblk; b += 32) {
+        const double2 v = part[(int64_t)b * ncols * 3 + t];
+        s.x += v.x;
+        s.y += v.y;
     }
-    double2 s = p[0];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) {
-        s.x += p[k].x;
-        s.y += p[k].y;
+    for (int o = 16; o > 0; o >>= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
     }
-    alpha[t] = make_double2(s.x / E0, s.y / E0);
+    if (lane == 0) alpha[t] = make_double2(s.x / E0, s.y / E0);
 }
 
 int launch_polarizability(const wfq_geom *g, int64_t ncols, const double2 *q, double E0,
@@ -373,7 +369,7 @@ int launch_polarizability(const wfq_geom *g, int64_t ncols, const double2 *q, do
     dim3 grid(nblk, (unsigned)((ncols + 63) / 64));
     k_alpha_partial<<<grid, 64, 0, s>>>(g->n, ncols, q, g->xyz, part.ptr); note_launch();
     WFQ_CUDA(cudaGetLastError());
-    k_alpha_final<<<(unsigned)((ncols * 3 + 127) / 128), 128, 0, s>>>(nblk, ncols, part.ptr, E0,
+    k_alpha_final<<<(unsigned)((ncols * 3 + 3) / 4), 128, 0, s>>>(nblk, ncols, part.ptr, E0,
                                                                        alpha_dev); note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
