@@ -6,15 +6,23 @@
 // Roles (18 warps):
 //   warp 0     : TMEM allocation; one lane loads, per stage, the Xhi / Xlo tiles (TMA) and
 //                the 32 atom records of the stage's K block (bulk copy, own barrier).
-//   warp 1     : one lane issues tcgen05.mma (three products per 16-atom K step).
-//   warps 2-17 : generate the 128 x 32 D tile of every stage -- one row per thread, one
-//                16-byte chunk (8 atoms) per group of four warps -- as bf16 hi and lo,
-//                written straight into the 64-byte-swizzled K-major layout the MMA
-//                descriptors expect; then a proxy fence and one arrival per warp on the
-//                stage's full-barrier.
+//   warp 1     : one lane issues tcgen05.mma (three products per 16-atom K step), from a
+//                warp-uniform loop.
+//   warps 2-17 : generate the 128 x 32 D tile of every stage -- one row per thread, in 16-byte
+//                chunks of 8 atoms -- as bf16 hi and lo, written straight into the
+//                64-byte-swizzled K-major layout the MMA descriptors expect; then a proxy fence
+//                and one arrival per warp on the stage's full-barrier.  GROUPS groups of WPS
+//                warps take the stages in turn, a thread 16 / WPS chunks of its row.
 //   warps 2-5  : also the epilogue (TMEM -> registers -> U), as in gemm_tc.cuh.
 // Work split and waits are those of gemm_tc.cuh (stream-K over (row tile, k block) units,
 // at most two CTAs per tile, bounded barrier waits).
+//
+// What bounds it, 99828 atoms x 32 real columns (9.97e9 pairs): about 1000 clocks per stage of
+// 4096 pairs, of which the ring alone (waits, six MMAs, commit; no pair generated) takes 690, and
+// the generators slow the issuing warp on its scheduler by the rest: more of them is slower (six
+// groups 10.0 ms, seven 9.1, four 8.2).  13.1 ms before; without 64-bit divisions for the stage and
+// the k block 10.2; four groups, so that a thread waits, fences and arrives once per 32 pairs
+// instead of 8, 9.8; MMAs from a warp-uniform loop 8.3 (with one group that made no difference).
 #pragma once
 
 #include "gemm_tc.cuh"
@@ -22,9 +30,22 @@
 namespace wfq {
 namespace tc {
 
-constexpr int MF_GEN_WARPS = 16;
 constexpr uint32_t MF_ATOM_BYTES = BK * 16;   // 32 float4 atom records per stage
-constexpr int MF_THREADS = 64 + 32 * MF_GEN_WARPS;
+constexpr int mf_threads(int wps, int groups) { return 64 + 32 * wps * groups; }
+
+// Stage and phase of a role's position in the ring.  A 64-bit division per stage (and one for its k
+// block) is some 40 instructions, as many as eight pairs' arithmetic needs for two of them.
+struct StageRing {
+    int stages, s = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void advance(int by) {   // by <= stages
+        s += by;
+        if (s >= stages) {
+            s -= stages;
+            ph ^= 1u;
+        }
+    }
+};
 
 struct MfParams {
     Params p;
@@ -63,7 +84,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
                  : "memory");
 }
 
-__global__ void __launch_bounds__(MF_THREADS, 1)
+template <int WPS, int GROUPS>
+__global__ void __launch_bounds__(mf_threads(WPS, GROUPS), 1)
     k_gemm3_mf(const __grid_constant__ CUtensorMap tm_xhi, const __grid_constant__ CUtensorMap tm_xlo,
                const MfParams mp) {
     const Params &p = mp.p;
@@ -87,7 +109,7 @@ __global__ void __launch_bounds__(MF_THREADS, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
-            mbar_init(smem_u32(full + s), 1 + MF_GEN_WARPS);
+            mbar_init(smem_u32(full + s), 1 + WPS);
             mbar_init(smem_u32(empty + s), 1);
             mbar_init(smem_u32(atoms_full + s), 1);
         }
@@ -111,60 +133,62 @@ __global__ void __launch_bounds__(MF_THREADS, 1)
     const uint32_t b_tx = 2u * p.b_bytes;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------------------------------------------------- TMA producer (X only)
+        // -------------------------------------------------------------- TMA producer (X only)
+        {
+            const bool el = elect_one();
             int64_t it = 0;
-            int64_t last_it[MAX_STAGES];
-            for (int s = 0; s < MAX_STAGES; ++s) last_it[s] = -1;
             bool aborted = false;
-            for (int64_t u = u_begin; u < u_end; ++u, ++it) {
-                const int s = (int)(it % p.stages);
-                const uint32_t ph = (uint32_t)((it / p.stages) & 1);
-                if (!mbar_wait(smem_u32(empty + s), ph ^ 1u, p, 1, abort_flag)) {
+            int kb = (int)(u_begin % p.kblocks);
+            StageRing r{p.stages};
+            for (int64_t u = u_begin; u < u_end; ++u, ++it, r.advance(1), kb = kb + 1 < p.kblocks ? kb + 1 : 0) {
+                if (!mbar_wait(smem_u32(empty + r.s), r.ph ^ 1u, p, 1, abort_flag)) aborted = true;
+                if (__any_sync(0xffffffffu, aborted)) {
                     aborted = true;
                     break;
                 }
-                const int kb = (int)(u % p.kblocks);
-                const uint32_t base = smem_base + (uint32_t)s * p.stage_bytes;
-                const uint32_t fb = smem_u32(full + s);
-                const uint32_t ab = smem_u32(atoms_full + s);
-                mbar_expect_tx(ab, MF_ATOM_BYTES);
-                bulk_load(base + atoms_off, mp.atoms_p + (int64_t)kb * BK, MF_ATOM_BYTES, ab);
-                mbar_expect_tx(fb, b_tx);
-                for (int j = 0; j < p.nsplit; ++j) {
-                    tma_load_2d(base + 2 * A_BYTES + (uint32_t)(j * p.nchunk * ROWB), &tm_xhi, fb, kb * BK,
-                                j * p.nchunk);
-                    tma_load_2d(base + 2 * A_BYTES + p.b_bytes + (uint32_t)(j * p.nchunk * ROWB), &tm_xlo, fb,
-                                kb * BK, j * p.nchunk);
+                const uint32_t base = smem_base + (uint32_t)r.s * p.stage_bytes;
+                const uint32_t fb = smem_u32(full + r.s), ab = smem_u32(atoms_full + r.s);
+                if (el) {
+                    mbar_expect_tx(ab, MF_ATOM_BYTES);
+                    bulk_load(base + atoms_off, mp.atoms_p + (int64_t)kb * BK, MF_ATOM_BYTES, ab);
+                    mbar_expect_tx(fb, b_tx);
                 }
-                last_it[s] = it;
-            }
-            if (aborted)
-                for (int s = 0; s < p.stages; ++s)
-                    if (last_it[s] >= 0) {
-                        volatile int no_abort = 0;
-                        const uint32_t par = (uint32_t)((last_it[s] / p.stages) & 1);
-                        mbar_wait(smem_u32(atoms_full + s), par, p, 1, &no_abort);
-                        mbar_wait(smem_u32(full + s), par, p, 1, &no_abort);
+                for (int j = 0; j < p.nsplit; ++j)
+                    if (el) {
+                        tma_load_2d(base + 2 * A_BYTES + (uint32_t)(j * p.nchunk * ROWB), &tm_xhi, fb, kb * BK,
+                                    j * p.nchunk);
+                        tma_load_2d(base + 2 * A_BYTES + p.b_bytes + (uint32_t)(j * p.nchunk * ROWB), &tm_xlo, fb,
+                                    kb * BK, j * p.nchunk);
                     }
+            }
+            // an aborted kernel waits for its own loads in flight: the last p.stages issued
+            if (aborted)
+                for (int64_t k = it > p.stages ? it - p.stages : 0; k < it; ++k) {
+                    volatile int no_abort = 0;
+                    const int s = (int)(k % p.stages);
+                    const uint32_t par = (uint32_t)((k / p.stages) & 1);
+                    mbar_wait(smem_u32(atoms_full + s), par, p, 1, &no_abort);
+                    mbar_wait(smem_u32(full + s), par, p, 1, &no_abort);
+                }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------------------------------------------------- MMA issuer
+        // -------------------------------------------------------------- MMA issuer
+        {
+            const bool el = elect_one();
             const uint32_t idesc = idesc_bf16(BM, p.nchunk);
-            int64_t it = 0, seg = 0;
+            int64_t seg = 0;
             int64_t u = u_begin;
             bool aborted = false;
+            StageRing r{p.stages};
             while (u < u_end && !aborted) {
                 const int64_t tile = u / p.kblocks;
                 const int64_t seg_end = u_end < (tile + 1) * p.kblocks ? u_end : (tile + 1) * p.kblocks;
                 if (!mbar_wait(smem_u32(acc_empty), (uint32_t)((seg & 1) ^ 1), p, 3, abort_flag)) break;
                 tc_fence_after();
                 bool first = true;
-                for (; u < seg_end; ++u, ++it) {
-                    const int s = (int)(it % p.stages);
-                    const uint32_t ph = (uint32_t)((it / p.stages) & 1);
-                    if (!mbar_wait(smem_u32(full + s), ph, p, 2, abort_flag)) {
+                for (; u < seg_end; ++u, r.advance(1)) {
+                    const int s = r.s;
+                    if (!mbar_wait(smem_u32(full + s), r.ph, p, 2, abort_flag)) {
                         aborted = true;
                         break;
                     }
@@ -180,40 +204,43 @@ __global__ void __launch_bounds__(MF_THREADS, 1)
                             const uint64_t b_hi = desc_k_sw64(base + 2 * A_BYTES + boff);
                             const uint64_t b_lo = desc_k_sw64(base + 2 * A_BYTES + p.b_bytes + boff);
                             const uint32_t d = tmem + (uint32_t)(j * p.nchunk);
-                            umma_bf16(d, a_hi, b_hi, idesc, first ? 0u : 1u);
-                            umma_bf16(d, a_hi, b_lo, idesc, 1u);
-                            umma_bf16(d, a_lo, b_hi, idesc, 1u);
+                            if (el) umma_bf16(d, a_hi, b_hi, idesc, first ? 0u : 1u);
+                            if (el) umma_bf16(d, a_hi, b_lo, idesc, 1u);
+                            if (el) umma_bf16(d, a_lo, b_hi, idesc, 1u);
                         }
                         first = false;
                     }
-                    umma_commit(smem_u32(empty + s));
+                    if (el) umma_commit(smem_u32(empty + s));
                 }
                 if (aborted) break;
-                umma_commit(smem_u32(acc_full));
+                if (el) umma_commit(smem_u32(acc_full));
                 ++seg;
             }
-            umma_commit(smem_u32(drain));
+            if (el) umma_commit(smem_u32(drain));
             volatile int no_abort = 0;
             mbar_wait(smem_u32(drain), 0u, p, 5, &no_abort);
         }
     } else {
         // ---------------------------------------------------------- D-tile generators
-        const int gt = threadIdx.x - 64;           // 0..511
+        const int gt = (threadIdx.x - 64) % (32 * WPS);
+        const int group = (threadIdx.x - 64) / (32 * WPS);
         const int row = gt & (BM - 1);             // tile row of this thread
-        const int kc = gt >> 7;                    // 16-byte chunk (8 atoms) of the 64-byte row
+        constexpr int CHUNKS = 16 / WPS;           // its 16-byte chunks (8 atoms) of the 64-byte row
+        const int c_begin = (gt >> 7) * CHUNKS;
         const bool epi = warp < 6;                 // warps 2-5 also run the epilogue
         const int quad = warp & 3;
         const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
         const int epi_row = quad * 32 + lane;
         const bool vec = ((p.ldu & 3) == 0) && ((reinterpret_cast<uintptr_t>(p.U) & 15) == 0);
         const float eta_from_w = 0.7978845608028654f;   // sqrt(2/pi): eta = sqrt(2/pi) / width (Eq. 4)
-        int64_t it = 0, seg = 0;
-        int64_t u = u_begin;
+        int64_t u = u_begin + group;               // group g generates the stages g, g + GROUPS, ...
         bool aborted = false;
-        while (u < u_end && !aborted) {
-            const int64_t tile = u / p.kblocks;
-            const int64_t seg_end = u_end < (tile + 1) * p.kblocks ? u_end : (tile + 1) * p.kblocks;
-            const int64_t seg_begin = u;
+        StageRing r{p.stages};
+        r.advance(group);
+        int64_t seg = 0, seg_end;
+        for (int64_t seg_begin = u_begin; seg_begin < u_end && !aborted; seg_begin = seg_end) {
+            const int64_t tile = seg_begin / p.kblocks;
+            seg_end = u_end < (tile + 1) * p.kblocks ? u_end : (tile + 1) * p.kblocks;
             const int gi = (int)(tile * BM + row);
             const float4 ai = mp.atoms[gi];
             const bool row_ok = gi < p.n;
@@ -222,19 +249,20 @@ __global__ void __launch_bounds__(MF_THREADS, 1)
             // the row atom as packed operands (the same value in both lanes)
             const float2 aix2 = make_float2(ai.x, ai.x), aiy2 = make_float2(ai.y, ai.y);
             const float2 aiz2 = make_float2(ai.z, ai.z), wa2_2 = make_float2(wa2, wa2);
-            for (; u < seg_end; ++u, ++it) {
-                const int s = (int)(it % p.stages);
-                const uint32_t ph = (uint32_t)((it / p.stages) & 1);
+            int k0 = (int)(u - tile * p.kblocks) * BK;
+            for (; u < seg_end; u += GROUPS, k0 += GROUPS * BK, r.advance(GROUPS)) {
+                const int s = r.s;
                 // the k-atom records land only after the stage was released by the MMAs,
                 // so this one wait covers both
-                if (!mbar_wait(smem_u32(atoms_full + s), ph, p, 6, abort_flag)) {
+                if (!mbar_wait(smem_u32(atoms_full + s), r.ph, p, 6, abort_flag)) aborted = true;
+                if (__any_sync(0xffffffffu, aborted)) {   // the warp leaves together
                     aborted = true;
                     break;
                 }
-                const int k0 = (int)(u % p.kblocks) * BK;
                 const uint32_t base = smem_base + (uint32_t)s * p.stage_bytes;
                 const float4 *atoms_s = reinterpret_cast<const float4 *>(smem + (size_t)s * p.stage_bytes + atoms_off);
-                {
+#pragma unroll 1
+                for (int kc = c_begin; kc < c_begin + CHUNKS; ++kc) {
                     const int kb0 = k0 + kc * 8;
                     float dv[8], r2v[8], s2v[8];
                     // the chunk's 8 atoms as 4 pairs, two k-atoms per packed FP32x2 operation
@@ -389,11 +417,20 @@ inline cudaError_t launch_group_mf(const float4 *atoms, const float4 *atoms_p, i
         return cudaErrorInvalidValue;
     const int64_t grid = grid_size(mtiles, num_sms);
     const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 512;
-    static std::atomic<uint64_t> smem_set{0};
     if (smem > (size_t)kMaxDynSmem) return cudaErrorInvalidValue;
-    cudaError_t e = allow_max_smem(k_gemm3_mf, smem_set);
+    auto run = [&](auto kernel, std::atomic<uint64_t> &smem_set, int threads) {
+        cudaError_t e = allow_max_smem(kernel, smem_set);
+        if (e == cudaSuccess) kernel<<<(unsigned)grid, threads, smem, s>>>(m_xhi, m_xlo, mp);
+        return e;
+    };
+    // Four groups need a stage each.  Blocks of more than 256 real columns have fewer (or no
+    // spare one): all 16 warps on one stage then (40000 atoms x 256 columns: 2.49 ms with four
+    // groups, 2.63 with one; x 384: 3.28 and 3.23; x 32: 1.53 and 1.90).
+    static std::atomic<uint64_t> set_grouped{0}, set_one{0};
+    constexpr int WPS = 4, GROUPS = 4;
+    const cudaError_t e = p.stages >= GROUPS ? run(k_gemm3_mf<WPS, GROUPS>, set_grouped, mf_threads(WPS, GROUPS))
+                                             : run(k_gemm3_mf<16, 1>, set_one, mf_threads(16, 1));
     if (e != cudaSuccess) return e;
-    k_gemm3_mf<<<(unsigned)grid, MF_THREADS, smem, s>>>(m_xhi, m_xlo, mp);
     return cudaGetLastError();
 }
 
