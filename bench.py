@@ -92,15 +92,12 @@ def store_for(name, wfq, solver="gmres"):
     return wfq.STORE_FP64 | wfq.STORE_BF16X2 | wfq.STORE_F32X2
 
 
-# DRAM bytes per stored D entry that ncu measured for one k_dgemv_df launch (cnt8k, N = 8200:
-# 549.3 MB read + written for 8200 x 8320 stored entries of the FP32 pair planes).
+# DRAM bytes per stored D entry that ncu measured for one k_dgemv_df launch (the BEM operator's
+# product; 8200-atom tube: 549.3 MB read + written for 8200 x 8320 stored entries of the FP32 pair planes).
 DGEMV_DRAM_BYTES_PER_ENTRY = 549.3e6 / (8200.0 * 8320.0)
 
 # Algorithmic bytes of one block apply of D: the FP32 D (4 bytes per entry) read once.
 ALG_BYTES_PER_ENTRY = 4.0
-
-# FP32 lane-instructions per second of the whole GPU: 152 SMs x 128 lanes x 2070 MHz.
-FP32_LANE_OPS_PER_S = 152 * 128 * 2.07e9
 
 # Minimum FP32-pipe instructions to generate one D entry as a bf16 hi/lo pair on the
 # matrix-free path: 3 coordinate differences, 3 for r^2, 1 for sigma^2, 1 far/near test,
@@ -434,42 +431,22 @@ def run_ours(args, rank, world, dist):
     # columns converge): 6 N^2 C tensor flops (three bf16 products of 2 N^2 C each).
     peaks, peak_src = load_peaks()
     roof = None
-    if gv_n and gv_ms >= gemm_ms and store & wfq.STORE_F32X2_SYM and not store & wfq.STORE_F32X2:
-        # shifted solver on the symmetric tiles: half of D streamed, each tile used for two
-        # products, so the double-float arithmetic bounds it: 12 FP32-pipe instructions per
-        # (entry, vector) product, N^2 x ndir products per launch
-        avg_s = gv_ms / gv_n * 1e-3
-        achieved = 12.0 * n * n * nd / avg_s / 1e12
-        peak = FP32_LANE_OPS_PER_S / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "FP32 Tinst/s",
-                "frac": achieved / peak, "traffic": None,
-                "kernel": "k_dsymv_df + k_dsymv_finish (symmetric double-float D product)", "launches": gv_n,
-                "avg_ms": gv_ms / gv_n, "bytes_per_launch": gv_bytes / gv_n,
-                "hbm_achieved_gbs": gv_bytes / gv_n / avg_s / 1e9,
-                "hbm_frac": gv_bytes / gv_n / avg_s / 1e9 / peaks["hbm_gbs"],
-                "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2070 MHz (one FP32 instruction per lane "
-                               "per clock); work: 12 instructions per double-float multiply-add"}
-    elif gv_n and gv_ms >= gemm_ms:
+    if gv_n and gv_ms >= gemm_ms:
         # shifted solver: the dominant kernel is the D product of the Arnoldi vectors.
         # Algorithmic bytes per launch: 4 bytes per D entry (the FP32 D read once per block
-        # apply), N^2 entries.  The kernel itself stores D as FP32 pairs (8 bytes per entry
-        # for ~2^-48 products); its utilisation of HBM on those stored bytes is reported
-        # beside the fraction, under its own name.
+        # apply), N^2 entries.  The kernel reads the upper triangle of the FP32 pairs (8 bytes
+        # for ~2^-48 of an entry) and uses every block twice: the same count.
         avg_s = gv_ms / gv_n * 1e-3
         alg_bytes = ALG_BYTES_PER_ENTRY * float(n) * float(n)
         achieved_gbs = alg_bytes / avg_s / 1e9
         peak = peaks["hbm_gbs"]
-        stored = gv_bytes / gv_n
         roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": peak, "unit": "GB/s",
-                "frac": achieved_gbs / peak,
-                "traffic": DGEMV_DRAM_BYTES_PER_ENTRY * n * (-(-n // 128) * 128),
-                "traffic_source": "ncu dram__bytes_read+write of k_dgemv_df at N = 8200 "
-                                  "(the committed profile summary of that kernel), scaled per D entry to this N",
-                "kernel": "k_dgemv_df (double-float D product of the real Arnoldi vectors)", "launches": gv_n,
-                "avg_ms": gv_ms / gv_n, "algorithmic_bytes_per_launch": alg_bytes,
+                "frac": achieved_gbs / peak, "traffic": None,
+                "kernel": "k_gemv_digits (D product of the real Arnoldi vectors by digit slices, tcgen05)",
+                "launches": gv_n, "avg_ms": gv_ms / gv_n, "algorithmic_bytes_per_launch": alg_bytes,
                 "algorithmic_bytes_rule": "4 bytes per D entry x N^2 entries (FP32 D streamed once per block apply)",
-                "stored_bytes_per_launch": stored,
-                "hbm_util_of_stored_bytes": stored / avg_s / 1e9 / peak,
+                "stored_bytes_per_launch": alg_bytes,
+                "hbm_util_of_stored_bytes": achieved_gbs / peak,
                 "peak_source": peak_src + " hbm_gbs (STREAM-style copy)"}
     elif gemm_n:
         gemm_avg_ms = gemm_ms / gemm_n
@@ -1068,7 +1045,7 @@ def run_serve(args, rank, world, dist):
         achieved = gv_bytes / (gv_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": None,
-                "kernel": "k_dgemv_df (double-float D product of the real Arnoldi vectors)", "launches": gv_n,
+                "kernel": "k_gemv_digits / k_dgemv_df (D product of the real Arnoldi vectors)", "launches": gv_n,
                 "avg_ms": gv_ms / gv_n, "peak_source": peak_src + " hbm_gbs (STREAM-style copy)",
                 "note": "launch times measured while batches on other worker streams share the GPU"}
     elif gemm_n:

@@ -585,7 +585,7 @@ cudaError_t launch_c(const CUtensorMap &m, const SymvParams &sp, int grid, cudaS
 }  // namespace
 
 // Needs a symmetric D (not the BEM operator: with every column block and no transposed products it
-// gained 10% there, but its Krylov spaces amplify the start's own rounding past 1e-9 of q).  All
+// gained 10% there, but its Krylov spaces amplify the rounding of either product past 1e-9 of q).  All
 // rows share one exponent (a column's sum runs over the rows), so the rows' bounds must not differ
 // by more than 2^3: a row then loses at most 3 of its 55 bits.
 bool gemv_digits_usable(const wfq_geom *g) {
