@@ -12,7 +12,8 @@
 //                chunks of 8 atoms -- as bf16 hi and lo, written straight into the
 //                64-byte-swizzled K-major layout the MMA descriptors expect; then a proxy fence
 //                and one arrival per warp on the stage's full-barrier.  GROUPS groups of WPS
-//                warps take the stages in turn, a thread 16 / WPS chunks of its row.
+//                warps take the stages in turn, a thread 16 / WPS chunks of its row; the ring's
+//                depth is a multiple of GROUPS, so a slot is always the same group's (mf_plan.h).
 //   warps 2-5  : also the epilogue (TMEM -> registers -> U), as in gemm_tc.cuh.
 // Work split and waits are those of gemm_tc.cuh (stream-K over (row tile, k block) units,
 // at most two CTAs per tile, bounded barrier waits).
@@ -26,6 +27,7 @@
 #pragma once
 
 #include "gemm_tc.cuh"
+#include "mf_plan.h"
 
 namespace wfq {
 namespace tc {
@@ -400,6 +402,8 @@ inline cudaError_t launch_group_mf(const float4 *atoms, const float4 *atoms_p, i
     p.stages = (int)((kMaxDynSmem - 2048) / p.stage_bytes);
     if (p.stages > MAX_STAGES) p.stages = MAX_STAGES;
     if (stages_req >= 2 && stages_req < p.stages) p.stages = stages_req;   // a shallower pipeline (autotuner)
+    const MfPlan plan = mf_plan(p.stages);
+    p.stages = plan.stages;
     int tcols = 32;
     while (tcols < cpad) tcols <<= 1;
     p.tmem_cols = tcols;
@@ -427,9 +431,9 @@ inline cudaError_t launch_group_mf(const float4 *atoms, const float4 *atoms_p, i
     // spare one): all 16 warps on one stage then (40000 atoms x 256 columns: 2.49 ms with four
     // groups, 2.63 with one; x 384: 3.28 and 3.23; x 32: 1.53 and 1.90).
     static std::atomic<uint64_t> set_grouped{0}, set_one{0};
-    constexpr int WPS = 4, GROUPS = 4;
-    const cudaError_t e = p.stages >= GROUPS ? run(k_gemm3_mf<WPS, GROUPS>, set_grouped, mf_threads(WPS, GROUPS))
-                                             : run(k_gemm3_mf<16, 1>, set_one, mf_threads(16, 1));
+    constexpr int WPS = 16 / MF_GROUPS;
+    const cudaError_t e = plan.groups == MF_GROUPS ? run(k_gemm3_mf<WPS, MF_GROUPS>, set_grouped, mf_threads(WPS, MF_GROUPS))
+                                                   : run(k_gemm3_mf<16, 1>, set_one, mf_threads(16, 1));
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

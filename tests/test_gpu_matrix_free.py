@@ -37,3 +37,20 @@ def test_product_at_the_edges_of_the_stage_groups(W, ctx, orc, S, n, ncplx):
         z, xc = sysm.z(om[c]), x[:, c].astype(np.complex128)
         ref = _oracle_apply(orc, sysm, z, xc)
         assert np.max(np.abs(y[:, c] - ref) / _mixed_bound(sysm, z, xc)) <= TAU_MIXED
+
+
+@pytest.mark.parametrize("ncplx", [48, 64, 80, 96])   # 7, 6, 6 and 5 stages fit
+def test_many_stages_where_the_ring_is_cut_to_whole_groups(W, ctx, orc, S, ncplx):
+    xyz = S.random_cluster(2300, seed=8)
+    p = _carbon(S, r0=2.7)
+    g = W.Geometry(ctx, xyz, p, store=0)
+    sysm = orc.System(xyz, p)
+    om = S.ev(np.linspace(0.3, 1.5, ncplx))
+    x = S.random_complex((len(xyz), ncplx), seed=3).astype(np.complex64)
+    y = np.empty_like(x)
+    for _ in range(3):
+        g.apply(om, x, y, prec=W.PREC_MIXED)
+    for c in (0, ncplx // 2, ncplx - 1):
+        z, xc = sysm.z(om[c]), x[:, c].astype(np.complex128)
+        ref = _oracle_apply(orc, sysm, z, xc)
+        assert np.max(np.abs(y[:, c] - ref) / _mixed_bound(sysm, z, xc)) <= TAU_MIXED
