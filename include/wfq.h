@@ -169,6 +169,12 @@ int64_t wfq_kernel_launches(void);
  * pool's in-use high-water mark.  out: host, 4 values, caller-owned. */
 int wfq_memory_stats(wfq_ctx *ctx, int64_t *out);
 
+/* Self-test of the kernels' bounded waits: lets one run out after limit_us (1..10000) microseconds
+ * while the rest of its warp may see the wait succeed.  out (host, 3 values): lanes of the warp whose
+ * wait succeeded when every lane decides alone, the same when the warp decides together (as the
+ * kernels do; 0 or 32), and the non-zero code the wait recorded. */
+int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out);
+
 /* Kernel timing (profiling aid).  While enabled, the library records a pair of CUDA
  * events on the launching stream around every launch of the kernels below;
  * wfq_profile_read synchronises those events and returns the launch count and the

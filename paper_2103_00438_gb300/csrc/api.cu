@@ -279,6 +279,13 @@ int wfq_memory_stats(wfq_ctx *ctx, int64_t *out) {
     return WFQ_OK;
 }
 
+int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out) {
+    if (!ctx || !out) return fail(WFQ_EINVAL, "NULL argument");
+    if (limit_us < 1 || limit_us > 10000) return fail(WFQ_EINVAL, "limit_us must be in 1..10000");
+    DeviceGuard dg(ctx->device);
+    return selftest_wait(ctx, limit_us, out, nullptr);
+}
+
 int wfq_create(wfq_ctx **out, int device) {
     if (!out) return fail(WFQ_EINVAL, "ctx out-pointer is NULL");
     *out = nullptr;

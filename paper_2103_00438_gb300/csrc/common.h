@@ -235,6 +235,9 @@ struct KScope {
     ~KScope();
 };
 
+// Runs a bounded wait out on purpose and reports what the lanes of a warp saw (wfq_selftest_wait).
+int selftest_wait(wfq_ctx *ctx, int limit_us, int *out, cudaStream_t s);
+
 // WFQ_ETIMEOUT (and clears the flag) if a kernel reported a bounded wait that gave up.
 int check_device_error(wfq_ctx *ctx, cudaStream_t s);
 

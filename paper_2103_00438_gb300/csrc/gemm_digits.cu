@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
         for (int u = 0; u < nunits; ++u, advance()) {
             const int nh = halves();
             if (nh == 2 || (u & 1) == e) {
-                if (!tc::mbar_wait(tc::smem_u32(acc_full + e), uses & 1u, p, 4, abort_flag)) break;
+                if (!tc::mbar_wait_warp(tc::smem_u32(acc_full + e), uses & 1u, p, 4, abort_flag)) break;
                 ++uses;
                 tc::tc_fence_after();
 #pragma unroll
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
         uint32_t buf = 0, par = 0;
         auto step = [&](int j, const Regs &now, Regs &next) -> bool {
             if (j + 1 < nst) load(next);
-            if (!tc::mbar_wait(tc::smem_u32(a_empty + buf), par ^ 1u, p, 1, abort_flag)) return false;
+            if (!tc::mbar_wait_warp(tc::smem_u32(a_empty + buf), par ^ 1u, p, 1, abort_flag)) return false;
             convert(now, smem_base + buf * A_STAGE);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();

@@ -143,8 +143,7 @@ __global__ void __launch_bounds__(mf_threads(WPS, GROUPS), 1)
             int kb = (int)(u_begin % p.kblocks);
             StageRing r{p.stages};
             for (int64_t u = u_begin; u < u_end; ++u, ++it, r.advance(1), kb = kb + 1 < p.kblocks ? kb + 1 : 0) {
-                if (!mbar_wait(smem_u32(empty + r.s), r.ph ^ 1u, p, 1, abort_flag)) aborted = true;
-                if (__any_sync(0xffffffffu, aborted)) {
+                if (!mbar_wait_warp(smem_u32(empty + r.s), r.ph ^ 1u, p, 1, abort_flag)) {
                     aborted = true;
                     break;
                 }
@@ -256,8 +255,7 @@ __global__ void __launch_bounds__(mf_threads(WPS, GROUPS), 1)
                 const int s = r.s;
                 // the k-atom records land only after the stage was released by the MMAs,
                 // so this one wait covers both
-                if (!mbar_wait(smem_u32(atoms_full + s), r.ph, p, 6, abort_flag)) aborted = true;
-                if (__any_sync(0xffffffffu, aborted)) {   // the warp leaves together
+                if (!mbar_wait_warp(smem_u32(atoms_full + s), r.ph, p, 6, abort_flag)) {
                     aborted = true;
                     break;
                 }
@@ -338,7 +336,7 @@ __global__ void __launch_bounds__(mf_threads(WPS, GROUPS), 1)
             }
             // ---------------------------------------------------------- epilogue (warps 2-5)
             const bool whole_tile = (seg_begin == tile * p.kblocks) && (seg_end == (tile + 1) * p.kblocks);
-            if (!mbar_wait(smem_u32(acc_full), (uint32_t)(seg & 1), p, 4, abort_flag)) break;
+            if (!mbar_wait_warp(smem_u32(acc_full), (uint32_t)(seg & 1), p, 4, abort_flag)) break;
             tc_fence_after();
             const int64_t orow = tile * BM + epi_row;
             float *dst_row = p.U + orow * p.ldu;

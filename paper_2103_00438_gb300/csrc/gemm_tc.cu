@@ -56,6 +56,43 @@ int tuned_stages(const wfq_geom *g, int64_t key, cudaStream_t s, Launch launch) 
     return best;
 }
 
+// The bounded waits run out on purpose (wfq_selftest_wait): warp 0 waits for a barrier that nothing
+// completes until its lane 0, whose limit is the shortest, has given up; warp 1 then completes it, so that
+// the lanes see different things.  out: lanes of warp 0 whose wait succeeded, by mbar_wait (round 0) and
+// by mbar_wait_warp (round 1), and the code recorded.  Every loop here ends by its limit.
+__global__ void __launch_bounds__(64) k_selftest_wait(unsigned long long limit_ns, int *err, int *out) {
+    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ int abort_flag[2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int r = 0; r < 2; ++r) {
+            tc::mbar_init(tc::smem_u32(bar + r), 1);
+            abort_flag[r] = 0;
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    tc::Params p{};
+    p.err = err;
+    p.timeout_ns = lane == 0 ? limit_ns : 50 * limit_ns;
+    for (int r = 0; r < 2; ++r) {
+        volatile int *flag = abort_flag + r;
+        if (warp == 0) {
+            const bool ok = r == 0 ? tc::mbar_wait(tc::smem_u32(bar + r), 0u, p, 9, flag)
+                                   : tc::mbar_wait_warp(tc::smem_u32(bar + r), 0u, p, 9, flag);
+            const unsigned lanes = __ballot_sync(0xffffffffu, ok);
+            if (lane == 0) out[r] = __popc(lanes);
+        } else if (lane == 0) {
+            const uint64_t t0 = tc::global_ns();
+            while (!*flag && tc::global_ns() - t0 < 100 * limit_ns) {
+            }
+            tc::mbar_arrive(tc::smem_u32(bar + r));
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[2] = *err;
+}
+
 // autotuner keys of the GEMMs: bit 60 set (the GEMV keys stay below 2^40), kernel id, shape
 inline int64_t gemm_key(int kernel, int64_t npad, int64_t cpad) {
     return ((int64_t)1 << 60) | ((int64_t)kernel << 56) | (npad << 20) | cpad;
@@ -106,6 +143,18 @@ int gemm_3xbf16(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi, const
         cudaGetLastError();
         return fail(WFQ_ECUDA, "tensor-core GEMM: " + (msg.empty() ? std::string(cudaGetErrorString(e)) : msg));
     }
+    return WFQ_OK;
+}
+
+int selftest_wait(wfq_ctx *ctx, int limit_us, int *out, cudaStream_t s) {
+    DevBuf<int> buf;
+    WFQ_TRY(buf.alloc(ctx, 4, s));
+    WFQ_CUDA(cudaMemsetAsync(buf.ptr, 0, 4 * sizeof(int), s));
+    k_selftest_wait<<<1, 64, 0, s>>>(1000ull * (unsigned long long)limit_us, buf.ptr + 3, buf.ptr);
+    note_launch();
+    WFQ_CUDA(cudaGetLastError());
+    WFQ_CUDA(cudaMemcpyAsync(out, buf.ptr, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    WFQ_CUDA(cudaStreamSynchronize(s));
     return WFQ_OK;
 }
 

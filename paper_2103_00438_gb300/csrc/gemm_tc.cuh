@@ -82,6 +82,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const P
     }
 }
 
+// The same for a whole warp that goes on to a warp-wide instruction (__syncwarp, tcgen05.ld): true in
+// all lanes or in none.  mbar_wait decides per lane, and a lane that gave up would leave the others
+// waiting for it in that instruction while they hold up the block's last barrier.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const Params &p, int code,
+                                               volatile int *abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, p, code, abort_flag));
+}
+
 // Shared-memory matrix descriptor of a K-major operand tile stored as rows of 64 bytes
 // with the 64-byte swizzle (as written by TMA with CU_TENSOR_MAP_SWIZZLE_64B): 8-row
 // groups are 512 bytes apart (stride byte offset); the leading byte offset is not used
@@ -276,7 +284,7 @@ static __global__ void __launch_bounds__(NUM_THREADS, 1)
             const int64_t tile = u / p.kblocks;
             const int64_t seg_end = u_end < (tile + 1) * p.kblocks ? u_end : (tile + 1) * p.kblocks;
             const bool whole = (u == tile * p.kblocks) && (seg_end == (tile + 1) * p.kblocks);
-            if (!mbar_wait(smem_u32(acc_full), (uint32_t)(seg & 1), p, 4, abort_flag)) break;
+            if (!mbar_wait_warp(smem_u32(acc_full), (uint32_t)(seg & 1), p, 4, abort_flag)) break;
             tc_fence_after();
             const int64_t row = tile * BM + row_in_tile;
             float *dst_row = p.U + row * p.ldu;

@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
         for (int u = 0; u < nunits; ++u, advance()) {
             if (!row_read(u)) continue;
             const uint32_t slot = uses & 1u;
-            if (!tc::mbar_wait(tc::smem_u32(row_full + slot), (uses >> 1) & 1u, p, 4, abort_flag)) break;
+            if (!tc::mbar_wait_warp(tc::smem_u32(row_full + slot), (uses >> 1) & 1u, p, 4, abort_flag)) break;
             ++uses;
             tc::tc_fence_after();
             read_terms<C>(base + slot * SLOT, hi, lo);
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
         for (int u = 0; u < nunits; ++u, advance()) {
             if (col_steps() == 0) continue;
             const uint32_t slot = uses & 1u;
-            if (!tc::mbar_wait(tc::smem_u32(col_full + slot), (uses >> 1) & 1u, p, 4, abort_flag)) break;
+            if (!tc::mbar_wait_warp(tc::smem_u32(col_full + slot), (uses >> 1) & 1u, p, 4, abort_flag)) break;
             ++uses;
             tc::tc_fence_after();
             int64_t hi[C], lo[C];
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
         for (int u = 0; u < nunits; ++u) {
             const uint32_t s = u & 1, ph = (u >> 1) & 1;
             const uint32_t base = smem_base + s * SV_A;
-            if (!tc::mbar_wait(tc::smem_u32(a_empty + s), ph ^ 1u, p, 1, abort_flag)) break;
+            if (!tc::mbar_wait_warp(tc::smem_u32(a_empty + s), ph ^ 1u, p, 1, abort_flag)) break;
             convert(r0, base, 0);
             if (u + 1 < nunits) load(r0);
             convert(r1, base, 1);
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
             prefetch();
             if (u == 0 || cur.J == 2 * cur.a) {   // a block's own rows, for the transposed products
                 const uint32_t bs = blocks & 1;
-                if (!tc::mbar_wait(tc::smem_u32(bi_empty + bs), ((blocks >> 1) & 1) ^ 1u, p, 1, abort_flag)) {
+                if (!tc::mbar_wait_warp(tc::smem_u32(bi_empty + bs), ((blocks >> 1) & 1) ^ 1u, p, 1, abort_flag)) {
                     aborted = true;
                     break;
                 }
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
                 }
                 ++blocks;
             }
-            if (!tc::mbar_wait(tc::smem_u32(a_empty + s), ph ^ 1u, p, 1, abort_flag)) {
+            if (!tc::mbar_wait_warp(tc::smem_u32(a_empty + s), ph ^ 1u, p, 1, abort_flag)) {
                 aborted = true;
                 break;
             }

@@ -25,7 +25,7 @@ EXPORTS = ["wfq_create", "wfq_destroy", "wfq_last_error", "wfq_kernel_launches",
            "wfq_geometry_info", "wfq_apply", "wfq_rhs", "wfq_solve_gmres", "wfq_solve_gmres_shifted", "wfq_solve_qmr",
            "wfq_polarizability", "wfq_profile", "wfq_profile_read", "wfq_apply_mixed_noalloc",
            "wfq_server_create", "wfq_server_submit", "wfq_server_poll", "wfq_server_destroy",
-           "wfq_memory_stats", "wfq_cross_section", "wfq_fmm_build", "wfq_fmm_info"]
+           "wfq_memory_stats", "wfq_cross_section", "wfq_fmm_build", "wfq_fmm_info", "wfq_selftest_wait"]
 KT_GEMM_MIXED, KT_DAPPLY_FP64, KT_SPARSE, KT_ORTHO, KT_RESIDUAL, KT_DGEMV_DF, KT_FMM = 0, 1, 2, 3, 4, 5, 6
 
 
@@ -93,6 +93,7 @@ def load(path: str | None = None):
     L.wfq_server_destroy.argtypes = [_P]
     L.wfq_profile.argtypes = [_P, INT]
     L.wfq_memory_stats.argtypes = [_P, _P]
+    L.wfq_selftest_wait.argtypes = [_P, INT, _P]
     L.wfq_fmm_build.argtypes = [_P, INT]
     L.wfq_fmm_info.argtypes = [_P, _P]
     L.wfq_cross_section.argtypes = [_P, I64, _P, INT, _P, D, _P, _P, _P, _P]
@@ -187,6 +188,13 @@ class Context:
         out = np.zeros(4, dtype=np.int64)
         _check(_lib.wfq_memory_stats(self.h, out.ctypes.data))
         return dict(zip(("allocs", "pool_reserved", "pool_used", "pool_used_high"), (int(v) for v in out)))
+
+    def selftest_wait(self, limit_us: int = 1000):
+        """(lanes that saw a wait succeed deciding alone, the same deciding as a warp, code recorded)
+        of a bounded wait that runs out."""
+        out = np.zeros(3, dtype=np.int32)
+        _check(_lib.wfq_selftest_wait(self.h, int(limit_us), out.ctypes.data))
+        return tuple(int(v) for v in out)
 
     def close(self):
         if self.h:
