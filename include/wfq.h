@@ -175,6 +175,10 @@ int wfq_memory_stats(wfq_ctx *ctx, int64_t *out);
  * kernels do; 0 or 32), and the non-zero code the wait recorded. */
 int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out);
 
+/* Host-side failure injection: the next wfq_apply on the context runs as if one of its kernels'
+ * bounded waits had given up with `code` (non-zero; 0 takes the injection back). */
+int wfq_selftest_fail_next_apply(wfq_ctx *ctx, int code);
+
 /* Kernel timing (profiling aid).  While enabled, the library records a pair of CUDA
  * events on the launching stream around every launch of the kernels below;
  * wfq_profile_read synchronises those events and returns the launch count and the
@@ -266,7 +270,8 @@ int wfq_geometry_info(const wfq_geom *g, int64_t *n, int64_t *nnz, int64_t *devi
  * FP64 / DF use the stored FP64 D if present, else recompute D (matrix-free).  MIXED uses
  * the stored bf16 planes if present, else generates the D tiles from the coordinates on
  * the fly (matrix-free tensor-core path).  Asynchronous on `stream` when x and y are
- * device pointers. */
+ * device pointers.  If a kernel's bounded wait gives up, y is NaN throughout; a call with y in
+ * host memory, which waits for it, also returns WFQ_ETIMEOUT.  Later calls are not affected. */
 int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, void *y,
               int prec, void *stream);
 

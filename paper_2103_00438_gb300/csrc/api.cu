@@ -286,6 +286,12 @@ int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out) {
     return selftest_wait(ctx, limit_us, out, nullptr);
 }
 
+int wfq_selftest_fail_next_apply(wfq_ctx *ctx, int code) {
+    if (!ctx) return fail(WFQ_EINVAL, "context is NULL");
+    ctx->fail_next_apply.store(code);
+    return WFQ_OK;
+}
+
 int wfq_create(wfq_ctx **out, int device) {
     if (!out) return fail(WFQ_EINVAL, "ctx out-pointer is NULL");
     *out = nullptr;
@@ -632,7 +638,7 @@ int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, vo
     DeviceGuard dg(g->ctx->device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int64_t n = g->n, nc = n * ncplx;
-    std::vector<double2> zh(ncplx);
+    std::vector<double2> zh(ncplx + 1);   // the shifts, then the call's error word
     if (g->op == OP_BEM && prec == WFQ_PREC_MIXED && !g->Dhi)
         return fail(WFQ_EUNSUPPORTED, "the mixed apply of a BEM geometry needs WFQ_STORE_BF16X2");
     const ShiftModel zm = shift_model(g);
@@ -641,9 +647,14 @@ int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, vo
         if (!(std::isfinite(zh[c].x) && std::isfinite(zh[c].y)))
             return fail(WFQ_EINVAL, "z(omega) is not finite (BEM: omega = 0 or eps_in = eps_out)");
     }
+    const int injected = g->ctx->fail_next_apply.exchange(0);
+    std::memcpy(&zh[ncplx], &injected, sizeof(int));
     DevBuf<double2> z;
-    WFQ_TRY(z.alloc(g->ctx, ncplx, s));
-    WFQ_CUDA(cudaMemcpyAsync(z.ptr, zh.data(), sizeof(double2) * ncplx, cudaMemcpyHostToDevice, s));
+    WFQ_TRY(z.alloc(g->ctx, ncplx + 1, s));
+    WFQ_CUDA(cudaMemcpyAsync(z.ptr, zh.data(), sizeof(double2) * (ncplx + 1), cudaMemcpyHostToDevice, s));
+    // A wait that gives up is recorded for this call alone: y becomes NaN, and a call that waits for
+    // its y in host memory returns WFQ_ETIMEOUT.
+    int *err = reinterpret_cast<int *>(z.ptr + ncplx), err_h = 0;
     if (prec == WFQ_PREC_FP64 || prec == WFQ_PREC_DF) {
         Staged<double2> X, Y;
         WFQ_TRY(X.in(g->ctx, static_cast<const double2 *>(x), nc, true, s));
@@ -651,10 +662,11 @@ int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, vo
         DevBuf<double2> U;
         WFQ_TRY(U.alloc(g->ctx, nc, s));
         if (prec == WFQ_PREC_DF)
-            WFQ_TRY(d_apply_df(g, ncplx, X.dev, U.ptr, s));
+            WFQ_TRY(d_apply_df(g, ncplx, X.dev, U.ptr, s, err));
         else
-            WFQ_TRY(d_apply_fp64(g, ncplx, X.dev, U.ptr, s));
-        WFQ_TRY(sparse_shift_fp64(g, ncplx, U.ptr, X.dev, z.ptr, Y.dev, s));
+            WFQ_TRY(d_apply_fp64(g, ncplx, X.dev, U.ptr, s, err));
+        WFQ_TRY(sparse_shift_fp64(g, ncplx, U.ptr, X.dev, z.ptr, Y.dev, s, err));
+        if (Y.host) WFQ_CUDA(cudaMemcpyAsync(&err_h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         WFQ_TRY(Y.out(s));
     } else {
         Staged<float2> X, Y;
@@ -667,12 +679,14 @@ int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, vo
             WFQ_TRY(d_apply_fmm(g, ncplx, X.dev, U.ptr, s));
         } else {
             WFQ_TRY(scratch.alloc(g->ctx, mixed_scratch_bytes(g, ncplx), s));
-            WFQ_TRY(d_apply_mixed(g, ncplx, X.dev, U.ptr, scratch.ptr, s));
+            WFQ_TRY(d_apply_mixed(g, ncplx, X.dev, U.ptr, scratch.ptr, s, err));
         }
-        WFQ_TRY(sparse_shift_fp32(g, ncplx, U.ptr, X.dev, z.ptr, Y.dev, s));
+        WFQ_TRY(sparse_shift_fp32(g, ncplx, U.ptr, X.dev, z.ptr, Y.dev, s, err));
+        if (Y.host) WFQ_CUDA(cudaMemcpyAsync(&err_h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         WFQ_TRY(Y.out(s));
     }
     WFQ_CUDA(cudaGetLastError());
+    if (err_h != 0) return fail(WFQ_ETIMEOUT, "a bounded device-side wait gave up (code " + std::to_string(err_h) + ")");
     return WFQ_OK;
 }
 

@@ -2,6 +2,8 @@
 //   u = D x              (dense; FP64 stored / FP64 recomputed / 3xBF16 tensor cores)
 //   y = Kbar u - P u - z x   (sparse neighbour term of Eq. 16-17 plus the shift of Eq. 14)
 // Block vectors are atom-major: (atom i, complex column c) at i * cc + c.
+#include <math_constants.h>
+
 #include "common.h"
 #include "dfloat.cuh"
 
@@ -406,11 +408,11 @@ __global__ void __launch_bounds__(256) k_dotf_df(int64_t n, int64_t C, const flo
     }
 }
 
-int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s) {
+int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
     // symmetric float-pair tiles: read them, 4 real vectors per pass (the product that
     // regenerates D from the coordinates' float pairs held the true residual of a 1.5e5-atom
     // sodium sphere near 5e-7, where the stored pairs reach 5e-9)
-    if (!g->D64 && !g->Dfh && g->Dsym) return d_apply_pairs_df(g, cc, X, U, s);
+    if (!g->D64 && !g->Dfh && g->Dsym) return d_apply_pairs_df(g, cc, X, U, s, err);
     if (!g->D64 && !g->Dfh) {
         // matrix-free double-float product
         WFQ_TRY(require_wfq(g));
@@ -434,14 +436,14 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
         return WFQ_OK;
     }
     const int64_t n = g->n, C = 2 * cc;
-    if (C <= 8 && g->D64) return d_apply_fp64(g, cc, X, U, s);   // few columns: memory bound, FP64 GEMV
-    if (!g->digits_ok) return g->Dfh ? d_apply_pairs_df(g, cc, X, U, s) : d_apply_fp64(g, cc, X, U, s);
+    if (C <= 8 && g->D64) return d_apply_fp64(g, cc, X, U, s, err);   // few columns: memory bound, FP64 GEMV
+    if (!g->digits_ok) return g->Dfh ? d_apply_pairs_df(g, cc, X, U, s, err) : d_apply_fp64(g, cc, X, U, s, err);
     // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
     // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     DevBuf<int> bad;
     WFQ_TRY(bad.alloc(g->ctx, 1, s));
-    return digits_product(g, 7, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), bad.ptr, s);
+    return digits_product(g, 7, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), bad.ptr, s, err);
 }
 
 template <int C>
@@ -455,7 +457,7 @@ static void launch_dgemv64(int64_t n, const double *D, const double *x, double *
         k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u);
 }
 
-int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s) {
+int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
     const int64_t n = g->n, C = 2 * cc;
     // The FP64 GEMV takes about 2e-6 n^2 C us (FP64 pipe), the digit slices 45 + 4e-6 n^2 whatever
     // C is up to 32: from 2 columns and 4096 atoms on the latter (6000 atoms, 2 columns: 188 against
@@ -463,7 +465,7 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     const bool few_by_digits = g->digits_ok && C >= 4 && n >= 4096;
     // no FP64 D but stored float pairs: their double-float product (2^-48 per product, on
     // the FP32 pipes and at 8 or 4 bytes per entry) instead of regenerating D in FP64
-    if (!g->D64 && (g->Dfh || g->Dsym) && C <= 8) return d_apply_pairs_df(g, cc, X, U, s);
+    if (!g->D64 && (g->Dfh || g->Dsym) && C <= 8) return d_apply_pairs_df(g, cc, X, U, s, err);
     const double *x = reinterpret_cast<const double *>(X);
     double *u = reinterpret_cast<double *>(U);
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
@@ -483,7 +485,7 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
             // 10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
             DevBuf<int> bad;
             WFQ_TRY(bad.alloc(g->ctx, 1, s));
-            WFQ_TRY(digits_product(g, 8, C, x, u, bad.ptr, s));
+            WFQ_TRY(digits_product(g, 8, C, x, u, bad.ptr, s, err));
             k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, bad.ptr);
         } else if (g->D64) {
             k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, nullptr);
@@ -510,6 +512,13 @@ struct CplxT<float2> {
     using R = float;
 };
 
+// v, or NaN when a product's bounded wait gave up: what it left of U is not the product.
+template <class V>
+__device__ __forceinline__ V unless_failed(V v, const int *err) {
+    if (err != nullptr && *err != 0) v.x = v.y = CUDART_NAN_F;
+    return v;
+}
+
 // Many columns: lpc lanes (a power of two, at most 32) per atom row over complex columns, so a
 // warp covers 32 / lpc rows; blockIdx.y: chunk of lpc columns.  A block's rows are consecutive
 // and work on the same columns, so that the neighbours they share come from L1, and four
@@ -523,7 +532,7 @@ __global__ void __launch_bounds__(512) k_sparse_cols(int64_t n, int64_t cc, int 
                                                      const int32_t *__restrict__ col,
                                                      const VAL *__restrict__ val,
                                                      const V *__restrict__ U, const V *__restrict__ X,
-                                                     const double2 *__restrict__ z, V *__restrict__ Y) {
+                                                     const double2 *__restrict__ z, V *__restrict__ Y, const int *err) {
     using R = typename CplxT<V>::R;
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lpc;
     const int64_t c = (int64_t)blockIdx.y * lpc + (threadIdx.x & (lpc - 1));
@@ -559,7 +568,7 @@ __global__ void __launch_bounds__(512) k_sparse_cols(int64_t n, int64_t cc, int 
     V out;
     out.x = ax - (zr * xv.x - zi * xv.y);
     out.y = ay - (zr * xv.y + zi * xv.x);
-    Y[i * cc + c] = out;
+    Y[i * cc + c] = unless_failed(out, err);
 }
 
 // Few columns (cc <= 4): one warp per atom row, lanes over neighbours.
@@ -568,7 +577,7 @@ __global__ void __launch_bounds__(128) k_sparse_nbrs(int64_t n, const int64_t *_
                                                      const int32_t *__restrict__ col,
                                                      const VAL *__restrict__ val,
                                                      const V *__restrict__ U, const V *__restrict__ X,
-                                                     const double2 *__restrict__ z, V *__restrict__ Y) {
+                                                     const double2 *__restrict__ z, V *__restrict__ Y, const int *err) {
     using R = typename CplxT<V>::R;
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
@@ -611,7 +620,7 @@ __global__ void __launch_bounds__(128) k_sparse_nbrs(int64_t n, const int64_t *_
             V out;
             out.x = ax[c] - (zr * xv.x - zi * xv.y);
             out.y = ay[c] - (zr * xv.y + zi * xv.x);
-            Y[i * CC + c] = out;
+            Y[i * CC + c] = unless_failed(out, err);
         }
     }
 }
@@ -620,7 +629,7 @@ __global__ void __launch_bounds__(128) k_sparse_nbrs(int64_t n, const int64_t *_
 template <class V>
 __global__ void __launch_bounds__(256) k_shift_only(int64_t total, int64_t cc, const V *__restrict__ U,
                                                     const V *__restrict__ X, const double2 *__restrict__ z,
-                                                    V *__restrict__ Y) {
+                                                    V *__restrict__ Y, const int *err) {
     using R = typename CplxT<V>::R;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= total) return;
@@ -630,31 +639,31 @@ __global__ void __launch_bounds__(256) k_shift_only(int64_t total, int64_t cc, c
     V out;
     out.x = u.x - (zr * xv.x - zi * xv.y);
     out.y = u.y - (zr * xv.y + zi * xv.x);
-    Y[e] = out;
+    Y[e] = unless_failed(out, err);
 }
 
 template <class V, class VAL>
 static int sparse_shift_impl(const wfq_geom *g, int64_t cc, const V *U, const V *X, const double2 *z,
-                             V *Y, const VAL *val, cudaStream_t s) {
+                             V *Y, const VAL *val, cudaStream_t s, const int *err) {
     const int64_t n = g->n;
     unsigned blocks = (unsigned)((n * 32 + 127) / 128);
     KScope ks(g->ctx, WFQ_KT_SPARSE, s);
     if (g->op == OP_BEM) {
         const int64_t total = n * cc;
-        k_shift_only<V><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(total, cc, U, X, z, Y); note_launch();
+        k_shift_only<V><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(total, cc, U, X, z, Y, err); note_launch();
         WFQ_CUDA(cudaGetLastError());
         return WFQ_OK;
     }
     switch (cc) {
-        case 1: k_sparse_nbrs<V, VAL, 1><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
-        case 2: k_sparse_nbrs<V, VAL, 2><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
-        case 3: k_sparse_nbrs<V, VAL, 3><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
-        case 4: k_sparse_nbrs<V, VAL, 4><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y); note_launch(); break;
+        case 1: k_sparse_nbrs<V, VAL, 1><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y, err); note_launch(); break;
+        case 2: k_sparse_nbrs<V, VAL, 2><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y, err); note_launch(); break;
+        case 3: k_sparse_nbrs<V, VAL, 3><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y, err); note_launch(); break;
+        case 4: k_sparse_nbrs<V, VAL, 4><<<blocks, 128, 0, s>>>(n, g->rowptr, g->col, val, U, X, z, Y, err); note_launch(); break;
         default: {
             int lpc = 8;
             while (lpc < cc && lpc < 32) lpc *= 2;
             const dim3 grid((unsigned)((n * lpc + 511) / 512), (unsigned)((cc + lpc - 1) / lpc));
-            k_sparse_cols<V, VAL><<<grid, 512, 0, s>>>(n, cc, lpc, g->rowptr, g->col, val, U, X, z, Y); note_launch();
+            k_sparse_cols<V, VAL><<<grid, 512, 0, s>>>(n, cc, lpc, g->rowptr, g->col, val, U, X, z, Y, err); note_launch();
         }
     }
     WFQ_CUDA(cudaGetLastError());
@@ -662,13 +671,13 @@ static int sparse_shift_impl(const wfq_geom *g, int64_t cc, const V *U, const V 
 }
 
 int sparse_shift_fp64(const wfq_geom *g, int64_t cc, const double2 *U, const double2 *X,
-                      const double2 *z, double2 *Y, cudaStream_t s) {
-    return sparse_shift_impl<double2, double>(g, cc, U, X, z, Y, g->val64, s);
+                      const double2 *z, double2 *Y, cudaStream_t s, const int *err) {
+    return sparse_shift_impl<double2, double>(g, cc, U, X, z, Y, g->val64, s, err);
 }
 
 int sparse_shift_fp32(const wfq_geom *g, int64_t cc, const float2 *U, const float2 *X,
-                      const double2 *z, float2 *Y, cudaStream_t s) {
-    return sparse_shift_impl<float2, float>(g, cc, U, X, z, Y, g->val32, s);
+                      const double2 *z, float2 *Y, cudaStream_t s, const int *err) {
+    return sparse_shift_impl<float2, float>(g, cc, U, X, z, Y, g->val32, s, err);
 }
 
 // ------------------------------------------------------------------ mixed: split + GEMM
@@ -711,7 +720,7 @@ size_t mixed_scratch_bytes(const wfq_geom *g, int64_t cc) {
 }
 
 int d_apply_mixed(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, void *scratch,
-                  cudaStream_t s) {
+                  cudaStream_t s, int *err) {
     // without stored planes, the fast-multipole product when its tree is built (at large N
     // both faster and, at order >= 6, closer to D than the generated 3xBF16 tiles)
     if (!g->Dhi && g->fmm && cc <= 256) return d_apply_fmm(g, cc, X, U, s);
@@ -722,8 +731,8 @@ int d_apply_mixed(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, voi
     dim3 grid((unsigned)(npad / 32), (unsigned)((cpad + 31) / 32));
     k_split_bf16<<<grid, 256, 0, s>>>(g->n, npad, C, cpad, reinterpret_cast<const float *>(X), xhi, xlo); note_launch();
     WFQ_CUDA(cudaGetLastError());
-    if (g->Dhi) return gemm_3xbf16(g, cpad, xhi, xlo, reinterpret_cast<float *>(U), C, s);
-    return gemm_3xbf16_mf(g, cpad, xhi, xlo, reinterpret_cast<float *>(U), C, s);
+    if (g->Dhi) return gemm_3xbf16(g, cpad, xhi, xlo, reinterpret_cast<float *>(U), C, s, err);
+    return gemm_3xbf16_mf(g, cpad, xhi, xlo, reinterpret_cast<float *>(U), C, s, err);
 }
 
 }  // namespace wfq

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <map>
 #include <mutex>
@@ -138,6 +139,7 @@ struct wfq_ctx {
     int num_sms = 0;
     cudaMemPool_t pool = nullptr;
     int *dev_err = nullptr;   // device flag: non-zero after a bounded wait in a kernel gave up
+    std::atomic<int> fail_next_apply{0};   // wfq_selftest_fail_next_apply
     wfq::KernelTimer timer;
     // autotuner results: kernel tiling chosen by timing, per problem key (kept across
     // geometries of the same shape)
@@ -269,20 +271,24 @@ int launch_polarizability(const wfq_geom *g, int64_t ncols, const double2 *q, do
 
 // ------------------------------------------------------------------ operator pieces
 // Block vectors are atom-major: element (atom i, complex column c) at i * cc + c.
+// err: device word in which a kernel records that a bounded wait gave up (its product is then not
+// complete); null: the context's, which the solvers read.  sparse_shift_*, the last step of an apply,
+// writes NaN when its err (null: none) is set.
 
 // U = D X in FP64 (stored FP64 D if present, else recomputed from the coordinates).
-int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
+int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
 
 // U = D X to double-float accuracy (about 48 significant bits) or better: exact digit slices
 // for more than 4 complex columns on stored planes, else double-float or FP64 kernels.  Used
 // for the refinement residual of mixed-precision solves.
-int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
+int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
 
 // U = D X for C real columns (row-major) by S = 7 or 8 exact digit slices on the tensor cores
 // (gemm_digits.cu): S = 8 from the FP64 D, S = 7 from the FP32 pair planes, else the FP64 D.
 // Needs g->digits_ok.  bad: device int, set to 1 when a column of X has an Inf or NaN (its
 // results are NaN), else 0.
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s);
+int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s,
+                   int *err = nullptr);
 
 // U = D V for C <= 4 real vectors by exact digit slices from the stored float pairs (symmetric
 // tiles or full planes; gemv_digits.cu).  Buffers of one stream's products: digit planes of the
@@ -298,12 +304,13 @@ size_t gemv_digits_plane_elems(const wfq_geom *g);
 // digits of the vectors X (element i of vector c at i si + c sc)
 int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s);
 // U (same indexing) = D times the vectors whose digits are in w
-int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s);
+int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s,
+                        int *err = nullptr);
 
 // U = D X for at most 4 complex columns with double-float products (~2^-48 per product)
 // from the stored float pairs (full planes or symmetric tiles) -- the FP64-grade product of
 // geometries that store no FP64 D (shifted.cu).
-int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
+int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
 // The same for a geometry with no stored D: D regenerated per product in double-float
 // (the shifted solver's matrix-free GEMV), at most 4 complex columns.
 int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);
@@ -313,7 +320,7 @@ int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 
 // scratch: at least mixed_scratch_bytes(g, cc) bytes of device memory.
 size_t mixed_scratch_bytes(const wfq_geom *g, int64_t cc);
 int d_apply_mixed(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, void *scratch,
-                  cudaStream_t s);
+                  cudaStream_t s, int *err = nullptr);
 
 // Fast-multipole D product (fmm.cu): build the tree and operators of an order, free them,
 // their device bytes, the tree summary of wfq_fmm_info, and U = D X with it (FP32).
@@ -325,19 +332,19 @@ int d_apply_fmm(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, cudaS
 
 // Y = Kbar U - P U - z_c X   (z: device, cc values); BEM geometries: Y = U - z_c X
 int sparse_shift_fp64(const wfq_geom *g, int64_t cc, const double2 *U, const double2 *X,
-                      const double2 *z, double2 *Y, cudaStream_t s);
+                      const double2 *z, double2 *Y, cudaStream_t s, const int *err = nullptr);
 int sparse_shift_fp32(const wfq_geom *g, int64_t cc, const float2 *U, const float2 *X,
-                      const double2 *z, float2 *Y, cudaStream_t s);
+                      const double2 *z, float2 *Y, cudaStream_t s, const int *err = nullptr);
 
 // U[n x ldu] (fp32, row-major) = Dhi.Xhi + Dhi.Xlo + Dlo.Xhi where Xhi/Xlo are
 // [cpad x npad] bf16 (K-major), cpad a multiple of 64 and >= ldu.  Only rows < n and
 // columns < ldu of U are written.
 int gemm_3xbf16(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi,
-                const __nv_bfloat16 *Xlo, float *U, int64_t ldu, cudaStream_t s);
+                const __nv_bfloat16 *Xlo, float *U, int64_t ldu, cudaStream_t s, int *err = nullptr);
 
 // As gemm_3xbf16 with the D tiles generated from the atom records (matrix-free).
 int gemm_3xbf16_mf(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi,
-                   const __nv_bfloat16 *Xlo, float *U, int64_t ldu, cudaStream_t s);
+                   const __nv_bfloat16 *Xlo, float *U, int64_t ldu, cudaStream_t s, int *err = nullptr);
 
 // ------------------------------------------------------------------ solvers
 

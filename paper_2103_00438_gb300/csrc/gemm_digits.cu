@@ -595,7 +595,8 @@ cudaError_t launch_digits(const CUtensorMap &m, const DigitParams &dp, int grid,
 
 }  // namespace
 
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s) {
+int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s,
+                   int *err) {
     wfq_ctx *ctx = g->ctx;
     const int64_t n = g->n, npad = g->npad;
     const int nhalf = (int)((C + DG_HALF - 1) / DG_HALF);
@@ -620,7 +621,7 @@ int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double 
     WFQ_CUDA(cudaGetLastError());
     DigitParams dp{};
     dp.p.n = n;
-    dp.p.err = ctx->dev_err;
+    dp.p.err = err ? err : ctx->dev_err;
     dp.p.timeout_ns = 4000000000ull;
     dp.C = C;
     dp.nhalf = nhalf;

@@ -101,7 +101,8 @@ inline int64_t gemm_key(int kernel, int64_t npad, int64_t cpad) {
 }  // namespace
 
 int gemm_3xbf16_mf(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi, const __nv_bfloat16 *Xlo, float *U,
-                   int64_t ldu, cudaStream_t s) {
+                   int64_t ldu, cudaStream_t s, int *err) {
+    if (!err) err = g->ctx->dev_err;
     std::string msg;
     int launches = 0;
     // timing twelve launches costs seconds at a million atoms (1.4 s per launch): large
@@ -109,12 +110,12 @@ int gemm_3xbf16_mf(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi, co
     const int st = g->npad > 262144 ? 0 : tuned_stages(g, gemm_key(2, g->npad, cpad), s, [&](int stg) {
         int l = 0;
         const cudaError_t e = tc::gemm3_mf(g->atom32, g->atom32p, g->n, g->npad, Xhi, Xlo, cpad, U, ldu, g->ctx->num_sms,
-                                           g->ctx->dev_err, s, &l, nullptr, stg);
+                                           err, s, &l, nullptr, stg);
         for (int i = 0; i < l; ++i) note_launch();
         return e;
     });
     KScope ks(g->ctx, WFQ_KT_GEMM_MIXED, s, 6.0 * (double)g->n * (double)g->n * (double)ldu);
-    cudaError_t e = tc::gemm3_mf(g->atom32, g->atom32p, g->n, g->npad, Xhi, Xlo, cpad, U, ldu, g->ctx->num_sms, g->ctx->dev_err,
+    cudaError_t e = tc::gemm3_mf(g->atom32, g->atom32p, g->n, g->npad, Xhi, Xlo, cpad, U, ldu, g->ctx->num_sms, err,
                                  s, &launches, &msg, st);
     for (int i = 0; i < launches; ++i) note_launch();
     if (e != cudaSuccess) {
@@ -125,19 +126,20 @@ int gemm_3xbf16_mf(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi, co
 }
 
 int gemm_3xbf16(const wfq_geom *g, int64_t cpad, const __nv_bfloat16 *Xhi, const __nv_bfloat16 *Xlo, float *U,
-                int64_t ldu, cudaStream_t s) {
+                int64_t ldu, cudaStream_t s, int *err) {
+    if (!err) err = g->ctx->dev_err;
     std::string msg;
     int launches = 0;
     const int st = tuned_stages(g, gemm_key(1, g->npad, cpad), s, [&](int stg) {
         int l = 0;
         const cudaError_t e = tc::gemm3_tc(g->Dhi, g->Dlo, g->n, g->npad, Xhi, Xlo, cpad, U, ldu, g->ctx->num_sms,
-                                           g->ctx->dev_err, s, &l, nullptr, stg);
+                                           err, s, &l, nullptr, stg);
         for (int i = 0; i < l; ++i) note_launch();
         return e;
     });
     KScope ks(g->ctx, WFQ_KT_GEMM_MIXED, s, 6.0 * (double)g->n * (double)g->n * (double)ldu);
     cudaError_t e = tc::gemm3_tc(g->Dhi, g->Dlo, g->n, g->npad, Xhi, Xlo, cpad, U, ldu, g->ctx->num_sms,
-                                 g->ctx->dev_err, s, &launches, &msg, st);
+                                 err, s, &launches, &msg, st);
     for (int i = 0; i < launches; ++i) note_launch();
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -606,11 +606,12 @@ int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int
     return WFQ_OK;
 }
 
-int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s) {
+int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s,
+                        int *err) {
     const int64_t n = g->n;
     SymvParams sp{};
     sp.p.n = n;
-    sp.p.err = g->ctx->dev_err;
+    sp.p.err = err ? err : g->ctx->dev_err;
     sp.p.timeout_ns = 4000000000ull;
     sp.T = (int)((n + SV_K - 1) / SV_K);
     const int64_t A = (sp.T + 1) / 2;

@@ -19,25 +19,32 @@ constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;  // 32 MiB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
-// Device address of g_noalloc_scratch per device, looked up once per device with that
+// Set by a kernel whose bounded wait gave up; cleared at the start of each call.
+static __device__ int g_noalloc_err;
+
+// Device addresses of g_noalloc_scratch and g_noalloc_err per device, looked up once per device with that
 // device current (in host code the symbol is only a host-side stand-in).
 constexpr int kMaxDevices = 64;
 static std::mutex g_noalloc_mu;
 static void *g_noalloc_addr[kMaxDevices] = {};
+static void *g_noalloc_err_addr[kMaxDevices] = {};
 
-static int noalloc_scratch(int device, void **out) {
+static int noalloc_scratch(int device, void **out, int **err) {
     if (device < 0 || device >= kMaxDevices) return fail(WFQ_EINVAL, "device index out of range");
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
     if (!g_noalloc_addr[device]) {
-        void *p = nullptr;
+        void *p = nullptr, *pe = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (e != cudaSuccess || p == nullptr) {
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&pe, g_noalloc_err);
+        if (e != cudaSuccess || p == nullptr || pe == nullptr) {
             cudaGetLastError();
             return fail(WFQ_ECUDA, std::string("cudaGetSymbolAddress(static scratch): ") + cudaGetErrorString(e));
         }
+        g_noalloc_err_addr[device] = pe;
         g_noalloc_addr[device] = p;
     }
     *out = g_noalloc_addr[device];
+    *err = static_cast<int *>(g_noalloc_err_addr[device]);
     return WFQ_OK;
 }
 
@@ -49,8 +56,9 @@ struct NoallocOmega {
     double w[kNoAllocMaxCols];
 };
 
-__global__ void k_noalloc_z(int64_t ncplx, ShiftModel m, NoallocOmega om, double2 *__restrict__ z) {
+__global__ void k_noalloc_z(int64_t ncplx, ShiftModel m, NoallocOmega om, double2 *__restrict__ z, int *err) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c == 0) *err = 0;
     if (c >= ncplx) return;
     z[c] = z_eval(m, om.w[c]);
 }
@@ -92,7 +100,8 @@ extern "C" int wfq_apply_mixed_noalloc(wfq_geom *g, int64_t ncplx, const double 
             break;
         }
         void *base = nullptr;
-        if ((rc = noalloc_scratch(g->ctx->device, &base)) != WFQ_OK) break;
+        int *err = nullptr;
+        if ((rc = noalloc_scratch(g->ctx->device, &base, &err)) != WFQ_OK) break;
         unsigned char *b = static_cast<unsigned char *>(base);
         double2 *z = reinterpret_cast<double2 *>(b);
         float2 *u = reinterpret_cast<float2 *>(b + z_bytes);
@@ -100,15 +109,15 @@ extern "C" int wfq_apply_mixed_noalloc(wfq_geom *g, int64_t ncplx, const double 
         cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
         NoallocOmega om;
         for (int64_t c = 0; c < ncplx; ++c) om.w[c] = omega[c];
-        k_noalloc_z<<<(unsigned)((ncplx + 127) / 128), 128, 0, s>>>(ncplx, shift_model(g), om, z);
+        k_noalloc_z<<<(unsigned)((ncplx + 127) / 128), 128, 0, s>>>(ncplx, shift_model(g), om, z, err);
         note_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) {
             rc = fail(WFQ_ECUDA, std::string("z kernel: ") + cudaGetErrorString(e));
             break;
         }
-        if ((rc = d_apply_mixed(g, ncplx, static_cast<const float2 *>(x), u, planes, s)) != WFQ_OK) break;
-        rc = sparse_shift_fp32(g, ncplx, u, static_cast<const float2 *>(x), z, static_cast<float2 *>(y), s);
+        if ((rc = d_apply_mixed(g, ncplx, static_cast<const float2 *>(x), u, planes, s, err)) != WFQ_OK) break;
+        rc = sparse_shift_fp32(g, ncplx, u, static_cast<const float2 *>(x), z, static_cast<float2 *>(y), s, err);
     } while (0);
     if (prev >= 0 && prev != g->ctx->device) cudaSetDevice(prev);
     return rc;

@@ -1077,7 +1077,7 @@ __global__ void k_cols_gather(int64_t n, int C, const double *__restrict__ Ud, d
 
 }  // namespace
 
-int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s) {
+int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
     const int64_t n = g->n;
     const int C = (int)(2 * cc);
     if (!(g->Dfh || g->Dsym)) return fail(WFQ_EUNSUPPORTED, "float-pair product: needs stored pairs");
@@ -1098,7 +1098,7 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
             // rows past 8 cg and atoms past n stay zero
             WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
             WFQ_TRY(gemv_digits_split(g, cg, reinterpret_cast<const double *>(X) + d0, C, 1, w, s));
-            WFQ_TRY(gemv_digits_product(g, cg, w, reinterpret_cast<double *>(U) + d0, C, 1, s));
+            WFQ_TRY(gemv_digits_product(g, cg, w, reinterpret_cast<double *>(U) + d0, C, 1, s, err));
         }
         return WFQ_OK;
     }

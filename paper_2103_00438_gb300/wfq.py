@@ -25,7 +25,8 @@ EXPORTS = ["wfq_create", "wfq_destroy", "wfq_last_error", "wfq_kernel_launches",
            "wfq_geometry_info", "wfq_apply", "wfq_rhs", "wfq_solve_gmres", "wfq_solve_gmres_shifted", "wfq_solve_qmr",
            "wfq_polarizability", "wfq_profile", "wfq_profile_read", "wfq_apply_mixed_noalloc",
            "wfq_server_create", "wfq_server_submit", "wfq_server_poll", "wfq_server_destroy",
-           "wfq_memory_stats", "wfq_cross_section", "wfq_fmm_build", "wfq_fmm_info", "wfq_selftest_wait"]
+           "wfq_memory_stats", "wfq_cross_section", "wfq_fmm_build", "wfq_fmm_info", "wfq_selftest_wait",
+           "wfq_selftest_fail_next_apply"]
 KT_GEMM_MIXED, KT_DAPPLY_FP64, KT_SPARSE, KT_ORTHO, KT_RESIDUAL, KT_DGEMV_DF, KT_FMM = 0, 1, 2, 3, 4, 5, 6
 
 
@@ -94,6 +95,7 @@ def load(path: str | None = None):
     L.wfq_profile.argtypes = [_P, INT]
     L.wfq_memory_stats.argtypes = [_P, _P]
     L.wfq_selftest_wait.argtypes = [_P, INT, _P]
+    L.wfq_selftest_fail_next_apply.argtypes = [_P, INT]
     L.wfq_fmm_build.argtypes = [_P, INT]
     L.wfq_fmm_info.argtypes = [_P, _P]
     L.wfq_cross_section.argtypes = [_P, I64, _P, INT, _P, D, _P, _P, _P, _P]
@@ -195,6 +197,10 @@ class Context:
         out = np.zeros(3, dtype=np.int32)
         _check(_lib.wfq_selftest_wait(self.h, int(limit_us), out.ctypes.data))
         return tuple(int(v) for v in out)
+
+    def selftest_fail_next_apply(self, code: int = 9):
+        """The next apply on this context runs as if a kernel's bounded wait had given up."""
+        _check(_lib.wfq_selftest_fail_next_apply(self.h, int(code)))
 
     def close(self):
         if self.h:
