@@ -558,8 +558,7 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     };
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);
     if ((rc = galloc(g, &g->elem, n))) return bail(rc);
-    if ((rc = galloc(g, &g->rowptr, (n + 1) + (n + 1) / 2))) return bail(rc);   // empty sparse term, row exponents
-    g->dexp = reinterpret_cast<int *>(g->rowptr + n + 1);
+    if ((rc = galloc(g, &g->rowptr, n + 1))) return bail(rc);   // empty sparse term
     if ((rc = galloc(g, &g->D64, (size_t)n * n))) return bail(rc);
     if (store & WFQ_STORE_BF16X2) {
         if ((rc = galloc(g, &g->Dhi, (size_t)g->npad * g->npad))) return bail(rc);
@@ -585,25 +584,12 @@ int wfq_build_bem_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const dou
     if (e == cudaSuccess) e = cudaMemcpy(g->elem, el.data(), sizeof(elem64_t) * n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(g->rowptr, 0, sizeof(int64_t) * (n + 1));
     if (e == cudaSuccess) e = cudaMemset(close, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(g->dexp, 0x80, sizeof(int) * n);   // kDexpNone
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("upload: ") + cudaGetErrorString(e)));
     if ((rc = launch_build_bem(g, close, nullptr))) return done(rc);
     int close_h = 0;
     e = cudaMemcpy(&close_h, close, sizeof(int), cudaMemcpyDeviceToHost);   // synchronises the build
     if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM build: ") + cudaGetErrorString(e)));
     if (close_h) return done(fail(WFQ_EINVAL, "two surface elements closer than 1e-8 bohr"));
-    // row exponents: a row of zeros (possible on a flat surface) takes any scale
-    std::vector<int> dexp(n);
-    e = cudaMemcpy(dexp.data(), g->dexp, sizeof(int) * n, cudaMemcpyDeviceToHost);
-    bool none = false;
-    for (int64_t i = 0; i < n; ++i)
-        if (dexp[i] == kDexpNone) {
-            dexp[i] = 0;
-            none = true;
-        }
-    set_exponent_range(g, dexp);
-    if (e == cudaSuccess && none) e = cudaMemcpy(g->dexp, dexp.data(), sizeof(int) * n, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return done(fail(WFQ_ECUDA, std::string("BEM row exponents: ") + cudaGetErrorString(e)));
     done(WFQ_OK);
     *out = g;
     return WFQ_OK;

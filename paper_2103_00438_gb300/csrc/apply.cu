@@ -199,6 +199,68 @@ __global__ void __launch_bounds__(256) k_dotf(int64_t n, int64_t C, const atom64
     }
 }
 
+// ------------------------------------------------------------------ double-float stored D
+
+// U[n x C] = D[n x n] X[n x C] with double-float products (df_mac): every FP64 operand
+// split into a float pair (hi = fp32(v), lo = fp32(v - hi): 48 significant bits).  This
+// runs on the FP32 pipes, which GB300 has far more of than FP64.  PL: D comes from the
+// stored FP32 pair planes (no FP64 arithmetic at all); else it is split from the FP64 D.
+
+template <bool PL>
+__global__ void __launch_bounds__(256) k_dgemm_df(int64_t n, int64_t C, const double *__restrict__ D,
+                                                  const float *__restrict__ Fh, const float *__restrict__ Fl,
+                                                  int64_t ldf, const double *__restrict__ X, double *__restrict__ U) {
+    __shared__ float Ah[16][64], Al[16][64], Bh[16][64], Bl[16][64];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
+    float sh[4][4] = {}, sl[4][4] = {};
+    for (int64_t k0 = 0; k0 < n; k0 += 16) {
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const int e = tid + l * 256;
+            const int r = e >> 4, kk = e & 15;
+            const int64_t gi = m0 + r, gk = k0 + kk;
+            if (PL) {
+                const bool in = gi < n && gk < n;
+                Ah[kk][r] = in ? Fh[gi * ldf + gk] : 0.f;
+                Al[kk][r] = in ? Fl[gi * ldf + gk] : 0.f;
+            } else {
+                df_split((gi < n && gk < n) ? D[gi * n + gk] : 0.0, Ah[kk][r], Al[kk][r]);
+            }
+            const int kb = e >> 6, cb = e & 63;
+            const int64_t bk = k0 + kb, bc = n0 + cb;
+            df_split((bk < n && bc < C) ? X[bk * C + bc] : 0.0, Bh[kb][cb], Bl[kb][cb]);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int kk = 0; kk < 16; ++kk) {
+            float ah[4], al[4], bh[4], bl[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                ah[t] = Ah[kk][ty * 4 + t];
+                al[t] = Al[kk][ty * 4 + t];
+                bh[t] = Bh[kk][tx * 4 + t];
+                bl[t] = Bl[kk][tx * 4 + t];
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) df_mac(ah[r], al[r], bh[c], bl[c], sh[r][c], sl[r][c]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t gi = m0 + ty * 4 + r;
+        if (gi >= n) continue;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int64_t gc = n0 + tx * 4 + c;
+            if (gc < C) U[gi * C + gc] = (double)sh[r][c] + (double)sl[r][c];
+        }
+    }
+}
+
 // ------------------------------------------------------------------ double-float matrix-free D
 
 // Exact a - b of two floats as an unevaluated sum (Knuth's two-difference).
@@ -348,8 +410,7 @@ int d_gemv_df_mf(const wfq_geom *g, int C, const float *xh, const float *xl, dou
     return WFQ_OK;
 }
 
-// U[n x C] = D[n x n] X[n x C] with double-float products (df_mac) on the FP32 pipes, the D
-// tile generated per use (matrix-free); TN columns per thread.
+// As k_dgemm_df with the D tile generated per use (matrix-free); TN columns per thread.
 template <int TN>
 __global__ void __launch_bounds__(256) k_dotf_df(int64_t n, int64_t C, const float4 *__restrict__ adf,
                                                  const atom64_t *__restrict__ a64, const double *__restrict__ eta,
@@ -437,13 +498,27 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     }
     const int64_t n = g->n, C = 2 * cc;
     if (C <= 8 && g->D64) return d_apply_fp64(g, cc, X, U, s, err);   // few columns: memory bound, FP64 GEMV
-    if (!g->digits_ok) return g->Dfh ? d_apply_pairs_df(g, cc, X, U, s, err) : d_apply_fp64(g, cc, X, U, s, err);
-    // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
-    // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.
+    const double *x = reinterpret_cast<const double *>(X);
+    double *u = reinterpret_cast<double *>(U);
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-    DevBuf<int> bad;
-    WFQ_TRY(bad.alloc(g->ctx, 1, s));
-    return digits_product(g, 7, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), bad.ptr, s, err);
+    // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
+    // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.  Below
+    // 128 atoms its launches take longer than they save (us per apply of 16 columns, pairs: 40
+    // atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
+    if (g->digits_ok && n >= 128) {
+        DevBuf<int> bad;
+        WFQ_TRY(bad.alloc(g->ctx, 1, s));
+        return digits_product(g, 7, C, x, u, bad.ptr, s, err);
+    }
+    dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
+    if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
+    if (g->Dfh)
+        k_dgemm_df<true><<<grid, 256, 0, s>>>(n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u);
+    else
+        k_dgemm_df<false><<<grid, 256, 0, s>>>(n, C, g->D64, nullptr, nullptr, 0, x, u);
+    note_launch();
+    WFQ_CUDA(cudaGetLastError());
+    return WFQ_OK;
 }
 
 template <int C>

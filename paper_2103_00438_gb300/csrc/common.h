@@ -172,9 +172,11 @@ struct wfq_geom {
     float4 *atomdf = nullptr;   // 2 per atom: (xh, xl, yh, yl), (zh, zl, width, 0) float pairs
     double *eta = nullptr;      // n
     int *dexp = nullptr;        // n, stored FP64 D, FP32 planes or tiles: |D_ij| < 2^dexp[i]
-                                // (in the allocation of eta, of rowptr for BEM geometries)
+                                // (in the allocation of eta; null for BEM geometries)
     int dexp_min = 0, dexp_max = 0;
-    bool digits_ok = false;     // every dexp within +-kDigitExpMax (the digit-slice products)
+    // Digit-slice products: omega-FQ with every dexp within +-kDigitExpMax.  Not BEM: they hold an
+    // entry to a fraction of its row's bound, and a BEM entry may be any fraction of it, down to 0.
+    bool digits_ok = false;
     wfq::elem64_t *elem = nullptr;   // BEM geometries: n element records
 
     // Kbar CSR (device)
@@ -255,9 +257,7 @@ int build_kbar_csr(int64_t n, const double *xyz, const wfq_params &p, std::vecto
 
 int launch_build_d(const wfq_geom *g, cudaStream_t s);
 // BEM geometries: the operator's entries into the requested storages; *close is set
-// non-zero (device int) when two elements lie closer than 1e-8 bohr.  Also g->dexp, each
-// row's largest exponent (kDexpNone for a row of zeros).
-constexpr int kDexpNone = -0x7f7f7f80;   // bytes of 0x80
+// non-zero (device int) when two elements lie closer than 1e-8 bohr.
 int launch_build_bem(const wfq_geom *g, int *close, cudaStream_t s);
 int launch_rhs(const wfq_geom *g, int ndir, const double *dirs_dev, double E0, double *R,
                cudaStream_t s);

@@ -589,7 +589,7 @@ cudaError_t launch_c(const CUtensorMap &m, const SymvParams &sp, int grid, cudaS
 // rows share one exponent (a column's sum runs over the rows), so the rows' bounds must not differ
 // by more than 2^3: a row then loses at most 3 of its 55 bits.
 bool gemv_digits_usable(const wfq_geom *g) {
-    return g->digits_ok && (g->Dfh || g->Dsym) && g->op == OP_WFQ && g->dexp_max - g->dexp_min <= 3;
+    return g->digits_ok && (g->Dfh || g->Dsym) && g->dexp_max - g->dexp_min <= 3;
 }
 
 size_t gemv_digits_plane_elems(const wfq_geom *g) { return (size_t)SV_ROWS * g->npad; }

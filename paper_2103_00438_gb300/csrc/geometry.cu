@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256) k_build_d(const atom64_t *__restrict__ at
 __global__ void k_build_bem(const elem64_t *__restrict__ el, int64_t n, int64_t npad, int64_t lim,
                             double *__restrict__ D64, __nv_bfloat16 *__restrict__ hi,
                             __nv_bfloat16 *__restrict__ lo, int64_t ldf, float *__restrict__ fh,
-                            float *__restrict__ fl, int *__restrict__ close, int *__restrict__ dexp) {
+                            float *__restrict__ fl, int *__restrict__ close) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t i = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= lim || j >= lim) return;
@@ -206,10 +206,6 @@ __global__ void k_build_bem(const elem64_t *__restrict__ el, int64_t n, int64_t 
                 v = a.area * (a.nx * dx + a.ny * dy + a.nz * dz) / (r2 * sqrt(r2));
             }
         }
-        // the row's largest exponent (a warp's lanes share the row): |v| < 2^(field - 1022)
-        const unsigned mask = __activemask();
-        const int f = __reduce_max_sync(mask, (__double2hiint(v) >> 20) & 0x7ff);
-        if (f > 0 && (threadIdx.x & 31) == __ffs(mask) - 1) atomicMax(dexp + i, f - 1022);
     }
     if (D64 && i < n && j < n) D64[i * n + j] = v;
     if (fh && i < n && j < ldf) {
@@ -231,7 +227,7 @@ int launch_build_bem(const wfq_geom *g, int *close, cudaStream_t s) {
     dim3 grid((unsigned)((lim + 63) / 64), (unsigned)((lim + 3) / 4));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "stored BEM operator with more than 262140 rows");
     k_build_bem<<<grid, block, 0, s>>>(g->elem, g->n, g->npad, lim, g->D64, g->Dhi, g->Dlo, g->ldf, g->Dfh, g->Dfl,
-                                       close, g->dexp); note_launch();
+                                       close); note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
 }
