@@ -110,9 +110,14 @@ typedef struct {
 
 /* Arithmetic of an apply / of the inner Krylov iterations. */
 enum {
-    WFQ_PREC_FP64 = 0,     /* FP64 operator, complex128 vectors (more than 4 columns on a stored
-                              FP64 D: 8 exact digits per operand on the tensor cores, at least
-                              as accurate as FP64 sums) */
+    WFQ_PREC_FP64 = 0,     /* FP64 operator, complex128 vectors.  An omega-FQ geometry with a stored
+                              FP64 D and more than 4 columns (2 and more from 4096 atoms): D.x by
+                              8 digits of 8 bits per operand on the tensor cores, integer sums.
+                              What they leave out is absolute -- per atom at most 2^-58 of the
+                              powers of two above the row's and the column's largest entries -- so
+                              columns for which that can exceed the bound of FP64 sums (a few
+                              entries dominate: the sum of |x| is small beside the largest) take
+                              plain FP64 sums instead, column by column, as other blocks do */
     WFQ_PREC_MIXED = 1,    /* D.x from 3 bf16 products (hi.hi + hi.lo + lo.hi) with FP32
                               accumulation on the tensor cores, D from the stored bf16 planes
                               or generated from the coordinates -- or, without stored planes
@@ -122,12 +127,13 @@ enum {
                               residuals use the WFQ_PREC_DF product (on a geometry with no
                               stored D, D regenerated in FP64 once that product's rounding
                               holds a residual at a floor) */
-    WFQ_PREC_DF = 2,       /* wfq_apply and the refinement residuals: complex128 vectors, D.x to
-                              double-float accuracy (~2^-48 relative per product) or better:
-                              more than 4 columns on the stored FP64 D or FP32 pair planes by
-                              exact digit slices on the tensor cores (7 signed 8-bit digits of
-                              D and x, integer sums); up to 4 columns the FP64 GEMV of the
-                              stored FP64 D, else float pairs: digit slices of the upper
+    WFQ_PREC_DF = 2,       /* wfq_apply and the refinement residuals: complex128 vectors, D.x with
+                              the error bound of double-float sums (~2^-48 relative per product)
+                              or a smaller one: more than 4 columns on the stored FP64 D or FP32
+                              pair planes by 7 digits per operand as above (2^-50; from 128 atoms
+                              on, omega-FQ geometries; dominated columns and other blocks in
+                              double-float); up to 4 columns as WFQ_PREC_FP64 on a stored FP64 D,
+                              else float pairs: digit slices of the upper
                               triangle (symmetric tiles, or 3072 atoms and more on the planes;
                               row bounds sqrt(2) eta_i within a factor of 8), or double-float
                               accumulation on the FP32 pipes (smaller planes, or D regenerated

@@ -429,6 +429,20 @@ int wfq_build_geometry(wfq_ctx *ctx, int64_t n, const double *xyz, const double 
         dexp.resize(n);
         for (int64_t i = 0; i < n; ++i) dexp[i] = std::ilogb(1.4142135623730951 * eta_h[i]) + 1;
         set_exponent_range(g, dexp);
+        // D decreases with the distance and the widths: at the diagonal of the bounding box with the
+        // largest widths (w = sqrt(2 / pi) / eta, Eq. 4) it is below every entry.
+        double d2 = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            double lo = xyz[k], hi = xyz[k];
+            for (int64_t i = 1; i < n; ++i) {
+                lo = std::min(lo, xyz[3 * i + k]);
+                hi = std::max(hi, xyz[3 * i + k]);
+            }
+            d2 += (hi - lo) * (hi - lo);
+        }
+        const double smax = 2.0 / (std::sqrt(3.14159265358979323846) * *std::min_element(eta_h.begin(), eta_h.end()));
+        const double r = std::max(std::sqrt(d2), 1e-6 * smax);
+        g->dmin = std::erf(r / smax) / r;
     }
 
     if ((rc = galloc(g, &g->xyz, 3 * n))) return bail(rc);

@@ -15,10 +15,17 @@ namespace wfq {
 // that every X element read from L2 serves RW D rows; D rows are read coalesced.  Bound by the
 // FP64 pipe (1.7 operations per clock per SM), so below 9728 atoms, where 4 rows a warp would
 // leave SMs idle, a warp takes 1 or 2: 1014 atoms, C = 2: 9.5 us, 26.2 with 4 rows.  The order of
-// a row's sum does not depend on RW.
+// a row's sum does not depend on RW.  cols: as k_dgemm.
 template <int C, int RW>
 __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restrict__ D,
-                                               const double *__restrict__ X, double *__restrict__ U) {
+                                               const double *__restrict__ X, double *__restrict__ U,
+                                               const DigitCols cols) {
+    if (cols.cmax) {
+        bool any = false;
+#pragma unroll
+        for (int c = 0; c < C; ++c) any = any || col_plain(cols, c, true);
+        if (!any) return;
+    }
     int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     int64_t i0 = warp * RW;
@@ -72,20 +79,23 @@ __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restri
         for (int r = 0; r < RW; ++r)
             if (i0 + r < n)
 #pragma unroll
-                for (int c = 0; c < C; ++c) U[(i0 + r) * C + c] = acc[r][c];
+                for (int c = 0; c < C; ++c)
+                    if (col_plain(cols, c, true)) U[(i0 + r) * C + c] = acc[r][c];
     }
 }
 
 // ------------------------------------------------------------------ FP64 stored D: many columns
 
-// U[n x C] = D[n x n] X[n x C], row-major, 64 x 64 tiles, 4 x 4 outputs per thread.  Runs only
-// when only_if is null or *only_if is set: it is what the digit-slice product (gemm_digits.cu)
-// leaves to plain FP64 -- columns with an Inf or NaN, whose signs and NaNs it reproduces, and
-// geometries whose entries lie outside the digits' exponent range.
+// U[n x C] = D[n x n] X[n x C], row-major, 64 x 64 tiles, 4 x 4 outputs per thread: every column
+// for geometries that the digit slices (gemm_digits.cu) do not serve, else the columns that they
+// leave (cols; blocks without one return at once).
 __global__ void __launch_bounds__(256) k_dgemm(int64_t n, int64_t C, const double *__restrict__ D,
                                                const double *__restrict__ X, double *__restrict__ U,
-                                               const int *__restrict__ only_if) {
-    if (only_if && *only_if == 0) return;
+                                               const DigitCols cols) {
+    if (cols.cmax) {
+        const int64_t c = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
+        if (!__syncthreads_or(c < C && col_plain(cols, c, true))) return;
+    }
     __shared__ double As[16][65];
     __shared__ double Bs[16][64];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -125,7 +135,7 @@ __global__ void __launch_bounds__(256) k_dgemm(int64_t n, int64_t C, const doubl
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             int64_t gc = n0 + tx * 4 + c;
-            if (gc < C) U[gi * C + gc] = acc[r][c];
+            if (gc < C && col_plain(cols, gc, true)) U[gi * C + gc] = acc[r][c];
         }
     }
 }
@@ -204,12 +214,18 @@ __global__ void __launch_bounds__(256) k_dotf(int64_t n, int64_t C, const atom64
 // U[n x C] = D[n x n] X[n x C] with double-float products (df_mac): every FP64 operand
 // split into a float pair (hi = fp32(v), lo = fp32(v - hi): 48 significant bits).  This
 // runs on the FP32 pipes, which GB300 has far more of than FP64.  PL: D comes from the
-// stored FP32 pair planes (no FP64 arithmetic at all); else it is split from the FP64 D.
+// stored FP32 pair planes (no FP64 arithmetic at all); else it is split from the FP64 D.  cols: as
+// k_dgemm, columns that are not finite excepted (NaN from the digits).
 
 template <bool PL>
 __global__ void __launch_bounds__(256) k_dgemm_df(int64_t n, int64_t C, const double *__restrict__ D,
                                                   const float *__restrict__ Fh, const float *__restrict__ Fl,
-                                                  int64_t ldf, const double *__restrict__ X, double *__restrict__ U) {
+                                                  int64_t ldf, const double *__restrict__ X, double *__restrict__ U,
+                                                  const DigitCols cols) {
+    if (cols.cmax) {
+        const int64_t c = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
+        if (!__syncthreads_or(c < C && col_plain(cols, c, false))) return;
+    }
     __shared__ float Ah[16][64], Al[16][64], Bh[16][64], Bl[16][64];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
@@ -256,7 +272,7 @@ __global__ void __launch_bounds__(256) k_dgemm_df(int64_t n, int64_t C, const do
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const int64_t gc = n0 + tx * 4 + c;
-            if (gc < C) U[gi * C + gc] = (double)sh[r][c] + (double)sl[r][c];
+            if (gc < C && col_plain(cols, gc, false)) U[gi * C + gc] = (double)sh[r][c] + (double)sl[r][c];
         }
     }
 }
@@ -505,31 +521,28 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.  Below
     // 128 atoms its launches take longer than they save (us per apply of 16 columns, pairs: 40
     // atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
-    if (g->digits_ok && n >= 128) {
-        DevBuf<int> bad;
-        WFQ_TRY(bad.alloc(g->ctx, 1, s));
-        return digits_product(g, 7, C, x, u, bad.ptr, s, err);
-    }
+    DigitColsBuf cols;
+    if (g->digits_ok && n >= 128) WFQ_TRY(digits_product(g, 7, C, x, u, cols, s, err));
     dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
     if (g->Dfh)
-        k_dgemm_df<true><<<grid, 256, 0, s>>>(n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u);
+        k_dgemm_df<true><<<grid, 256, 0, s>>>(n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u, cols.dc);
     else
-        k_dgemm_df<false><<<grid, 256, 0, s>>>(n, C, g->D64, nullptr, nullptr, 0, x, u);
+        k_dgemm_df<false><<<grid, 256, 0, s>>>(n, C, g->D64, nullptr, nullptr, 0, x, u, cols.dc);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
 }
 
 template <int C>
-static void launch_dgemv64(int64_t n, const double *D, const double *x, double *u, cudaStream_t s) {
+static void launch_dgemv64(int64_t n, const double *D, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
     auto blocks = [&](int rw) { return (unsigned)(((n + rw - 1) / rw + 7) / 8); };
     if (n >= 9728)   // 16 warps an SM on 152 SMs
-        k_dgemv<C, 4><<<blocks(4), 256, 0, s>>>(n, D, x, u);
+        k_dgemv<C, 4><<<blocks(4), 256, 0, s>>>(n, D, x, u, cols);
     else if (n >= 4864)
-        k_dgemv<C, 2><<<blocks(2), 256, 0, s>>>(n, D, x, u);
+        k_dgemv<C, 2><<<blocks(2), 256, 0, s>>>(n, D, x, u, cols);
     else
-        k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u);
+        k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u, cols);
 }
 
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
@@ -544,32 +557,28 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     const double *x = reinterpret_cast<const double *>(X);
     double *u = reinterpret_cast<double *>(U);
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-    if (g->D64 && C <= 8 && !few_by_digits) {
+    DigitColsBuf cols;
+    // eight exact digits on the tensor cores; dominated columns and those that are not finite in
+    // plain FP64.  10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
+    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) WFQ_TRY(digits_product(g, 8, C, x, u, cols, s, err));
+    if (g->D64 && C <= 8) {
         switch (C) {
-            case 2: launch_dgemv64<2>(n, g->D64, x, u, s); break;
-            case 4: launch_dgemv64<4>(n, g->D64, x, u, s); break;
-            case 6: launch_dgemv64<6>(n, g->D64, x, u, s); break;
-            default: launch_dgemv64<8>(n, g->D64, x, u, s); break;
+            case 2: launch_dgemv64<2>(n, g->D64, x, u, cols.dc, s); break;
+            case 4: launch_dgemv64<4>(n, g->D64, x, u, cols.dc, s); break;
+            case 6: launch_dgemv64<6>(n, g->D64, x, u, cols.dc, s); break;
+            default: launch_dgemv64<8>(n, g->D64, x, u, cols.dc, s); break;
         }
-        note_launch();
     } else {
         dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
         if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "FP64 apply: too many rows");
-        if (g->D64 && g->digits_ok) {
-            // eight exact digits on the tensor cores; columns that are not finite in FP64.
-            // 10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
-            DevBuf<int> bad;
-            WFQ_TRY(bad.alloc(g->ctx, 1, s));
-            WFQ_TRY(digits_product(g, 8, C, x, u, bad.ptr, s, err));
-            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, bad.ptr);
-        } else if (g->D64) {
-            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, nullptr);
+        if (g->D64) {
+            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, cols.dc);
         } else {
             WFQ_TRY(require_wfq(g));
             k_dotf<<<grid, 256, 0, s>>>(n, C, g->atom64, g->eta, x, u);
         }
-        note_launch();
     }
+    note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
 }

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/wfq.h"
+#include "digit_cols.cuh"
 
 namespace wfq {
 
@@ -174,6 +175,7 @@ struct wfq_geom {
     int *dexp = nullptr;        // n, stored FP64 D, FP32 planes or tiles: |D_ij| < 2^dexp[i]
                                 // (in the allocation of eta; null for BEM geometries)
     int dexp_min = 0, dexp_max = 0;
+    double dmin = 0.0;          // with dexp: no entry of D is below it
     // Digit-slice products: omega-FQ with every dexp within +-kDigitExpMax.  Not BEM: they hold an
     // entry to a fraction of its row's bound, and a BEM entry may be any fraction of it, down to 0.
     bool digits_ok = false;
@@ -285,9 +287,16 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
 
 // U = D X for C real columns (row-major) by S = 7 or 8 exact digit slices on the tensor cores
 // (gemm_digits.cu): S = 8 from the FP64 D, S = 7 from the FP32 pair planes, else the FP64 D.
-// Needs g->digits_ok.  bad: device int, set to 1 when a column of X has an Inf or NaN (its
-// results are NaN), else 0.
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s,
+// Needs g->digits_ok.  Columns of X with an Inf or NaN give NaN; those that few entries dominate are
+// not written: plain kernels take them, by cols (allocated here, on s).
+struct DigitColsBuf {
+    DevBuf<unsigned long long> buf;
+    DigitCols dc{nullptr, nullptr, 0};
+    void set(const wfq_geom *g, int S, int64_t C);
+};
+// 2^8 2^log2_ratio 2^max(E) / dmin (digit_cols.cuh), capped
+unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio);
+int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err = nullptr);
 
 // U = D V for C <= 4 real vectors by exact digit slices from the stored float pairs (symmetric

@@ -9,11 +9,13 @@
 // them stay below 2^24, so the FP32 accumulators of the tensor cores hold every partial sum
 // exactly.  The digit products d_a e_b with a + b = w < S share one accumulator (weight
 // 2^(-8w)); each 128-atom chunk's accumulators are read back, converted to integers and added
-// to a 96-bit integer per output.  Nothing is rounded before the final conversion to FP64, so
+// to a 96-bit integer per output.  Nothing is rounded before the final conversion to FP64 (but
+// for S = 7 the weights 4 to 6 of a chunk, as one float), and a chunk's sum is one integer, so
 // the result does not depend on how the work is split; what is left out is the digits past the
-// S-th (2^-63 or 2^-55 of the row's and column's bound) and the digit products with
-// a + b >= S.  S = 8 stands for FP64 products, S = 7 for double-float ones: the error against
-// exact sums is below that of the plain FP64 and double-float chains for both.
+// S-th (2^-62 or 2^-54 of the row's and column's bound) and the digit products with
+// a + b >= S.  S = 8 stands for FP64 products, S = 7 for double-float ones; columns whose sum of
+// magnitudes is too small beside their largest entry for the bounds above to be below those of plain
+// sums are left to plain kernels (digit_cols.cuh).
 //
 // Why: GB300 has about 2 FP64 FMAs per clock per SM (0.5e12/s) and the double-float product
 // costs 12 FP32 operations; the tensor cores do 36 (S = 8) or 28 (S = 7) fp16 digit products
@@ -46,8 +48,10 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "common.h"
+#include "digit_cols.cuh"
 #include "gemm_tc.cuh"
 
 namespace wfq {
@@ -81,6 +85,7 @@ struct DigitParams {
     int64_t ld;
     const int *dexp;     // n: |D_ij| < 2^dexp[i]
     unsigned long long *acc;   // [n][C][2]: sums in units of 2^-24 and of 2^-56
+    DigitCols cols;
 };
 
 // v 2^(8S - 2 - E) as an integer (|v| < 2^E), truncated for S = 8, rounded for S = 7; done on
@@ -151,6 +156,11 @@ __device__ __forceinline__ void add96(uint32_t &t0, uint32_t &t1, uint32_t &t2, 
 template <int S, int SRC>
 __global__ void __launch_bounds__(DG_THREADS, 1)
     k_gemm_digits(const __grid_constant__ CUtensorMap tm_x, const DigitParams dp) {
+    {   // nothing to do when plain sums take every column
+        bool mine = false;
+        for (int64_t c = threadIdx.x; c < dp.C; c += DG_THREADS) mine = mine || col_state(dp.cols, c) == COL_DIGITS;
+        if (!__syncthreads_or(mine)) return;
+    }
     const Params &p = dp.p;
     constexpr uint32_t A_STAGE = S * DG_A_BYTES;
     constexpr uint32_t B_HALF = S * DG_HALF * ROWB;   // one half's X digit planes of a stage
@@ -172,7 +182,6 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int64_t u_begin = dp.units * (int64_t)blockIdx.x / gridDim.x;
     const int64_t u_end = dp.units * ((int64_t)blockIdx.x + 1) / gridDim.x;
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < DG_STAGES; ++s) {
             tc::mbar_init(tc::smem_u32(b_full + s), 1);
@@ -258,8 +267,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
                         lo = (int64_t)__float2int_rn(v[0]) * 16777216 + (int64_t)__float2int_rn(v[1]) * 65536 +
                              (int64_t)__float2int_rn(v[2]) * 256 + __float2int_rn(v[3]);
                     } else {
-                        // weights 4 to 6 as one float in units of 2^-7 of weight 4: rounded at
-                        // 2^-24 of s_4, 2^-51 of the bounds' product
+                        // weights 4 to 6 as one float in units of 2^-7 of weight 4: exact below
+                        // 2^24 units (as for digits of varying signs), else rounded at 2^-24 of
+                        // s_4, at most 2^-52 of the bounds' product per nonzero entry
                         const float f = fmaf(v[0], 128.f, fmaf(v[1], 0.5f, v[2] * 0.001953125f));
                         lo = (int64_t)__float2int_rn(f) * 131072;
                     }
@@ -531,46 +541,54 @@ __device__ __forceinline__ int col_exp(unsigned long long bits) {
 // 64 atoms x 32 columns.
 template <int S>
 __global__ void __launch_bounds__(256) k_split_digits(int64_t n, int64_t npad, int64_t C, const double *__restrict__ X,
-                                                      const unsigned long long *__restrict__ cmax,
-                                                      __half *__restrict__ planes) {
+                                                      DigitCols cols, __half *__restrict__ planes) {
     __shared__ uint64_t t[64][33];
+    __shared__ unsigned qsum[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int64_t a0 = (int64_t)blockIdx.x * 64, c = (int64_t)blockIdx.y * 32 + tx;
-    const unsigned long long mb = c < C ? cmax[c] : 0ull;
+    const unsigned long long mb = c < C ? cols.cmax[c] : 0ull;
     const bool finite = mb < 0x7ff0000000000000ull;
     const int e = col_exp(mb);
+    unsigned q = 0;   // 2^8 |x| / 2^e
 #pragma unroll
     for (int r = ty; r < 64; r += 8) {
         const int64_t a = a0 + r;
         const double v = (a < n && c < C && finite) ? X[a * C + c] : 0.0;
-        t[r][tx] = biased<S>(fixed_point<S>(v, e));
+        const int64_t f = fixed_point<S>(v, e);
+        q += (unsigned)((uint64_t)(f < 0 ? -f : f) >> (8 * S - 10));
+        t[r][tx] = biased<S>(f);
     }
+    qsum[ty][tx] = q;
     __syncthreads();
+    if (ty == 0 && c < C) {
 #pragma unroll
-    for (int q = ty; q < 32; q += 8) {
-        const uint64_t v0 = t[2 * tx][q], v1 = t[2 * tx + 1][q];
+        for (int k = 1; k < 8; ++k) q += qsum[k][tx];
+        atomicAdd(cols.csum + c, q);
+    }
+#pragma unroll
+    for (int cr = ty; cr < 32; cr += 8) {
+        const uint64_t v0 = t[2 * tx][cr], v1 = t[2 * tx + 1][cr];
 #pragma unroll
         for (int d = 0; d < S; ++d) {
             const int sft = 8 * (S - 1 - d);
             const uint32_t w = (uint32_t)((v0 >> sft) & 0xffu) | ((uint32_t)((v1 >> sft) & 0xffu) << 8);
-            const int64_t row = ((int64_t)blockIdx.y * S + d) * DG_HALF + q;
+            const int64_t row = ((int64_t)blockIdx.y * S + d) * DG_HALF + cr;
             *reinterpret_cast<uint32_t *>(planes + row * npad + a0 + 2 * tx) = digits_f16(w, false);
         }
     }
 }
 
-// U = 2^(E_i + e_c + unit) (acc0 + acc1 2^-32); a column that is not finite gives NaN and
-// sets *bad.
+// U = 2^(E_i + e_c + unit) (acc0 + acc1 2^-32); a column that is not finite gives NaN; columns of
+// the plain sums are left to them.
 __global__ void __launch_bounds__(256) k_digits_finish(int64_t n, int64_t C, const unsigned long long *__restrict__ acc,
-                                                       const int *__restrict__ dexp,
-                                                       const unsigned long long *__restrict__ cmax,
-                                                       int unit, double *__restrict__ U, int *__restrict__ bad) {
+                                                       const int *__restrict__ dexp, DigitCols cols, int unit,
+                                                       double *__restrict__ U) {
     const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= n * C) return;
     const int64_t i = e / C, c = e - i * C;
-    const unsigned long long mb = cmax[c];
-    if (mb >= 0x7ff0000000000000ull) {
-        if (i == 0) *bad = 1;
+    const ColState st = col_state(cols, c);
+    if (st == COL_PLAIN) return;
+    if (st == COL_NOT_FINITE) {
         U[e] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
@@ -579,7 +597,7 @@ __global__ void __launch_bounds__(256) k_digits_finish(int64_t n, int64_t C, con
     const long long hi = (long long)a.x + (long long)(a.y >> 32);
     const unsigned lo = (unsigned)a.y;
     const double v = fma((double)lo, 0x1p-32, (double)hi);
-    U[e] = scalbn(v, dexp[i] + col_exp(mb) + unit);
+    U[e] = scalbn(v, dexp[i] + col_exp(cols.cmax[c]) + unit);
 }
 
 template <int S, int SRC>
@@ -595,28 +613,42 @@ cudaError_t launch_digits(const CUtensorMap &m, const DigitParams &dp, int grid,
 
 }  // namespace
 
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, int *bad, cudaStream_t s,
+void DigitColsBuf::set(const wfq_geom *g, int S, int64_t C) {
+    dc.cmax = buf.ptr;
+    dc.csum = reinterpret_cast<unsigned *>(buf.ptr + C);
+    // What is left out per entry, in 2^(E + e): products with a + b = S, (S - 1) 2^(14 - 8 S) against 2^12,
+    // the truncated or rounded last digits and, S = 7, the float of weights 4 to 6 (2^-24 of 5 2^14 2^7 in
+    // its units): below 2^-58 (S = 8), 2^-50 (S = 7).
+    dc.thr = digit_sum_threshold(g, S == 8 ? -58 + 53 : -50 + 48);
+}
+
+unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio) {
+    const double t = std::ceil(std::ldexp(1.0, 8 + log2_ratio + g->dexp_max) / g->dmin);
+    return t < 4294967295.0 ? (unsigned)t : 4294967295u;
+}
+
+int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err) {
     wfq_ctx *ctx = g->ctx;
     const int64_t n = g->n, npad = g->npad;
     const int nhalf = (int)((C + DG_HALF - 1) / DG_HALF);
     const bool pairs = S == 7 && g->Dfh != nullptr;
     DevBuf<__half> planes;
-    DevBuf<unsigned long long> acc, cmax;
+    DevBuf<unsigned long long> acc;
     WFQ_TRY(planes.alloc(ctx, (size_t)nhalf * S * DG_HALF * npad, s));
     WFQ_TRY(acc.alloc(ctx, (size_t)2 * n * C, s));
-    WFQ_TRY(cmax.alloc(ctx, (size_t)C, s));
+    WFQ_TRY(cols.buf.alloc(ctx, (size_t)C + (C + 1) / 2, s));
+    cols.set(g, S, C);
     WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 2 * n * C, s));
-    WFQ_CUDA(cudaMemsetAsync(cmax.ptr, 0, sizeof(unsigned long long) * C, s));
-    WFQ_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
+    WFQ_CUDA(cudaMemsetAsync(cols.buf.ptr, 0, sizeof(unsigned long long) * ((size_t)C + (C + 1) / 2), s));
     const int64_t rpb = std::max<int64_t>(32, round_up((n + 4 * ctx->num_sms - 1) / (4 * ctx->num_sms), 8));
-    k_col_absmax<<<dim3((unsigned)((n + rpb - 1) / rpb), (unsigned)nhalf), 256, 0, s>>>(n, C, rpb, X, cmax.ptr);
+    k_col_absmax<<<dim3((unsigned)((n + rpb - 1) / rpb), (unsigned)nhalf), 256, 0, s>>>(n, C, rpb, X, cols.dc.cmax);
     note_launch();
     const dim3 sg((unsigned)(npad / 64), (unsigned)nhalf);
     if (S == 8)
-        k_split_digits<8><<<sg, 256, 0, s>>>(n, npad, C, X, cmax.ptr, planes.ptr);
+        k_split_digits<8><<<sg, 256, 0, s>>>(n, npad, C, X, cols.dc, planes.ptr);
     else
-        k_split_digits<7><<<sg, 256, 0, s>>>(n, npad, C, X, cmax.ptr, planes.ptr);
+        k_split_digits<7><<<sg, 256, 0, s>>>(n, npad, C, X, cols.dc, planes.ptr);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     DigitParams dp{};
@@ -634,6 +666,7 @@ int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double 
     dp.ld = g->ldf;
     dp.dexp = g->dexp;
     dp.acc = acc.ptr;
+    dp.cols = cols.dc;
     std::string msg;
     CUtensorMap m;
     const uint32_t rows = (uint32_t)S * DG_HALF;
@@ -649,8 +682,8 @@ int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double 
         cudaGetLastError();
         return fail(WFQ_ECUDA, std::string("digit-slice GEMM: ") + cudaGetErrorString(e));
     }
-    k_digits_finish<<<(unsigned)((n * C + 255) / 256), 256, 0, s>>>(n, C, acc.ptr, g->dexp, cmax.ptr,
-                                                                          pairs ? -35 : -36, U, bad);
+    k_digits_finish<<<(unsigned)((n * C + 255) / 256), 256, 0, s>>>(n, C, acc.ptr, g->dexp, cols.dc,
+                                                                    pairs ? -35 : -36, U);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

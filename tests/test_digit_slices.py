@@ -69,3 +69,43 @@ def test_accumulators_stay_exact():
     # S = 7: weights 4 to 6 as one float in units of 2^-7 of weight 4 fits 31 bits
     assert s[4] * 128 + s[5] // 2 + s[6] // 512 < 2 ** 31
     assert math.log2(s[0]) + 24 + math.log2(2 ** 21 / 128) < 63   # sums of 2^21 atoms
+
+
+def _worst(S):
+    """Fixed-point integers whose digits are all extreme (127 or -128), and random ones."""
+    rng = np.random.default_rng(S)
+    out = []
+    for pick in ([127] * S, [-128] * S, [127, -128] * 4, [-128, 127] * 4):
+        d = [max(-63, min(63, pick[0]))] + list(pick[1:S])
+        out.append(sum(v * 256 ** (S - 1 - a) for a, v in enumerate(d)))
+    out += [int(v) for v in rng.integers(-2 ** 53, 2 ** 53, 200)]
+    return out
+
+
+@pytest.mark.parametrize("S,u", [(8, -58), (7, -50)])
+def test_what_a_product_leaves_out(S, u):
+    """D_ij x_j from the digit products with a + b < S and the last digits of both operands: within
+    2^u of the bounds' product, the constant of csrc/digit_cols.cuh's threshold."""
+    unit = Fraction(2) ** (8 * S - 2)          # operands in units of their bound / unit
+    last = 1 if S == 8 else 2                  # S = 7 from float pairs: two roundings of half 2^(E - 53)
+    for f in _worst(S):
+        for h in _worst(S)[:40]:
+            df, dh = digits((f + BIAS[S]) % 2 ** 64, S), digits((h + BIAS[S]) % 2 ** 64, S)
+            kept = sum(df[a] * dh[b] * 256 ** (2 * S - 2 - a - b) for a in range(S) for b in range(S - a))
+            err = abs(Fraction(kept - f * h)) / unit ** 2 + (last * abs(Fraction(h)) + abs(Fraction(f)) + last) / unit ** 2
+            assert err <= Fraction(2) ** u
+
+
+def test_what_a_chunk_of_one_sign_rounds():
+    """S = 7: weights 4 to 6 of a 128-atom chunk as one float, all digits extreme: with the products
+    left out still within 2^-50 of the bounds' product per entry."""
+    for n in (1, 16, 128):
+        s = [n * (w + 1) * 128 * 128 for w in range(7)]
+        f = np.float32(s[6]) * np.float32(2.0 ** -9)
+        f = np.float32(np.float64(s[5]) * 0.5 + np.float64(f))
+        f = np.float32(np.float64(s[4]) * 128 + np.float64(f))
+        exact = Fraction(s[4]) * 128 + Fraction(s[5], 2) + Fraction(s[6], 512)
+        got = Fraction(int(np.rint(f)))
+        # in units of 2^-7 of weight 4; weight 4 is 2^-32 of weight 0, 2^12 of which is the bound
+        err = abs(got - exact) / 2 ** 7 / 2 ** 32 / 2 ** 12
+        assert err + n * Fraction(6 * 2 ** 14, 2 ** 68) + n * Fraction(3, 2 ** 54) <= n * Fraction(1, 2 ** 50) + Fraction(1, 2 ** 52)

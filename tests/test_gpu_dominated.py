@@ -32,7 +32,7 @@ def _column(kind, n, rng):
     if kind == "spread":
         x[:] = (rng.uniform(0.5, 1, n) + 1j * rng.uniform(0.5, 1, n)) * 10.0 ** rng.uniform(-14, 0, n)
         x[rng.integers(n)] = 0.7 + 0.6j
-    else:
+    else:   # "mixed": five entries, beside another kind of column
         k = rng.choice(n, 1 if kind == "one" else 5, replace=False)
         x[k] = rng.uniform(0.5, 1, len(k)) + 1j * rng.uniform(0.5, 1, len(k))
     return x
@@ -67,3 +67,58 @@ def test_bem_columns(W, ctx, S, prec, planes, ncplx, kind):
     ref = A.astype(np.longdouble) @ x.astype(np.clongdouble) - z * x
     bound = _tau(prec, m) * (B @ (np.abs(x.real) + np.abs(x.imag)) + np.abs(z) * np.abs(x))
     assert np.all(np.abs(y - ref) <= bound)
+
+
+def _far_pair(S, n):
+    """Two clusters 1e5 bohr apart: the entries of D between them are 2^-17 of its largest."""
+    a = S.random_cluster(n - n // 3, seed=n)
+    b = S.random_cluster(n // 3, seed=n + 1)
+    return np.concatenate([a, b + np.array([1e5, 0.0, 0.0])])
+
+
+def _check(W, ctx, orc, S, n, ncplx, store, prec, kind, zero_imag=False):
+    """As for BEM, through the neighbour term; a double-float sum of m entries within (m + 8) 2^-48 s
+    (a rounding of at most 2^-48 s in each step)."""
+    xyz = _far_pair(S, n)
+    p = S.carbon_params(1.51)
+    p["r0"] = 2.7
+    D = orc.d_matrix(xyz, np.full(n, p["eta"]))
+    rowptr, col, val = orc.kbar_csr(xyz, p, cutoff_eps=p["cutoff_eps"])
+    flag = {"fp64": W.STORE_FP64, "pairs": W.STORE_F32X2, "sym": W.STORE_F32X2_SYM}[store]
+    g = W.Geometry(ctx, xyz, p, store=flag)
+    rng = np.random.default_rng(n + ncplx)
+    x = np.stack([_column(kind, n, rng) for _ in range(ncplx)], axis=1)
+    if kind == "mixed":
+        x[:, 0] = S.random_complex((n, 1), seed=2)[:, 0]   # a column for the digits beside the others
+    if zero_imag:
+        x = x.real + 0j
+    om = np.linspace(0.01, 0.1, ncplx)
+    z = np.array([orc.z_of_omega(w, p) for w in om])
+    y = np.empty_like(x)
+    g.apply(om, x, y, prec=W.PREC_FP64 if prec == "fp64" else W.PREC_DF)
+    u = (D @ x.real.astype(np.longdouble)) + 1j * (D @ x.imag.astype(np.longdouble))
+    s = D @ (np.abs(x.real) + np.abs(x.imag))
+    m = np.count_nonzero(x, axis=0)
+    tau = (m + 16) * 2.0 ** -53 if prec == "fp64" else (m + 8) * 2.0 ** -48 + 16 * 2.0 ** -53
+    for i in range(n):
+        q, k = col[rowptr[i]:rowptr[i + 1]], val[rowptr[i]:rowptr[i + 1]][:, None]
+        ref = (k * (u[q] - u[i])).sum(axis=0) - z * x[i]
+        scale = (k * (s[q] + s[i])).sum(axis=0) + np.abs(z) * (np.abs(x[i].real) + np.abs(x[i].imag))
+        assert np.all(np.abs(y[i] - ref) <= (tau + (len(q) + 8) * 2.0 ** -53) * scale), i
+
+
+@pytest.mark.parametrize("kind", ["one", "five", "spread", "mixed"])
+@pytest.mark.parametrize("store,prec", [("fp64", "fp64"), ("fp64", "df"), ("pairs", "df")])
+def test_blocks_of_columns(W, ctx, orc, S, store, prec, kind):
+    _check(W, ctx, orc, S, 451, 6, store, prec, kind)
+
+
+@pytest.mark.parametrize("store,prec", [("fp64", "fp64"), ("pairs", "df")])
+def test_a_block_without_a_column_for_the_digits(W, ctx, orc, S, store, prec):
+    _check(W, ctx, orc, S, 300, 33, store, prec, "one", zero_imag=True)
+
+
+@pytest.mark.parametrize("kind", ["one", "spread", "mixed"])
+@pytest.mark.parametrize("ncplx", [2, 3, 4])
+def test_few_columns_of_a_stored_fp64_operator(W, ctx, orc, S, ncplx, kind):
+    _check(W, ctx, orc, S, 4100, ncplx, "fp64", "fp64", kind)
