@@ -117,7 +117,9 @@ enum {
                               powers of two above the row's and the column's largest entries -- so
                               columns for which that can exceed the bound of FP64 sums (a few
                               entries dominate: the sum of |x| is small beside the largest) take
-                              plain FP64 sums instead, column by column, as other blocks do */
+                              plain FP64 sums instead, column by column, as other blocks do.
+                              Up to 4 columns without a stored FP64 D but with float pairs: as
+                              WFQ_PREC_DF from the tiles (on planes from 3072 atoms on) */
     WFQ_PREC_MIXED = 1,    /* D.x from 3 bf16 products (hi.hi + hi.lo + lo.hi) with FP32
                               accumulation on the tensor cores, D from the stored bf16 planes
                               or generated from the coordinates -- or, without stored planes
@@ -129,15 +131,15 @@ enum {
                               holds a residual at a floor) */
     WFQ_PREC_DF = 2,       /* wfq_apply and the refinement residuals: complex128 vectors, D.x with
                               the error bound of double-float sums (~2^-48 relative per product)
-                              or a smaller one: more than 4 columns on the stored FP64 D or FP32
-                              pair planes by 7 digits per operand as above (2^-50; from 128 atoms
-                              on, omega-FQ geometries; dominated columns and other blocks in
-                              double-float); up to 4 columns as WFQ_PREC_FP64 on a stored FP64 D,
-                              else float pairs: digit slices of the upper
-                              triangle (symmetric tiles, or 3072 atoms and more on the planes;
-                              row bounds sqrt(2) eta_i within a factor of 8), or double-float
-                              accumulation on the FP32 pipes (smaller planes, or D regenerated
-                              from the coordinates in double-float, near pairs in FP64) */
+                              or a smaller one.  Up to 4 columns on a stored FP64 D: as
+                              WFQ_PREC_FP64.  Else from the stored FP64 D or FP32 pair planes by 7
+                              digits per operand as above (2^-50), omega-FQ geometries of 96 atoms
+                              and more; from the symmetric tiles by digits of the upper triangle
+                              (2^-53 of the bounds; from 1100 / min(4, real columns) atoms on, row
+                              bounds sqrt(2) eta_i within a factor of 8; 4 real columns at a time);
+                              dominated columns and other blocks in double-float on the FP32 pipes,
+                              D regenerated from the coordinates where it is not stored (near
+                              pairs in FP64) */
     WFQ_PREC_FMM = 3       /* wfq_apply only: complex64 vectors, D.x by the fast multipole
                               method built with wfq_fmm_build (near field by Eq. 3, far field
                               1/r by Chebyshev interpolation), FP32 arithmetic */

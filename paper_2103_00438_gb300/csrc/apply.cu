@@ -518,11 +518,11 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     double *u = reinterpret_cast<double *>(U);
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     // many columns: seven exact digits on the tensor cores.  cnt20k, 384 real columns, from the
-    // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.  Below
-    // 128 atoms its launches take longer than they save (us per apply of 16 columns, pairs: 40
-    // atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
+    // pair planes: 7.3 ms against 69.9 ms for double-float multiply-adds on the FP32 pipes.  In the
+    // smallest structures its launches take longer than they save (us per apply of 16 columns, pairs:
+    // 40 atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
     DigitColsBuf cols;
-    if (g->digits_ok && n >= 128) WFQ_TRY(digits_product(g, 7, C, x, u, cols, s, err));
+    if (g->digits_ok && n >= 96) WFQ_TRY(digits_product(g, 7, C, x, u, cols, s, err));
     dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
     if (g->Dfh)

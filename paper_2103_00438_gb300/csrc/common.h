@@ -299,22 +299,37 @@ unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio);
 int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err = nullptr);
 
-// U = D V for C <= 4 real vectors by exact digit slices from the stored float pairs (symmetric
-// tiles or full planes; gemv_digits.cu).  Buffers of one stream's products: digit planes of the
-// vectors (gemv_digits_plane_elems, zeroed once), exponents and largest magnitudes (C each) and
-// the integer sums (2 n C, zeroed once; each product leaves them zeroed).
+// U = D V for real vectors, 4 at a time, by exact digit slices from the stored float pairs (symmetric
+// tiles or full planes; gemv_digits.cu).  Buffers of one stream's products of C vectors: digit planes
+// (gemv_digits_plane_elems per group of 4, zeroed once), exponents, largest magnitudes and sums of
+// magnitudes (C each) and the integer sums of a group (8 n, zeroed once; each product leaves them
+// zeroed).  A group with a vector that few entries dominate (VecSums) is left to double-float sums:
+// every step of both ways is launched, and those of the other one return at once.
 struct GemvDigits {
     uint16_t *planes;
     int *xexp;
     unsigned long long *vmax, *acc;
+    unsigned *vsum, thr;
+    bool complex_parts;   // vectors 2 k and 2 k + 1 are the parts of a complex column
+    VecSums sums() const { return VecSums{vsum, complex_parts ? vmax : nullptr, thr}; }
+};
+// Partial sums of the double-float product from the symmetric tiles (null rowpart: none).
+struct SymPartials {
+    const float2 *rowpart, *colpart;
+    const int *item_start;
+    int64_t T;
 };
 bool gemv_digits_usable(const wfq_geom *g);
 size_t gemv_digits_plane_elems(const wfq_geom *g);
-// digits of the vectors X (element i of vector c at i si + c sc)
+unsigned gemv_digits_threshold(const wfq_geom *g);
+// digits of the C vectors X (element i of vector c at i si + c sc); vsum follows vmax in memory
 int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s);
-// U (same indexing) = D times the vectors whose digits are in w
-int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s,
-                        int *err = nullptr);
+// the digit products of a group of C <= 4 vectors, into w.acc
+int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, cudaStream_t s, int *err = nullptr);
+// U (element i of vector c at i si + c sc) of the group: from w.acc, or from the double-float product --
+// sym's partial sums, else ud [C][n] (null: already in U)
+int gemv_digits_finish(const wfq_geom *g, int C, const GemvDigits &w, const SymPartials &sym, const double *ud, double *U,
+                       int64_t si, int64_t sc, cudaStream_t s);
 
 // U = D X for at most 4 complex columns with double-float products (~2^-48 per product)
 // from the stored float pairs (full planes or symmetric tiles) -- the FP64-grade product of

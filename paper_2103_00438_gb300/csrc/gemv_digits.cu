@@ -6,9 +6,10 @@
 //     D_ij = 2^(E - 10) sum_k d_k 2^(-11 k),  k < 5,  |d_k| <= 2048,
 //     v_j  = 2^(e - 5)  sum_m e_m 2^(-7 m),   m < 8,  |e_m| <= 64,
 // with one accumulator per (k, m, vector): sums of 128 products stay within 2^24.  The terms
-// with 11 k + 7 m <= 58 are kept (digits and terms left out: 2^-55 of the bounds and below);
-// each read-back adds them to 64-bit integers, so the result does not depend on the split of
-// the work.  The error against exact sums is below the double-float product's.
+// with 11 k + 7 m <= 56 are kept (digits and terms left out: 2^-53 of the bounds' product at
+// most); each read-back adds them to 64-bit integers, so the result does not depend on the split
+// of the work.  Vectors that few entries dominate, for which that bound can exceed the
+// double-float sums', are left to those (VecSums).
 //
 // Why: the double-float multiply-adds cost 12 FP32 operations per entry and vector.  A digit
 // split costs 12.5 packed instructions per entry for all vectors, and D being symmetric
@@ -47,7 +48,7 @@ namespace {
 using tc::Params;
 
 constexpr int SV_M = 128, SV_K = 64;                 // rows and columns of a stage
-constexpr int SV_ND = 5, SV_NE = 8;                  // digits of D, of a vector
+constexpr int SV_ND = 5;                             // digits of D (a vector has 8)
 constexpr int SV_ROWS = 32;                          // rows of the vector digit planes: m * C + v
 constexpr uint32_t SV_PLANE = SV_M * SV_K * 2;       // one digit plane of a stage
 constexpr uint32_t SV_A = SV_ND * SV_PLANE;
@@ -75,6 +76,7 @@ struct SymvParams {
     int64_t ld;
     int E;                  // |D_ij| < 2^E
     unsigned long long *acc;   // [C][n][2]: units 2^-28 and 2^-56
+    VecSums sums;
 };
 
 // descriptor of a tile of 128-byte rows with the 128-byte swizzle: 8-row groups 1024 bytes apart
@@ -130,6 +132,7 @@ __device__ __forceinline__ void read_terms(uint32_t base, int64_t (&hi)[C], int6
 
 template <int C, bool TILES>
 __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_constant__ CUtensorMap tm_x, const SymvParams sp) {
+    if (sp.sums.plain(C)) return;
     const Params &p = sp.p;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem =
@@ -526,23 +529,37 @@ __global__ void __launch_bounds__(256) k_vec_absmax(int64_t n, int64_t si, int64
 
 __global__ void __launch_bounds__(256) k_vec_digits(int64_t n, int64_t npad, int C, int64_t si, int64_t sc,
                                                     const double *__restrict__ X, const unsigned long long *__restrict__ vmax,
-                                                    __half *__restrict__ planes, int *__restrict__ xexp) {
+                                                    __half *__restrict__ planes, int *__restrict__ xexp,
+                                                    unsigned *__restrict__ vsum) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int c = blockIdx.y;
+    const int c = blockIdx.y, cg = min(4, C - (c & ~3));
     const unsigned long long mb = vmax[c];
     const int e = vec_exp(mb);
-    if (i == 0) xexp[c] = e;
-    if (i < n) put_vec_digits(X[i * si + c * sc], e, planes + (int64_t)c * npad + i, (int64_t)C * npad);
+    __half *dst = planes + (int64_t)(c >> 2) * SV_ROWS * npad + (int64_t)(c & 3) * npad + i;
+    unsigned q = 0;
+    if (i < n) q = put_vec_digits(X[i * si + c * sc], e, dst, (int64_t)cg * npad);
+    q = __reduce_add_sync(0xffffffffu, q);
+    if ((threadIdx.x & 31) == 0 && q > 0) atomicAdd(vsum + c, q);
+    if (i == 0) {
+        xexp[c] = e;
+        if (mb == 0ull || e == kVecNotFinite) vsum[c] = 0xffffffffu;   // nothing is added for these
+    }
 }
 
-// U[i si + c sc] = 2^(E + e_c - 43) (acc0 + acc1 2^-28); the sums are cleared for the next product
+// U[i si + c sc] = 2^(E + e_c - 43) (acc0 + acc1 2^-28), and the sums are cleared for the next
+// product; a group left to double-float sums takes theirs.
 __global__ void __launch_bounds__(256) k_gemv_digits_finish(int64_t n, int C, int64_t si, int64_t sc,
                                                             unsigned long long *__restrict__ acc, int E,
-                                                            const int *__restrict__ xexp,
-                                                            double *__restrict__ U) {
+                                                            const int *__restrict__ xexp, const VecSums sums,
+                                                            const SymPartials sym, const double *ud, double *U) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int c = blockIdx.y;
     if (i >= n) return;
+    if (sums.plain(C)) {
+        if (sym.rowpart) U[i * si + c * sc] = dsymv_sum(sym, C, i, c);
+        else if (ud) U[i * si + c * sc] = ud[c * n + i];
+        return;
+    }
     ulonglong2 *a = reinterpret_cast<ulonglong2 *>(acc) + (int64_t)c * n + i;
     const ulonglong2 s = *a;
     *a = make_ulonglong2(0ull, 0ull);
@@ -594,20 +611,24 @@ bool gemv_digits_usable(const wfq_geom *g) {
 
 size_t gemv_digits_plane_elems(const wfq_geom *g) { return (size_t)SV_ROWS * g->npad; }
 
+// What is left out per entry, in 2^(E + e): the terms with 11 k + 7 m > 56 (2^-55 at most), the last
+// digits of D and of the vector (2^-55 each) and the rounding of D's fourth remainder (2^-57): below 2^-53,
+// against 2^-48 |D_ij v_j| of double-float sums.
+unsigned gemv_digits_threshold(const wfq_geom *g) { return digit_sum_threshold(g, -53 + 48); }
+
 int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s) {
-    WFQ_CUDA(cudaMemsetAsync(w.vmax, 0, sizeof(unsigned long long) * C, s));
+    WFQ_CUDA(cudaMemsetAsync(w.vmax, 0, (sizeof(unsigned long long) + sizeof(unsigned)) * C, s));
     const unsigned nb = (unsigned)std::min<int64_t>((g->n + 255) / 256, 64);
     k_vec_absmax<<<dim3(nb, (unsigned)C), 256, 0, s>>>(g->n, si, sc, X, w.vmax);
     note_launch();
-    k_vec_digits<<<dim3((unsigned)((g->n + 255) / 256), (unsigned)C), 256, 0, s>>>(g->n, g->npad, C, si, sc, X, w.vmax,
-                                                                                  reinterpret_cast<__half *>(w.planes), w.xexp);
+    k_vec_digits<<<dim3((unsigned)((g->n + 255) / 256), (unsigned)C), 256, 0, s>>>(
+        g->n, g->npad, C, si, sc, X, w.vmax, reinterpret_cast<__half *>(w.planes), w.xexp, w.vsum);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
 }
 
-int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U, int64_t si, int64_t sc, cudaStream_t s,
-                        int *err) {
+int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, cudaStream_t s, int *err) {
     const int64_t n = g->n;
     SymvParams sp{};
     sp.p.n = n;
@@ -622,6 +643,7 @@ int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U
     sp.ld = g->ldf;
     sp.E = g->dexp_max;
     sp.acc = w.acc;
+    sp.sums = w.sums();
     std::string msg;
     CUtensorMap m;
     if (!make_x_map(&m, reinterpret_cast<const __half *>(w.planes), (uint64_t)g->npad, &msg)) return fail(WFQ_ECUDA, "digit-slice GEMV: " + msg);
@@ -633,7 +655,13 @@ int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, double *U
         cudaGetLastError();
         return fail(WFQ_ECUDA, std::string("digit-slice GEMV: ") + cudaGetErrorString(e));
     }
-    k_gemv_digits_finish<<<dim3((unsigned)((n + 255) / 256), (unsigned)C), 256, 0, s>>>(n, C, si, sc, w.acc, sp.E, w.xexp, U);
+    return WFQ_OK;
+}
+
+int gemv_digits_finish(const wfq_geom *g, int C, const GemvDigits &w, const SymPartials &sym, const double *ud, double *U,
+                       int64_t si, int64_t sc, cudaStream_t s) {
+    k_gemv_digits_finish<<<dim3((unsigned)((g->n + 255) / 256), (unsigned)C), 256, 0, s>>>(
+        g->n, C, si, sc, w.acc, g->dexp_max, w.xexp, w.sums(), sym, ud, U);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

@@ -72,6 +72,14 @@ constexpr int GV_WARPS = 8;      // warps per block
 constexpr int GV_CHUNK = 1024;   // x entries staged in shared memory per step
 constexpr int GV_NTILINGS = 4;
 
+// Whether a double-float kernel has the product: a group of vectors is the digit slices' unless one of them
+// is dominated; null vsum: whatever the vectors are.
+struct PlainIf {
+    VecSums sums;
+    __device__ __forceinline__ bool runs(int C) const { return !sums.vsum || sums.plain(C); }
+};
+constexpr PlainIf kAlways{{nullptr, nullptr, 0}};
+
 // U[d][i] = sum_j D_ij x[d][j] for C real vectors (direction-major, length n), with
 // double-float products.  Each warp owns ROWS rows and reads them with 16-byte loads
 // (four consecutive j per lane), TB steps of 128 columns at a time so that 2 * ROWS * TB
@@ -79,129 +87,137 @@ constexpr int GV_NTILINGS = 4;
 // chunk in shared memory as separate hi / lo planes so that a quarter-warp's 16-byte reads
 // are conflict-free.  PL: D from the FP32 pair planes (row pitch ld, a multiple of 4, zero
 // beyond n); else split from the FP64 D.  Entries past n contribute zero (x is zero there).
-template <int C, bool PL, int ROWS, int TB, int MINB>
+// LOOP: the launch beside a digit-slice product (pi) -- a few blocks that take the rows in turn, since
+// mostly they return at once, and 2500 blocks that do so took 12 us of a 20000-atom step.
+template <int C, bool PL, int ROWS, int TB, int MINB, bool LOOP = false>
 __global__ void __launch_bounds__(GV_WARPS * 32, MINB) k_dgemv_df(int64_t n, int64_t ld, const float *__restrict__ Fh,
                                                             const float *__restrict__ Fl,
                                                             const double *__restrict__ D64,
                                                             const float *__restrict__ xh,
-                                                            const float *__restrict__ xl, double *__restrict__ U) {
+                                                            const float *__restrict__ xl, double *__restrict__ U,
+                                                            const PlainIf pi) {
+    if (LOOP && !pi.runs(C)) return;
     __shared__ __align__(16) float sxh[C][GV_CHUNK];
     __shared__ __align__(16) float sxl[C][GV_CHUNK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t row0 = ((int64_t)blockIdx.x * GV_WARPS + warp) * ROWS;
-    // FP32 planes (PL): rows of ld floats, ld a multiple of 128, zero past column n, so a
-    // 128-column step that starts below n lies inside the row and needs no column check;
-    // rows past n read the last row (their results are dropped).  This lane's float4 of
-    // each row, as a pointer advanced by the step's float4 index.
-    const float4 *rowh[ROWS], *rowl[ROWS];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
-        if constexpr (PL) {
-            const int64_t i = row0 + r, ic = i < n ? i : n - 1;
-            rowh[r] = reinterpret_cast<const float4 *>(Fh + ic * ld) + lane;
-            rowl[r] = reinterpret_cast<const float4 *>(Fl + ic * ld) + lane;
-        } else {
-            rowh[r] = rowl[r] = nullptr;
-        }
-    }
-    // accumulators per (row, vector): even and odd columns in the two lanes of a float2
-    float2 sh2[ROWS][C], sl2[ROWS][C];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-        for (int d = 0; d < C; ++d) sh2[r][d] = sl2[r][d] = make_float2(0.f, 0.f);
-
-    for (int64_t j0 = 0; j0 < n; j0 += GV_CHUNK) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < C * GV_CHUNK; t += GV_WARPS * 32) {
-            const int d = t / GV_CHUNK, jj = t - d * GV_CHUNK;
-            const int64_t j = j0 + jj;
-            sxh[d][jj] = j < n ? xh[(int64_t)d * n + j] : 0.f;
-            sxl[d][jj] = j < n ? xl[(int64_t)d * n + j] : 0.f;
-        }
-        __syncthreads();
-        const int64_t trem = (n - j0 + 127) / 128;
-        const int tend = trem < GV_CHUNK / 128 ? (int)trem : GV_CHUNK / 128;
-        for (int t0 = 0; t0 < tend; t0 += TB) {
-            float4 dh[TB][ROWS], dl[TB][ROWS];
-#pragma unroll
-            for (int t = 0; t < TB; ++t) {
-                const int tt = t0 + t;
-                const int64_t j = j0 + tt * 128 + lane * 4;
-#pragma unroll
-                for (int r = 0; r < ROWS; ++r) {
-                    const int64_t i = row0 + r;
-                    if constexpr (PL) {
-                        if (tt < tend) {   // warp-uniform: the last chunk may end inside the TB group
-                            const int64_t q = (j0 >> 2) + tt * 32;
-                            dh[t][r] = __ldg(rowh[r] + q);
-                            dl[t][r] = __ldg(rowl[r] + q);
-                        } else {
-                            dh[t][r] = dl[t][r] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-                    } else if (i >= n || j >= n) {
-                        dh[t][r] = dl[t][r] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    } else {
-                        const double *row = D64 + i * n;
-                        float h[4], l[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) df_split(j + e < n ? __ldg(row + j + e) : 0.0, h[e], l[e]);
-                        dh[t][r] = make_float4(h[0], h[1], h[2], h[3]);
-                        dl[t][r] = make_float4(l[0], l[1], l[2], l[3]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < TB; ++t) {
-                const int jl = (t0 + t) * 128 + lane * 4;
-#pragma unroll
-                for (int d = 0; d < C; ++d) {
-                    const float4 xh4 = *reinterpret_cast<const float4 *>(&sxh[d][jl]);
-                    const float4 xl4 = *reinterpret_cast<const float4 *>(&sxl[d][jl]);
-#pragma unroll
-                    for (int r = 0; r < ROWS; ++r) {
-                        df_mac2(make_float2(dh[t][r].x, dh[t][r].y), make_float2(dl[t][r].x, dl[t][r].y),
-                                make_float2(xh4.x, xh4.y), make_float2(xl4.x, xl4.y), sh2[r][d], sl2[r][d]);
-                        df_mac2(make_float2(dh[t][r].z, dh[t][r].w), make_float2(dl[t][r].z, dl[t][r].w),
-                                make_float2(xh4.z, xh4.w), make_float2(xl4.z, xl4.w), sh2[r][d], sl2[r][d]);
-                    }
-                }
-            }
-        }
-    }
-    // the two lanes, then warp sums in double-float, fixed butterfly order
-    float sh[ROWS][C], sl[ROWS][C];
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-        for (int d = 0; d < C; ++d) {
-            sh[r][d] = sh2[r][d].x;
-            sl[r][d] = sl2[r][d].x;
-            df_add(sh[r][d], sl[r][d], sh2[r][d].y, sl2[r][d].y);
-        }
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-        for (int d = 0; d < C; ++d)
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const float oh = __shfl_xor_sync(0xffffffffu, sh[r][d], off);
-                const float ol = __shfl_xor_sync(0xffffffffu, sl[r][d], off);
-                df_add(sh[r][d], sl[r][d], oh, ol);
-            }
-    if (lane == 0) {
+    unsigned block = blockIdx.x;
+    do {
+        const int64_t row0 = ((int64_t)block * GV_WARPS + warp) * ROWS;
+        // FP32 planes (PL): rows of ld floats, ld a multiple of 128, zero past column n, so a
+        // 128-column step that starts below n lies inside the row and needs no column check;
+        // rows past n read the last row (their results are dropped).  This lane's float4 of
+        // each row, as a pointer advanced by the step's float4 index.
+        const float4 *rowh[ROWS], *rowl[ROWS];
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
-            const int64_t i = row0 + r;
-            if (i < n)
-#pragma unroll
-                for (int d = 0; d < C; ++d) U[(int64_t)d * n + i] = (double)sh[r][d] + (double)sl[r][d];
+            if constexpr (PL) {
+                const int64_t i = row0 + r, ic = i < n ? i : n - 1;
+                rowh[r] = reinterpret_cast<const float4 *>(Fh + ic * ld) + lane;
+                rowl[r] = reinterpret_cast<const float4 *>(Fl + ic * ld) + lane;
+            } else {
+                rowh[r] = rowl[r] = nullptr;
+            }
         }
-    }
+        // accumulators per (row, vector): even and odd columns in the two lanes of a float2
+        float2 sh2[ROWS][C], sl2[ROWS][C];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int d = 0; d < C; ++d) sh2[r][d] = sl2[r][d] = make_float2(0.f, 0.f);
+
+        for (int64_t j0 = 0; j0 < n; j0 += GV_CHUNK) {
+            __syncthreads();
+            for (int t = threadIdx.x; t < C * GV_CHUNK; t += GV_WARPS * 32) {
+                const int d = t / GV_CHUNK, jj = t - d * GV_CHUNK;
+                const int64_t j = j0 + jj;
+                sxh[d][jj] = j < n ? xh[(int64_t)d * n + j] : 0.f;
+                sxl[d][jj] = j < n ? xl[(int64_t)d * n + j] : 0.f;
+            }
+            __syncthreads();
+            const int64_t trem = (n - j0 + 127) / 128;
+            const int tend = trem < GV_CHUNK / 128 ? (int)trem : GV_CHUNK / 128;
+            for (int t0 = 0; t0 < tend; t0 += TB) {
+                float4 dh[TB][ROWS], dl[TB][ROWS];
+#pragma unroll
+                for (int t = 0; t < TB; ++t) {
+                    const int tt = t0 + t;
+                    const int64_t j = j0 + tt * 128 + lane * 4;
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        const int64_t i = row0 + r;
+                        if constexpr (PL) {
+                            if (tt < tend) {   // warp-uniform: the last chunk may end inside the TB group
+                                const int64_t q = (j0 >> 2) + tt * 32;
+                                dh[t][r] = __ldg(rowh[r] + q);
+                                dl[t][r] = __ldg(rowl[r] + q);
+                            } else {
+                                dh[t][r] = dl[t][r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                        } else if (i >= n || j >= n) {
+                            dh[t][r] = dl[t][r] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        } else {
+                            const double *row = D64 + i * n;
+                            float h[4], l[4];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) df_split(j + e < n ? __ldg(row + j + e) : 0.0, h[e], l[e]);
+                            dh[t][r] = make_float4(h[0], h[1], h[2], h[3]);
+                            dl[t][r] = make_float4(l[0], l[1], l[2], l[3]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < TB; ++t) {
+                    const int jl = (t0 + t) * 128 + lane * 4;
+#pragma unroll
+                    for (int d = 0; d < C; ++d) {
+                        const float4 xh4 = *reinterpret_cast<const float4 *>(&sxh[d][jl]);
+                        const float4 xl4 = *reinterpret_cast<const float4 *>(&sxl[d][jl]);
+#pragma unroll
+                        for (int r = 0; r < ROWS; ++r) {
+                            df_mac2(make_float2(dh[t][r].x, dh[t][r].y), make_float2(dl[t][r].x, dl[t][r].y),
+                                    make_float2(xh4.x, xh4.y), make_float2(xl4.x, xl4.y), sh2[r][d], sl2[r][d]);
+                            df_mac2(make_float2(dh[t][r].z, dh[t][r].w), make_float2(dl[t][r].z, dl[t][r].w),
+                                    make_float2(xh4.z, xh4.w), make_float2(xl4.z, xl4.w), sh2[r][d], sl2[r][d]);
+                        }
+                    }
+                }
+            }
+        }
+        // the two lanes, then warp sums in double-float, fixed butterfly order
+        float sh[ROWS][C], sl[ROWS][C];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int d = 0; d < C; ++d) {
+                sh[r][d] = sh2[r][d].x;
+                sl[r][d] = sl2[r][d].x;
+                df_add(sh[r][d], sl[r][d], sh2[r][d].y, sl2[r][d].y);
+            }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+            for (int d = 0; d < C; ++d)
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    const float oh = __shfl_xor_sync(0xffffffffu, sh[r][d], off);
+                    const float ol = __shfl_xor_sync(0xffffffffu, sl[r][d], off);
+                    df_add(sh[r][d], sl[r][d], oh, ol);
+                }
+        if (lane == 0) {
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) {
+                const int64_t i = row0 + r;
+                if (i < n)
+#pragma unroll
+                    for (int d = 0; d < C; ++d) U[(int64_t)d * n + i] = (double)sh[r][d] + (double)sl[r][d];
+            }
+        }
+        block += gridDim.x;
+    } while (LOOP && (int64_t)block * (GV_WARPS * ROWS) < n);
 }
 
-// ---- the same product from the symmetric tiled storage (upper-triangle 64 x 64 tiles), for
-// hardnesses too far apart for the digit slices (gemv_digits_usable):
+// ---- the same product from the symmetric tiled storage (upper-triangle 64 x 64 tiles), for what
+// the digit slices leave (gemv_digits_usable, VecSums):
 // every stored tile (I, J), I < J, serves both U_I += D_IJ x_J and U_J += D_IJ^T x_I, so D is
 // read once for the triangle instead of the full matrix -- half the memory; the time is
 // that of the full-plane product (both are bound by issue of the double-float arithmetic:
@@ -214,14 +230,14 @@ __global__ void __launch_bounds__(GV_WARPS * 32, MINB) k_dgemv_df(int64_t n, int
 constexpr int SY_T = (int)kSymTile;
 
 template <int C>
-__global__ void __launch_bounds__(256, 2) k_dsymv_df(int64_t n, int64_t T, const float *__restrict__ Dsym,
+__device__ __forceinline__ void dsymv_df_item(int item, int64_t n, int64_t T, const float *__restrict__ Dsym,
                                                      const SymItem *__restrict__ items,
                                                      const float *__restrict__ xh, const float *__restrict__ xl,
                                                      float2 *__restrict__ rowpart, float2 *__restrict__ colpart) {
     __shared__ __align__(16) float sxh[C][SY_T];
     __shared__ __align__(16) float sxl[C][SY_T];
     __shared__ float2 cred[16][SY_T * C];
-    const SymItem it = items[blockIdx.x];
+    const SymItem it = items[item];
     const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
     const int64_t I = it.I;
     float xih[4][C], xil[4][C], rh[4][C], rl[4][C];
@@ -304,28 +320,26 @@ __global__ void __launch_bounds__(256, 2) k_dsymv_df(int64_t n, int64_t T, const
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int d = 0; d < C; ++d)
-                rowpart[((int64_t)blockIdx.x * SY_T + tr * 4 + r) * C + d] = make_float2(rh[r][d], rl[r][d]);
+                rowpart[((int64_t)item * SY_T + tr * 4 + r) * C + d] = make_float2(rh[r][d], rl[r][d]);
+}
+
+// Beside a digit-slice product (pi) with a few blocks, as k_dgemv_df.
+template <int C>
+__global__ void __launch_bounds__(256, 2)
+    k_dsymv_df(int64_t n, int64_t T, const float *__restrict__ Dsym, const SymItem *__restrict__ items, int nitems,
+               const float *__restrict__ xh, const float *__restrict__ xl, float2 *__restrict__ rowpart,
+               float2 *__restrict__ colpart, const PlainIf pi) {
+    if (!pi.runs(C)) return;
+    for (int item = blockIdx.x; item < nitems; item += gridDim.x) dsymv_df_item<C>(item, n, T, Dsym, items, xh, xl, rowpart, colpart);
 }
 
 // U[d][i] = (row sums of the items of tile row K) + (column sums of tiles (I, K), I < K),
 // K = i / 64, added in that fixed order in double-float.
-__global__ void k_dsymv_finish(int64_t n, int C, int64_t T, const int *__restrict__ item_start,
-                               const float2 *__restrict__ rowpart, const float2 *__restrict__ colpart,
-                               double *__restrict__ U) {
+__global__ void k_dsymv_finish(int64_t n, int C, const SymPartials p, double *__restrict__ U) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n * C) return;
     const int d = (int)(e / n);
-    const int64_t i = e - (int64_t)d * n, K = i / SY_T, r = i % SY_T;
-    float sh = 0.f, sl = 0.f;
-    for (int q = item_start[K]; q < item_start[K + 1]; ++q) {
-        const float2 v = rowpart[((int64_t)q * SY_T + r) * C + d];
-        df_add(sh, sl, v.x, v.y);
-    }
-    for (int64_t I = 0; I < K; ++I) {
-        const float2 v = colpart[(sym_tile(I, K, T) * SY_T + r) * C + d];
-        df_add(sh, sl, v.x, v.y);
-    }
-    U[e] = (double)sh + (double)sl;
+    U[e] = dsymv_sum(p, C, e - (int64_t)d * n, d);
 }
 
 template <int C, bool PL>
@@ -333,10 +347,10 @@ void launch_dgemv(int tiling, int64_t n, int64_t ld, const float *Fh, const floa
                   const float *xh, const float *xl, double *U, cudaStream_t s) {
     const unsigned b1 = (unsigned)((n + GV_WARPS - 1) / GV_WARPS), b2 = (unsigned)((n + 2 * GV_WARPS - 1) / (2 * GV_WARPS));
     switch (tiling) {
-        case 1: k_dgemv_df<C, PL, 2, 4, 2><<<b2, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U); break;
-        case 2: k_dgemv_df<C, PL, 2, 2, 3><<<b2, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U); break;
-        case 3: k_dgemv_df<C, PL, 1, 8, 2><<<b1, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U); break;
-        default: k_dgemv_df<C, PL, 1, 4, 3><<<b1, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U); break;
+        case 1: k_dgemv_df<C, PL, 2, 4, 2><<<b2, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U, kAlways); break;
+        case 2: k_dgemv_df<C, PL, 2, 2, 3><<<b2, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U, kAlways); break;
+        case 3: k_dgemv_df<C, PL, 1, 8, 2><<<b1, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U, kAlways); break;
+        default: k_dgemv_df<C, PL, 1, 4, 3><<<b1, GV_WARPS * 32, 0, s>>>(n, ld, Fh, Fl, D64, xh, xl, U, kAlways); break;
     }
 }
 
@@ -349,6 +363,44 @@ void launch_dgemv_c(int cg, int tiling, int64_t n, int64_t ld, const float *Fh, 
         case 3: launch_dgemv<3, PL>(tiling, n, ld, Fh, Fl, D64, xh, xl, U, s); break;
         default: launch_dgemv<4, PL>(tiling, n, ld, Fh, Fl, D64, xh, xl, U, s); break;
     }
+}
+
+// The symmetric product of cg <= 4 vectors into its partial sums.
+void launch_dsymv(const wfq_geom *g, int cg, const float *xh, const float *xl, float2 *rowpart, float2 *colpart,
+                  const PlainIf &pi, cudaStream_t s) {
+    const int ni = (int)g->sym_nitems;
+    const unsigned grid = pi.sums.vsum ? (unsigned)std::min(ni, 2 * g->ctx->num_sms) : (unsigned)ni;
+    const int64_t n = g->n, T = g->sym_nt;
+    switch (cg) {
+        case 1: k_dsymv_df<1><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
+        case 2: k_dsymv_df<2><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
+        case 3: k_dsymv_df<3><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
+        default: k_dsymv_df<4><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
+    }
+    note_launch();
+}
+
+// The double-float product from the planes beside a digit-slice product (runs where pi says so).
+template <int C>
+void launch_dgemv_beside(const wfq_geom *g, const float *xh, const float *xl, double *U, const PlainIf &pi, cudaStream_t s) {
+    const unsigned b = (unsigned)std::min<int64_t>((g->n + GV_WARPS - 1) / GV_WARPS, 3 * g->ctx->num_sms);
+    k_dgemv_df<C, true, 1, 4, 3, true><<<b, GV_WARPS * 32, 0, s>>>(g->n, g->ldf, g->Dfh, g->Dfl, nullptr, xh, xl, U, pi);
+    note_launch();
+}
+void launch_dgemv_beside(const wfq_geom *g, int cg, const float *xh, const float *xl, double *U, const PlainIf &pi,
+                         cudaStream_t s) {
+    switch (cg) {
+        case 1: launch_dgemv_beside<1>(g, xh, xl, U, pi, s); break;
+        case 2: launch_dgemv_beside<2>(g, xh, xl, U, pi, s); break;
+        case 3: launch_dgemv_beside<3>(g, xh, xl, U, pi, s); break;
+        default: launch_dgemv_beside<4>(g, xh, xl, U, pi, s); break;
+    }
+}
+
+// Partial sums of the symmetric product: row and column parts of one group of cg vectors.
+size_t rowpart_elems(const wfq_geom *g, int cg) { return (size_t)g->sym_nitems * kSymTile * cg; }
+size_t colpart_elems(const wfq_geom *g, int cg) {
+    return (size_t)(g->sym_nt * (g->sym_nt + 1) / 2) * kSymTile * cg;
 }
 
 // W[d][i] = sum_p Kbar_ip (U[d][j_p] - U[d][i]) = ((Kbar - P) U)_i  (Eq. 16-17), FP64, for
@@ -474,7 +526,8 @@ constexpr int RU_ELEMS = 32 * RU_EPL;
 // sums are added in a fixed order.  Fused with the next step's reductions of the updated w:
 // NEXT_DOTS -- the partial dots of w with V_0 .. V_{nv-1} for the second Gram-Schmidt pass,
 // partial[(block * nv + k) * C + d]; NEXT_NORM -- the partial squared norm,
-// partial[block * C + d]; NEXT_NORM_MAX -- also the largest |w| of the block, pmax[block * C + d].
+// partial[block * C + d]; NEXT_NORM_MAX -- also the largest |w| of the block and its sum of |w|,
+// pmax[2 (block * C + d)] and the next.
 // Fixed orders throughout.
 enum { NEXT_DOTS = 1, NEXT_NORM = 2, NEXT_NORM_MAX = 3 };
 template <int NEXT>
@@ -484,7 +537,7 @@ __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int 
                                                                  double *__restrict__ pmax) {
     __shared__ double part[RU_SLICES][RU_ELEMS];
     __shared__ double wv[RU_ELEMS];
-    __shared__ double sqw[RU_ELEMS / 32], mxw[RU_ELEMS / 32];
+    __shared__ double sqw[RU_ELEMS / 32], mxw[RU_ELEMS / 32], abw[RU_ELEMS / 32];
     const int el = threadIdx.x & 31, sl = threadIdx.x >> 5;
     const int d = blockIdx.y;
     const int64_t i0 = (int64_t)blockIdx.x * RU_ELEMS;
@@ -533,12 +586,17 @@ __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int 
             if (el == 0) sqw[sl] = sq;
             if constexpr (NEXT == NEXT_NORM_MAX) {   // magnitudes as integers: order of the bits, NaN and Inf largest
                 unsigned long long mx = (unsigned long long)__double_as_longlong(wn) & 0x7fffffffffffffffull;
+                double ab = fabs(wn);
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) {
                     const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
                     mx = o > mx ? o : mx;
+                    ab += __shfl_xor_sync(0xffffffffu, ab, off);
                 }
-                if (el == 0) mxw[sl] = __longlong_as_double((long long)mx);
+                if (el == 0) {
+                    mxw[sl] = __longlong_as_double((long long)mx);
+                    abw[sl] = ab;
+                }
             }
         }
     }
@@ -551,12 +609,16 @@ __global__ void __launch_bounds__(32 * RU_SLICES) k_rupdate_next(int64_t n, int 
             partial[(int64_t)blockIdx.x * C + d] = sq;
             if constexpr (NEXT == NEXT_NORM_MAX) {
                 unsigned long long mx = 0;
+                double ab = 0.0;
 #pragma unroll
                 for (int q = 0; q < RU_ELEMS / 32; ++q) {
                     const unsigned long long o = (unsigned long long)__double_as_longlong(mxw[q]);
                     mx = o > mx ? o : mx;
+                    ab += abw[q];
                 }
-                pmax[(int64_t)blockIdx.x * C + d] = __longlong_as_double((long long)mx);
+                double *p = pmax + 2 * ((int64_t)blockIdx.x * C + d);
+                p[0] = __longlong_as_double((long long)mx);
+                p[1] = ab;
             }
         }
         return;
@@ -594,28 +656,33 @@ struct NextVec {
     __half *planes;
     int *xexp;
     int64_t gs, npad;
-    const double *pmax;   // largest |w| per block of k_rupdate_next
+    const double *pmax;   // largest |w| and sum of |w| per block of k_rupdate_next
+    unsigned *vsum, thr;  // VecSums
 };
 
 // The norms of the C directions from their nrb partial squares (every block reduces them
 // in the same fixed order: lane-strided sums, a butterfly), H(j + 1, j) = hn[d] = norm
 // (block 0), then v = w / norm with v's float-pair split, as k_rscale, or its digits (division
-// is monotonic: max |v| is max |w| / norm as computed).  Four elements per thread.
+// is monotonic: max |v| is max |w| / norm as computed) unless its group is left to double-float
+// sums.  Four elements per thread.
 template <bool DIG>
 __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restrict__ partial, int m, int j,
                               double *__restrict__ H, double *__restrict__ hn, const double *__restrict__ w,
                               double *__restrict__ v, NextVec nx) {
-    extern __shared__ double nrm[];   // [C], then C exponents
+    extern __shared__ double nrm[];   // [C], then C exponents and sums of magnitudes
     int *vex = reinterpret_cast<int *>(nrm + C);
+    unsigned *vsm = reinterpret_cast<unsigned *>(vex + C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int d = warp; d < C; d += blockDim.x / 32) {
-        double sv = 0.0;
+        double sv = 0.0, ab = 0.0;
         unsigned long long mx = 0;
         for (int rb = lane; rb < nrb; rb += 32) {
             sv += partial[(int64_t)rb * C + d];
             if constexpr (DIG) {
-                const unsigned long long o = (unsigned long long)__double_as_longlong(nx.pmax[(int64_t)rb * C + d]);
+                const double2 p = reinterpret_cast<const double2 *>(nx.pmax)[(int64_t)rb * C + d];
+                const unsigned long long o = (unsigned long long)__double_as_longlong(p.x);
                 mx = o > mx ? o : mx;
+                ab += p.y;
             }
         }
 #pragma unroll
@@ -624,6 +691,7 @@ __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restric
             if constexpr (DIG) {
                 const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
                 mx = o > mx ? o : mx;
+                ab += __shfl_xor_sync(0xffffffffu, ab, off);
             }
         }
         if (lane == 0) {
@@ -632,7 +700,12 @@ __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restric
             if constexpr (DIG) {
                 const double vm = nr > 0.0 ? __longlong_as_double((long long)mx) / nr : 0.0;
                 vex[d] = vec_exp((unsigned long long)__double_as_longlong(vm) & 0x7fffffffffffffffull);
-                if (blockIdx.x == 0) nx.xexp[d] = vex[d];
+                const bool sums = vm > 0.0 && vex[d] != kVecNotFinite;
+                vsm[d] = sums ? (unsigned)fmin(scalbn(ab / nr, 8 - vex[d]), 4294967294.0) : 0xffffffffu;
+                if (blockIdx.x == 0) {
+                    nx.xexp[d] = vex[d];
+                    nx.vsum[d] = vsm[d];
+                }
             }
             if (blockIdx.x == 0) {
                 H[((int64_t)d * m + j) * (m + 1) + j + 1] = nr;
@@ -648,8 +721,8 @@ __global__ void k_rscale_norm(int64_t n, int C, int nrb, const double *__restric
         const double h = nrm[d];
         const double t = h > 0.0 ? w[e] / h : 0.0;
         v[e] = t;
-        if constexpr (DIG) {
-            const int cg = min(4, C - (d & ~3));
+        const int cg = min(4, C - (d & ~3));
+        if (DIG && !VecSums{vsm + (d & ~3), nullptr, nx.thr}.plain(cg)) {
             put_vec_digits(t, vex[d], nx.planes + (d >> 2) * nx.gs + (d & 3) * nx.npad + (e - d * n), cg * nx.npad);
         } else {
             df_split(t, nx.xh[e], nx.xl[e]);
@@ -866,8 +939,9 @@ struct Arnoldi {
     bool digits = false;               // D products by digit slices (gemv_digits.cu)
     DevBuf<uint16_t> planes;           // vector digits, a set for every 4 directions
     DevBuf<int> xexp;
-    DevBuf<unsigned long long> vmax, acc;
+    DevBuf<unsigned long long> vmax, acc;   // vmax: largest magnitudes, then sums of magnitudes
     DevBuf<double> pmax;
+    unsigned thr = 0;
 
     int init(wfq_geom *geom, int ndir, int m, cudaStream_t stream) {
         g = geom;
@@ -879,26 +953,25 @@ struct Arnoldi {
         digits = use_gemv_digits(g);
         if (digits) {
             const size_t np = gemv_digits_plane_elems(g) * ((C + 3) / 4);
+            thr = gemv_digits_threshold(g);
             WFQ_TRY(planes.alloc(g->ctx, np, s));
             WFQ_TRY(xexp.alloc(g->ctx, C, s));
-            WFQ_TRY(vmax.alloc(g->ctx, C, s));
+            WFQ_TRY(vmax.alloc(g->ctx, C + (C + 1) / 2, s));
             WFQ_TRY(acc.alloc(g->ctx, (size_t)8 * n, s));
             WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
             WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 8 * n, s));
-        } else {
-            WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
-            WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
         }
+        WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
+        WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
         WFQ_TRY(U.alloc(g->ctx, (size_t)n * C, s));
         WFQ_TRY(partial.alloc(g->ctx, (size_t)nrb * (m + 1) * C, s));
         nbru = (int)((n + RU_ELEMS - 1) / RU_ELEMS);
         WFQ_TRY(partial_f.alloc(g->ctx, (size_t)nbru * (m + 1) * C, s));
         WFQ_TRY(coef.alloc(g->ctx, (size_t)(m + 1) * C, s));
-        if (digits) WFQ_TRY(pmax.alloc(g->ctx, (size_t)nbru * C, s));
-        if (g->Dsym && !g->Dfh && !digits) {
-            const int64_t T = g->sym_nt, cg = std::min<int64_t>(C, 4);
-            WFQ_TRY(rowpart.alloc(g->ctx, (size_t)g->sym_nitems * kSymTile * cg, s));
-            WFQ_TRY(colpart.alloc(g->ctx, (size_t)(T * (T + 1) / 2) * kSymTile * cg, s));
+        if (digits) WFQ_TRY(pmax.alloc(g->ctx, (size_t)2 * nbru * C, s));
+        if (g->Dsym && !g->Dfh) {
+            WFQ_TRY(rowpart.alloc(g->ctx, rowpart_elems(g, std::min(C, 4)), s));
+            WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
         }
         return WFQ_OK;
     }
@@ -946,26 +1019,36 @@ struct Arnoldi {
         return best;
     }
 
+    unsigned *vsum() const { return reinterpret_cast<unsigned *>(vmax.ptr + C); }
     GemvDigits work(int d0) const {
-        return GemvDigits{planes.ptr + (size_t)(d0 / 4) * gemv_digits_plane_elems(g), xexp.ptr + d0, vmax.ptr + d0, acc.ptr};
+        return GemvDigits{planes.ptr + (size_t)(d0 / 4) * gemv_digits_plane_elems(g), xexp.ptr + d0, vmax.ptr + d0,
+                          acc.ptr, vsum() + d0, thr, false};
     }
     NextVec next() const {
         return NextVec{xh.ptr, xl.ptr, reinterpret_cast<__half *>(planes.ptr), xexp.ptr, (int64_t)gemv_digits_plane_elems(g),
-                       g->npad, pmax.ptr};
+                       g->npad, pmax.ptr, vsum(), thr};
     }
+    SymPartials partials() const { return SymPartials{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt}; }
     // digits of v [C][n] (the start vectors; later ones get theirs in k_rscale_norm)
-    int split(const double *v) {
-        for (int d0 = 0; digits && d0 < C; d0 += 4)
-            WFQ_TRY(gemv_digits_split(g, std::min(4, C - d0), v + (int64_t)d0 * n, 1, n, work(d0), s));
-        return WFQ_OK;
-    }
+    int split(const double *v) { return digits ? gemv_digits_split(g, C, v, 1, n, work(0), s) : WFQ_OK; }
 
     // u = D v; xh / xl (or the digit planes) already hold v (written when v was normalised)
     int dmul(double *u) {
         if (digits) {
             for (int d0 = 0; d0 < C; d0 += 4) {
+                const int cg = std::min(4, C - d0);
+                const GemvDigits w = work(d0);
+                const PlainIf pi{w.sums()};
+                const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
+                double *pu = u + (int64_t)d0 * n;
                 KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, 8.0 * (double)n * (double)n);
-                WFQ_TRY(gemv_digits_product(g, std::min(4, C - d0), work(d0), u + (int64_t)d0 * n, 1, n, s));
+                WFQ_TRY(gemv_digits_product(g, cg, w, s));
+                if (g->Dfh) {
+                    launch_dgemv_beside(g, cg, ph, pxl, pu, pi, s);
+                } else {
+                    launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
+                }
+                WFQ_TRY(gemv_digits_finish(g, cg, w, partials(), nullptr, pu, 1, n, s));
             }
             return WFQ_OK;
         }
@@ -984,16 +1067,8 @@ struct Arnoldi {
                 const int cg = std::min(4, C - d0);
                 const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
                 KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, dbytes);
-                const unsigned items = (unsigned)g->sym_nitems;
-                switch (cg) {
-                    case 1: k_dsymv_df<1><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rowpart.ptr, colpart.ptr); break;
-                    case 2: k_dsymv_df<2><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rowpart.ptr, colpart.ptr); break;
-                    case 3: k_dsymv_df<3><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rowpart.ptr, colpart.ptr); break;
-                    default: k_dsymv_df<4><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rowpart.ptr, colpart.ptr); break;
-                }
-                note_launch();
-                k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, T, g->sym_item_start, rowpart.ptr, colpart.ptr,
-                                                           u + (int64_t)d0 * n);
+                launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, kAlways, s);
+                k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, partials(), u + (int64_t)d0 * n);
                 note_launch();
             }
             WFQ_CUDA(cudaGetLastError());
@@ -1059,12 +1134,15 @@ struct Arnoldi {
 
 // Real column r of an atom-major complex block X (n x cc; r = 2c + 0/1 for the real and
 // imaginary parts of column c) split into direction-major float pairs xh/xl [C][n].
-__global__ void k_cols_split(int64_t n, int C, const double *__restrict__ X, float *__restrict__ xh,
-                             float *__restrict__ xl) {
+// X has ld real columns a row; pi: groups of 4 columns (complex parts) of the digit slices are left out.
+__global__ void k_cols_split(int64_t n, int C, int64_t ld, const double *__restrict__ X, float *__restrict__ xh,
+                             float *__restrict__ xl, const PlainIf pi) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n * C) return;
     const int64_t r = e / n, i = e - r * n;
-    df_split(X[i * C + r], xh[e], xl[e]);
+    const int r4 = (int)r & ~3;
+    if (pi.sums.vsum && !VecSums{pi.sums.vsum + r4, pi.sums.vmax + r4, pi.sums.thr}.plain(min(4, C - r4))) return;
+    df_split(X[i * ld + r], xh[e], xl[e]);
 }
 
 // U (atom-major complex block, real column r at i * C + r) = Ud [C][n]
@@ -1081,33 +1159,66 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
     const int64_t n = g->n;
     const int C = (int)(2 * cc);
     if (!(g->Dfh || g->Dsym)) return fail(WFQ_EUNSUPPORTED, "float-pair product: needs stored pairs");
-    if (use_gemv_digits(g)) {
+    const double *x = reinterpret_cast<const double *>(X);
+    double *u = reinterpret_cast<double *>(U);
+    DevBuf<float> xh, xl;
+    DevBuf<double> ud;
+    DevBuf<float2> rowpart, colpart;
+    const bool sym = !g->Dfh;
+    auto partials = [&] { return SymPartials{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt}; };
+    // An apply's digits cost more launches than a solver's.  From the tiles, us per apply of 1, 2 and 16
+    // columns, digits against double-float: 160 atoms 44 / 30, 46 / 39, 178 / 191; 320 atoms 44 / 35, 45 / 47,
+    // 185 / 259; 640 atoms 45 / 45, 47 / 70, 195 / 431.
+    if (use_gemv_digits(g) && (g->Dfh || n * std::min(C, 4) >= 1100)) {
+        // blocks of 32 real columns, groups of 4: workspace of one block
+        constexpr int CB = 32;
+        const int cb0 = std::min(C, CB);
         DevBuf<uint16_t> planes;
         DevBuf<int> xexp;
-        DevBuf<unsigned long long> vmax, acc;
-        const size_t np = gemv_digits_plane_elems(g);
+        DevBuf<unsigned long long> stats, acc;
+        const size_t gp = gemv_digits_plane_elems(g), np = gp * ((cb0 + 3) / 4);
         WFQ_TRY(planes.alloc(g->ctx, np, s));
-        WFQ_TRY(xexp.alloc(g->ctx, 4, s));
-        WFQ_TRY(vmax.alloc(g->ctx, 4, s));
+        WFQ_TRY(xexp.alloc(g->ctx, cb0, s));
+        WFQ_TRY(stats.alloc(g->ctx, cb0 + (cb0 + 1) / 2, s));
         WFQ_TRY(acc.alloc(g->ctx, (size_t)8 * n, s));
+        WFQ_TRY(xh.alloc(g->ctx, (size_t)n * cb0, s));
+        WFQ_TRY(xl.alloc(g->ctx, (size_t)n * cb0, s));
+        if (sym) {
+            WFQ_TRY(rowpart.alloc(g->ctx, rowpart_elems(g, std::min(C, 4)), s));
+            WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
+        } else {
+            WFQ_TRY(ud.alloc(g->ctx, (size_t)n * std::min(C, 4), s));
+        }
+        // atoms past n stay zero; rows of digits that a group of fewer columns leaves are not read back
+        WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
         WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 8 * n, s));
-        const GemvDigits w{planes.ptr, xexp.ptr, vmax.ptr, acc.ptr};
         KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-        for (int d0 = 0; d0 < C; d0 += 4) {
-            const int cg = std::min(4, C - d0);
-            // rows past 8 cg and atoms past n stay zero
-            WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
-            WFQ_TRY(gemv_digits_split(g, cg, reinterpret_cast<const double *>(X) + d0, C, 1, w, s));
-            WFQ_TRY(gemv_digits_product(g, cg, w, reinterpret_cast<double *>(U) + d0, C, 1, s, err));
+        for (int b0 = 0; b0 < C; b0 += CB) {
+            const int cb = std::min(CB, C - b0);
+            GemvDigits w{planes.ptr, xexp.ptr, stats.ptr, acc.ptr, reinterpret_cast<unsigned *>(stats.ptr + cb),
+                         gemv_digits_threshold(g), true};
+            WFQ_TRY(gemv_digits_split(g, cb, x + b0, C, 1, w, s));
+            k_cols_split<<<nblk(n * cb), 256, 0, s>>>(n, cb, C, x + b0, xh.ptr, xl.ptr, PlainIf{w.sums()});
+            note_launch();
+            for (int d0 = 0; d0 < cb; d0 += 4, w.planes += gp, w.xexp += 4, w.vmax += 4, w.vsum += 4) {
+                const int cg = std::min(4, cb - d0);
+                const PlainIf pi{w.sums()};
+                const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
+                WFQ_TRY(gemv_digits_product(g, cg, w, s, err));
+                if (sym) {
+                    launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
+                } else {
+                    launch_dgemv_beside(g, cg, ph, pxl, ud.ptr, pi, s);
+                }
+                WFQ_TRY(gemv_digits_finish(g, cg, w, partials(), ud.ptr, u + b0 + d0, C, 1, s));
+            }
         }
         return WFQ_OK;
     }
-    DevBuf<float> xh, xl;
-    DevBuf<double> ud, rowpart, colpart;
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(ud.alloc(g->ctx, (size_t)n * C, s));
-    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr);
+    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr, kAlways);
     note_launch();
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     if (g->Dfh) {
@@ -1118,22 +1229,12 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
             note_launch();
         }
     } else {
-        const int64_t T = g->sym_nt;
-        WFQ_TRY(rowpart.alloc(g->ctx, (size_t)g->sym_nitems * kSymTile * 4 * 2, s));
-        WFQ_TRY(colpart.alloc(g->ctx, (size_t)(T * (T + 1) / 2) * kSymTile * 4 * 2, s));
-        float2 *rp = reinterpret_cast<float2 *>(rowpart.ptr), *cp = reinterpret_cast<float2 *>(colpart.ptr);
+        WFQ_TRY(rowpart.alloc(g->ctx, rowpart_elems(g, std::min(C, 4)), s));
+        WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
         for (int d0 = 0; d0 < C; d0 += 4) {
             const int cg = std::min(4, C - d0);
-            const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
-            const unsigned items = (unsigned)g->sym_nitems;
-            switch (cg) {
-                case 1: k_dsymv_df<1><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rp, cp); break;
-                case 2: k_dsymv_df<2><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rp, cp); break;
-                case 3: k_dsymv_df<3><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rp, cp); break;
-                default: k_dsymv_df<4><<<items, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ph, pxl, rp, cp); break;
-            }
-            note_launch();
-            k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, T, g->sym_item_start, rp, cp, ud.ptr + (int64_t)d0 * n);
+            launch_dsymv(g, cg, xh.ptr + (int64_t)d0 * n, xl.ptr + (int64_t)d0 * n, rowpart.ptr, colpart.ptr, kAlways, s);
+            k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, partials(), ud.ptr + (int64_t)d0 * n);
             note_launch();
         }
     }
@@ -1152,7 +1253,7 @@ int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(ud.alloc(g->ctx, (size_t)n * C, s));
-    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr);
+    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr, kAlways);
     note_launch();
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     for (int d0 = 0; d0 < C; d0 += 4)
@@ -1257,6 +1358,10 @@ int solve_gmres_shifted(wfq_geom *g, const SolveArgs &a, cudaStream_t s) {
         WFQ_CUDA(cudaStreamWaitEvent(s, side.join, 0));
         return WFQ_OK;
     };
+    const size_t sm_norm = (sizeof(double) + 2 * sizeof(int)) * C;   // k_rscale_norm
+    if (sm_norm > 48 * 1024)
+        WFQ_CUDA(cudaFuncSetAttribute(ar.digits ? k_rscale_norm<true> : k_rscale_norm<false>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     for (int j = 0; j < m; ++j) {
         double *dvj = DV.ptr + (int64_t)j * vstride;
         double *w = V.ptr + (int64_t)(j + 1) * vstride;
@@ -1279,16 +1384,15 @@ int solve_gmres_shifted(wfq_geom *g, const SolveArgs &a, cudaStream_t s) {
                                                                   H.ptr, ar.coef.ptr, hn.ptr);
             note_launch();
             const dim3 gu((unsigned)ar.nbru, (unsigned)C);
-            const size_t sm = (sizeof(double) + sizeof(int)) * C;
             if (ar.digits) {
                 k_rupdate_next<NEXT_NORM_MAX><<<gu, 32 * RU_SLICES, 0, s>>>(n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w,
                                                                             ar.partial_f.ptr, ar.pmax.ptr);
-                k_rscale_norm<true><<<nblk(n * C, 1024), 256, sm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
+                k_rscale_norm<true><<<nblk(n * C, 1024), 256, sm_norm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
                                                                        hn.ptr, w, w, ar.next());
             } else {
                 k_rupdate_next<NEXT_NORM><<<gu, 32 * RU_SLICES, 0, s>>>(n, (int)C, nv, V.ptr, vstride, ar.coef.ptr, w,
                                                                         ar.partial_f.ptr, nullptr);
-                k_rscale_norm<false><<<nblk(n * C, 1024), 256, sm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
+                k_rscale_norm<false><<<nblk(n * C, 1024), 256, sm_norm, s>>>(n, (int)C, ar.nbru, ar.partial_f.ptr, m, j, H.ptr,
                                                                         hn.ptr, w, w, ar.next());
             }
             note_launch();

@@ -7,6 +7,9 @@
 
 #include <cstdint>
 
+#include "dfloat.cuh"
+#include "common.h"
+
 namespace wfq {
 
 constexpr int kVecDigits = 8;
@@ -30,15 +33,34 @@ __device__ __forceinline__ int vec_exp(unsigned long long bits) {
     return ex == 0x7ff ? kVecNotFinite : ex > 0 ? ex - 1022 : -1021;
 }
 
-// x = 2^(e - 5) sum_m e_m 2^(-7 m), |e_m| <= 64, as fp16 at dst[m * stride]
-__device__ __forceinline__ void put_vec_digits(double x, int e, __half *dst, int64_t stride) {
+// x = 2^(e - 5) sum_m e_m 2^(-7 m), |e_m| <= 64, as fp16 at dst[m * stride].  Returns
+// floor(2^8 |x| / 2^e).
+__device__ __forceinline__ unsigned put_vec_digits(double x, int e, __half *dst, int64_t stride) {
     const uint64_t bias = 0x81020408102040ull;   // 64 (128^8 - 1) / 127
-    const uint64_t g = e == kVecNotFinite ? bias : (uint64_t)fixed_point54(x, e) + bias;
+    const int64_t f = e == kVecNotFinite ? 0 : fixed_point54(x, e);
+    const uint64_t g = (uint64_t)f + bias;
 #pragma unroll
     for (int m = 0; m < kVecDigits; ++m) {
         const unsigned short u = (unsigned short)(0x6400u | (uint32_t)((g >> (7 * (kVecDigits - 1 - m))) & 127u));
         dst[m * stride] = __hsub(__ushort_as_half(u), __ushort_as_half(0x6440u));   // 1024 + u - 1088
     }
+    return (unsigned)((uint64_t)(f < 0 ? -f : f) >> 46);
+}
+
+// Row i, vector d of C from the symmetric product's partial sums: the items of tile row K = i / 64,
+// then the tiles (I, K), I < K, in double-float in that order.
+__device__ __forceinline__ double dsymv_sum(const SymPartials &p, int C, int64_t i, int d) {
+    const int64_t K = i / kSymTile, r = i % kSymTile;
+    float sh = 0.f, sl = 0.f;
+    for (int q = p.item_start[K]; q < p.item_start[K + 1]; ++q) {
+        const float2 v = p.rowpart[((int64_t)q * kSymTile + r) * C + d];
+        df_add(sh, sl, v.x, v.y);
+    }
+    for (int64_t I = 0; I < K; ++I) {
+        const float2 v = p.colpart[(sym_tile(I, K, p.T) * kSymTile + r) * C + d];
+        df_add(sh, sl, v.x, v.y);
+    }
+    return (double)sh + (double)sl;
 }
 
 }  // namespace wfq

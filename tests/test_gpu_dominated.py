@@ -122,3 +122,42 @@ def test_a_block_without_a_column_for_the_digits(W, ctx, orc, S, store, prec):
 @pytest.mark.parametrize("ncplx", [2, 3, 4])
 def test_few_columns_of_a_stored_fp64_operator(W, ctx, orc, S, ncplx, kind):
     _check(W, ctx, orc, S, 4100, ncplx, "fp64", "fp64", kind)
+
+
+@pytest.mark.parametrize("kind", ["one", "five", "spread", "mixed"])
+@pytest.mark.parametrize("n,ncplx,store", [(451, 1, "sym"), (451, 2, "sym"), (700, 3, "sym"), (700, 19, "sym"),
+                                           (3100, 1, "pairs"), (3100, 3, "pairs")])
+def test_few_columns_from_float_pairs(W, ctx, orc, S, n, ncplx, store, kind):
+    _check(W, ctx, orc, S, n, ncplx, store, "df", kind)
+
+
+@pytest.mark.parametrize("store", ["sym", "pairs"])
+def test_a_zero_imaginary_part_needs_no_other_sums(W, ctx, orc, S, store):
+    _check(W, ctx, orc, S, 3100 if store == "pairs" else 451, 2, store, "df", "mixed", zero_imag=True)
+
+
+@pytest.mark.parametrize("store", ["sym", "pairs"])
+@pytest.mark.parametrize("ndir", [1, 3, 6])
+def test_a_solve_from_localised_start_vectors(W, ctx, orc, S, store, ndir):
+    """A flake's right-hand side is zero but at its edge: the first Arnoldi vectors may go to the
+    double-float sums, later ones to the digits.
+    q against LU within 1e-7, as for the other solves to 1e-10."""
+    xyz = S.honeycomb_flake(23 if store == "pairs" else 9)   # 3174 and 486 atoms
+    p = S.carbon_params(1.51)
+    g = W.Geometry(ctx, xyz, p, store=W.STORE_F32X2 if store == "pairs" else W.STORE_F32X2_SYM)
+    rng = np.random.default_rng(ndir)
+    dirs = rng.standard_normal((ndir, 3))
+    dirs[:, 2] = 0.0
+    om = S.ev([0.8])
+    q, _, status = g.solve_gmres_shifted(om, dirs, rel_tol=1e-10, max_iter=2000, prec=W.PREC_FP64)
+    assert status == "WFQ_OK"
+    D = orc.d_matrix(xyz, np.full(len(xyz), p["eta"]))
+    rowptr, col, val = orc.kbar_csr(xyz, p, cutoff_eps=p["cutoff_eps"])
+    K = np.zeros_like(D)
+    for i in range(len(xyz)):
+        K[i, col[rowptr[i]:rowptr[i + 1]]] = val[rowptr[i]:rowptr[i + 1]]
+    A = K @ D - K.sum(axis=1)[:, None] * D
+    A = A.astype(complex)
+    A[np.arange(len(xyz)), np.arange(len(xyz))] -= orc.z_of_omega(om[0], p)
+    ref = np.linalg.solve(A, g.rhs(dirs, E0=1.0).astype(complex))
+    assert np.linalg.norm(q - ref) <= 1e-7 * np.linalg.norm(ref)
