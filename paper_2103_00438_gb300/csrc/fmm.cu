@@ -64,6 +64,9 @@ struct Fmm {
     int32_t *near_start = nullptr;   // nleaf + 1: near leaves of each leaf (CSR)
     int32_t *near_leaf = nullptr;    // nnear: leaf index
     int8_t *near_delta = nullptr;    // nnear: offset code, sum_d (src_d - tgt_d + 1) 3^d
+    int64_t ngroups = 0;             // targets of the near field: up to 32 atoms of one leaf
+    int32_t *tgt_leaf = nullptr;     // ngroups: leaf index
+    int32_t *tgt_first = nullptr;    // ngroups: first atom
     float *Tm = nullptr;             // 2^dim x P x Pp: M2M weights [octant][child node][parent node]
     float *Tl = nullptr;             // 2^dim x P x Pp: the same [octant][parent node][child node], for L2L
     float *K = nullptr;              // 7^dim x P x P: M2L kernel for boxes of half-width 1
@@ -129,7 +132,7 @@ struct FmmDev {
     float h;                          // leaf side
     int nslots;
     const int32_t *perm, *leaf_start, *parent, *child_lo, *child_hi, *m2l_box, *m2l_src;
-    const int32_t *near_start, *near_leaf;
+    const int32_t *near_start, *near_leaf, *tgt_leaf, *tgt_first;
     const int16_t *slot_off;
     const int8_t *octant, *near_delta, *m2l_level;
     const float4 *atl;
@@ -360,80 +363,187 @@ __global__ void __launch_bounds__(32 * M2L_WARPS, 2)
     }
 }
 
-// L2P and the near field: a warp per leaf, a lane per target atom, 4 CQ columns (blockIdx.y) in
-// registers, so a pair's D_ij is computed once for them (once per 8 columns before: 1431 us for
-// the 250k-atom disk, order 6, 32 columns, against 726).  Sources, their X rows and the leaf's
-// local coefficients are uniform in the warp and come through L1.
+// M2L of small trees, where the boxes of an octant fill few blocks (k_fmm_m2l waits for L2 in every slot, 5
+// to 7 us, whatever the number of boxes): a block per (box, 32 columns, 64 or more target nodes).  Steps
+// of MB_KC source nodes of a slot: K's rows for the block's target nodes and the source's multipoles come by
+// asynchronous copies into two stages of shared memory, one step ahead.  Warps over groups of 8
+// target nodes, a lane per column (lpb of them; 32 / lpb node groups a warp).  The same sums in the same
+// order as k_fmm_m2l.
+constexpr int MB_KC = 32;
+__device__ __forceinline__ void copy_async(float *dst, const float *src, bool vec) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (vec) asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__global__ void __launch_bounds__(256) k_fmm_m2l_box(FmmDev f, int64_t C, int64_t nm2l, int noct, M2lGrid gr, int lpb,
+                                                     int rows, const float *__restrict__ M, float *__restrict__ Lc) {
+    extern __shared__ __align__(16) float sm[];   // two stages of K [MB_KC][rows], M [MB_KC][lpb]
+    const int P = f.P, stage = MB_KC * (rows + lpb);
+    const int64_t pos = blockIdx.x, PC = (int64_t)P * C, col0 = (int64_t)blockIdx.y * 32;
+    int oc = 0;
+    while (oc + 1 < noct && pos >= gr.first[oc + 1]) ++oc;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rb = blockIdx.z * rows, nr = min(rows, P - rb);
+    const int c = lane & (lpb - 1), r0 = (warp * (32 / lpb) + lane / lpb) * 8;
+    const bool ok = col0 + c < C && r0 < nr;
+    const bool vec = (P & 3) == 0;   // rows of K by 16 bytes (C is a multiple of 4)
+    const int total = f.dim == 2 ? 6 * 8 : 6 * 57;  // offset code of -d: total - code
+    const int nc = (int)min((int64_t)lpb, C - col0);
+    auto source = [&](int sl) { return __ldg(f.m2l_src + (int64_t)sl * nm2l + pos); };
+    auto next_slot = [&](int sl) {
+        while (sl < f.nslots && source(sl) < 0) ++sl;
+        return sl;
+    };
+    auto fetch = [&](int sl, int k0, float *dst) {   // K[-offset] is K[offset] transposed: its rows are source nodes
+        const int nk = min(MB_KC, P - k0), w = vec ? 4 : 1;
+        const float *Ko = f.K + ((int64_t)(total - f.slot_off[oc * f.nslots + sl]) * P + k0) * P + rb;
+        for (int q = threadIdx.x; q < nk * (nr / w); q += 256) {
+            const int k = q / (nr / w), r = (q - k * (nr / w)) * w;
+            copy_async(dst + k * rows + r, Ko + (int64_t)k * P + r, vec);
+        }
+        const float *Ms = M + (int64_t)source(sl) * PC + (int64_t)k0 * C + col0;
+        float *dm = dst + MB_KC * rows;
+        for (int q = threadIdx.x; q < nk * (nc / 4); q += 256) {
+            const int k = q / (nc / 4), r = (q - k * (nc / 4)) * 4;
+            copy_async(dm + k * lpb + r, Ms + (int64_t)k * C + r, true);
+        }
+    };
+    float acc[8] = {};
+    int sl = next_slot(0), k0 = 0, buf = 0;
+    if (sl < f.nslots) fetch(sl, 0, sm);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    while (sl < f.nslots) {
+        const int nk = min(MB_KC, P - k0);
+        k0 += MB_KC;
+        if (k0 >= P) {
+            k0 = 0;
+            sl = next_slot(sl + 1);
+        }
+        if (sl < f.nslots) fetch(sl, k0, sm + (buf ^ 1) * stage);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 1;" ::: "memory");   // this step's copies; the next one's go on
+        __syncthreads();
+        if (ok) {
+            const float *sK = sm + buf * stage + r0, *sM = sm + buf * stage + MB_KC * rows + c;
+#pragma unroll 4
+            for (int k = 0; k < nk; ++k) {
+                const float m = sM[k * lpb];
+                const float4 a = *reinterpret_cast<const float4 *>(sK + k * rows);
+                const float4 b = *reinterpret_cast<const float4 *>(sK + k * rows + 4);
+                acc[0] = fmaf(a.x, m, acc[0]);
+                acc[1] = fmaf(a.y, m, acc[1]);
+                acc[2] = fmaf(a.z, m, acc[2]);
+                acc[3] = fmaf(a.w, m, acc[3]);
+                acc[4] = fmaf(b.x, m, acc[4]);
+                acc[5] = fmaf(b.y, m, acc[5]);
+                acc[6] = fmaf(b.z, m, acc[6]);
+                acc[7] = fmaf(b.w, m, acc[7]);
+            }
+        }
+        __syncthreads();   // before the next fetch overwrites this stage
+        buf ^= 1;
+    }
+    if (!ok) return;
+    const float scale = gr.inv_a[f.m2l_level[pos]];
+    float *o = Lc + (int64_t)f.m2l_box[pos] * PC + col0 + c;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (rb + r0 + i < P && r0 + i < nr) o[(int64_t)(rb + r0 + i) * C] = scale * acc[i];
+}
+
+// L2P and the near field: a warp per 32 atoms of a leaf (tgt_leaf, tgt_first), a lane per target
+// atom, 4 CQ columns (blockIdx.y) in registers, so a pair's D_ij is computed once for them (once per 8 columns: 1431 us for the
+// 250k-atom disk, order 6, 32 columns, against 726; sources staged by 32 took the apply from 2.57
+// to 2.41 ms).  X rows and the leaf's local coefficients are uniform in the warp and come through L1.
+// Bound by the chain of each source (distance, erf, multiply-adds) where warps are few: a leaf
+// to a warp took 116 ms for an apply of 16 columns of a 15k-atom sphere (64 leaves) that takes 2.3.
 template <int CQ>
-__global__ void __launch_bounds__(128) k_fmm_l2p_near(FmmDev f, int64_t nleaf, int64_t C, int64_t Cp, int far,
+__global__ void __launch_bounds__(128) k_fmm_l2p_near(FmmDev f, int64_t ngroups, int64_t C, int64_t Cp, int far,
                                                       const float *__restrict__ Xs, const float *__restrict__ Lc,
                                                       float *__restrict__ U) {
     __shared__ float sW[4][3][kMaxP][32];
+    __shared__ float4 sS[4][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t b = (int64_t)blockIdx.x * 4 + warp;
-    if (b >= nleaf) return;
+    const int64_t grp = (int64_t)blockIdx.x * 4 + warp;
+    if (grp >= ngroups) return;
+    const int64_t b = f.tgt_leaf[grp];
     const int64_t col0 = (int64_t)blockIdx.y * (4 * CQ);
-    const int k0 = f.leaf_start[b], k1 = f.leaf_start[b + 1];
+    const int k1 = f.leaf_start[b + 1];
     const float a = 0.5f * f.h;
-    for (int base = k0; base < k1; base += 32) {
-        const int i = base + lane;
-        const bool act = i < k1;
-        const float4 qi = act ? f.atl[i] : make_float4(0.f, 0.f, 0.f, 1.f);
-        float2 lo[CQ], hi[CQ];
+    const int i = f.tgt_first[grp] + lane;
+    const bool act = i < k1;
+    const float4 qi = act ? f.atl[i] : make_float4(0.f, 0.f, 0.f, 1.f);
+    float2 lo[CQ], hi[CQ];
 #pragma unroll
-        for (int q = 0; q < CQ; ++q) lo[q] = hi[q] = make_float2(0.f, 0.f);
-        auto add = [&](float d, const float4 *x) {
+    for (int q = 0; q < CQ; ++q) lo[q] = hi[q] = make_float2(0.f, 0.f);
+    auto add = [&](float d, const float4 *x) {
 #pragma unroll
-            for (int q = 0; q < CQ; ++q) {
-                if (col0 + 4 * q >= Cp) break;
-                const float4 v = __ldg(x + q);
-                lo[q] = __ffma2_rn(make_float2(d, d), make_float2(v.x, v.y), lo[q]);
-                hi[q] = __ffma2_rn(make_float2(d, d), make_float2(v.z, v.w), hi[q]);
-            }
-        };
-        if (far && f.L >= 2) {
-            const float y[3] = {qi.x / a, qi.y / a, qi.z / a};
-            float tk[kMaxP];
-            for (int d = 0; d < f.dim; ++d) {   // node_weights into shared memory
-                tk[0] = 1.f;
-                if (f.p > 1) tk[1] = y[d];
-                for (int k = 2; k < f.p; ++k) tk[k] = 2.f * y[d] * tk[k - 1] - tk[k - 2];
-                const float inv = 1.f / f.p;
-                for (int m = 0; m < f.p; ++m) {
-                    float s = 0.f;
-                    for (int k = 1; k < f.p; ++k) s = fmaf(f.cheb[m * f.p + k], tk[k], s);
-                    sW[warp][d][m][lane] = inv + 2.f * inv * s;
-                }
-            }
-            __syncwarp();
-            const float *Lb = Lc + (f.leaf0 + b) * (int64_t)f.P * Cp + col0;
-            if (f.dim == 2) {
-                for (int m0 = 0; m0 < f.p; ++m0) {
-                    const float w0 = sW[warp][0][m0][lane];
-                    for (int m1 = 0; m1 < f.p; ++m1, Lb += Cp)
-                        add(w0 * sW[warp][1][m1][lane], reinterpret_cast<const float4 *>(Lb));
-                }
-            } else {
-                for (int m0 = 0; m0 < f.p; ++m0)
-                    for (int m1 = 0; m1 < f.p; ++m1) {
-                        const float w01 = sW[warp][0][m0][lane] * sW[warp][1][m1][lane];
-                        for (int m2 = 0; m2 < f.p; ++m2, Lb += Cp)
-                            add(w01 * sW[warp][2][m2][lane], reinterpret_cast<const float4 *>(Lb));
-                    }
-            }
-            __syncwarp();
+        for (int q = 0; q < CQ; ++q) {
+            if (col0 + 4 * q >= Cp) break;
+            const float4 v = __ldg(x + q);
+            lo[q] = __ffma2_rn(make_float2(d, d), make_float2(v.x, v.y), lo[q]);
+            hi[q] = __ffma2_rn(make_float2(d, d), make_float2(v.z, v.w), hi[q]);
         }
-        const float etai = act ? f.eta[i] : 0.f;
-        for (int e = f.near_start[b]; e < f.near_start[b + 1]; ++e) {
-            const int nb = f.near_leaf[e];
-            const int dc = f.near_delta[e];
-            const float ox = ((dc % 3) - 1) * f.h, oy = ((dc / 3) % 3 - 1) * f.h, oz = (dc / 9 - 1) * f.h;
-            const int s1 = f.leaf_start[nb + 1];
-            for (int j = f.leaf_start[nb]; j < s1; ++j) {
-                float4 sj = __ldg(f.atl + j);
-                sj.x += ox;   // source position in the target leaf's frame
-                sj.y += oy;
-                sj.z += oz;
+    };
+    if (far && f.L >= 2) {
+        const float y[3] = {qi.x / a, qi.y / a, qi.z / a};
+        float tk[kMaxP];
+        for (int d = 0; d < f.dim; ++d) {   // node_weights into shared memory
+            tk[0] = 1.f;
+            if (f.p > 1) tk[1] = y[d];
+            for (int k = 2; k < f.p; ++k) tk[k] = 2.f * y[d] * tk[k - 1] - tk[k - 2];
+            const float inv = 1.f / f.p;
+            for (int m = 0; m < f.p; ++m) {
+                float s = 0.f;
+                for (int k = 1; k < f.p; ++k) s = fmaf(f.cheb[m * f.p + k], tk[k], s);
+                sW[warp][d][m][lane] = inv + 2.f * inv * s;
+            }
+        }
+        __syncwarp();
+        const float *Lb = Lc + (f.leaf0 + b) * (int64_t)f.P * Cp + col0;
+        if (f.dim == 2) {
+            for (int m0 = 0; m0 < f.p; ++m0) {
+                const float w0 = sW[warp][0][m0][lane];
+                for (int m1 = 0; m1 < f.p; ++m1, Lb += Cp)
+                    add(w0 * sW[warp][1][m1][lane], reinterpret_cast<const float4 *>(Lb));
+            }
+        } else {
+            for (int m0 = 0; m0 < f.p; ++m0)
+                for (int m1 = 0; m1 < f.p; ++m1) {
+                    const float w01 = sW[warp][0][m0][lane] * sW[warp][1][m1][lane];
+                    for (int m2 = 0; m2 < f.p; ++m2, Lb += Cp)
+                        add(w01 * sW[warp][2][m2][lane], reinterpret_cast<const float4 *>(Lb));
+                }
+        }
+        __syncwarp();
+    }
+    const float etai = act ? f.eta[i] : 0.f;
+    for (int e = f.near_start[b]; e < f.near_start[b + 1]; ++e) {
+        const int nb = f.near_leaf[e];
+        const int dc = f.near_delta[e];
+        const float ox = ((dc % 3) - 1) * f.h, oy = ((dc / 3) % 3 - 1) * f.h, oz = (dc / 9 - 1) * f.h;
+        const int s1 = f.leaf_start[nb + 1];
+        for (int c0 = f.leaf_start[nb]; c0 < s1; c0 += 32) {
+            // 32 sources at a time: their records through shared memory, their X rows on the way into
+            // L1 (one by one each source waited for L2: 1.1 us a source and warp with 32 columns)
+            __syncwarp();
+            if (c0 + lane < s1) {
+                float4 v = __ldg(f.atl + c0 + lane);
+                v.x += ox;   // source position in the target leaf's frame
+                v.y += oy;
+                v.z += oz;
+                sS[warp][lane] = v;
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(Xs + (int64_t)(c0 + lane) * Cp + col0));
+            }
+            __syncwarp();
+            const int je = min(c0 + 32, s1);
+            for (int j = c0; j < je; ++j) {
+                const float4 sj = sS[warp][j - c0];
+                float4 xv[CQ];   // on their way while D_ij is computed
+#pragma unroll
+                for (int q = 0; q < CQ; ++q)
+                    xv[q] = col0 + 4 * q < Cp ? __ldg(reinterpret_cast<const float4 *>(Xs + (int64_t)j * Cp + col0) + q)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
                 const float dx = qi.x - sj.x, dy = qi.y - sj.y, dz = qi.z - sj.z;
                 const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                 const float s2 = fmaf(qi.w, qi.w, sj.w * sj.w);
@@ -445,18 +555,22 @@ __global__ void __launch_bounds__(128) k_fmm_l2p_near(FmmDev f, int64_t nleaf, i
                     d = r2 > 1e-24f ? erff(r2 * rinv * sinv) * rinv : 1.1283791670955126f * sinv;
                 }
                 if (j == i) d = etai;
-                add(d, reinterpret_cast<const float4 *>(Xs + (int64_t)j * Cp + col0));
+#pragma unroll
+                for (int q = 0; q < CQ; ++q) {
+                    lo[q] = __ffma2_rn(make_float2(d, d), make_float2(xv[q].x, xv[q].y), lo[q]);
+                    hi[q] = __ffma2_rn(make_float2(d, d), make_float2(xv[q].z, xv[q].w), hi[q]);
+                }
             }
         }
-        if (act) {
-            float *Ui = U + (int64_t)f.perm[i] * C + col0;
+    }
+    if (act) {
+        float *Ui = U + (int64_t)f.perm[i] * C + col0;
 #pragma unroll
-            for (int q = 0; q < CQ; ++q) {
-                const float v[4] = {lo[q].x, lo[q].y, hi[q].x, hi[q].y};
+        for (int q = 0; q < CQ; ++q) {
+            const float v[4] = {lo[q].x, lo[q].y, hi[q].x, hi[q].y};
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (col0 + 4 * q + j < C) Ui[4 * q + j] = v[j];
-            }
+            for (int j = 0; j < 4; ++j)
+                if (col0 + 4 * q + j < C) Ui[4 * q + j] = v[j];
         }
     }
 }
@@ -480,6 +594,8 @@ FmmDev dev_view(const Fmm *f) {
     d.slot_off = f->slot_off;
     d.near_start = f->near_start;
     d.near_leaf = f->near_leaf;
+    d.tgt_leaf = f->tgt_leaf;
+    d.tgt_first = f->tgt_first;
     d.octant = f->octant;
     d.near_delta = f->near_delta;
     d.atl = f->atl;
@@ -498,6 +614,7 @@ void fmm_free(Fmm *f) {
     if (!f) return;
     void *ptrs[] = {f->perm, f->leaf_start, f->atl, f->eta, f->parent, f->child_lo, f->child_hi, f->octant,
                     f->m2l_box, f->m2l_level, f->m2l_src, f->slot_off, f->near_start, f->near_leaf, f->near_delta,
+                    f->tgt_leaf, f->tgt_first,
                     f->Tm, f->Tl, f->K, f->cheb};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -767,6 +884,15 @@ int fmm_build(wfq_geom *g, int order, Fmm **out) {
     WFQ_TRY(upload(ctx, f, &f->near_start, near_start));
     WFQ_TRY(upload(ctx, f, &f->near_leaf, near_leaf));
     WFQ_TRY(upload(ctx, f, &f->near_delta, near_delta));
+    std::vector<int32_t> tgt_leaf, tgt_first;
+    for (int64_t b = 0; b < f->nleaf; ++b)
+        for (int32_t i = leaf_start[b]; i < leaf_start[b + 1]; i += 32) {
+            tgt_leaf.push_back((int32_t)b);
+            tgt_first.push_back(i);
+        }
+    f->ngroups = (int64_t)tgt_leaf.size();
+    WFQ_TRY(upload(ctx, f, &f->tgt_leaf, tgt_leaf));
+    WFQ_TRY(upload(ctx, f, &f->tgt_first, tgt_first));
     WFQ_TRY(upload(ctx, f, &f->Tm, Tm));
     WFQ_TRY(upload(ctx, f, &f->Tl, Tl));
     WFQ_TRY(upload(ctx, f, &f->K, K));
@@ -823,7 +949,20 @@ int d_apply_fmm(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, cudaS
         const dim3 grid((unsigned)tiles, cols32, (unsigned)((P + 2 * best - 1) / (2 * best)));
         const size_t sm = sizeof(float) * (size_t)P * 2 * best;   // at most 256 x 36 floats
         const unsigned th = 32 * M2L_WARPS;
-        switch (best) {
+        const int nodes = 64 * (32 / lpb), rows = (int)std::min<int64_t>(nodes, round_up(P, 8));
+        const dim3 gbox((unsigned)f->nm2l, cols32, (unsigned)((P + rows - 1) / rows));
+        // A slot takes a block of boxes of one octant about 0.1 us per source node (2 blocks an SM at a
+        // time); box by box the interactions take about 1 / 70 us per 64 x 64 nodes and 32 columns.
+        // us, octant / box: 15k-atom sphere 1277 / 199, 30k 1549 / 552 (1682 / 972 with 32 columns), 20000-atom
+        // tube 664 / 173; a 74k-atom disk's apply 474 / 691.
+        const double waves = std::ceil((double)grid.x * grid.y * grid.z / (2.0 * g->ctx->num_sms));
+        const bool by_box = (double)f->nil * cols32 * P * P / 4096.0 / 70.0 < 0.1 * f->nslots * P * waves;
+        if (by_box) {
+            const size_t smb = sizeof(float) * 2 * MB_KC * (size_t)(rows + lpb);
+            if (smb > 48 * 1024)
+                WFQ_CUDA(cudaFuncSetAttribute(k_fmm_m2l_box, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb));
+            k_fmm_m2l_box<<<gbox, 256, smb, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, rows, M.ptr, Lc.ptr);
+        } else switch (best) {
             case 18: k_fmm_m2l<18><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
             case 16: k_fmm_m2l<16><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
             case 13: k_fmm_m2l<13><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
@@ -837,18 +976,20 @@ int d_apply_fmm(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, cudaS
         }
         WFQ_CUDA(cudaGetLastError());
     }
-    // columns per thread: 32, or the fewest multiple of 4 that holds them
-    const unsigned nl4 = (unsigned)((f->nleaf + 3) / 4);
+    // columns per thread: the fewest multiple of 4 (4, 8, 16, 32) that holds them, but fewer, with D_ij
+    // computed again for the others, while that leaves under 16 warps an SM (a warp's sources are a chain)
+    int cq = Cp > 16 ? 8 : Cp > 8 ? 4 : Cp > 4 ? 2 : 1;
+    auto warps = [&](int q) { return f->ngroups * ((Cp + 4 * q - 1) / (4 * q)); };
+    while (cq > 2 && warps(cq) < 16 * (int64_t)g->ctx->num_sms) cq /= 2;
+    const dim3 gnear((unsigned)((f->ngroups + 3) / 4), (unsigned)((Cp + 4 * cq - 1) / (4 * cq)));
     const int far = L >= 2 ? 1 : 0;
     float *Uf = reinterpret_cast<float *>(U);
-    if (Cp > 16)
-        k_fmm_l2p_near<8><<<dim3(nl4, cols32), 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
-    else if (Cp > 8)
-        k_fmm_l2p_near<4><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
-    else if (Cp > 4)
-        k_fmm_l2p_near<2><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
-    else
-        k_fmm_l2p_near<1><<<nl4, 128, 0, s>>>(fd, f->nleaf, C, Cp, far, Xs.ptr, Lc.ptr, Uf);
+    switch (cq) {
+        case 8: k_fmm_l2p_near<8><<<gnear, 128, 0, s>>>(fd, f->ngroups, C, Cp, far, Xs.ptr, Lc.ptr, Uf); break;
+        case 4: k_fmm_l2p_near<4><<<gnear, 128, 0, s>>>(fd, f->ngroups, C, Cp, far, Xs.ptr, Lc.ptr, Uf); break;
+        case 2: k_fmm_l2p_near<2><<<gnear, 128, 0, s>>>(fd, f->ngroups, C, Cp, far, Xs.ptr, Lc.ptr, Uf); break;
+        default: k_fmm_l2p_near<1><<<gnear, 128, 0, s>>>(fd, f->ngroups, C, Cp, far, Xs.ptr, Lc.ptr, Uf); break;
+    }
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
