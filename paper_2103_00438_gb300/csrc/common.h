@@ -322,8 +322,10 @@ struct SymPartials {
 bool gemv_digits_usable(const wfq_geom *g);
 size_t gemv_digits_plane_elems(const wfq_geom *g);
 unsigned gemv_digits_threshold(const wfq_geom *g);
-// digits of the C vectors X (element i of vector c at i si + c sc); vsum follows vmax in memory
-int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s);
+// digits of the C vectors X (element i of vector c at i si + c sc), and their float pairs [C][n] unless
+// xh is null; vsum follows vmax in memory
+int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, float *xh,
+                      float *xl, cudaStream_t s);
 // the digit products of a group of C <= 4 vectors, into w.acc
 int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, cudaStream_t s, int *err = nullptr);
 // U (element i of vector c at i si + c sc) of the group: from w.acc, or from the double-float product --

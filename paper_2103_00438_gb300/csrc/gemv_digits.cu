@@ -530,14 +530,19 @@ __global__ void __launch_bounds__(256) k_vec_absmax(int64_t n, int64_t si, int64
 __global__ void __launch_bounds__(256) k_vec_digits(int64_t n, int64_t npad, int C, int64_t si, int64_t sc,
                                                     const double *__restrict__ X, const unsigned long long *__restrict__ vmax,
                                                     __half *__restrict__ planes, int *__restrict__ xexp,
-                                                    unsigned *__restrict__ vsum) {
+                                                    unsigned *__restrict__ vsum, float *__restrict__ xh,
+                                                    float *__restrict__ xl) {
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int c = blockIdx.y, cg = min(4, C - (c & ~3));
     const unsigned long long mb = vmax[c];
     const int e = vec_exp(mb);
     __half *dst = planes + (int64_t)(c >> 2) * SV_ROWS * npad + (int64_t)(c & 3) * npad + i;
     unsigned q = 0;
-    if (i < n) q = put_vec_digits(X[i * si + c * sc], e, dst, (int64_t)cg * npad);
+    if (i < n) {
+        const double x = X[i * si + c * sc];
+        q = put_vec_digits(x, e, dst, (int64_t)cg * npad);
+        if (xh) df_split(x, xh[c * n + i], xl[c * n + i]);
+    }
     q = __reduce_add_sync(0xffffffffu, q);
     if ((threadIdx.x & 31) == 0 && q > 0) atomicAdd(vsum + c, q);
     if (i == 0) {
@@ -616,13 +621,14 @@ size_t gemv_digits_plane_elems(const wfq_geom *g) { return (size_t)SV_ROWS * g->
 // against 2^-48 |D_ij v_j| of double-float sums.
 unsigned gemv_digits_threshold(const wfq_geom *g) { return digit_sum_threshold(g, -53 + 48); }
 
-int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, cudaStream_t s) {
+int gemv_digits_split(const wfq_geom *g, int C, const double *X, int64_t si, int64_t sc, const GemvDigits &w, float *xh,
+                      float *xl, cudaStream_t s) {
     WFQ_CUDA(cudaMemsetAsync(w.vmax, 0, (sizeof(unsigned long long) + sizeof(unsigned)) * C, s));
     const unsigned nb = (unsigned)std::min<int64_t>((g->n + 255) / 256, 64);
     k_vec_absmax<<<dim3(nb, (unsigned)C), 256, 0, s>>>(g->n, si, sc, X, w.vmax);
     note_launch();
     k_vec_digits<<<dim3((unsigned)((g->n + 255) / 256), (unsigned)C), 256, 0, s>>>(
-        g->n, g->npad, C, si, sc, X, w.vmax, reinterpret_cast<__half *>(w.planes), w.xexp, w.vsum);
+        g->n, g->npad, C, si, sc, X, w.vmax, reinterpret_cast<__half *>(w.planes), w.xexp, w.vsum, xh, xl);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

@@ -229,108 +229,105 @@ __global__ void __launch_bounds__(GV_WARPS * 32, MINB) k_dgemv_df(int64_t n, int
 // tile, stored in full, contributes only row sums.
 constexpr int SY_T = (int)kSymTile;
 
-template <int C>
-__device__ __forceinline__ void dsymv_df_item(int item, int64_t n, int64_t T, const float *__restrict__ Dsym,
-                                                     const SymItem *__restrict__ items,
+// LOOP: beside a digit-slice product (pi) with a few blocks, as k_dgemv_df.
+template <int C, bool LOOP>
+__global__ void __launch_bounds__(256, 2) k_dsymv_df(int64_t n, int64_t T, const float *__restrict__ Dsym,
+                                                     const SymItem *__restrict__ items, int nitems,
                                                      const float *__restrict__ xh, const float *__restrict__ xl,
-                                                     float2 *__restrict__ rowpart, float2 *__restrict__ colpart) {
+                                                     float2 *__restrict__ rowpart, float2 *__restrict__ colpart,
+                                                     const PlainIf pi) {
+    if (LOOP && !pi.runs(C)) return;
     __shared__ __align__(16) float sxh[C][SY_T];
     __shared__ __align__(16) float sxl[C][SY_T];
     __shared__ float2 cred[16][SY_T * C];
-    const SymItem it = items[item];
     const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
-    const int64_t I = it.I;
-    float xih[4][C], xil[4][C], rh[4][C], rl[4][C];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int64_t i = I * SY_T + tr * 4 + r;
-#pragma unroll
-        for (int d = 0; d < C; ++d) {
-            xih[r][d] = i < n ? xh[(int64_t)d * n + i] : 0.f;
-            xil[r][d] = i < n ? xl[(int64_t)d * n + i] : 0.f;
-            rh[r][d] = rl[r][d] = 0.f;
-        }
-    }
-    for (int J = it.J0; J < it.J1; ++J) {
-        const int64_t t = sym_tile(I, J, T);
-        const float *th = Dsym + t * 2 * SY_T * SY_T, *tl = th + SY_T * SY_T;
-        __syncthreads();   // the previous tile's shared-memory readers are done
-        if (tid < C * SY_T) {
-            const int d = tid / SY_T, c = tid % SY_T;
-            const int64_t j = (int64_t)J * SY_T + c;
-            sxh[d][c] = j < n ? xh[(int64_t)d * n + j] : 0.f;
-            sxl[d][c] = j < n ? xl[(int64_t)d * n + j] : 0.f;
-        }
-        float4 dh[4], dl[4];
+    int item = blockIdx.x;
+    do {
+        const SymItem it = items[item];
+        const int64_t I = it.I;
+        float xih[4][C], xil[4][C], rh[4][C], rl[4][C];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            dh[r] = __ldg(reinterpret_cast<const float4 *>(th + (tr * 4 + r) * SY_T + tc * 4));
-            dl[r] = __ldg(reinterpret_cast<const float4 *>(tl + (tr * 4 + r) * SY_T + tc * 4));
-        }
-        __syncthreads();
-        const bool diag = J == I;
-        float ch[4][C], cl[4][C];
+            const int64_t i = I * SY_T + tr * 4 + r;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int d = 0; d < C; ++d) ch[c][d] = cl[c][d] = 0.f;
-#pragma unroll
-        for (int d = 0; d < C; ++d) {
-            const float4 ah = *reinterpret_cast<const float4 *>(&sxh[d][tc * 4]);
-            const float4 al = *reinterpret_cast<const float4 *>(&sxl[d][tc * 4]);
-            const float xjh[4] = {ah.x, ah.y, ah.z, ah.w}, xjl[4] = {al.x, al.y, al.z, al.w};
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float vh[4] = {dh[r].x, dh[r].y, dh[r].z, dh[r].w};
-                const float vl[4] = {dl[r].x, dl[r].y, dl[r].z, dl[r].w};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    df_mac(vh[c], vl[c], xjh[c], xjl[c], rh[r][d], rl[r][d]);
-                    if (!diag) df_mac(vh[c], vl[c], xih[r][d], xil[r][d], ch[c][d], cl[c][d]);
-                }
+            for (int d = 0; d < C; ++d) {
+                xih[r][d] = i < n ? xh[(int64_t)d * n + i] : 0.f;
+                xil[r][d] = i < n ? xl[(int64_t)d * n + i] : 0.f;
+                rh[r][d] = rl[r][d] = 0.f;
             }
         }
-        if (!diag) {
+        for (int J = it.J0; J < it.J1; ++J) {
+            const int64_t t = sym_tile(I, J, T);
+            const float *th = Dsym + t * 2 * SY_T * SY_T, *tl = th + SY_T * SY_T;
+            __syncthreads();   // the previous tile's shared-memory readers are done
+            if (tid < C * SY_T) {
+                const int d = tid / SY_T, c = tid % SY_T;
+                const int64_t j = (int64_t)J * SY_T + c;
+                sxh[d][c] = j < n ? xh[(int64_t)d * n + j] : 0.f;
+                sxl[d][c] = j < n ? xl[(int64_t)d * n + j] : 0.f;
+            }
+            float4 dh[4], dl[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                dh[r] = __ldg(reinterpret_cast<const float4 *>(th + (tr * 4 + r) * SY_T + tc * 4));
+                dl[r] = __ldg(reinterpret_cast<const float4 *>(tl + (tr * 4 + r) * SY_T + tc * 4));
+            }
+            __syncthreads();
+            const bool diag = J == I;
+            float ch[4][C], cl[4][C];
 #pragma unroll
             for (int c = 0; c < 4; ++c)
 #pragma unroll
-                for (int d = 0; d < C; ++d) cred[tr][(tc * 4 + c) * C + d] = make_float2(ch[c][d], cl[c][d]);
-            __syncthreads();
-            if (tid < SY_T * C) {
-                float sh = 0.f, sl = 0.f;
+                for (int d = 0; d < C; ++d) ch[c][d] = cl[c][d] = 0.f;
 #pragma unroll
-                for (int q = 0; q < 16; ++q) df_add(sh, sl, cred[q][tid].x, cred[q][tid].y);
-                colpart[t * SY_T * C + tid] = make_float2(sh, sl);   // (column, direction) = (tid / C, tid % C)
+            for (int d = 0; d < C; ++d) {
+                const float4 ah = *reinterpret_cast<const float4 *>(&sxh[d][tc * 4]);
+                const float4 al = *reinterpret_cast<const float4 *>(&sxl[d][tc * 4]);
+                const float xjh[4] = {ah.x, ah.y, ah.z, ah.w}, xjl[4] = {al.x, al.y, al.z, al.w};
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float vh[4] = {dh[r].x, dh[r].y, dh[r].z, dh[r].w};
+                    const float vl[4] = {dl[r].x, dl[r].y, dl[r].z, dl[r].w};
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        df_mac(vh[c], vl[c], xjh[c], xjl[c], rh[r][d], rl[r][d]);
+                        if (!diag) df_mac(vh[c], vl[c], xih[r][d], xil[r][d], ch[c][d], cl[c][d]);
+                    }
+                }
+            }
+            if (!diag) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int d = 0; d < C; ++d) cred[tr][(tc * 4 + c) * C + d] = make_float2(ch[c][d], cl[c][d]);
+                __syncthreads();
+                if (tid < SY_T * C) {
+                    float sh = 0.f, sl = 0.f;
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) df_add(sh, sl, cred[q][tid].x, cred[q][tid].y);
+                    colpart[t * SY_T * C + tid] = make_float2(sh, sl);   // (column, direction) = (tid / C, tid % C)
+                }
             }
         }
-    }
-    // row sums over the 16 threads of a thread row (16 consecutive lanes), fixed butterfly
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int d = 0; d < C; ++d)
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) {
-                const float oh = __shfl_xor_sync(0xffffffffu, rh[r][d], off);
-                const float ol = __shfl_xor_sync(0xffffffffu, rl[r][d], off);
-                df_add(rh[r][d], rl[r][d], oh, ol);
-            }
-    if (tc == 0)
+        // row sums over the 16 threads of a thread row (16 consecutive lanes), fixed butterfly
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int d = 0; d < C; ++d)
-                rowpart[((int64_t)item * SY_T + tr * 4 + r) * C + d] = make_float2(rh[r][d], rl[r][d]);
-}
-
-// Beside a digit-slice product (pi) with a few blocks, as k_dgemv_df.
-template <int C>
-__global__ void __launch_bounds__(256, 2)
-    k_dsymv_df(int64_t n, int64_t T, const float *__restrict__ Dsym, const SymItem *__restrict__ items, int nitems,
-               const float *__restrict__ xh, const float *__restrict__ xl, float2 *__restrict__ rowpart,
-               float2 *__restrict__ colpart, const PlainIf pi) {
-    if (!pi.runs(C)) return;
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x) dsymv_df_item<C>(item, n, T, Dsym, items, xh, xl, rowpart, colpart);
+#pragma unroll
+                for (int off = 8; off > 0; off >>= 1) {
+                    const float oh = __shfl_xor_sync(0xffffffffu, rh[r][d], off);
+                    const float ol = __shfl_xor_sync(0xffffffffu, rl[r][d], off);
+                    df_add(rh[r][d], rl[r][d], oh, ol);
+                }
+        if (tc == 0)
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int d = 0; d < C; ++d)
+                    rowpart[((int64_t)item * SY_T + tr * 4 + r) * C + d] = make_float2(rh[r][d], rl[r][d]);
+        item += gridDim.x;
+    } while (LOOP && item < nitems);
 }
 
 // U[d][i] = (row sums of the items of tile row K) + (column sums of tiles (I, K), I < K),
@@ -365,19 +362,26 @@ void launch_dgemv_c(int cg, int tiling, int64_t n, int64_t ld, const float *Fh, 
     }
 }
 
-// The symmetric product of cg <= 4 vectors into its partial sums.
+// The symmetric product of cg <= 4 vectors into its partial sums, in full or beside a digit-slice product.
+template <int C>
+void launch_dsymv(const wfq_geom *g, const float *xh, const float *xl, float2 *rowpart, float2 *colpart, const PlainIf &pi,
+                  cudaStream_t s) {
+    const int ni = (int)g->sym_nitems;
+    if (pi.sums.vsum)
+        k_dsymv_df<C, true><<<std::min(ni, 2 * g->ctx->num_sms), 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh,
+                                                                               xl, rowpart, colpart, pi);
+    else
+        k_dsymv_df<C, false><<<ni, 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
+    note_launch();
+}
 void launch_dsymv(const wfq_geom *g, int cg, const float *xh, const float *xl, float2 *rowpart, float2 *colpart,
                   const PlainIf &pi, cudaStream_t s) {
-    const int ni = (int)g->sym_nitems;
-    const unsigned grid = pi.sums.vsum ? (unsigned)std::min(ni, 2 * g->ctx->num_sms) : (unsigned)ni;
-    const int64_t n = g->n, T = g->sym_nt;
     switch (cg) {
-        case 1: k_dsymv_df<1><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
-        case 2: k_dsymv_df<2><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
-        case 3: k_dsymv_df<3><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
-        default: k_dsymv_df<4><<<grid, 256, 0, s>>>(n, T, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi); break;
+        case 1: launch_dsymv<1>(g, xh, xl, rowpart, colpart, pi, s); break;
+        case 2: launch_dsymv<2>(g, xh, xl, rowpart, colpart, pi, s); break;
+        case 3: launch_dsymv<3>(g, xh, xl, rowpart, colpart, pi, s); break;
+        default: launch_dsymv<4>(g, xh, xl, rowpart, colpart, pi, s); break;
     }
-    note_launch();
 }
 
 // The double-float product from the planes beside a digit-slice product (runs where pi says so).
@@ -1030,7 +1034,7 @@ struct Arnoldi {
     }
     SymPartials partials() const { return SymPartials{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt}; }
     // digits of v [C][n] (the start vectors; later ones get theirs in k_rscale_norm)
-    int split(const double *v) { return digits ? gemv_digits_split(g, C, v, 1, n, work(0), s) : WFQ_OK; }
+    int split(const double *v) { return digits ? gemv_digits_split(g, C, v, 1, n, work(0), nullptr, nullptr, s) : WFQ_OK; }
 
     // u = D v; xh / xl (or the digit planes) already hold v (written when v was normalised)
     int dmul(double *u) {
@@ -1134,15 +1138,12 @@ struct Arnoldi {
 
 // Real column r of an atom-major complex block X (n x cc; r = 2c + 0/1 for the real and
 // imaginary parts of column c) split into direction-major float pairs xh/xl [C][n].
-// X has ld real columns a row; pi: groups of 4 columns (complex parts) of the digit slices are left out.
-__global__ void k_cols_split(int64_t n, int C, int64_t ld, const double *__restrict__ X, float *__restrict__ xh,
-                             float *__restrict__ xl, const PlainIf pi) {
+__global__ void k_cols_split(int64_t n, int C, const double *__restrict__ X, float *__restrict__ xh,
+                             float *__restrict__ xl) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n * C) return;
     const int64_t r = e / n, i = e - r * n;
-    const int r4 = (int)r & ~3;
-    if (pi.sums.vsum && !VecSums{pi.sums.vsum + r4, pi.sums.vmax + r4, pi.sums.thr}.plain(min(4, C - r4))) return;
-    df_split(X[i * ld + r], xh[e], xl[e]);
+    df_split(X[i * C + r], xh[e], xl[e]);
 }
 
 // U (atom-major complex block, real column r at i * C + r) = Ud [C][n]
@@ -1173,14 +1174,12 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
         // blocks of 32 real columns, groups of 4: workspace of one block
         constexpr int CB = 32;
         const int cb0 = std::min(C, CB);
-        DevBuf<uint16_t> planes;
         DevBuf<int> xexp;
-        DevBuf<unsigned long long> stats, acc;
-        const size_t gp = gemv_digits_plane_elems(g), np = gp * ((cb0 + 3) / 4);
-        WFQ_TRY(planes.alloc(g->ctx, np, s));
+        DevBuf<unsigned long long> stats, zeroed;   // zeroed: integer sums, then digit planes
+        const size_t gp = gemv_digits_plane_elems(g), words = (size_t)8 * n + gp * ((cb0 + 3) / 4) / 4;
+        WFQ_TRY(zeroed.alloc(g->ctx, words, s));
         WFQ_TRY(xexp.alloc(g->ctx, cb0, s));
         WFQ_TRY(stats.alloc(g->ctx, cb0 + (cb0 + 1) / 2, s));
-        WFQ_TRY(acc.alloc(g->ctx, (size_t)8 * n, s));
         WFQ_TRY(xh.alloc(g->ctx, (size_t)n * cb0, s));
         WFQ_TRY(xl.alloc(g->ctx, (size_t)n * cb0, s));
         if (sym) {
@@ -1190,16 +1189,13 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
             WFQ_TRY(ud.alloc(g->ctx, (size_t)n * std::min(C, 4), s));
         }
         // atoms past n stay zero; rows of digits that a group of fewer columns leaves are not read back
-        WFQ_CUDA(cudaMemsetAsync(planes.ptr, 0, sizeof(uint16_t) * np, s));
-        WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 8 * n, s));
+        WFQ_CUDA(cudaMemsetAsync(zeroed.ptr, 0, sizeof(unsigned long long) * words, s));
         KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
         for (int b0 = 0; b0 < C; b0 += CB) {
             const int cb = std::min(CB, C - b0);
-            GemvDigits w{planes.ptr, xexp.ptr, stats.ptr, acc.ptr, reinterpret_cast<unsigned *>(stats.ptr + cb),
-                         gemv_digits_threshold(g), true};
-            WFQ_TRY(gemv_digits_split(g, cb, x + b0, C, 1, w, s));
-            k_cols_split<<<nblk(n * cb), 256, 0, s>>>(n, cb, C, x + b0, xh.ptr, xl.ptr, PlainIf{w.sums()});
-            note_launch();
+            GemvDigits w{reinterpret_cast<uint16_t *>(zeroed.ptr + 8 * n), xexp.ptr, stats.ptr, zeroed.ptr,
+                         reinterpret_cast<unsigned *>(stats.ptr + cb), gemv_digits_threshold(g), true};
+            WFQ_TRY(gemv_digits_split(g, cb, x + b0, C, 1, w, xh.ptr, xl.ptr, s));
             for (int d0 = 0; d0 < cb; d0 += 4, w.planes += gp, w.xexp += 4, w.vmax += 4, w.vsum += 4) {
                 const int cg = std::min(4, cb - d0);
                 const PlainIf pi{w.sums()};
@@ -1218,7 +1214,7 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(ud.alloc(g->ctx, (size_t)n * C, s));
-    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr, kAlways);
+    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr);
     note_launch();
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     if (g->Dfh) {
@@ -1253,7 +1249,7 @@ int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(ud.alloc(g->ctx, (size_t)n * C, s));
-    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr, kAlways);
+    k_cols_split<<<nblk(n * C), 256, 0, s>>>(n, C, reinterpret_cast<const double *>(X), xh.ptr, xl.ptr);
     note_launch();
     KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
     for (int d0 = 0; d0 < C; d0 += 4)
