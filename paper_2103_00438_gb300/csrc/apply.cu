@@ -522,7 +522,10 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     // smallest structures its launches take longer than they save (us per apply of 16 columns, pairs:
     // 40 atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
     DigitColsBuf cols;
-    if (g->digits_ok && n >= 96) WFQ_TRY(digits_product(g, 7, C, x, u, cols, s, err));
+    if (g->digits_ok && n >= 96) {
+        WFQ_TRY(digits_product(g, false, C, x, u, cols, s, err));
+        if (cols.dc.thr <= kSumOfOne) return WFQ_OK;   // no column can be left
+    }
     dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
     if (g->Dfh)
@@ -560,7 +563,7 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     DigitColsBuf cols;
     // eight exact digits on the tensor cores; dominated columns and those that are not finite in
     // plain FP64.  10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
-    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) WFQ_TRY(digits_product(g, 8, C, x, u, cols, s, err));
+    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) WFQ_TRY(digits_product(g, true, C, x, u, cols, s, err));
     if (g->D64 && C <= 8) {
         switch (C) {
             case 2: launch_dgemv64<2>(n, g->D64, x, u, cols.dc, s); break;

@@ -285,18 +285,18 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
 // for the refinement residual of mixed-precision solves.
 int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
 
-// U = D X for C real columns (row-major) by S = 7 or 8 exact digit slices on the tensor cores
-// (gemm_digits.cu): S = 8 from the FP64 D, S = 7 from the FP32 pair planes, else the FP64 D.
-// Needs g->digits_ok.  Columns of X with an Inf or NaN give NaN; those that few entries dominate are
-// not written: plain kernels take them, by cols (allocated here, on s).
+// U = D X for C real columns (row-major) by exact digit slices on the tensor cores (gemm_digits.cu), to
+// the bound of FP64 sums (fp64: eight digits, from the FP64 D) or of double-float ones (from the FP32 pair
+// planes, else the FP64 D: seven digits, or eight if a column needs them).  Needs g->digits_ok.  Columns of
+// X with an Inf or NaN give NaN; those that few entries dominate are not written: plain kernels take
+// them, by cols (allocated here, on s).
 struct DigitColsBuf {
-    DevBuf<unsigned long long> buf;
-    DigitCols dc{nullptr, nullptr, 0};
-    void set(const wfq_geom *g, int S, int64_t C);
+    DevBuf<unsigned long long> buf;   // integer sums [n][C][2], then the columns' maxima and sums
+    DigitCols dc{nullptr, nullptr, 0, 0};
 };
 // 2^8 2^log2_ratio 2^max(E) / dmin (digit_cols.cuh), capped
 unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio);
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
+int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err = nullptr);
 
 // U = D V for real vectors, 4 at a time, by exact digit slices from the stored float pairs (symmetric

@@ -9,7 +9,8 @@
 // a column is taken in digits only then (the sum may be that of the other part of the complex
 // column: its error stands beside the same |y|).  csum: sum_j floor(2^8 |x_j| / 2^e), from the splitting kernel;
 // thr = 2^8 (u_d / u) 2^max(E) / dmin.  A 20000-atom tube of carbon asks for an average |x_j| of 0.004
-// (u_d / u = 2^-5) or 0.03 (2^-2) of 2^e; normal random columns have 0.1 to 0.2.
+// of 2^e in FP64 blocks (u_d / u = 2^-5, eight digits), 0.03 (2^-2, seven digits) or 0.0002 (2^-9, eight)
+// in double-float ones; normal random columns have 0.1 to 0.2, the charges of a solve down to 0.01.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -22,6 +23,7 @@ struct DigitCols {
     unsigned long long *cmax;   // bits of the largest |x| of each column (null: no columns to sort out)
     unsigned *csum;
     unsigned thr;
+    unsigned thr7;   // seven digits do when every column of the digits has this sum
 };
 
 // Whether real column c (its sum and largest magnitude) or its partner in a complex column, whose rows it
@@ -35,6 +37,8 @@ __device__ __forceinline__ bool sum_suffices(unsigned own, unsigned other, unsig
     if (up >= 0) return up > 31 || ((unsigned long long)other << up) >= thr;
     return -up < 32 && (other >> -up) >= thr;
 }
+
+constexpr unsigned kSumOfOne = 128;   // csum of a column that is not zero: at least its largest entry's
 
 enum ColState { COL_ZERO, COL_DIGITS, COL_PLAIN, COL_NOT_FINITE };
 

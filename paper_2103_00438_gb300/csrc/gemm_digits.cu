@@ -64,6 +64,7 @@ using tc::ROWB;
 
 constexpr int DG_CHUNK = 128;          // atoms per accumulator read-back: 2^14 * 8 * 128 = 2^24
 constexpr int DG_HALF = 32;            // columns per TMEM slot
+constexpr int DG_DIGITS = 8;           // digit planes of X (seven digits: the first seven)
 constexpr int DG_STAGES = 2;           // a third D stage (it fits for S = 7) measured slower: less L1
 constexpr int DG_EPI_WARPS = 16, DG_CONV_WARPS = 8;
 constexpr int DG_EPI_COLS = 2 * DG_HALF / (DG_EPI_WARPS / 4);   // columns an epilogue thread sums
@@ -126,6 +127,20 @@ __device__ __forceinline__ uint64_t biased_pair(float h, float l, float sh, floa
     return (uint64_t)((int64_t)it * 2147483648ll + ib);
 }
 
+// v 2^(61 - E) as an integer, truncated; |v| < 2^E.
+__device__ __forceinline__ int64_t fixed_float(float v, int E) {
+    const uint32_t b = __float_as_uint(v);
+    const int ex = (int)((b >> 23) & 0xffu), sh = max(ex, 1) - 89 - E;   // v = m 2^(ex - 150)
+    const uint64_t m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);
+    const int64_t f = (int64_t)(sh >= 0 ? m << min(sh, 38) : m >> min(-sh, 31));   // (38: memory past column n)
+    return (int)b < 0 ? -f : f;
+}
+
+// biased<8> of a float pair in units of 2^(E - 61).
+__device__ __forceinline__ uint64_t biased_pair8(float h, float l, int E) {
+    return (uint64_t)(fixed_float(h, E) + fixed_float(l, E)) + 0x8080808080808080ull;
+}
+
 // Two digits, bytes q and q + 1 of w (q = 0 or 2), as fp16: 0x6400 | u is 1024 + u.
 __device__ __forceinline__ uint32_t digits_f16(uint32_t w, bool upper) {
     const uint32_t b = __byte_perm(w, 0x64646464u, upper ? 0x4342u : 0x4140u);
@@ -154,13 +169,7 @@ __device__ __forceinline__ void add96(uint32_t &t0, uint32_t &t1, uint32_t &t2, 
 }
 
 template <int S, int SRC>
-__global__ void __launch_bounds__(DG_THREADS, 1)
-    k_gemm_digits(const __grid_constant__ CUtensorMap tm_x, const DigitParams dp) {
-    {   // nothing to do when plain sums take every column
-        bool mine = false;
-        for (int64_t c = threadIdx.x; c < dp.C; c += DG_THREADS) mine = mine || col_state(dp.cols, c) == COL_DIGITS;
-        if (!__syncthreads_or(mine)) return;
-    }
+__device__ __forceinline__ void gemm_digits(const CUtensorMap &tm_x, const DigitParams &dp) {
     const Params &p = dp.p;
     constexpr uint32_t A_STAGE = S * DG_A_BYTES;
     constexpr uint32_t B_HALF = S * DG_HALF * ROWB;   // one half's X digit planes of a stage
@@ -359,7 +368,12 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
             for (int q = 0; q < DG_ROWS; ++q) {
                 const int ex = (int)(f.ex << (24 - 8 * q)) >> 24;
                 uint64_t g[4];
-                if constexpr (SRC == SRC_PAIRS) {
+                if constexpr (SRC == SRC_PAIRS && S == 8) {
+                    g[0] = biased_pair8(f.a[q].x, f.b[q].x, ex);
+                    g[1] = biased_pair8(f.a[q].y, f.b[q].y, ex);
+                    g[2] = biased_pair8(f.a[q].z, f.b[q].z, ex);
+                    g[3] = biased_pair8(f.a[q].w, f.b[q].w, ex);
+                } else if constexpr (SRC == SRC_PAIRS) {
                     const float sh = __int_as_float((127 + 22 - ex) << 23);
                     const float sl = __int_as_float((127 + 53 - ex) << 23);
                     g[0] = biased_pair(f.a[q].x, f.b[q].x, sh, sl);
@@ -437,7 +451,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
                     tc::mbar_expect_tx(fb, (uint32_t)nh * B_HALF);
                     for (int h = 0; h < nh; ++h)
                         tc::tma_load_2d(smem_base + B_OFF + (2 * s + (uint32_t)h) * B_HALF, &tm_x, fb,
-                                        cur.kc * DG_CHUNK + st * BK, (2 * cur.grp + h) * S * DG_HALF);
+                                        cur.kc * DG_CHUNK + st * BK, (2 * cur.grp + h) * DG_DIGITS * DG_HALF);
                 }
             }
             if (aborted) {   // wait (bounded) for the copies of the last stages issued
@@ -508,6 +522,35 @@ __global__ void __launch_bounds__(DG_THREADS, 1)
     }
 }
 
+// Eight digits; or seven if they do for every column, else eight -- in one launch (DG_BOTH), or in two of
+// which one finds nothing to do (4 us): with both bodies in a kernel its registers spill, which
+// costs 4% (20000 atoms x 384 real columns 8.79 ms against 8.45).
+enum DigitMode { DG_EIGHT, DG_BOTH, DG_IF_SEVEN, DG_IF_EIGHT };
+constexpr int64_t DG_BOTH_MAX = 4096;   // atoms
+template <int SRC, DigitMode MODE>
+__global__ void __launch_bounds__(DG_THREADS, 1)
+    k_gemm_digits(const __grid_constant__ CUtensorMap tm7, const __grid_constant__ CUtensorMap tm8, const DigitParams dp) {
+    const DigitCols &cols = dp.cols;
+    bool mine = false, low = false;
+    for (int64_t c = threadIdx.x; c < dp.C; c += DG_THREADS)
+        if (col_state(cols, c) == COL_DIGITS) {
+            mine = true;
+            if constexpr (MODE != DG_EIGHT)
+                low = low || !sum_suffices(cols.csum[c], cols.csum[c ^ 1], cols.cmax[c], cols.cmax[c ^ 1], cols.thr7);
+        }
+    if (!__syncthreads_or(mine)) return;   // plain sums take every column
+    const bool eight = MODE == DG_EIGHT || __syncthreads_or(low);
+    if constexpr (MODE == DG_BOTH || MODE == DG_IF_SEVEN) {
+        if (!eight) {
+            gemm_digits<7, SRC>(tm7, dp);
+            return;
+        }
+    }
+    if constexpr (MODE != DG_IF_SEVEN) {
+        if (eight) gemm_digits<8, SRC>(tm8, dp);
+    }
+}
+
 // cmax[c] = the largest |x| of column c as its bit pattern (monotonic; 0x7ff0... and above:
 // not finite).  X: n x C row-major.  Block: 32 columns x 8 row lanes over a run of rows.
 __global__ void __launch_bounds__(256) k_col_absmax(int64_t n, int64_t C, int64_t rpb, const double *__restrict__ X,
@@ -539,9 +582,9 @@ __device__ __forceinline__ int col_exp(unsigned long long bits) {
 
 // X digits: planes [half][digit][32 columns][npad] fp16, zero past row n and column C.  Block:
 // 64 atoms x 32 columns.
-template <int S>
 __global__ void __launch_bounds__(256) k_split_digits(int64_t n, int64_t npad, int64_t C, const double *__restrict__ X,
                                                       DigitCols cols, __half *__restrict__ planes) {
+    constexpr int S = DG_DIGITS;
     __shared__ uint64_t t[64][33];
     __shared__ unsigned qsum[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -600,55 +643,67 @@ __global__ void __launch_bounds__(256) k_digits_finish(int64_t n, int64_t C, con
     U[e] = scalbn(v, dexp[i] + col_exp(cols.cmax[c]) + unit);
 }
 
-template <int S, int SRC>
-cudaError_t launch_digits(const CUtensorMap &m, const DigitParams &dp, int grid, cudaStream_t s) {
+template <int SRC, DigitMode MODE>
+int launch_digits(const __half *planes, const DigitParams &dp, int64_t npad, int grid, cudaStream_t s) {
+    constexpr int S = DG_DIGITS;
     constexpr size_t smem = (size_t)DG_STAGES * S * DG_A_BYTES + (size_t)DG_STAGES * 2 * S * DG_HALF * ROWB + 1024 + 256;
     static_assert(smem <= (size_t)tc::kMaxDynSmem, "digit stages exceed shared memory");
+    std::string msg;
+    CUtensorMap m7, m8;
+    const uint64_t rows = (uint64_t)dp.nhalf * DG_DIGITS * DG_HALF;
+    if (!tc::make_map(&m7, planes, (uint64_t)npad, rows, (uint64_t)npad, 7u * DG_HALF, &msg) ||
+        !tc::make_map(&m8, planes, (uint64_t)npad, rows, (uint64_t)npad, 8u * DG_HALF, &msg))
+        return fail(WFQ_ECUDA, "digit-slice GEMM: " + msg);
     static std::atomic<uint64_t> smem_set{0};
-    cudaError_t e = tc::allow_max_smem(k_gemm_digits<S, SRC>, smem_set);
-    if (e != cudaSuccess) return e;
-    k_gemm_digits<S, SRC><<<(unsigned)grid, DG_THREADS, smem, s>>>(m, dp);
-    return cudaGetLastError();
+    cudaError_t e = tc::allow_max_smem(k_gemm_digits<SRC, MODE>, smem_set);
+    if (e == cudaSuccess) {
+        k_gemm_digits<SRC, MODE><<<(unsigned)grid, DG_THREADS, smem, s>>>(m7, m8, dp);
+        note_launch();
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(WFQ_ECUDA, std::string("digit-slice GEMM: ") + cudaGetErrorString(e));
+    }
+    return WFQ_OK;
+}
+
+template <int SRC>
+int launch_double_float(const __half *planes, const DigitParams &dp, int64_t npad, int grid, cudaStream_t s) {
+    if (dp.p.n <= DG_BOTH_MAX) return launch_digits<SRC, DG_BOTH>(planes, dp, npad, grid, s);
+    WFQ_TRY((launch_digits<SRC, DG_IF_SEVEN>(planes, dp, npad, grid, s)));
+    return launch_digits<SRC, DG_IF_EIGHT>(planes, dp, npad, grid, s);
 }
 
 }  // namespace
-
-void DigitColsBuf::set(const wfq_geom *g, int S, int64_t C) {
-    dc.cmax = buf.ptr;
-    dc.csum = reinterpret_cast<unsigned *>(buf.ptr + C);
-    // What is left out per entry, in 2^(E + e): products with a + b = S, (S - 1) 2^(14 - 8 S) against 2^12,
-    // the truncated or rounded last digits and, S = 7, the float of weights 4 to 6 (2^-24 of 5 2^14 2^7 in
-    // its units): below 2^-58 (S = 8), 2^-50 (S = 7).
-    dc.thr = digit_sum_threshold(g, S == 8 ? -58 + 53 : -50 + 48);
-}
 
 unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio) {
     const double t = std::ceil(std::ldexp(1.0, 8 + log2_ratio + g->dexp_max) / g->dmin);
     return t < 4294967295.0 ? (unsigned)t : 4294967295u;
 }
 
-int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
+int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err) {
     wfq_ctx *ctx = g->ctx;
     const int64_t n = g->n, npad = g->npad;
     const int nhalf = (int)((C + DG_HALF - 1) / DG_HALF);
-    const bool pairs = S == 7 && g->Dfh != nullptr;
+    const bool pairs = !fp64 && g->Dfh != nullptr;
     DevBuf<__half> planes;
-    DevBuf<unsigned long long> acc;
-    WFQ_TRY(planes.alloc(ctx, (size_t)nhalf * S * DG_HALF * npad, s));
-    WFQ_TRY(acc.alloc(ctx, (size_t)2 * n * C, s));
-    WFQ_TRY(cols.buf.alloc(ctx, (size_t)C + (C + 1) / 2, s));
-    cols.set(g, S, C);
-    WFQ_CUDA(cudaMemsetAsync(acc.ptr, 0, sizeof(unsigned long long) * 2 * n * C, s));
-    WFQ_CUDA(cudaMemsetAsync(cols.buf.ptr, 0, sizeof(unsigned long long) * ((size_t)C + (C + 1) / 2), s));
+    const size_t words = (size_t)2 * n * C + C + (C + 1) / 2;
+    WFQ_TRY(planes.alloc(ctx, (size_t)nhalf * DG_DIGITS * DG_HALF * npad, s));
+    WFQ_TRY(cols.buf.alloc(ctx, words, s));
+    unsigned long long *acc = cols.buf.ptr, *cmax = acc + 2 * n * C;
+    // What is left out per entry, in 2^(E + e): products with a + b = S, (S - 1) 2^(14 - 8 S) against 2^12
+    // (2^11 from pairs), the truncated or rounded last digits and, S = 7, the float of weights 4 to 6 (2^-24
+    // of 5 2^14 2^7 in its units): below 2^-57 (S = 8), 2^-50 (S = 7); against 2^-53 or 2^-48.
+    cols.dc = fp64 ? DigitCols{cmax, reinterpret_cast<unsigned *>(cmax + C), digit_sum_threshold(g, -58 + 53), 0}
+                   : DigitCols{cmax, reinterpret_cast<unsigned *>(cmax + C), digit_sum_threshold(g, -57 + 48),
+                               digit_sum_threshold(g, -50 + 48)};
+    WFQ_CUDA(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * words, s));
     const int64_t rpb = std::max<int64_t>(32, round_up((n + 4 * ctx->num_sms - 1) / (4 * ctx->num_sms), 8));
-    k_col_absmax<<<dim3((unsigned)((n + rpb - 1) / rpb), (unsigned)nhalf), 256, 0, s>>>(n, C, rpb, X, cols.dc.cmax);
+    k_col_absmax<<<dim3((unsigned)((n + rpb - 1) / rpb), (unsigned)nhalf), 256, 0, s>>>(n, C, rpb, X, cmax);
     note_launch();
-    const dim3 sg((unsigned)(npad / 64), (unsigned)nhalf);
-    if (S == 8)
-        k_split_digits<8><<<sg, 256, 0, s>>>(n, npad, C, X, cols.dc, planes.ptr);
-    else
-        k_split_digits<7><<<sg, 256, 0, s>>>(n, npad, C, X, cols.dc, planes.ptr);
+    k_split_digits<<<dim3((unsigned)(npad / 64), (unsigned)nhalf), 256, 0, s>>>(n, npad, C, X, cols.dc, planes.ptr);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     DigitParams dp{};
@@ -665,25 +720,16 @@ int digits_product(const wfq_geom *g, int S, int64_t C, const double *X, double 
     dp.Fl = g->Dfl;
     dp.ld = g->ldf;
     dp.dexp = g->dexp;
-    dp.acc = acc.ptr;
+    dp.acc = acc;
     dp.cols = cols.dc;
-    std::string msg;
-    CUtensorMap m;
-    const uint32_t rows = (uint32_t)S * DG_HALF;
-    if (!tc::make_map(&m, reinterpret_cast<const __nv_bfloat16 *>(planes.ptr), (uint64_t)npad, (uint64_t)nhalf * rows,
-                      (uint64_t)npad, rows, &msg))
-        return fail(WFQ_ECUDA, "digit-slice GEMM: " + msg);
     const int grid = (int)std::min<int64_t>(ctx->num_sms, dp.units);
-    cudaError_t e = S == 8 ? launch_digits<8, SRC_FP64>(m, dp, grid, s)
-                    : pairs ? launch_digits<7, SRC_PAIRS>(m, dp, grid, s)
-                            : launch_digits<7, SRC_FP64>(m, dp, grid, s);
-    note_launch();
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return fail(WFQ_ECUDA, std::string("digit-slice GEMM: ") + cudaGetErrorString(e));
-    }
-    k_digits_finish<<<(unsigned)((n * C + 255) / 256), 256, 0, s>>>(n, C, acc.ptr, g->dexp, cols.dc,
-                                                                    pairs ? -35 : -36, U);
+    if (fp64)
+        WFQ_TRY((launch_digits<SRC_FP64, DG_EIGHT>(planes.ptr, dp, npad, grid, s)));
+    else if (pairs)
+        WFQ_TRY(launch_double_float<SRC_PAIRS>(planes.ptr, dp, npad, grid, s));
+    else
+        WFQ_TRY(launch_double_float<SRC_FP64>(planes.ptr, dp, npad, grid, s));
+    k_digits_finish<<<(unsigned)((n * C + 255) / 256), 256, 0, s>>>(n, C, acc, g->dexp, cols.dc, pairs ? -35 : -36, U);
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

@@ -109,3 +109,25 @@ def test_what_a_chunk_of_one_sign_rounds():
         # in units of 2^-7 of weight 4; weight 4 is 2^-32 of weight 0, 2^12 of which is the bound
         err = abs(got - exact) / 2 ** 7 / 2 ** 32 / 2 ** 12
         assert err + n * Fraction(6 * 2 ** 14, 2 ** 68) + n * Fraction(3, 2 ** 54) <= n * Fraction(1, 2 ** 50) + Fraction(1, 2 ** 52)
+
+
+def fixed_float(v, E):
+    """csrc/gemm_digits.cu's fixed_float: v 2^(61 - E), truncated, from the bits of a float."""
+    b = int(np.float32(v).view(np.uint32))
+    ex = (b >> 23) & 0xff
+    sh = max(ex, 1) - 89 - E
+    m = (b & 0x7fffff) | (0x800000 if ex else 0)
+    f = m << sh if sh >= 0 else m >> min(-sh, 31)
+    return -f if b >> 31 else f
+
+
+def test_float_pairs_in_eight_digits():
+    rng = np.random.default_rng(3)
+    vals = list(rng.uniform(-1, 1, 1000) * 2.0 ** rng.uniform(-40, 0, 1000)) + [0.0, 1.0 - 2.0 ** -53, 2.0 ** -30]
+    for v in vals:
+        h = np.float32(v)
+        l = np.float32(v - float(h))
+        f = fixed_float(h, 0) + fixed_float(l, 0)
+        d = digits((f + BIAS[8]) % 2 ** 64, 8)
+        assert sum(x * 256 ** (7 - a) for a, x in enumerate(d)) == f and abs(d[0]) <= 64
+        assert abs(Fraction(f) / 2 ** 61 - Fraction(float(h)) - Fraction(float(l))) < 2 * Fraction(1, 2 ** 61)

@@ -69,17 +69,17 @@ def test_bem_columns(W, ctx, S, prec, planes, ncplx, kind):
     assert np.all(np.abs(y - ref) <= bound)
 
 
-def _far_pair(S, n):
-    """Two clusters 1e5 bohr apart: the entries of D between them are 2^-17 of its largest."""
+def _far_pair(S, n, distance):
+    """Two clusters a distance apart: at 1e5 bohr the entries of D between them are 2^-17 of its largest."""
     a = S.random_cluster(n - n // 3, seed=n)
     b = S.random_cluster(n // 3, seed=n + 1)
-    return np.concatenate([a, b + np.array([1e5, 0.0, 0.0])])
+    return np.concatenate([a, b + np.array([distance, 0.0, 0.0])])
 
 
-def _check(W, ctx, orc, S, n, ncplx, store, prec, kind, zero_imag=False):
+def _check(W, ctx, orc, S, n, ncplx, store, prec, kind, zero_imag=False, distance=1e5):
     """As for BEM, through the neighbour term; a double-float sum of m entries within (m + 8) 2^-48 s
     (a rounding of at most 2^-48 s in each step)."""
-    xyz = _far_pair(S, n)
+    xyz = _far_pair(S, n, distance)
     p = S.carbon_params(1.51)
     p["r0"] = 2.7
     D = orc.d_matrix(xyz, np.full(n, p["eta"]))
@@ -88,6 +88,8 @@ def _check(W, ctx, orc, S, n, ncplx, store, prec, kind, zero_imag=False):
     g = W.Geometry(ctx, xyz, p, store=flag)
     rng = np.random.default_rng(n + ncplx)
     x = np.stack([_column(kind, n, rng) for _ in range(ncplx)], axis=1)
+    if kind == "random":
+        x = S.random_complex((n, ncplx), seed=2)
     if kind == "mixed":
         x[:, 0] = S.random_complex((n, 1), seed=2)[:, 0]   # a column for the digits beside the others
     if zero_imag:
@@ -116,6 +118,14 @@ def test_blocks_of_columns(W, ctx, orc, S, store, prec, kind):
 @pytest.mark.parametrize("store,prec", [("fp64", "fp64"), ("pairs", "df")])
 def test_a_block_without_a_column_for_the_digits(W, ctx, orc, S, store, prec):
     _check(W, ctx, orc, S, 300, 33, store, prec, "one", zero_imag=True)
+
+
+@pytest.mark.parametrize("kind", ["random", "mixed", "spread"])
+@pytest.mark.parametrize("store", ["fp64", "pairs"])
+@pytest.mark.parametrize("n,ncplx", [(451, 5), (300, 33), (97, 6)])
+def test_double_float_blocks_that_need_eight_digits(W, ctx, orc, S, n, ncplx, store, kind):
+    """3000 bohr apart, random columns pass the test of eight digits and not that of seven."""
+    _check(W, ctx, orc, S, n, ncplx, store, "df", kind, distance=3e3)
 
 
 @pytest.mark.parametrize("kind", ["one", "spread", "mixed"])
