@@ -599,10 +599,12 @@ struct CplxT<float2> {
     using R = float;
 };
 
-// v, or NaN when a product's bounded wait gave up: what it left of U is not the product.
+// v, or NaN when a product's bounded wait gave up (code, read early in the kernel): what it left of
+// U is not the product.
+__device__ __forceinline__ int wait_code(const int *err) { return err != nullptr ? *err : 0; }
 template <class V>
-__device__ __forceinline__ V unless_failed(V v, const int *err) {
-    if (err != nullptr && *err != 0) v.x = v.y = CUDART_NAN_F;
+__device__ __forceinline__ V unless_failed(V v, int code) {
+    if (code != 0) v.x = v.y = CUDART_NAN_F;
     return v;
 }
 
@@ -624,6 +626,7 @@ __global__ void __launch_bounds__(512) k_sparse_cols(int64_t n, int64_t cc, int 
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / lpc;
     const int64_t c = (int64_t)blockIdx.y * lpc + (threadIdx.x & (lpc - 1));
     if (i >= n || c >= cc) return;
+    const int code = wait_code(err);
     const int64_t p0 = rowptr[i], p1 = rowptr[i + 1];
     const V *Uc = U + c;
     const V ui = Uc[i * cc];
@@ -655,7 +658,7 @@ __global__ void __launch_bounds__(512) k_sparse_cols(int64_t n, int64_t cc, int 
     V out;
     out.x = ax - (zr * xv.x - zi * xv.y);
     out.y = ay - (zr * xv.y + zi * xv.x);
-    Y[i * cc + c] = unless_failed(out, err);
+    Y[i * cc + c] = unless_failed(out, code);
 }
 
 // Few columns (cc <= 4): one warp per atom row, lanes over neighbours.
@@ -669,6 +672,7 @@ __global__ void __launch_bounds__(128) k_sparse_nbrs(int64_t n, const int64_t *_
     int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (i >= n) return;
+    const int code = wait_code(err);
     const int64_t p0 = rowptr[i], p1 = rowptr[i + 1];
     V ui[CC];
     R ax[CC], ay[CC];
@@ -707,7 +711,7 @@ __global__ void __launch_bounds__(128) k_sparse_nbrs(int64_t n, const int64_t *_
             V out;
             out.x = ax[c] - (zr * xv.x - zi * xv.y);
             out.y = ay[c] - (zr * xv.y + zi * xv.x);
-            Y[i * CC + c] = unless_failed(out, err);
+            Y[i * CC + c] = unless_failed(out, code);
         }
     }
 }
@@ -720,13 +724,14 @@ __global__ void __launch_bounds__(256) k_shift_only(int64_t total, int64_t cc, c
     using R = typename CplxT<V>::R;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= total) return;
+    const int code = wait_code(err);
     const double2 zc = z[e % cc];
     const R zr = (R)zc.x, zi = (R)zc.y;
     const V u = U[e], xv = X[e];
     V out;
     out.x = u.x - (zr * xv.x - zi * xv.y);
     out.y = u.y - (zr * xv.y + zi * xv.x);
-    Y[e] = unless_failed(out, err);
+    Y[e] = unless_failed(out, code);
 }
 
 template <class V, class VAL>
@@ -749,8 +754,14 @@ static int sparse_shift_impl(const wfq_geom *g, int64_t cc, const V *U, const V 
         default: {
             int lpc = 8;
             while (lpc < cc && lpc < 32) lpc *= 2;
-            const dim3 grid((unsigned)((n * lpc + 511) / 512), (unsigned)((cc + lpc - 1) / lpc));
-            k_sparse_cols<V, VAL><<<grid, 512, 0, s>>>(n, cc, lpc, g->rowptr, g->col, val, U, X, z, Y, err); note_launch();
+            // Blocks of 512 threads share the most neighbours; in FP64, bound by the pipe, small structures
+            // need more SMs (us per FP64 apply, 512 / 128 threads: 120 atoms x 5 columns 61 / 53, 1000 x 5
+            // 71 / 57, 4000 x 5 126 / 118; FP32 the same or slower).
+            const int64_t chunks = (cc + lpc - 1) / lpc;
+            int bt = 512;
+            while (sizeof(V) == sizeof(double2) && bt > 128 && (n * lpc + bt - 1) / bt * chunks < 2 * g->ctx->num_sms) bt /= 2;
+            const dim3 grid((unsigned)((n * lpc + bt - 1) / bt), (unsigned)chunks);
+            k_sparse_cols<V, VAL><<<grid, bt, 0, s>>>(n, cc, lpc, g->rowptr, g->col, val, U, X, z, Y, err); note_launch();
         }
     }
     WFQ_CUDA(cudaGetLastError());
