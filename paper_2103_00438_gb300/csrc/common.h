@@ -294,6 +294,8 @@ struct DigitColsBuf {
     DevBuf<unsigned long long> buf;   // integer sums [n][C][2], then the columns' maxima and sums
     DigitCols dc{nullptr, nullptr, 0, 0};
 };
+// Device bytes of a digits_product of C columns (0 where the geometry takes none).
+size_t digits_workspace(const wfq_geom *g, int64_t C);
 // 2^8 2^log2_ratio 2^max(E) / dmin (digit_cols.cuh), capped
 unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio);
 int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
@@ -337,6 +339,8 @@ int gemv_digits_finish(const wfq_geom *g, int C, const GemvDigits &w, const SymP
 // from the stored float pairs (full planes or symmetric tiles) -- the FP64-grade product of
 // geometries that store no FP64 D (shifted.cu).
 int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
+// Its device bytes for C real columns.
+size_t pairs_df_workspace(const wfq_geom *g, int64_t C);
 // The same for a geometry with no stored D: D regenerated per product in double-float
 // (the shifted solver's matrix-free GEMV), at most 4 complex columns.
 int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s);

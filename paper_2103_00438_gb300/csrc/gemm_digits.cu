@@ -682,6 +682,15 @@ unsigned digit_sum_threshold(const wfq_geom *g, int log2_ratio) {
     return t < 4294967295.0 ? (unsigned)t : 4294967295u;
 }
 
+static size_t plane_elems(const wfq_geom *g, int64_t C) {
+    return (size_t)((C + DG_HALF - 1) / DG_HALF) * DG_DIGITS * DG_HALF * g->npad;
+}
+static size_t sum_words(const wfq_geom *g, int64_t C) { return (size_t)2 * g->n * C + C + (C + 1) / 2; }
+
+size_t digits_workspace(const wfq_geom *g, int64_t C) {
+    return g->digits_ok && (g->D64 || g->Dfh) ? plane_elems(g, C) * sizeof(__half) + sum_words(g, C) * sizeof(unsigned long long) : 0;
+}
+
 int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, double *U, DigitColsBuf &cols, cudaStream_t s,
                    int *err) {
     wfq_ctx *ctx = g->ctx;
@@ -689,8 +698,8 @@ int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, dou
     const int nhalf = (int)((C + DG_HALF - 1) / DG_HALF);
     const bool pairs = !fp64 && g->Dfh != nullptr;
     DevBuf<__half> planes;
-    const size_t words = (size_t)2 * n * C + C + (C + 1) / 2;
-    WFQ_TRY(planes.alloc(ctx, (size_t)nhalf * DG_DIGITS * DG_HALF * npad, s));
+    const size_t words = sum_words(g, C);
+    WFQ_TRY(planes.alloc(ctx, plane_elems(g, C), s));
     WFQ_TRY(cols.buf.alloc(ctx, words, s));
     unsigned long long *acc = cols.buf.ptr, *cmax = acc + 2 * n * C;
     // What is left out per entry, in 2^(E + e): products with a + b = S, (S - 1) 2^(14 - 8 S) against 2^12

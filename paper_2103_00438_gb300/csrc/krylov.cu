@@ -1017,7 +1017,8 @@ size_t solve_footprint(const wfq_geom *g, int64_t cc, int m, int prec) {
     b += (size_t)(m + 2) * (size_t)(m + 1) * cc * 48;           // Hessenberg, rotations
     b += (size_t)std::min<int64_t>((int64_t)(n + 127) / 128, 304) * cc * 64 * sizeof(double2);  // partials
     if (mixed) b += 3 * nc * sizeof(float2) + (size_t)round_up(2 * cc, 32) * (size_t)g->npad * 4;
-    return b;
+    // the residuals' products: digit slices, or float pairs where nothing else is stored
+    return b + (g->D64 || g->Dfh ? digits_workspace(g, 2 * cc) : pairs_df_workspace(g, 2 * cc));
 }
 
 // Continue the columns `cols` of a solve from their iterate in a.q: block GMRES(m) at

@@ -928,6 +928,8 @@ bool use_gemv_digits(const wfq_geom *g) {
     return gemv_digits_usable(g) && (!g->Dfh || g->n >= 3072);
 }
 
+constexpr int kPairsBlock = 32;   // real columns an apply from float pairs splits at a time
+
 struct Arnoldi {
     wfq_geom *g;
     cudaStream_t s;
@@ -1172,7 +1174,7 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
     // 185 / 259; 640 atoms 45 / 45, 47 / 70, 195 / 431.
     if (use_gemv_digits(g) && (g->Dfh || n * std::min(C, 4) >= 1100)) {
         // blocks of 32 real columns, groups of 4: workspace of one block
-        constexpr int CB = 32;
+        constexpr int CB = kPairsBlock;
         const int cb0 = std::min(C, CB);
         DevBuf<int> xexp;
         DevBuf<unsigned long long> stats, zeroed;   // zeroed: integer sums, then digit planes
@@ -1261,12 +1263,28 @@ int d_apply_mf_gemv_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 
     return WFQ_OK;
 }
 
+size_t pairs_df_workspace(const wfq_geom *g, int64_t C) {
+    if (!(g->Dfh || g->Dsym)) return 0;
+    const size_t n = (size_t)g->n, cb = use_gemv_digits(g) ? (size_t)std::min<int64_t>(C, kPairsBlock) : (size_t)C;
+    const int cg = (int)std::min<int64_t>(C, 4);
+    size_t b = n * cb * 16;
+    if (use_gemv_digits(g)) b += gemv_digits_plane_elems(g) * ((cb + 3) / 4) * 2 + n * 64;
+    if (!g->Dfh) b += (rowpart_elems(g, cg) + colpart_elems(g, cg)) * sizeof(float2);
+    return b;
+}
+
 size_t shifted_footprint(const wfq_geom *g, int64_t ncols, int ndir, int m) {
     if (m <= 0) m = 600;
     const size_t n = (size_t)g->n, C = (size_t)ndir, nc = (size_t)ncols;
     size_t b = (size_t)(2 * m + 1) * n * C * 8;                                // Arnoldi vectors, D v_k
     b += (size_t)m * (m + 1) / 2 * nc * 16 + (size_t)(3 * m + 2) * nc * 16;   // rotated H, rotations, g, y
     b += n * nc * 16 * 9;                                                     // q, D q, residual blocks
+    b += C * m * (m + 1) * 8;                                                 // Hessenberg matrices
+    b += (n / 128 + 1 + n / 1024 + 1) * (m + 1) * C * 8;                      // partial dots
+    b += 3 * n * C * 8;                                                       // R, U, float pairs of the vectors
+    if (use_gemv_digits(g)) b += gemv_digits_plane_elems(g) * ((C + 3) / 4) * 2 + n * 64;   // digits, integer sums
+    if (g->Dsym && !g->Dfh)
+        b += (rowpart_elems(g, (int)std::min<size_t>(C, 4)) + colpart_elems(g, (int)std::min<size_t>(C, 4))) * sizeof(float2);
     return b;
 }
 
