@@ -187,6 +187,10 @@ int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out);
  * bounded waits had given up with `code` (non-zero; 0 takes the injection back). */
 int wfq_selftest_fail_next_apply(wfq_ctx *ctx, int code);
 
+/* Host-side failure injection: of the context's device allocations from now on the nth (1: the next;
+ * 0: none) fails as if the memory were used up, once. */
+int wfq_selftest_fail_alloc(wfq_ctx *ctx, int nth);
+
 /* Kernel timing (profiling aid).  While enabled, the library records a pair of CUDA
  * events on the launching stream around every launch of the kernels below;
  * wfq_profile_read synchronises those events and returns the launch count and the

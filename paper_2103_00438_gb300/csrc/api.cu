@@ -49,7 +49,9 @@ int dalloc(wfq_ctx *ctx, void **p, size_t bytes, cudaStream_t s) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     note_alloc();
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, s);
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (ctx->fail_alloc.load(std::memory_order_relaxed) <= 0 || ctx->fail_alloc.fetch_sub(1) != 1)
+        e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -289,6 +291,13 @@ int wfq_selftest_wait(wfq_ctx *ctx, int limit_us, int *out) {
 int wfq_selftest_fail_next_apply(wfq_ctx *ctx, int code) {
     if (!ctx) return fail(WFQ_EINVAL, "context is NULL");
     ctx->fail_next_apply.store(code);
+    return WFQ_OK;
+}
+
+int wfq_selftest_fail_alloc(wfq_ctx *ctx, int nth) {
+    if (!ctx) return fail(WFQ_EINVAL, "context is NULL");
+    if (nth < 0) return fail(WFQ_EINVAL, "nth must be >= 0");
+    ctx->fail_alloc.store(nth);
     return WFQ_OK;
 }
 

@@ -523,8 +523,9 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     // 40 atoms 48 against 33, 120 atoms 66 against 68, 240 atoms 76 against 109).
     DigitColsBuf cols;
     if (g->digits_ok && n >= 96) {
-        WFQ_TRY(digits_product(g, false, C, x, u, cols, s, err));
-        if (cols.dc.thr <= kSumOfOne) return WFQ_OK;   // no column can be left
+        const int rc = digits_product(g, false, C, x, u, cols, s, err);
+        if (rc == WFQ_OK && cols.dc.thr <= kSumOfOne) return WFQ_OK;   // no column can be left
+        if (rc != WFQ_OK && rc != WFQ_ENOMEM) return rc;               // no memory: all columns below
     }
     dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
@@ -563,7 +564,11 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     DigitColsBuf cols;
     // eight exact digits on the tensor cores; dominated columns and those that are not finite in
     // plain FP64.  10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
-    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) WFQ_TRY(digits_product(g, true, C, x, u, cols, s, err));
+    // Without memory for them plain FP64 takes all, which needs none.
+    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) {
+        const int rc = digits_product(g, true, C, x, u, cols, s, err);
+        if (rc != WFQ_OK && rc != WFQ_ENOMEM) return rc;
+    }
     if (g->D64 && C <= 8) {
         switch (C) {
             case 2: launch_dgemv64<2>(n, g->D64, x, u, cols.dc, s); break;

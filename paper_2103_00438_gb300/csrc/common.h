@@ -141,6 +141,7 @@ struct wfq_ctx {
     cudaMemPool_t pool = nullptr;
     int *dev_err = nullptr;   // device flag: non-zero after a bounded wait in a kernel gave up
     std::atomic<int> fail_next_apply{0};   // wfq_selftest_fail_next_apply
+    std::atomic<int> fail_alloc{0};        // wfq_selftest_fail_alloc: allocations to the one that fails
     wfq::KernelTimer timer;
     // autotuner results: kernel tiling chosen by timing, per problem key (kept across
     // geometries of the same shape)
@@ -289,7 +290,7 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
 // the bound of FP64 sums (fp64: eight digits, from the FP64 D) or of double-float ones (from the FP32 pair
 // planes, else the FP64 D: seven digits, or eight if a column needs them).  Needs g->digits_ok.  Columns of
 // X with an Inf or NaN give NaN; those that few entries dominate are not written: plain kernels take
-// them, by cols (allocated here, on s).
+// them, by cols (allocated here, on s).  WFQ_ENOMEM: nothing was launched, and cols has every column.
 struct DigitColsBuf {
     DevBuf<unsigned long long> buf;   // integer sums [n][C][2], then the columns' maxima and sums
     DigitCols dc{nullptr, nullptr, 0, 0};

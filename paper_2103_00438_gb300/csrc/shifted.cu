@@ -1158,60 +1158,69 @@ __global__ void k_cols_gather(int64_t n, int C, const double *__restrict__ Ud, d
 
 }  // namespace
 
+// d_apply_pairs_df by digit slices.  WFQ_ENOMEM: nothing was launched.
+static int pairs_by_digits(const wfq_geom *g, int C, const double *x, double *u, cudaStream_t s, int *err) {
+    const int64_t n = g->n;
+    const bool sym = !g->Dfh;
+    DevBuf<float> xh, xl;
+    DevBuf<double> ud;
+    DevBuf<float2> rowpart, colpart;
+    // blocks of 32 real columns, groups of 4: workspace of one block
+    constexpr int CB = kPairsBlock;
+    const int cb0 = std::min(C, CB);
+    DevBuf<int> xexp;
+    DevBuf<unsigned long long> stats, zeroed;   // zeroed: integer sums, then digit planes
+    const size_t gp = gemv_digits_plane_elems(g), words = (size_t)8 * n + gp * ((cb0 + 3) / 4) / 4;
+    WFQ_TRY(zeroed.alloc(g->ctx, words, s));
+    WFQ_TRY(xexp.alloc(g->ctx, cb0, s));
+    WFQ_TRY(stats.alloc(g->ctx, cb0 + (cb0 + 1) / 2, s));
+    WFQ_TRY(xh.alloc(g->ctx, (size_t)n * cb0, s));
+    WFQ_TRY(xl.alloc(g->ctx, (size_t)n * cb0, s));
+    if (sym) {
+        WFQ_TRY(rowpart.alloc(g->ctx, rowpart_elems(g, std::min(C, 4)), s));
+        WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
+    } else {
+        WFQ_TRY(ud.alloc(g->ctx, (size_t)n * std::min(C, 4), s));
+    }
+    // atoms past n stay zero; rows of digits that a group of fewer columns leaves are not read back
+    WFQ_CUDA(cudaMemsetAsync(zeroed.ptr, 0, sizeof(unsigned long long) * words, s));
+    KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
+    for (int b0 = 0; b0 < C; b0 += CB) {
+        const int cb = std::min(CB, C - b0);
+        GemvDigits w{reinterpret_cast<uint16_t *>(zeroed.ptr + 8 * n), xexp.ptr, stats.ptr, zeroed.ptr,
+                     reinterpret_cast<unsigned *>(stats.ptr + cb), gemv_digits_threshold(g), true};
+        WFQ_TRY(gemv_digits_split(g, cb, x + b0, C, 1, w, xh.ptr, xl.ptr, s));
+        for (int d0 = 0; d0 < cb; d0 += 4, w.planes += gp, w.xexp += 4, w.vmax += 4, w.vsum += 4) {
+            const int cg = std::min(4, cb - d0);
+            const PlainIf pi{w.sums()};
+            const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
+            WFQ_TRY(gemv_digits_product(g, cg, w, s, err));
+            if (sym) {
+                launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
+            } else {
+                launch_dgemv_beside(g, cg, ph, pxl, ud.ptr, pi, s);
+            }
+            const SymPartials sp{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt};
+            WFQ_TRY(gemv_digits_finish(g, cg, w, sp, ud.ptr, u + b0 + d0, C, 1, s));
+        }
+    }
+    return WFQ_OK;
+}
+
 int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
     const int64_t n = g->n;
     const int C = (int)(2 * cc);
     if (!(g->Dfh || g->Dsym)) return fail(WFQ_EUNSUPPORTED, "float-pair product: needs stored pairs");
-    const double *x = reinterpret_cast<const double *>(X);
-    double *u = reinterpret_cast<double *>(U);
     DevBuf<float> xh, xl;
     DevBuf<double> ud;
     DevBuf<float2> rowpart, colpart;
-    const bool sym = !g->Dfh;
     auto partials = [&] { return SymPartials{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt}; };
     // An apply's digits cost more launches than a solver's.  From the tiles, us per apply of 1, 2 and 16
     // columns, digits against double-float: 160 atoms 44 / 30, 46 / 39, 178 / 191; 320 atoms 44 / 35, 45 / 47,
     // 185 / 259; 640 atoms 45 / 45, 47 / 70, 195 / 431.
     if (use_gemv_digits(g) && (g->Dfh || n * std::min(C, 4) >= 1100)) {
-        // blocks of 32 real columns, groups of 4: workspace of one block
-        constexpr int CB = kPairsBlock;
-        const int cb0 = std::min(C, CB);
-        DevBuf<int> xexp;
-        DevBuf<unsigned long long> stats, zeroed;   // zeroed: integer sums, then digit planes
-        const size_t gp = gemv_digits_plane_elems(g), words = (size_t)8 * n + gp * ((cb0 + 3) / 4) / 4;
-        WFQ_TRY(zeroed.alloc(g->ctx, words, s));
-        WFQ_TRY(xexp.alloc(g->ctx, cb0, s));
-        WFQ_TRY(stats.alloc(g->ctx, cb0 + (cb0 + 1) / 2, s));
-        WFQ_TRY(xh.alloc(g->ctx, (size_t)n * cb0, s));
-        WFQ_TRY(xl.alloc(g->ctx, (size_t)n * cb0, s));
-        if (sym) {
-            WFQ_TRY(rowpart.alloc(g->ctx, rowpart_elems(g, std::min(C, 4)), s));
-            WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
-        } else {
-            WFQ_TRY(ud.alloc(g->ctx, (size_t)n * std::min(C, 4), s));
-        }
-        // atoms past n stay zero; rows of digits that a group of fewer columns leaves are not read back
-        WFQ_CUDA(cudaMemsetAsync(zeroed.ptr, 0, sizeof(unsigned long long) * words, s));
-        KScope ks(g->ctx, WFQ_KT_DAPPLY_FP64, s, 2.0 * (double)n * (double)n * (double)C);
-        for (int b0 = 0; b0 < C; b0 += CB) {
-            const int cb = std::min(CB, C - b0);
-            GemvDigits w{reinterpret_cast<uint16_t *>(zeroed.ptr + 8 * n), xexp.ptr, stats.ptr, zeroed.ptr,
-                         reinterpret_cast<unsigned *>(stats.ptr + cb), gemv_digits_threshold(g), true};
-            WFQ_TRY(gemv_digits_split(g, cb, x + b0, C, 1, w, xh.ptr, xl.ptr, s));
-            for (int d0 = 0; d0 < cb; d0 += 4, w.planes += gp, w.xexp += 4, w.vmax += 4, w.vsum += 4) {
-                const int cg = std::min(4, cb - d0);
-                const PlainIf pi{w.sums()};
-                const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
-                WFQ_TRY(gemv_digits_product(g, cg, w, s, err));
-                if (sym) {
-                    launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
-                } else {
-                    launch_dgemv_beside(g, cg, ph, pxl, ud.ptr, pi, s);
-                }
-                WFQ_TRY(gemv_digits_finish(g, cg, w, partials(), ud.ptr, u + b0 + d0, C, 1, s));
-            }
-        }
-        return WFQ_OK;
+        const int rc = pairs_by_digits(g, C, reinterpret_cast<const double *>(X), reinterpret_cast<double *>(U), s, err);
+        if (rc != WFQ_ENOMEM) return rc;   // else the double-float sums below, with less of it
     }
     WFQ_TRY(xh.alloc(g->ctx, (size_t)n * C, s));
     WFQ_TRY(xl.alloc(g->ctx, (size_t)n * C, s));

@@ -26,7 +26,7 @@ EXPORTS = ["wfq_create", "wfq_destroy", "wfq_last_error", "wfq_kernel_launches",
            "wfq_polarizability", "wfq_profile", "wfq_profile_read", "wfq_apply_mixed_noalloc",
            "wfq_server_create", "wfq_server_submit", "wfq_server_poll", "wfq_server_destroy",
            "wfq_memory_stats", "wfq_cross_section", "wfq_fmm_build", "wfq_fmm_info", "wfq_selftest_wait",
-           "wfq_selftest_fail_next_apply"]
+           "wfq_selftest_fail_next_apply", "wfq_selftest_fail_alloc"]
 KT_GEMM_MIXED, KT_DAPPLY_FP64, KT_SPARSE, KT_ORTHO, KT_RESIDUAL, KT_DGEMV_DF, KT_FMM = 0, 1, 2, 3, 4, 5, 6
 
 
@@ -96,6 +96,7 @@ def load(path: str | None = None):
     L.wfq_memory_stats.argtypes = [_P, _P]
     L.wfq_selftest_wait.argtypes = [_P, INT, _P]
     L.wfq_selftest_fail_next_apply.argtypes = [_P, INT]
+    L.wfq_selftest_fail_alloc.argtypes = [_P, INT]
     L.wfq_fmm_build.argtypes = [_P, INT]
     L.wfq_fmm_info.argtypes = [_P, _P]
     L.wfq_cross_section.argtypes = [_P, I64, _P, INT, _P, D, _P, _P, _P, _P]
@@ -201,6 +202,10 @@ class Context:
     def selftest_fail_next_apply(self, code: int = 9):
         """The next apply on this context runs as if a kernel's bounded wait had given up."""
         _check(_lib.wfq_selftest_fail_next_apply(self.h, int(code)))
+
+    def selftest_fail_alloc(self, nth: int):
+        """The nth device allocation from now on (0: none) fails as if the memory were used up."""
+        _check(_lib.wfq_selftest_fail_alloc(self.h, int(nth)))
 
     def close(self):
         if self.h:
