@@ -5,7 +5,7 @@ Workload (default "cnt20k"): armchair (10,10) carbon nanotube, 500 unit cells,
 N = 20,000 atoms; 64 frequencies evenly over 0.05-2.0 eV x 3 field directions =
 192 (omega, direction) solves per step, run as ONE launch of the default solver,
 shifted GMRES: one real Arnoldi process per field direction serves all 64
-frequencies (double-float D products from the FP32 pair planes, FP64 basis,
+frequencies (D products by exact digit slices of the FP32 pair planes, FP64 basis,
 per-frequency Givens), every column's FP64 true residual checked to 1e-8, then the
 polarizability.  `--solver gmres` runs the block form instead: the 192 columns as
 one mixed-precision GMRES(50) (3xBF16 tensor-core D products, complex64 basis) with
@@ -98,6 +98,25 @@ DGEMV_DRAM_BYTES_PER_ENTRY = 549.3e6 / (8200.0 * 8320.0)
 
 # Algorithmic bytes of one block apply of D: the FP32 D (4 bytes per entry) read once.
 ALG_BYTES_PER_ENTRY = 4.0
+
+
+def shifted_product(n, store, wfq):
+    """The D product of the shifted solver's Arnoldi vectors on an omega-FQ geometry, as the library
+    dispatches it: kernel, compute dtype and a description.  Its bytes per launch are the library's
+    own count (wfq_profile_read)."""
+    digits = ("k_gemv_digits (digit slices of the upper triangle, tcgen05)", "f16 digit slices (exact sums)+f64",
+              "D products by exact digit slices of the float pairs")
+    if store & wfq.STORE_F32X2:
+        return digits if n >= 3072 else ("k_dgemv_df (double-float, FP32 pair planes)", "f32x2(double-float)+f64",
+                                         "double-float D products (FP32 pair planes)")
+    if store & wfq.STORE_F32X2_SYM:
+        return digits
+    if store & wfq.STORE_FP64:
+        return ("k_dgemv_df (double-float, split from the FP64 D)", "f32x2(double-float)+f64",
+                "double-float D products (FP64 D split per use)")
+    return ("k_dotf_dfv (double-float, D regenerated)", "f32x2(double-float)+f64",
+            "double-float D products (D regenerated from the coordinates)")
+
 
 # Minimum FP32-pipe instructions to generate one D entry as a bf16 hi/lo pair on the
 # matrix-free path: 3 coordinate differences, 3 for r^2, 1 for sigma^2, 1 far/near test,
@@ -430,23 +449,25 @@ def run_ours(args, rank, world, dist):
     # the library from the columns that launch actually carried (the block narrows as
     # columns converge): 6 N^2 C tensor flops (three bf16 products of 2 N^2 C each).
     peaks, peak_src = load_peaks()
+    product = shifted_product(n, store, wfq)
     roof = None
     if gv_n and gv_ms >= gemm_ms:
         # shifted solver: the dominant kernel is the D product of the Arnoldi vectors.
         # Algorithmic bytes per launch: 4 bytes per D entry (the FP32 D read once per block
-        # apply), N^2 entries.  The kernel reads the upper triangle of the FP32 pairs (8 bytes
-        # for ~2^-48 of an entry) and uses every block twice: the same count.
+        # apply), N^2 entries.  Stored bytes: what the kernel that ran reads of D, as the library
+        # counts it (digit slices: the upper triangle of the pairs, 8 bytes an entry, every block used
+        # twice; double-float kernels: 8 bytes per entry of the matrix; 0 where D is not stored).
         avg_s = gv_ms / gv_n * 1e-3
         alg_bytes = ALG_BYTES_PER_ENTRY * float(n) * float(n)
         achieved_gbs = alg_bytes / avg_s / 1e9
         peak = peaks["hbm_gbs"]
         roof = {"bound": "hbm", "achieved": achieved_gbs, "peak": peak, "unit": "GB/s",
                 "frac": achieved_gbs / peak, "traffic": None,
-                "kernel": "k_gemv_digits (D product of the real Arnoldi vectors by digit slices, tcgen05)",
+                "kernel": product[0] + ": D product of the real Arnoldi vectors",
                 "launches": gv_n, "avg_ms": gv_ms / gv_n, "algorithmic_bytes_per_launch": alg_bytes,
                 "algorithmic_bytes_rule": "4 bytes per D entry x N^2 entries (FP32 D streamed once per block apply)",
-                "stored_bytes_per_launch": alg_bytes,
-                "hbm_util_of_stored_bytes": achieved_gbs / peak,
+                "stored_bytes_per_launch": gv_bytes / gv_n if gv_bytes else None,
+                "hbm_util_of_stored_bytes": gv_bytes / gv_n / avg_s / 1e9 / peak if gv_bytes else None,
                 "peak_source": peak_src + " hbm_gbs (STREAM-style copy)"}
     elif gemm_n:
         gemm_avg_ms = gemm_ms / gemm_n
@@ -464,13 +485,13 @@ def run_ours(args, rank, world, dist):
     out = {"metric": "freq-point solves/s", "value": value, "unit": "solves/s", "n_gpus": world,
            "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-           "dtype": "f32x2(double-float)+f64" if args.solver == "shifted" else "bf16x3+f32+f64",
+           "dtype": product[1] if args.solver == "shifted" else "bf16x3+f32+f64",
            "data": "synthetic",
            "config": {"workload": args.workload, "n_atoms": n, "nfreq": nf, "ndir": nd, "columns": ncols,
                       "solver": {"gmres": f"gmres({args.m})", "qmr": "qmr",
                                  "shifted": "shifted gmres (one real Arnoldi per direction, all frequencies)"}[args.solver],
-                      "precision": ("double-float D products (FP32 pair planes), FP64 Arnoldi basis and "
-                                    "per-frequency Givens, FP64-accuracy true residual"
+                      "precision": (product[2] + ", FP64 Arnoldi basis and per-frequency Givens, "
+                                    "FP64-accuracy true residual"
                                     if args.solver == "shifted" else
                                     "mixed: 3xBF16 D products, complex64 basis, FP64 refinement"),
                       "rel_tol": 1e-8, "parallelism": f"replicas{world}",

@@ -202,8 +202,8 @@ enum {
     WFQ_KT_ORTHO = 3,        /* Arnoldi orthogonalisation of one GMRES step (projections,
                                 norm, Givens, scaling) / the vector updates of a QMR step */
     WFQ_KT_RESIDUAL = 4,     /* FP64 true residual of a cycle (gathers, product, norms) */
-    WFQ_KT_DGEMV_DF = 5,     /* shifted GMRES: double-float D product of the real Arnoldi
-                                vectors (one launch per group of <= 4 directions) */
+    WFQ_KT_DGEMV_DF = 5,     /* shifted GMRES: D product of the real Arnoldi vectors, by digit slices
+                                or in double-float (one per group of <= 4 directions) */
     WFQ_KT_FMM = 6,          /* the fast-multipole D product (all its passes) */
     WFQ_KT_COUNT = 7
 };
@@ -214,7 +214,8 @@ int wfq_profile(wfq_ctx *ctx, int enable);
 /* Launches, summed device milliseconds and summed work of kernel class `kind` (WFQ_KT_*).
  * Work: WFQ_KT_GEMM_MIXED -- tensor flops of the three bf16 products, 6 N^2 C per launch
  * (C = real columns of that launch); WFQ_KT_DAPPLY_FP64 -- 2 N^2 C flops; WFQ_KT_DGEMV_DF --
- * algorithmic bytes of D read, 8 N^2 (the entries; padding columns not counted); WFQ_KT_FMM
+ * bytes of D read: 8 per entry, of the full matrix (padding columns not counted) or, digit slices and
+ * symmetric tiles, of the 64 x 64 tiles on and above the diagonal; 0 where D is not stored; WFQ_KT_FMM
  * -- N^2, the pair interactions the product stands for; others 0.
  * Any out-pointer may be NULL. */
 int wfq_profile_read(wfq_ctx *ctx, int kind, int64_t *launches, double *total_ms, double *work);

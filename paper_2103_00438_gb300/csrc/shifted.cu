@@ -1041,13 +1041,16 @@ struct Arnoldi {
     // u = D v; xh / xl (or the digit planes) already hold v (written when v was normalised)
     int dmul(double *u) {
         if (digits) {
+            // the tiles above the diagonal and on it, of the planes likewise (8 bytes an entry)
+            const double T = (double)((n + kSymTile - 1) / kSymTile);
+            const double dbytes = T * (T + 1) / 2 * kSymTile * kSymTile * 8.0;
             for (int d0 = 0; d0 < C; d0 += 4) {
                 const int cg = std::min(4, C - d0);
                 const GemvDigits w = work(d0);
                 const PlainIf pi{w.sums()};
                 const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
                 double *pu = u + (int64_t)d0 * n;
-                KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, 8.0 * (double)n * (double)n);
+                KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, dbytes);
                 WFQ_TRY(gemv_digits_product(g, cg, w, s));
                 if (g->Dfh) {
                     launch_dgemv_beside(g, cg, ph, pxl, pu, pi, s);
