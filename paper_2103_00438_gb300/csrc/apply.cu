@@ -13,8 +13,8 @@ namespace wfq {
 
 // U[i][:] = sum_k D[i][k] X[k][:] for C real columns (C <= 8): each warp owns RW rows so
 // that every X element read from L2 serves RW D rows; D rows are read coalesced.  Bound by the
-// FP64 pipe (1.7 operations per clock per SM), so below 9728 atoms, where 4 rows a warp would
-// leave SMs idle, a warp takes 1 or 2: 1014 atoms, C = 2: 9.5 us, 26.2 with 4 rows.  The order of
+// FP64 pipe (1.7 operations per clock per SM), so below 64 atoms per SM (9728 on 152), where 4 rows
+// a warp would leave SMs idle, a warp takes 1 or 2: 1014 atoms, C = 2: 9.5 us, 26.2 with 4 rows.  The order of
 // a row's sum does not depend on RW.  cols: as k_dgemm.
 template <int C, int RW>
 __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restrict__ D,
@@ -539,11 +539,13 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
 }
 
 template <int C>
-static void launch_dgemv64(int64_t n, const double *D, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
+static void launch_dgemv64(const wfq_geom *g, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
+    const int64_t n = g->n, sms = g->ctx->num_sms;
+    const double *D = g->D64;
     auto blocks = [&](int rw) { return (unsigned)(((n + rw - 1) / rw + 7) / 8); };
-    if (n >= 9728)   // 16 warps an SM on 152 SMs
+    if (n >= 64 * sms)   // 16 warps an SM
         k_dgemv<C, 4><<<blocks(4), 256, 0, s>>>(n, D, x, u, cols);
-    else if (n >= 4864)
+    else if (n >= 32 * sms)
         k_dgemv<C, 2><<<blocks(2), 256, 0, s>>>(n, D, x, u, cols);
     else
         k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u, cols);
@@ -571,10 +573,10 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     }
     if (g->D64 && C <= 8) {
         switch (C) {
-            case 2: launch_dgemv64<2>(n, g->D64, x, u, cols.dc, s); break;
-            case 4: launch_dgemv64<4>(n, g->D64, x, u, cols.dc, s); break;
-            case 6: launch_dgemv64<6>(n, g->D64, x, u, cols.dc, s); break;
-            default: launch_dgemv64<8>(n, g->D64, x, u, cols.dc, s); break;
+            case 2: launch_dgemv64<2>(g, x, u, cols.dc, s); break;
+            case 4: launch_dgemv64<4>(g, x, u, cols.dc, s); break;
+            case 6: launch_dgemv64<6>(g, x, u, cols.dc, s); break;
+            default: launch_dgemv64<8>(g, x, u, cols.dc, s); break;
         }
     } else {
         dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));

@@ -427,7 +427,8 @@ inline cudaError_t launch_group_mf(const float4 *atoms, const float4 *atoms_p, i
     };
     // Four groups need a stage each.  Blocks of more than 256 real columns have fewer (or no
     // spare one): all 16 warps on one stage then (40000 atoms x 256 columns: 2.49 ms with four
-    // groups, 2.63 with one; x 384: 3.28 and 3.23; x 32: 1.53 and 1.90).
+    // groups, 2.63 with one; x 384: 3.28 and 3.23; x 32: 1.53 and 1.90).  Of a tube's 40000 atoms, with the
+    // ring cut to four stages: x 96 1.87 ms, x 128 1.89, x 192 1.95, x 256 1.96.
     static std::atomic<uint64_t> set_grouped{0}, set_one{0};
     constexpr int WPS = 16 / MF_GROUPS;
     const cudaError_t e = plan.groups == MF_GROUPS ? run(k_gemm3_mf<WPS, MF_GROUPS>, set_grouped, mf_threads(WPS, MF_GROUPS))

@@ -151,9 +151,10 @@ struct DStores {
     }
 };
 
-// D by 64 x 64 tiles of the upper triangle, one block each: D_ji has the same bits as D_ij (the
-// squares and sums of Eq. 3 are the same), so a tile's entries are computed once and written twice,
-// the second time transposed through shared memory.  Bound by the FP64 pipe (about 30 operations an
+// D by 64 x 64 tiles of the upper triangle, one block each: D_ji is D_ij (Eq. 3), so a tile's entries
+// are computed once and written twice, the second time transposed through shared memory.  (Computed
+// apart they have the same bits for equal widths; for others the fused sum of the widths' squares
+// may round differently.)  Bound by the FP64 pipe (about 30 operations an
 // entry, 1.7 per clock per SM) until its writes: 10000 atoms into float pairs 3.10 ms, 5.15 with every
 // entry computed.  Tile t of the triangle, columns I = 0 .. J first.
 constexpr int BD_T = 64;
