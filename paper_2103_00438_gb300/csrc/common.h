@@ -231,6 +231,24 @@ struct DevBuf {
 // Counts kernel launches made by the library (wfq_kernel_launches).
 void note_launch();
 
+// Launch of a kernel whose blocks may be scheduled as the blocks of the kernel before it on the stream
+// leave.  Every thread of it calls wait_for_previous() before it reads or writes memory: that returns
+// once the kernel before has completed.
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Records start/end events around the launches made in its scope when timing is on.
 struct KScope {
     wfq_ctx *ctx;

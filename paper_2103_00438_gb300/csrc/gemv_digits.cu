@@ -132,7 +132,7 @@ __device__ __forceinline__ void read_terms(uint32_t base, int64_t (&hi)[C], int6
 
 template <int C, bool TILES>
 __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_constant__ CUtensorMap tm_x, const SymvParams sp) {
-    if (sp.sums.plain(C)) return;
+    const bool skip = sp.sums.plain(C);   // read while the block sets up
     const Params &p = sp.p;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem =
@@ -185,6 +185,11 @@ __global__ void __launch_bounds__(SV_THREADS, 1) k_gemv_digits(const __grid_cons
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (skip) {
+        if (warp == SV_TMA_WARP)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        return;
+    }
     const uint32_t smem_base = tc::smem_u32(smem);
 
     // position of a unit: row block a, column block J from 2 a, advanced in order
@@ -557,6 +562,7 @@ __global__ void __launch_bounds__(256) k_gemv_digits_finish(int64_t n, int C, in
                                                             unsigned long long *__restrict__ acc, int E,
                                                             const int *__restrict__ xexp, const VecSums sums,
                                                             const SymPartials sym, const double *ud, double *U) {
+    wait_for_previous();
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     const int c = blockIdx.y;
     if (i >= n) return;
@@ -666,8 +672,8 @@ int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, cudaStrea
 
 int gemv_digits_finish(const wfq_geom *g, int C, const GemvDigits &w, const SymPartials &sym, const double *ud, double *U,
                        int64_t si, int64_t sc, cudaStream_t s) {
-    k_gemv_digits_finish<<<dim3((unsigned)((g->n + 255) / 256), (unsigned)C), 256, 0, s>>>(
-        g->n, C, si, sc, w.acc, g->dexp_max, w.xexp, w.sums(), sym, ud, U);
+    WFQ_CUDA(launch_overlapped(k_gemv_digits_finish, dim3((unsigned)((g->n + 255) / 256), (unsigned)C), dim3(256), s, g->n, C,
+                               si, sc, w.acc, g->dexp_max, w.xexp, w.sums(), sym, ud, U));
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

@@ -96,7 +96,10 @@ __global__ void __launch_bounds__(GV_WARPS * 32, MINB) k_dgemv_df(int64_t n, int
                                                             const float *__restrict__ xh,
                                                             const float *__restrict__ xl, double *__restrict__ U,
                                                             const PlainIf pi) {
-    if (LOOP && !pi.runs(C)) return;
+    if (LOOP) {
+        wait_for_previous();
+        if (!pi.runs(C)) return;
+    }
     __shared__ __align__(16) float sxh[C][GV_CHUNK];
     __shared__ __align__(16) float sxl[C][GV_CHUNK];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -236,7 +239,10 @@ __global__ void __launch_bounds__(256, 2) k_dsymv_df(int64_t n, int64_t T, const
                                                      const float *__restrict__ xh, const float *__restrict__ xl,
                                                      float2 *__restrict__ rowpart, float2 *__restrict__ colpart,
                                                      const PlainIf pi) {
-    if (LOOP && !pi.runs(C)) return;
+    if (LOOP) {
+        wait_for_previous();
+        if (!pi.runs(C)) return;
+    }
     __shared__ __align__(16) float sxh[C][SY_T];
     __shared__ __align__(16) float sxl[C][SY_T];
     __shared__ float2 cred[16][SY_T * C];
@@ -364,40 +370,41 @@ void launch_dgemv_c(int cg, int tiling, int64_t n, int64_t ld, const float *Fh, 
 
 // The symmetric product of cg <= 4 vectors into its partial sums, in full or beside a digit-slice product.
 template <int C>
-void launch_dsymv(const wfq_geom *g, const float *xh, const float *xl, float2 *rowpart, float2 *colpart, const PlainIf &pi,
+cudaError_t launch_dsymv(const wfq_geom *g, const float *xh, const float *xl, float2 *rowpart, float2 *colpart, const PlainIf &pi,
                   cudaStream_t s) {
     const int ni = (int)g->sym_nitems;
-    if (pi.sums.vsum)
-        k_dsymv_df<C, true><<<std::min(ni, 2 * g->ctx->num_sms), 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh,
-                                                                               xl, rowpart, colpart, pi);
-    else
-        k_dsymv_df<C, false><<<ni, 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
     note_launch();
+    if (pi.sums.vsum)
+        return launch_overlapped(k_dsymv_df<C, true>, dim3((unsigned)std::min(ni, 2 * g->ctx->num_sms)), dim3(256), s, g->n,
+                                 g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
+    k_dsymv_df<C, false><<<ni, 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
+    return cudaGetLastError();
 }
-void launch_dsymv(const wfq_geom *g, int cg, const float *xh, const float *xl, float2 *rowpart, float2 *colpart,
+cudaError_t launch_dsymv(const wfq_geom *g, int cg, const float *xh, const float *xl, float2 *rowpart, float2 *colpart,
                   const PlainIf &pi, cudaStream_t s) {
     switch (cg) {
-        case 1: launch_dsymv<1>(g, xh, xl, rowpart, colpart, pi, s); break;
-        case 2: launch_dsymv<2>(g, xh, xl, rowpart, colpart, pi, s); break;
-        case 3: launch_dsymv<3>(g, xh, xl, rowpart, colpart, pi, s); break;
-        default: launch_dsymv<4>(g, xh, xl, rowpart, colpart, pi, s); break;
+        case 1: return launch_dsymv<1>(g, xh, xl, rowpart, colpart, pi, s);
+        case 2: return launch_dsymv<2>(g, xh, xl, rowpart, colpart, pi, s);
+        case 3: return launch_dsymv<3>(g, xh, xl, rowpart, colpart, pi, s);
+        default: return launch_dsymv<4>(g, xh, xl, rowpart, colpart, pi, s);
     }
 }
 
 // The double-float product from the planes beside a digit-slice product (runs where pi says so).
 template <int C>
-void launch_dgemv_beside(const wfq_geom *g, const float *xh, const float *xl, double *U, const PlainIf &pi, cudaStream_t s) {
+cudaError_t launch_dgemv_beside(const wfq_geom *g, const float *xh, const float *xl, double *U, const PlainIf &pi, cudaStream_t s) {
     const unsigned b = (unsigned)std::min<int64_t>((g->n + GV_WARPS - 1) / GV_WARPS, 3 * g->ctx->num_sms);
-    k_dgemv_df<C, true, 1, 4, 3, true><<<b, GV_WARPS * 32, 0, s>>>(g->n, g->ldf, g->Dfh, g->Dfl, nullptr, xh, xl, U, pi);
     note_launch();
+    return launch_overlapped(k_dgemv_df<C, true, 1, 4, 3, true>, dim3(b), dim3(GV_WARPS * 32), s, g->n, g->ldf, g->Dfh, g->Dfl,
+                             nullptr, xh, xl, U, pi);
 }
-void launch_dgemv_beside(const wfq_geom *g, int cg, const float *xh, const float *xl, double *U, const PlainIf &pi,
+cudaError_t launch_dgemv_beside(const wfq_geom *g, int cg, const float *xh, const float *xl, double *U, const PlainIf &pi,
                          cudaStream_t s) {
     switch (cg) {
-        case 1: launch_dgemv_beside<1>(g, xh, xl, U, pi, s); break;
-        case 2: launch_dgemv_beside<2>(g, xh, xl, U, pi, s); break;
-        case 3: launch_dgemv_beside<3>(g, xh, xl, U, pi, s); break;
-        default: launch_dgemv_beside<4>(g, xh, xl, U, pi, s); break;
+        case 1: return launch_dgemv_beside<1>(g, xh, xl, U, pi, s);
+        case 2: return launch_dgemv_beside<2>(g, xh, xl, U, pi, s);
+        case 3: return launch_dgemv_beside<3>(g, xh, xl, U, pi, s);
+        default: return launch_dgemv_beside<4>(g, xh, xl, U, pi, s);
     }
 }
 
@@ -1053,9 +1060,9 @@ struct Arnoldi {
                 KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, dbytes);
                 WFQ_TRY(gemv_digits_product(g, cg, w, s));
                 if (g->Dfh) {
-                    launch_dgemv_beside(g, cg, ph, pxl, pu, pi, s);
+                    WFQ_CUDA(launch_dgemv_beside(g, cg, ph, pxl, pu, pi, s));
                 } else {
-                    launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
+                    WFQ_CUDA(launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s));
                 }
                 WFQ_TRY(gemv_digits_finish(g, cg, w, partials(), nullptr, pu, 1, n, s));
             }
@@ -1076,7 +1083,7 @@ struct Arnoldi {
                 const int cg = std::min(4, C - d0);
                 const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
                 KScope ks(g->ctx, WFQ_KT_DGEMV_DF, s, dbytes);
-                launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, kAlways, s);
+                WFQ_CUDA(launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, kAlways, s));
                 k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, partials(), u + (int64_t)d0 * n);
                 note_launch();
             }
@@ -1199,9 +1206,9 @@ static int pairs_by_digits(const wfq_geom *g, int C, const double *x, double *u,
             const float *ph = xh.ptr + (int64_t)d0 * n, *pxl = xl.ptr + (int64_t)d0 * n;
             WFQ_TRY(gemv_digits_product(g, cg, w, s, err));
             if (sym) {
-                launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s);
+                WFQ_CUDA(launch_dsymv(g, cg, ph, pxl, rowpart.ptr, colpart.ptr, pi, s));
             } else {
-                launch_dgemv_beside(g, cg, ph, pxl, ud.ptr, pi, s);
+                WFQ_CUDA(launch_dgemv_beside(g, cg, ph, pxl, ud.ptr, pi, s));
             }
             const SymPartials sp{rowpart.ptr, colpart.ptr, g->sym_item_start, g->sym_nt};
             WFQ_TRY(gemv_digits_finish(g, cg, w, sp, ud.ptr, u + b0 + d0, C, 1, s));
@@ -1243,7 +1250,7 @@ int d_apply_pairs_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U
         WFQ_TRY(colpart.alloc(g->ctx, colpart_elems(g, std::min(C, 4)), s));
         for (int d0 = 0; d0 < C; d0 += 4) {
             const int cg = std::min(4, C - d0);
-            launch_dsymv(g, cg, xh.ptr + (int64_t)d0 * n, xl.ptr + (int64_t)d0 * n, rowpart.ptr, colpart.ptr, kAlways, s);
+            WFQ_CUDA(launch_dsymv(g, cg, xh.ptr + (int64_t)d0 * n, xl.ptr + (int64_t)d0 * n, rowpart.ptr, colpart.ptr, kAlways, s));
             k_dsymv_finish<<<nblk(n * cg), 256, 0, s>>>(n, cg, partials(), ud.ptr + (int64_t)d0 * n);
             note_launch();
         }
