@@ -9,6 +9,15 @@
 
 namespace wfq {
 
+// A plain product of 256-thread blocks: in full, or (cols) what a digit-slice product leaves, mostly nothing.
+template <class... P, class... A>
+static cudaError_t launch_plain(void (*kernel)(P...), dim3 grid, const DigitCols &cols, cudaStream_t s, A... args) {
+    note_launch();
+    if (cols.cmax) return launch_overlapped(kernel, grid, dim3(256), 0, s, args..., cols);
+    kernel<<<grid, 256, 0, s>>>(args..., cols);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ FP64 stored D: few columns
 
 // U[i][:] = sum_k D[i][k] X[k][:] for C real columns (C <= 8): each warp owns RW rows so
@@ -20,6 +29,7 @@ template <int C, int RW>
 __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restrict__ D,
                                                const double *__restrict__ X, double *__restrict__ U,
                                                const DigitCols cols) {
+    wait_for_previous();
     if (cols.cmax) {
         bool any = false;
 #pragma unroll
@@ -92,6 +102,7 @@ __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restri
 __global__ void __launch_bounds__(256) k_dgemm(int64_t n, int64_t C, const double *__restrict__ D,
                                                const double *__restrict__ X, double *__restrict__ U,
                                                const DigitCols cols) {
+    wait_for_previous();
     if (cols.cmax) {
         const int64_t c = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
         if (!__syncthreads_or(c < C && col_plain(cols, c, true))) return;
@@ -222,6 +233,7 @@ __global__ void __launch_bounds__(256) k_dgemm_df(int64_t n, int64_t C, const do
                                                   const float *__restrict__ Fh, const float *__restrict__ Fl,
                                                   int64_t ldf, const double *__restrict__ X, double *__restrict__ U,
                                                   const DigitCols cols) {
+    wait_for_previous();
     if (cols.cmax) {
         const int64_t c = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
         if (!__syncthreads_or(c < C && col_plain(cols, c, false))) return;
@@ -530,25 +542,19 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
     if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "double-float apply: too many rows");
     if (g->Dfh)
-        k_dgemm_df<true><<<grid, 256, 0, s>>>(n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u, cols.dc);
+        WFQ_CUDA(launch_plain(k_dgemm_df<true>, grid, cols.dc, s, n, C, nullptr, g->Dfh, g->Dfl, g->ldf, x, u));
     else
-        k_dgemm_df<false><<<grid, 256, 0, s>>>(n, C, g->D64, nullptr, nullptr, 0, x, u, cols.dc);
-    note_launch();
-    WFQ_CUDA(cudaGetLastError());
+        WFQ_CUDA(launch_plain(k_dgemm_df<false>, grid, cols.dc, s, n, C, g->D64, nullptr, nullptr, 0, x, u));
     return WFQ_OK;
 }
 
 template <int C>
-static void launch_dgemv64(const wfq_geom *g, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
+static cudaError_t launch_dgemv64(const wfq_geom *g, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
     const int64_t n = g->n, sms = g->ctx->num_sms;
-    const double *D = g->D64;
-    auto blocks = [&](int rw) { return (unsigned)(((n + rw - 1) / rw + 7) / 8); };
-    if (n >= 64 * sms)   // 16 warps an SM
-        k_dgemv<C, 4><<<blocks(4), 256, 0, s>>>(n, D, x, u, cols);
-    else if (n >= 32 * sms)
-        k_dgemv<C, 2><<<blocks(2), 256, 0, s>>>(n, D, x, u, cols);
-    else
-        k_dgemv<C, 1><<<blocks(1), 256, 0, s>>>(n, D, x, u, cols);
+    auto blocks = [&](int rw) { return dim3((unsigned)(((n + rw - 1) / rw + 7) / 8)); };
+    if (n >= 64 * sms) return launch_plain(k_dgemv<C, 4>, blocks(4), cols, s, n, g->D64, x, u);   // 16 warps an SM
+    if (n >= 32 * sms) return launch_plain(k_dgemv<C, 2>, blocks(2), cols, s, n, g->D64, x, u);
+    return launch_plain(k_dgemv<C, 1>, blocks(1), cols, s, n, g->D64, x, u);
 }
 
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
@@ -573,22 +579,22 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     }
     if (g->D64 && C <= 8) {
         switch (C) {
-            case 2: launch_dgemv64<2>(g, x, u, cols.dc, s); break;
-            case 4: launch_dgemv64<4>(g, x, u, cols.dc, s); break;
-            case 6: launch_dgemv64<6>(g, x, u, cols.dc, s); break;
-            default: launch_dgemv64<8>(g, x, u, cols.dc, s); break;
+            case 2: WFQ_CUDA(launch_dgemv64<2>(g, x, u, cols.dc, s)); break;
+            case 4: WFQ_CUDA(launch_dgemv64<4>(g, x, u, cols.dc, s)); break;
+            case 6: WFQ_CUDA(launch_dgemv64<6>(g, x, u, cols.dc, s)); break;
+            default: WFQ_CUDA(launch_dgemv64<8>(g, x, u, cols.dc, s)); break;
         }
     } else {
         dim3 grid((unsigned)((C + 63) / 64), (unsigned)((n + 63) / 64));
         if (grid.y > 65535u) return fail(WFQ_EUNSUPPORTED, "FP64 apply: too many rows");
         if (g->D64) {
-            k_dgemm<<<grid, 256, 0, s>>>(n, C, g->D64, x, u, cols.dc);
+            WFQ_CUDA(launch_plain(k_dgemm, grid, cols.dc, s, n, C, g->D64, x, u));
         } else {
             WFQ_TRY(require_wfq(g));
             k_dotf<<<grid, 256, 0, s>>>(n, C, g->atom64, g->eta, x, u);
+            note_launch();
         }
     }
-    note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;
 }

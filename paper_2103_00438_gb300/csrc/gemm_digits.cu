@@ -531,6 +531,7 @@ template <int SRC, DigitMode MODE>
 __global__ void __launch_bounds__(DG_THREADS, 1)
     k_gemm_digits(const __grid_constant__ CUtensorMap tm7, const __grid_constant__ CUtensorMap tm8, const DigitParams dp) {
     const DigitCols &cols = dp.cols;
+    if constexpr (MODE == DG_IF_EIGHT) wait_for_previous();
     bool mine = false, low = false;
     for (int64_t c = threadIdx.x; c < dp.C; c += DG_THREADS)
         if (col_state(cols, c) == COL_DIGITS) {
@@ -626,6 +627,7 @@ __global__ void __launch_bounds__(256) k_split_digits(int64_t n, int64_t npad, i
 __global__ void __launch_bounds__(256) k_digits_finish(int64_t n, int64_t C, const unsigned long long *__restrict__ acc,
                                                        const int *__restrict__ dexp, DigitCols cols, int unit,
                                                        double *__restrict__ U) {
+    wait_for_previous();
     const int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (e >= n * C) return;
     const int64_t i = e / C, c = e - i * C;
@@ -657,9 +659,13 @@ int launch_digits(const __half *planes, const DigitParams &dp, int64_t npad, int
     static std::atomic<uint64_t> smem_set{0};
     cudaError_t e = tc::allow_max_smem(k_gemm_digits<SRC, MODE>, smem_set);
     if (e == cudaSuccess) {
-        k_gemm_digits<SRC, MODE><<<(unsigned)grid, DG_THREADS, smem, s>>>(m7, m8, dp);
         note_launch();
-        e = cudaGetLastError();
+        if constexpr (MODE == DG_IF_EIGHT) {
+            e = launch_overlapped(k_gemm_digits<SRC, MODE>, dim3((unsigned)grid), dim3(DG_THREADS), smem, s, m7, m8, dp);
+        } else {
+            k_gemm_digits<SRC, MODE><<<(unsigned)grid, DG_THREADS, smem, s>>>(m7, m8, dp);
+            e = cudaGetLastError();
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -738,7 +744,8 @@ int digits_product(const wfq_geom *g, bool fp64, int64_t C, const double *X, dou
         WFQ_TRY(launch_double_float<SRC_PAIRS>(planes.ptr, dp, npad, grid, s));
     else
         WFQ_TRY(launch_double_float<SRC_FP64>(planes.ptr, dp, npad, grid, s));
-    k_digits_finish<<<(unsigned)((n * C + 255) / 256), 256, 0, s>>>(n, C, acc, g->dexp, cols.dc, pairs ? -35 : -36, U);
+    WFQ_CUDA(launch_overlapped(k_digits_finish, dim3((unsigned)((n * C + 255) / 256)), dim3(256), 0, s, n, C, acc, g->dexp,
+                               cols.dc, pairs ? -35 : -36, U));
     note_launch();
     WFQ_CUDA(cudaGetLastError());
     return WFQ_OK;

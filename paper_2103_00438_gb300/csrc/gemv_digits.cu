@@ -672,7 +672,7 @@ int gemv_digits_product(const wfq_geom *g, int C, const GemvDigits &w, cudaStrea
 
 int gemv_digits_finish(const wfq_geom *g, int C, const GemvDigits &w, const SymPartials &sym, const double *ud, double *U,
                        int64_t si, int64_t sc, cudaStream_t s) {
-    WFQ_CUDA(launch_overlapped(k_gemv_digits_finish, dim3((unsigned)((g->n + 255) / 256), (unsigned)C), dim3(256), s, g->n, C,
+    WFQ_CUDA(launch_overlapped(k_gemv_digits_finish, dim3((unsigned)((g->n + 255) / 256), (unsigned)C), dim3(256), 0, s, g->n, C,
                                si, sc, w.acc, g->dexp_max, w.xexp, w.sums(), sym, ud, U));
     note_launch();
     WFQ_CUDA(cudaGetLastError());

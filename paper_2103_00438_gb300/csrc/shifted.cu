@@ -375,7 +375,7 @@ cudaError_t launch_dsymv(const wfq_geom *g, const float *xh, const float *xl, fl
     const int ni = (int)g->sym_nitems;
     note_launch();
     if (pi.sums.vsum)
-        return launch_overlapped(k_dsymv_df<C, true>, dim3((unsigned)std::min(ni, 2 * g->ctx->num_sms)), dim3(256), s, g->n,
+        return launch_overlapped(k_dsymv_df<C, true>, dim3((unsigned)std::min(ni, 2 * g->ctx->num_sms)), dim3(256), 0, s, g->n,
                                  g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
     k_dsymv_df<C, false><<<ni, 256, 0, s>>>(g->n, g->sym_nt, g->Dsym, g->sym_items, ni, xh, xl, rowpart, colpart, pi);
     return cudaGetLastError();
@@ -395,7 +395,7 @@ template <int C>
 cudaError_t launch_dgemv_beside(const wfq_geom *g, const float *xh, const float *xl, double *U, const PlainIf &pi, cudaStream_t s) {
     const unsigned b = (unsigned)std::min<int64_t>((g->n + GV_WARPS - 1) / GV_WARPS, 3 * g->ctx->num_sms);
     note_launch();
-    return launch_overlapped(k_dgemv_df<C, true, 1, 4, 3, true>, dim3(b), dim3(GV_WARPS * 32), s, g->n, g->ldf, g->Dfh, g->Dfl,
+    return launch_overlapped(k_dgemv_df<C, true, 1, 4, 3, true>, dim3(b), dim3(GV_WARPS * 32), 0, s, g->n, g->ldf, g->Dfh, g->Dfl,
                              nullptr, xh, xl, U, pi);
 }
 cudaError_t launch_dgemv_beside(const wfq_geom *g, int cg, const float *xh, const float *xl, double *U, const PlainIf &pi,
