@@ -314,7 +314,7 @@ int wfq_apply(wfq_geom *g, int64_t ncplx, const double *omega, const void *x, vo
  *     threads or devices' streams without ordering) race on it and must be
  *     serialised by the caller.
  *   - Needs WFQ_STORE_BF16X2 (else WFQ_EUNSUPPORTED).  No device memory is allocated
- *     or freed by this call. */
+ *     or freed by this call.  y is NaN if a kernel's bounded wait gave up. */
 int wfq_apply_mixed_noalloc(wfq_geom *g, int64_t ncplx, const double *omega, const void *x,
                             void *y, void *stream);
 

@@ -24,13 +24,13 @@ static cudaError_t launch_plain(void (*kernel)(P...), dim3 grid, const DigitCols
 // that every X element read from L2 serves RW D rows; D rows are read coalesced.  Bound by the
 // FP64 pipe (1.7 operations per clock per SM), so below 64 atoms per SM (9728 on 152), where 4 rows
 // a warp would leave SMs idle, a warp takes 1 or 2: 1014 atoms, C = 2: 9.5 us, 26.2 with 4 rows.  The order of
-// a row's sum does not depend on RW.  cols: as k_dgemm.
-template <int C, int RW>
+// a row's sum does not depend on RW.  REST: what a digit-slice product leaves (cols), as k_dgemm.
+template <int C, int RW, bool REST>
 __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restrict__ D,
                                                const double *__restrict__ X, double *__restrict__ U,
                                                const DigitCols cols) {
-    wait_for_previous();
-    if (cols.cmax) {
+    if constexpr (REST) {
+        wait_for_previous();
         bool any = false;
 #pragma unroll
         for (int c = 0; c < C; ++c) any = any || col_plain(cols, c, true);
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) k_dgemv(int64_t n, const double *__restri
             if (i0 + r < n)
 #pragma unroll
                 for (int c = 0; c < C; ++c)
-                    if (col_plain(cols, c, true)) U[(i0 + r) * C + c] = acc[r][c];
+                    if (!REST || col_plain(cols, c, true)) U[(i0 + r) * C + c] = acc[r][c];
     }
 }
 
@@ -548,13 +548,17 @@ int d_apply_df(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cuda
     return WFQ_OK;
 }
 
+template <int C, int RW>
+static cudaError_t launch_dgemv64(const wfq_geom *g, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
+    const dim3 blocks((unsigned)(((g->n + RW - 1) / RW + 7) / 8));
+    return cols.cmax ? launch_plain(k_dgemv<C, RW, true>, blocks, cols, s, g->n, g->D64, x, u)
+                     : launch_plain(k_dgemv<C, RW, false>, blocks, cols, s, g->n, g->D64, x, u);
+}
 template <int C>
 static cudaError_t launch_dgemv64(const wfq_geom *g, const double *x, double *u, const DigitCols &cols, cudaStream_t s) {
     const int64_t n = g->n, sms = g->ctx->num_sms;
-    auto blocks = [&](int rw) { return dim3((unsigned)(((n + rw - 1) / rw + 7) / 8)); };
-    if (n >= 64 * sms) return launch_plain(k_dgemv<C, 4>, blocks(4), cols, s, n, g->D64, x, u);   // 16 warps an SM
-    if (n >= 32 * sms) return launch_plain(k_dgemv<C, 2>, blocks(2), cols, s, n, g->D64, x, u);
-    return launch_plain(k_dgemv<C, 1>, blocks(1), cols, s, n, g->D64, x, u);
+    if (n >= 64 * sms) return launch_dgemv64<C, 4>(g, x, u, cols, s);   // 16 warps an SM
+    return n >= 32 * sms ? launch_dgemv64<C, 2>(g, x, u, cols, s) : launch_dgemv64<C, 1>(g, x, u, cols, s);
 }
 
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {

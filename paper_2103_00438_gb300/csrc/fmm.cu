@@ -959,8 +959,8 @@ int d_apply_fmm(const wfq_geom *g, int64_t cc, const float2 *X, float2 *U, cudaS
         const bool by_box = (double)f->nil * cols32 * P * P / 4096.0 / 70.0 < 0.1 * f->nslots * P * waves;
         if (by_box) {
             const size_t smb = sizeof(float) * 2 * MB_KC * (size_t)(rows + lpb);
-            if (smb > 48 * 1024)
-                WFQ_CUDA(cudaFuncSetAttribute(k_fmm_m2l_box, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smb));
+            if (smb > 48 * 1024)   // at most 67 KiB (256 nodes); the limit is the process's, never one launch's
+                WFQ_CUDA(cudaFuncSetAttribute(k_fmm_m2l_box, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024));
             k_fmm_m2l_box<<<gbox, 256, smb, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, rows, M.ptr, Lc.ptr);
         } else switch (best) {
             case 18: k_fmm_m2l<18><<<grid, th, sm, s>>>(fd, Cp, f->nm2l, noct, gr, lpb, M.ptr, Lc.ptr); break;
