@@ -1401,8 +1401,8 @@ int solve_gmres_shifted(wfq_geom *g, const SolveArgs &a, cudaStream_t s) {
         WFQ_TRY(ar.dmul(dvj));
         // w = (Kbar - P) D v_j, the first classical Gram-Schmidt pass's dots; each update of
         // the two passes forms the partial reductions of the next step (the second pass's
-        // dots, then the norm): 9 launches per step with the D product and the Givens step
-        // (12 with a launch per reduction).  Finishing the first pass's dots inside the first
+        // dots, then the norm): 9 launches per step with a D product of one kernel and the Givens
+        // step (12 with a launch per reduction).  Finishing the first pass's dots inside the first
         // update as well (8 launches) measured slower: 102.3-102.7 against 101.1 ms per
         // cnt20k step, the finish then a serial prologue of every update block.
         WFQ_TRY(ar.sparse(dvj, w));
