@@ -561,12 +561,19 @@ static cudaError_t launch_dgemv64(const wfq_geom *g, const double *x, double *u,
     return n >= 32 * sms ? launch_dgemv64<C, 2>(g, x, u, cols, s) : launch_dgemv64<C, 1>(g, x, u, cols, s);
 }
 
+// The FP64 GEMV takes about 2e-6 n^2 C us (FP64 pipe), the digit slices 45 + 4e-6 n^2 whatever
+// C is up to 32: from 2 columns and 4096 atoms on the latter (6000 atoms, 2 columns: 188 against
+// 435 us per apply; 10000 atoms, 4 columns: 463 against 2017).
+static bool few_by_digits(const wfq_geom *g, int64_t C) { return g->digits_ok && C >= 4 && g->n >= 4096; }
+
+bool apply_waits(const wfq_geom *g, int64_t cc, int prec) {
+    if (prec == WFQ_PREC_FMM) return false;
+    if (prec == WFQ_PREC_MIXED) return g->Dhi || !g->fmm || cc > 256;
+    return !(g->D64 && cc <= 4 && !few_by_digits(g, 2 * cc));
+}
+
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err) {
     const int64_t n = g->n, C = 2 * cc;
-    // The FP64 GEMV takes about 2e-6 n^2 C us (FP64 pipe), the digit slices 45 + 4e-6 n^2 whatever
-    // C is up to 32: from 2 columns and 4096 atoms on the latter (6000 atoms, 2 columns: 188 against
-    // 435 us per apply; 10000 atoms, 4 columns: 463 against 2017).
-    const bool few_by_digits = g->digits_ok && C >= 4 && n >= 4096;
     // no FP64 D but stored float pairs: their double-float product (2^-48 per product, on
     // the FP32 pipes and at 8 or 4 bytes per entry) instead of regenerating D in FP64
     if (!g->D64 && (g->Dfh || g->Dsym) && C <= 8) return d_apply_pairs_df(g, cc, X, U, s, err);
@@ -577,7 +584,7 @@ int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cu
     // eight exact digits on the tensor cores; dominated columns and those that are not finite in
     // plain FP64.  10k-atom sphere, 32 real columns: 0.38 ms against 20.5 ms for the FP64 kernel.
     // Without memory for them plain FP64 takes all, which needs none.
-    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits)) {
+    if (g->D64 && g->digits_ok && (C > 8 || few_by_digits(g, C))) {
         const int rc = digits_product(g, true, C, x, u, cols, s, err);
         if (rc != WFQ_OK && rc != WFQ_ENOMEM) return rc;
     }

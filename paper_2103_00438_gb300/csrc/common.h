@@ -297,6 +297,8 @@ int launch_polarizability(const wfq_geom *g, int64_t ncols, const double2 *q, do
 // complete); null: the context's, which the solvers read.  sparse_shift_*, the last step of an apply,
 // writes NaN when its err (null: none) is set.
 
+// Whether an apply may run a kernel with bounded waits (true for some that run none).
+bool apply_waits(const wfq_geom *g, int64_t cc, int prec);
 // U = D X in FP64 (stored FP64 D if present, else recomputed from the coordinates).
 int d_apply_fp64(const wfq_geom *g, int64_t cc, const double2 *X, double2 *U, cudaStream_t s, int *err = nullptr);
 
