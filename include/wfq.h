@@ -133,9 +133,9 @@ enum {
                               the error bound of double-float sums (~2^-48 relative per product)
                               or a smaller one.  Up to 4 columns on a stored FP64 D: as
                               WFQ_PREC_FP64.  Else from the stored FP64 D or FP32 pair planes by 7
-                              digits per operand as above (2^-50), omega-FQ geometries of 96 atoms
-                              and more; from the symmetric tiles by digits of the upper triangle
-                              (2^-53 of the bounds; from 1100 / min(4, real columns) atoms on, row
+                              digits per operand as above (2^-50; 8 where a column needs them),
+                              omega-FQ geometries of 96 atoms and more; from the symmetric tiles by
+                              digits of the upper triangle (2^-53 of the bounds; from 1100 / min(4, real columns) atoms on, row
                               bounds sqrt(2) eta_i within a factor of 8; 4 real columns at a time);
                               dominated columns and other blocks in double-float on the FP32 pipes,
                               D regenerated from the coordinates where it is not stored (near

@@ -13,7 +13,8 @@
 // for S = 7 the weights 4 to 6 of a chunk, as one float), and a chunk's sum is one integer, so
 // the result does not depend on how the work is split; what is left out is the digits past the
 // S-th (2^-62 or 2^-54 of the row's and column's bound) and the digit products with
-// a + b >= S.  S = 8 stands for FP64 products, S = 7 for double-float ones; columns whose sum of
+// a + b >= S.  S = 8 stands for FP64 products, S = 7 for double-float ones (8 for blocks with a
+// column that needs it; X is always split into 8); columns whose sum of
 // magnitudes is too small beside their largest entry for the bounds above to be below those of plain
 // sums are left to plain kernels (digit_cols.cuh).
 //
